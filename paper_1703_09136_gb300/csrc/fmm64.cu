@@ -389,6 +389,54 @@ hfmm_status down64_lists(hfmm_plan_s* P, int l, int nrhs, const cd* mult, cd* lo
     return HFMM_OK;
 }
 
+// M2M from the leaves up to lmin (leaf multipoles in place), with the spectra
+// of the diagonal levels: on the tensor cores (split64.cu) where the plan holds
+// the operators' slices, else one FP64 thread per output coefficient.
+static hfmm_status upward64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
+    const int L = P->L;
+    if (P->s6_ready) {
+        HFMM_TRY(split64_begin(P, st));
+        HFMM_TRY(split64_exponent(P, L, false, nrhs, st));
+    }
+    for (int l = L - 1; l >= P->lmin; --l) {
+        LevelInfo& lv = P->lev[l];
+        if (P->s6_ready) HFMM_TRY(split64_m2m(P, l, nrhs, st));
+        else {
+            m2m_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(
+                P->lev[l + 1].mult, lv.t_m2m, P->lev[l + 1].p, lv.p, nrhs, lv.mult);
+            ++P->launches;
+            HFMM_CUDA_TRY(cudaGetLastError());
+        }
+        if (lv.diag_logq) HFMM_TRY(diag_src(P, l, nrhs, st));
+    }
+    return HFMM_OK;
+}
+
+// L2L, free-space and reaction M2L of every level, lmin .. L.
+static hfmm_status downward64(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t st) {
+    const int L = P->L;
+    for (int l = P->lmin; l <= L; ++l) {
+        LevelInfo& lv = P->lev[l];
+        const bool has_parent = l > P->lmin;
+        const bool dg = lv.diag_logq > 0;   // translations in diagonal form after the L2L
+        if (P->s6_ready) HFMM_TRY(split64_down(P, l, nrhs, parts, st));
+        else {
+            downward_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(
+                P->leaf_begin, L, l, P->lmin, nrhs, lv.p, has_parent ? P->lev[l - 1].p : 0,
+                has_parent ? P->lev[l - 1].loc : nullptr, has_parent ? P->lev[l - 1].t_l2l : nullptr,
+                lv.mult, lv.nv && !dg ? lv.v_begin : nullptr, lv.v_src, lv.v_off, lv.t_free,
+                lv.nr && !dg ? lv.r_begin : nullptr, lv.r_src, lv.r_tab, lv.t_react, parts, lv.loc);
+            ++P->launches;
+            HFMM_CUDA_TRY(cudaGetLastError());
+        }
+        if (dg) {
+            HFMM_TRY(diag_m2l(P, l, nrhs, parts, st));
+            if (P->s6_ready && l < L) HFMM_TRY(split64_exponent(P, l, true, nrhs, st));
+        }
+    }
+    return HFMM_OK;
+}
+
 hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, bool adjoint,
                        cudaStream_t st) {
     const int64_t n = P->n;
@@ -425,31 +473,19 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
                 P->st_bytes[HFMM_STAGE_P2M] = C * n + 16.0 * n + C * lv.nbox * lv.ncoef;
             }
             tm.begin(HFMM_STAGE_M2M);
+            HFMM_TRY(upward64(P, nrhs, st));
             for (int l = L - 1; l >= P->lmin; --l) {
-                LevelInfo& lv = P->lev[l];
-                m2m_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(P->lev[l + 1].mult, lv.t_m2m, P->lev[l + 1].p, lv.p,
-                                                            nrhs, lv.mult);
-                ++P->launches;
-                HFMM_CUDA_TRY(cudaGetLastError());
-                if (lv.diag_logq) HFMM_TRY(diag_src(P, l, nrhs, st));
+                const LevelInfo& lv = P->lev[l];
                 P->st_flops[HFMM_STAGE_M2M] += MAC * 4.0 * lv.nbox * lv.ncoef * P->lev[l + 1].ncoef;
                 P->st_bytes[HFMM_STAGE_M2M] += C * (4.0 * lv.nbox * P->lev[l + 1].ncoef + lv.nbox * lv.ncoef);
             }
             tm.end(HFMM_STAGE_M2M);
             // step 3: downward pass
             tm.begin(HFMM_STAGE_DOWN);
+            HFMM_TRY(downward64(P, nrhs, parts, st));
             for (int l = P->lmin; l <= L; ++l) {
-                LevelInfo& lv = P->lev[l];
-                const bool has_parent = l > P->lmin;
-                const bool dg = lv.diag_logq > 0;   // translations in diagonal form after the L2L
-                downward_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(
-                    P->leaf_begin, L, l, P->lmin, nrhs, lv.p, has_parent ? P->lev[l - 1].p : 0,
-                    has_parent ? P->lev[l - 1].loc : nullptr, has_parent ? P->lev[l - 1].t_l2l : nullptr,
-                    lv.mult, lv.nv && !dg ? lv.v_begin : nullptr, lv.v_src, lv.v_off, lv.t_free,
-                    lv.nr && !dg ? lv.r_begin : nullptr, lv.r_src, lv.r_tab, lv.t_react, parts, lv.loc);
-                ++P->launches;
-                HFMM_CUDA_TRY(cudaGetLastError());
-                if (dg) HFMM_TRY(diag_m2l(P, l, nrhs, parts, st));
+                const LevelInfo& lv = P->lev[l];
+                const bool has_parent = l > P->lmin, dg = lv.diag_logq > 0;
                 double pairs = 0.0;
                 if (parts & HFMM_PART_FAR_FREE) pairs += (double)lv.nv;
                 if (parts & HFMM_PART_FAR_REACT) pairs += (double)lv.nr;
@@ -796,24 +832,8 @@ hfmm_status field_grad_fp64(hfmm_plan_s* P, int nrhs, cd* fx, cd* fy, cudaStream
         HFMM_CUDA_TRY(cudaGetLastError());
         if (lv.diag_logq) HFMM_TRY(diag_src(P, L, nrhs, st));
     }
-    for (int l = L - 1; l >= P->lmin; --l) {
-        LevelInfo& lv = P->lev[l];
-        m2m_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(P->lev[l + 1].mult, lv.t_m2m, P->lev[l + 1].p, lv.p, nrhs, lv.mult);
-        HFMM_CUDA_TRY(cudaGetLastError());
-        if (lv.diag_logq) HFMM_TRY(diag_src(P, l, nrhs, st));
-    }
-    for (int l = P->lmin; l <= L; ++l) {
-        LevelInfo& lv = P->lev[l];
-        const bool has_parent = l > P->lmin;
-        const bool dg = lv.diag_logq > 0;
-        downward_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(
-            P->leaf_begin, L, l, P->lmin, nrhs, lv.p, has_parent ? P->lev[l - 1].p : 0,
-            has_parent ? P->lev[l - 1].loc : nullptr, has_parent ? P->lev[l - 1].t_l2l : nullptr, lv.mult,
-            lv.nv && !dg ? lv.v_begin : nullptr, lv.v_src, lv.v_off, lv.t_free, lv.nr && !dg ? lv.r_begin : nullptr,
-            lv.r_src, lv.r_tab, lv.t_react, HFMM_PART_ALL, lv.loc);
-        HFMM_CUDA_TRY(cudaGetLastError());
-        if (dg) HFMM_TRY(diag_m2l(P, l, nrhs, HFMM_PART_ALL, st));
-    }
+    HFMM_TRY(upward64(P, nrhs, st));
+    HFMM_TRY(downward64(P, nrhs, HFMM_PART_ALL, st));
     {
         LevelInfo& lv = P->lev[L];
         const int chunk = pick_chunk_grad(lv.p);
@@ -849,6 +869,7 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
         HFMM_TRY(plan_alloc(P, (void**)&P->grad_buf, 5 * bytes));
         HFMM_TRY(build_direct_grad(P, st));
         HFMM_TRY(build_near64_grad(P, st));
+        HFMM_TRY(build_split64(P, st));
     }
     cd* ux = P->grad_buf;
     cd* uy = ux + (size_t)n * P->max_rhs;

@@ -99,6 +99,12 @@ struct LevelInfo {
     cd* diag_spec = nullptr;
     double diag_err = -1.0;
     int64_t nonempty = 0;         // non-empty boxes (set by the diagonal-form check)
+    // FP64 translations on the tensor cores (split64.cu): power-of-two scales
+    // log2 s(n), operator digit slices and the exponents of the operator families
+    // (lists, L2L into this level, M2M into this level)
+    const int* s6_sx = nullptr;
+    uint4 *s6_free = nullptr, *s6_react = nullptr, *s6_l2l = nullptr, *s6_m2m = nullptr;
+    int* s6_Eop = nullptr;
 };
 
 // Diagonal form: kept on a level when its weighted difference to the dense
@@ -223,6 +229,11 @@ struct hfmm_plan_s {
     float* tc_part = nullptr;       // partial sums of split launches (levels with few tiles)
     size_t tc_part_floats = 0;
 
+    // FP64 translations on the tensor cores (split64.cu): slices built, and the
+    // exponents of every level's expansions [multipoles, locals][level][max_rhs]
+    bool s6_ready = false;
+    int* s6_E = nullptr;
+
     // table quadrature: panel-count scale (hfmm_options.quad_scale) and the
     // node-doubling check's largest weighted relative difference and where
     // (level, dx, ysum; level -1 for a directly summed block)
@@ -306,6 +317,12 @@ void adaptive_destroy(AdaptiveTree* T);
 hfmm_status diag_src(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st);
 hfmm_status diag_m2l(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st);
 double diag_flops(const hfmm_plan_s* P, int l, int nrhs, int parts);
+// split64.cu
+hfmm_status build_split64(hfmm_plan_s* P, cudaStream_t st);
+hfmm_status split64_begin(hfmm_plan_s* P, cudaStream_t st);
+hfmm_status split64_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st);
+hfmm_status split64_m2m(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st);
+hfmm_status split64_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st);
 hfmm_status build_near64_grad(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, bool adjoint,
                        cudaStream_t st);

@@ -1,0 +1,699 @@
+// FP64 translations (M2M, L2L, free-space and reaction M2L) as exact-slice
+// products on the tensor cores.
+//
+// Every translation is a real matrix-vector product of length 2 nc (interleaved
+// real and imaginary parts).  The operand and the operator are written as
+// fixed-point numbers of 53 bits and cut into six signed base-512 digits,
+//     x = 2^(E - 53) sum_i d_i 512^(5 - i),  |d_i| <= 256,
+// (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms
+// 59, 2012): a digit is an f16 number, a digit product is below 2^16, and a sum
+// of up to four of them over 64 terms stays within 2^24, so f16 x f16 -> FP32
+// mma.sync accumulates them without rounding.  The 21 digit products
+// with i + j <= 5 are summed per order i + j: orders 0 .. 3 leave the tensor
+// core every 64 terms as integers (int32, over all sources of a target), the two
+// lowest orders stay in FP32 (their rounding is below 2^-60 of the largest
+// term).  What is dropped (orders >= 6) is below the FP64 rounding of the row.
+//
+// Scaling: expansions are scaled by powers of two close to
+// s_l(n) = min(1, (k R_l / 2)^n / n!) (a~_n = a_n / s, b~_n = b_n s), which makes
+// every operator entry O(1); the exponent E is one number per level, kind
+// of expansion and right-hand side (largest scaled coefficient, found by the
+// kernel that writes the expansions) and one per operator family.  The stored
+// expansions stay unscaled, so every other kernel reads them as before.  A level
+// that holds an infinity or a NaN makes every output of that right-hand side NaN.
+//
+// What bounds it: GB300's FP64 pipe runs at 1.0 TFLOP/s (a warp-wide FMA every 16
+// clocks per SM), mma.sync f16 at 600 TFLOP/s: 21 products leave 28 TFLOP/s.
+// Measured (one GB300, two layers, 262,144 points, one right-hand side): leaf
+// level (order 15, 430k free-space and 49k reaction translations, 3.8 GFLOP)
+// 5.73 -> 0.63 ms, all levels 12.0 -> 1.55 ms, M2M 0.72 -> 0.17 ms; the result
+// differs from the FP64 kernels' by 2e-13 (1e-14 at orders where those cancel
+// less), and both are equally far from the direct sum.
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "plan.cuh"
+
+namespace {
+
+constexpr int ND = 6;                    // digits
+constexpr int S6_MAXW = 8;               // m-tiles (warps) per CTA
+constexpr int S6_NONE = -(1 << 24);      // exponent of an all-zero level (or below)
+constexpr int S6_NAN = 1 << 20;          // exponent of a level with an infinity or a NaN
+constexpr double S6_MAX_BYTES = 16e9;    // operator slices of one plan
+
+// largest E with |v 2^shift| < 2^E (S6_NONE for zero)
+__device__ __forceinline__ int s6_exponent(double v, int shift) {
+    const long long b = __double_as_longlong(v);
+    const int e = (int)((b >> 52) & 2047);
+    if (e == 2047) return S6_NAN;
+    if (e == 0) return (b & 0xfffffffffffffll) ? -1021 + shift : S6_NONE;
+    return e - 1022 + shift;
+}
+
+// v 2^shift 2^(BITS - E) rounded to an integer plus the digit bias, |v 2^shift| < 2^E
+template <int BITS>
+__device__ __forceinline__ long long s6_fixed(double v, int shift, int E) {
+    const long long b = __double_as_longlong(v);
+    int e = (int)((b >> 52) & 2047);
+    unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
+    if (e) m |= 1ull << 52; else e = 1;
+    const int s = E - shift - e + 1075 - BITS;            // right shift, >= 0 for BITS = 53
+    if (s > 0) m = s > 54 ? 0ull : (m + (1ull << (s - 1))) >> s;
+    const long long x = b < 0 ? -(long long)m : (long long)m;
+    // + 256 sum_{i = 0 .. 4} 512^i: the low five fields then hold digit + 256
+    return x + 0x100804020100ll;
+}
+
+// field of digit i (0 = most significant), digit + 256 in [0, 512]
+__device__ __forceinline__ unsigned s6_field(long long xb, int i) {
+    return i == 0 ? (unsigned)((int)(xb >> 45) + 256) : (unsigned)(xb >> (9 * (ND - 1 - i))) & 511u;
+}
+
+// two digits as f16 (1024 + field as bits 0x6400 | field, minus 1280)
+__device__ __forceinline__ unsigned s6_half2(unsigned f0, unsigned f1) {
+    unsigned h = 0x64006400u + (f0 | (f1 << 16)), r;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x65006500u));
+    return r;
+}
+
+// ---------------------------------------------------------------------------
+// plan time: operator slices in the A-fragment order of mma.m16n8k16
+// ---------------------------------------------------------------------------
+enum { S6_FREE = 0, S6_REACT = 1, S6_L2L = 2, S6_M2M = 3 };
+
+struct S6Op {
+    const cd* T;
+    int kind, nop, po, pi;           // orders of the outputs and the inputs
+    const int* sxo;                  // log2 s of the output level, per |order|
+    const int* sxi;
+};
+
+__device__ __forceinline__ cd s6_entry(const S6Op& o, int op, int j, int m, int* sh) {
+    // output order j, input order m; *sh = -(in_shift + out_shift)
+    const int so = o.sxo[abs(j)], si = o.sxi[abs(m)];
+    if (o.kind == S6_FREE) {
+        *sh = so + si;
+        return o.T[(int64_t)op * (4 * o.po + 1) + (m - j) + 2 * o.po];
+    }
+    if (o.kind == S6_REACT) {
+        *sh = so + si;
+        cd v = o.T[(int64_t)op * (4 * o.po + 1) + (-m - j) + 2 * o.po];
+        return (m & 1) ? cneg(v) : v;
+    }
+    const int nmax = o.po + o.pi, w = 2 * nmax + 1;
+    *sh = o.kind == S6_L2L ? so - si : si - so;
+    return o.T[(int64_t)op * w + nmax + (m - j)];         // J_{n-m}(c - P) or J_{m-j}(P - c)
+}
+
+__global__ void s6_op_exponent_kernel(S6Op o, int* __restrict__ E) {
+    const int no = 2 * o.po + 1, ni = 2 * o.pi + 1;
+    const int64_t total = (int64_t)o.nop * no * ni;
+    int e = S6_NONE;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int op = (int)(i / (no * ni)), r = (int)(i % (no * ni));
+        int sh;
+        const cd v = s6_entry(o, op, r / ni - o.po, r % ni - o.pi, &sh);
+        e = max(e, max(s6_exponent(v.x, sh), s6_exponent(v.y, sh)));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) atomicMax(E, e);
+}
+
+// one thread per (op, m-tile, k-step, lane): its eight entries' digits
+__global__ void s6_op_slice_kernel(S6Op o, const int* __restrict__ Ep, uint4* __restrict__ out) {
+    const int no = 2 * o.po + 1, ni = 2 * o.pi + 1;
+    const int MT = (2 * no + 15) / 16, KS = (2 * ni + 15) / 16;
+    const int64_t total = (int64_t)o.nop * MT * KS * 32;
+    const int E = *Ep;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int lane = (int)(i & 31);
+        const int64_t blk = i >> 5;                        // (op, mt, ks)
+        const int ks = (int)(blk % KS), mt = (int)((blk / KS) % MT), op = (int)(blk / ((int64_t)KS * MT));
+        const int g = lane >> 2, t = lane & 3;
+        unsigned f[ND][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int row = 16 * mt + g + (q & 1) * 8, m = (16 * ks + (q >> 1) * 8) / 2 + t;   // columns 2m, 2m + 1
+            const int j = row >> 1;
+            long long x0 = 0x100804020100ll, x1 = 0x100804020100ll;
+            if (j < no && m < ni) {
+                int sh;
+                const cd v = s6_entry(o, op, j - o.po, m - o.pi, &sh);
+                // [[Re, -Im], [Im, Re]]
+                x0 = s6_fixed<52>((row & 1) ? v.y : v.x, sh, E);
+                x1 = s6_fixed<52>((row & 1) ? v.x : -v.y, sh, E);
+            }
+#pragma unroll
+            for (int d = 0; d < ND; ++d) f[d][q] = s6_half2(s6_field(x0, d), s6_field(x1, d));
+        }
+#pragma unroll
+        for (int d = 0; d < ND; ++d) out[(blk * ND + d) * 32 + lane] = make_uint4(f[d][0], f[d][1], f[d][2], f[d][3]);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// level exponents of expansions written by other kernels
+// ---------------------------------------------------------------------------
+__global__ void s6_exponent_kernel(const cd* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
+                                   int sign, int* __restrict__ E) {
+    const int nc = 2 * p + 1, r = blockIdx.y;
+    int e = S6_NONE;
+    const int64_t total = nbox * nc;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = i / nc;
+        const int m = (int)(i % nc) - p;
+        const cd v = a[(b * nrhs + r) * nc + m + p];
+        const int sh = sign * sx[abs(m)];
+        e = max(e, max(s6_exponent(v.x, sh), s6_exponent(v.y, sh)));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0 && e > S6_NONE) atomicMax(E + r, e);
+}
+
+// ---------------------------------------------------------------------------
+// the product kernel
+// ---------------------------------------------------------------------------
+// One operator family of a launch: sources, their order, scale signs, slices.
+struct S6Fam {
+    const cd* src;
+    const uint4* ops;
+    const int* Eop;                  // exponent of the family
+    const int* Esrc;                 // [nrhs] exponent of the source expansions
+    const int* sx;                   // log2 s of the source level
+    int p, sign;                     // source order; in_shift = sign * sx
+};
+
+struct S6Args {
+    int l, L, mode;                  // mode 0: M2M (targets 16 NT consecutive boxes), 1: downward
+    int nrhs, p;                     // output order
+    int tiles;
+    const int32_t* lb;               // leaf ranges (downward: empty targets are skipped)
+    S6Fam shift;                     // M2M or L2L (src null: none)
+    S6Fam list;                      // M2L sources (src null: none); ops = free-space operators
+    const uint4* rops;               // reaction operators (null: none)
+    int vlist, rlist, lstar;         // lists to run; first level whose bottom-row pair is admissible
+    int rows;                        // box rows covered by the launch (downward)
+    int accumulate;                  // add to the outputs
+    const int* sxo;
+    int osign;                       // out_shift = osign * sxo
+    cd* out;
+    int* Eout;                       // [nrhs], or null
+};
+
+__device__ __forceinline__ void s6_mma(float (&c)[4], const uint4& a, const uint2& b) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
+// A step of a tile: operator and the sources of its columns.
+struct S6Step {
+    int fam;                         // 0 shift, 1 list
+    const uint4* op;
+    int dx, sy, child;               // list: source (ix - dx, sy); shift: child position (mode 0)
+};
+
+// Steps of a downward tile (row iy, columns ix0, ix0 + 2, ..., ncol of them):
+// 0 the L2L, then the offsets (dx, dy), |dx|, |dy| <= 3 outside the 3 x 3
+// neighbourhood whose parents touch, then the reaction pairs (source row,
+// dx).  Returns false where a step does not exist for this tile.
+struct S6Tile {
+    int iy, ix0, ncol, n;            // n boxes per row
+    int nshift, nv, nr, rspan, ropt0;
+};
+
+__device__ __forceinline__ int s6_steps(const S6Args& A, S6Tile& T) {
+    T.nshift = A.shift.src ? (A.mode == 0 ? 4 : 1) : 0;
+    T.nv = T.nr = 0;
+    if (A.mode == 1) {
+        T.nv = A.vlist ? 36 : 0;      // 6 x 6 offsets of the parents' neighbourhood
+        if (A.rlist && T.iy < 2) {
+            T.ropt0 = (T.iy == 1 || A.l == A.lstar) ? 0 : 1;      // first admissible source row
+            const int opts = min(2, T.n) - T.ropt0;
+            T.rspan = T.n + 2 * (T.ncol - 1);
+            T.nr = opts > 0 ? opts * T.rspan : 0;
+        }
+    }
+    return T.nshift + T.nv + T.nr;
+}
+
+__device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s, int MT, int KSs, int KSl, S6Step& st) {
+    if (s < T.nshift) {
+        st.fam = 0;
+        st.child = A.mode == 0 ? s : (T.ix0 & 1) + 2 * (T.iy & 1);
+        st.op = A.shift.ops + (int64_t)st.child * MT * KSs * (ND * 32);
+        return true;
+    }
+    s -= T.nshift;
+    st.fam = 1;
+    if (s < T.nv) {
+        // source = parent's neighbourhood: sx = 2 (ixP + a) + u, a = -1 .. 1, u = 0, 1
+        const int ox = s % 6 - 2 - (T.ix0 & 1), oy = s / 6 - 2 - (T.iy & 1);   // source - target
+        if (abs(ox) < 2 && abs(oy) < 2) return false;
+        st.sy = T.iy + oy;
+        if (st.sy < 0 || st.sy >= T.n) return false;
+        st.dx = -ox;
+        if (T.ix0 + 2 * (T.ncol - 1) + ox < 0 || T.ix0 + ox >= T.n) return false;
+        st.op = A.list.ops + (int64_t)((st.dx + 3) * 7 + (-oy + 3)) * MT * KSl * (ND * 32);
+        return true;
+    }
+    s -= T.nv;
+    st.sy = T.ropt0 + s / T.rspan;
+    st.dx = T.ix0 + 2 * (T.ncol - 1) - s % T.rspan;              // sources from right to left cover [0, n)
+    const int dxm = T.n - 1;
+    if (abs(st.dx) > dxm) return false;
+    st.op = A.rops + (int64_t)((st.dx + dxm) * 3 + T.iy + st.sy) * MT * KSl * (ND * 32);
+    return true;
+}
+
+// A CTA owns 8 NT target boxes of one row and one column parity (they share every
+// operator) and up to eight m-tiles of 16 output rows, one per warp; it walks the
+// steps, slices the sources' 64-term chunks into shared memory (integer work on
+// the otherwise idle ALUs: slicing on the fly costs a tenth of the products and
+// saves a pass over memory) and multiplies them with the operator fragments, which
+// each warp reads from L2 as it needs them.  Levels with few tiles split a tile's
+// steps over a cluster of up to eight CTAs and add the partial sums in rank order
+// through distributed shared memory, so results do not depend on timing.
+template <int NT>
+__global__ void __launch_bounds__(S6_MAXW * 32, 1) s6_kernel(const __grid_constant__ S6Args A) {
+    // digits of the sources of one 64-term chunk, in B-fragment order, two buffers
+    __shared__ __align__(16) uint2 Bs[2][ND][4][NT][32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    const int S = (int)cluster_size(), rank = (int)cluster_rank();
+    const int tile = blockIdx.x / S, r = blockIdx.z;
+    const int no = 2 * A.p + 1, MT = (2 * no + 15) / 16;
+    const int mper = (MT + gridDim.y - 1) / gridDim.y;
+    const int mt = blockIdx.y * mper + wid;
+    const bool has_m = wid < mper && mt < MT;
+    constexpr int NC = 8 * NT;
+    S6Tile T;
+    int64_t box0 = 0;
+    T.n = 1 << A.l;
+    if (A.mode == 0) {
+        box0 = (int64_t)tile * NC;
+        T.iy = T.ix0 = 0;
+        T.ncol = NC;
+    } else {
+        const int per = max(1, T.n >> 1), G = (per + NC - 1) / NC, par = T.n > 1 ? 2 : 1;
+        T.iy = tile / (par * G);
+        const int c = (tile / G) % par, g = tile % G;
+        T.ix0 = 2 * NC * g + c;
+        T.ncol = min(NC, per - NC * g);
+    }
+    const int64_t nbox = (int64_t)1 << (2 * A.l);
+    auto target = [&](int col) -> int64_t {
+        if (A.mode == 0) return box0 + col < nbox ? box0 + col : -1;
+        if (col >= T.ncol) return -1;
+        const int64_t b = morton((uint32_t)(T.ix0 + 2 * col), (uint32_t)T.iy);
+        int32_t lo, hi;
+        box_range(A.lb, A.L, A.l, b, &lo, &hi);
+        return hi > lo ? b : -1;
+    };
+    {   // nothing to do where every target is empty (the same for all CTAs of the cluster)
+        bool any = false;
+        for (int c = 0; c < NC; ++c) any |= target(c) >= 0;
+        if (!any) return;
+    }
+    const int nsteps = s6_steps(A, T);
+    const int nis = A.shift.src ? 2 * A.shift.p + 1 : 0, nil = A.list.src ? 2 * A.list.p + 1 : 0;
+    const int KSs = (2 * nis + 15) / 16, KSl = (2 * nil + 15) / 16;
+
+    float acc[NT][ND][4];
+    int iacc[NT][4][4];
+    double dacc[NT][4];
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            dacc[t][v] = 0.0;
+#pragma unroll
+            for (int o = 0; o < 4; ++o) iacc[t][o][v] = 0;
+#pragma unroll
+            for (int o = 0; o < ND; ++o) acc[t][o][v] = 0.0f;
+        }
+    int Es = 0;                       // exponent of the family being staged
+    int since = 0;                    // chunks since the integers were last folded
+    // dacc += (digit sums) 2^(Esrc + Eop - 42): order o weighs 2^(9 (10 - o)) of 2^-105
+    auto fold = [&](int E) {
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const long long x = ((long long)iacc[t][0][v] << 27) + ((long long)iacc[t][1][v] << 18) +
+                                    ((long long)iacc[t][2][v] << 9) + (long long)iacc[t][3][v];
+                const float lo = acc[t][4][v] + acc[t][5][v] * (1.0f / 512.0f);
+                const double d = (double)x + (double)lo * (1.0 / 512.0);
+                dacc[t][v] += scalbn(d, E);
+                iacc[t][0][v] = iacc[t][1][v] = iacc[t][2][v] = iacc[t][3][v] = 0;
+                acc[t][4][v] = acc[t][5][v] = 0.0f;
+            }
+        since = 0;
+    };
+    int Ef[2] = {0, 0};               // fold exponents per family
+    bool bad = false;
+    if (A.shift.src) {
+        const int e = A.shift.Esrc[r];
+        bad |= e >= S6_NAN / 2;
+        Ef[0] = max(e, S6_NONE) + max(*A.shift.Eop, S6_NONE) - 42;
+    }
+    if (A.list.src) {
+        const int e = A.list.Esrc[r];
+        bad |= e >= S6_NAN / 2;
+        Ef[1] = max(e, S6_NONE) + max(*A.list.Eop, S6_NONE) - 42;
+    }
+
+    int buf = 0, prev_fam = -1;
+    for (int s = rank; s < nsteps; s += S) {
+        S6Step st;
+        if (!s6_step(A, T, s, MT, KSs, KSl, st)) continue;
+        const S6Fam& F = st.fam ? A.list : A.shift;
+        const int ni = st.fam ? nil : nis, KS = st.fam ? KSl : KSs;
+        if (prev_fam >= 0 && st.fam != prev_fam) fold(Ef[prev_fam]);
+        prev_fam = st.fam;
+        Es = F.Esrc[r];
+        const uint4* op = st.op + (int64_t)mt * KS * (ND * 32) + lane;
+        for (int k0 = 0; k0 < KS; k0 += 4) {
+            const int nk = min(4, KS - k0);
+            // stage: warp w < 4 slices columns w, w + 4, ...; lane = complex coefficient of the chunk
+            const int m = 8 * k0 + lane;
+            if (wid < 4) {
+                cd v[2 * NT];
+                const int sh = m < ni ? F.sign * F.sx[abs(m - F.p)] : 0;
+#pragma unroll
+                for (int u = 0; u < 2 * NT; ++u) {
+                    const int c = 4 * u + wid;
+                    int64_t b = -1;
+                    if (m < ni) {
+                        if (st.fam == 0) {
+                            if (A.mode == 0) b = box0 + c < nbox ? 4 * (box0 + c) + st.child : -1;
+                            else if (c < T.ncol) b = morton((uint32_t)((T.ix0 >> 1) + c), (uint32_t)(T.iy >> 1));
+                        } else if (c < T.ncol) {
+                            const int sx = T.ix0 + 2 * c - st.dx;
+                            if (sx >= 0 && sx < T.n) b = morton((uint32_t)sx, (uint32_t)st.sy);
+                        }
+                    }
+                    v[u] = b >= 0 ? __ldg(F.src + (b * A.nrhs + r) * ni + m) : cmk(0.0, 0.0);
+                }
+                const int kk = lane >> 3, reg = (lane >> 2) & 1;
+#pragma unroll
+                for (int u = 0; u < 2 * NT; ++u) {
+                    const int c = 4 * u + wid, fl = (c & 7) * 4 + (lane & 3);
+                    const long long xr = s6_fixed<53>(v[u].x, sh, Es), xi = s6_fixed<53>(v[u].y, sh, Es);
+#pragma unroll
+                    for (int d = 0; d < ND; ++d)
+                        reinterpret_cast<unsigned*>(&Bs[buf][d][kk][c >> 3][fl])[reg] =
+                            s6_half2(s6_field(xr, d), s6_field(xi, d));
+                }
+            }
+            __syncthreads();
+            if (has_m) {
+#pragma unroll
+                for (int t = 0; t < NT; ++t)
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) acc[t][o][v] = 0.0f;
+                for (int kk = 0; kk < nk; ++kk) {
+                    uint4 a[ND];
+#pragma unroll
+                    for (int d = 0; d < ND; ++d) a[d] = __ldg(op + (int64_t)((k0 + kk) * ND + d) * 32);
+#pragma unroll
+                    for (int t = 0; t < NT; ++t) {
+                        uint2 bb[ND];
+#pragma unroll
+                        for (int d = 0; d < ND; ++d) bb[d] = Bs[buf][d][kk][t][lane];
+#pragma unroll
+                        for (int i = 0; i < ND; ++i)
+#pragma unroll
+                            for (int j = 0; j < ND - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < NT; ++t)
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) iacc[t][o][v] += __float2int_rn(acc[t][o][v]);
+                if (++since == 120) fold(Ef[st.fam]);     // 120 x 2^24 < 2^31
+            }
+            buf ^= 1;
+        }
+    }
+    if (prev_fam >= 0) fold(Ef[prev_fam]);
+
+    // partial sums of the cluster's CTAs, added in rank order by rank 0
+    double* part = reinterpret_cast<double*>(&Bs[0][0][0][0][0]);   // [warp][NT][4][32]: 8 NT x 1 KB <= 24 KB NT / 2
+    if (S > 1) {
+        __syncthreads();
+        if (rank != 0 && has_m)
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) part[((wid * NT + t) * 4 + v) * 32 + lane] = dacc[t][v];
+        cluster_sync();
+        if (rank == 0 && has_m)
+            for (int q = 1; q < S; ++q) {
+                uint32_t local = (uint32_t)__cvta_generic_to_shared(part), remote;
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(q));
+#pragma unroll
+                for (int t = 0; t < NT; ++t)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        double x;
+                        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x)
+                                     : "r"(remote + (uint32_t)(((wid * NT + t) * 4 + v) * 32 + lane) * 8u));
+                        dacc[t][v] += x;
+                    }
+            }
+        cluster_sync();
+        if (rank != 0) return;
+    }
+    if (!has_m) return;
+    int e = S6_NONE;
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int row = 16 * mt + (lane >> 2) + (v >> 1) * 8, c = 8 * t + 2 * (lane & 3) + (v & 1);
+            const int64_t b = target(c);
+            if (row >= 2 * no || b < 0) continue;
+            const int sh = A.sxo[abs((row >> 1) - A.p)];
+            double* o = reinterpret_cast<double*>(A.out + (b * A.nrhs + r) * no) + row;
+            double x = bad ? nan : scalbn(dacc[t][v], A.osign * sh);
+            if (A.accumulate) x += *o;
+            *o = x;
+            e = max(e, s6_exponent(x, -A.osign * sh));
+        }
+    if (A.Eout) {
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0 && e > S6_NONE) atomicMax(A.Eout + r, e);
+    }
+}
+
+template <int NT>
+hfmm_status s6_launch(const S6Args& A, int tiles, int steps, cudaStream_t st) {
+    const int MT = (2 * (2 * A.p + 1) + 15) / 16;
+    const int gy = (MT + S6_MAXW - 1) / S6_MAXW, W = std::max(4, (MT + gy - 1) / gy);
+    // CTAs per tile: split the steps over a cluster while the launch leaves SMs idle
+    int S = 1;
+    while (S < 8 && (int64_t)tiles * gy * A.nrhs * S * 2 <= 4 * 152 && 2 * S <= steps) S *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(tiles * S), (unsigned)gy, (unsigned)A.nrhs);
+    cfg.blockDim = dim3(32 * W);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = S;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    HFMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, s6_kernel<NT>, A));
+    return HFMM_OK;
+}
+
+// Columns per tile: 16 where that still fills the GPU (each operator slice is
+// read once per tile), else 8.
+hfmm_status s6_run(S6Args& A, cudaStream_t st) {
+    const int64_t n = (int64_t)1 << A.l;
+    const int MT = (2 * (2 * A.p + 1) + 15) / 16, gy = (MT + S6_MAXW - 1) / S6_MAXW;
+    auto tiles = [&](int nc) -> int64_t {
+        if (A.mode == 0) return (n * n + nc - 1) / nc;
+        const int64_t per = std::max<int64_t>(1, n >> 1);
+        return (int64_t)A.rows * (n > 1 ? 2 : 1) * ((per + nc - 1) / nc);
+    };
+    const int steps = A.mode == 0 ? 4 : 1 + (A.vlist ? 27 : 0) + (A.rlist ? (int)std::min<int64_t>(n, 1 << 20) : 0);
+    const bool wide = (A.mode == 0 || (n >> 1) > 8) && tiles(16) * gy * A.nrhs >= 2 * 152;
+    A.tiles = (int)tiles(wide ? 16 : 8);
+    return wide ? s6_launch<2>(A, A.tiles, steps, st) : s6_launch<1>(A, A.tiles, steps, st);
+}
+
+S6Fam s6_fam(const cd* src, const LevelInfo& sl, const uint4* ops, const int* Eop, const int* Esrc,
+             int sign) {
+    S6Fam f{};
+    f.src = src;
+    f.ops = ops;
+    f.Eop = Eop;
+    f.Esrc = Esrc;
+    f.sx = sl.s6_sx;
+    f.p = sl.p;
+    f.sign = sign;
+    return f;
+}
+
+}  // namespace
+
+// Operator slices of every level (plan time, or a mixed plan's first gradient).
+// A plan whose slices would pass the byte budget keeps the FP64 kernels.
+hfmm_status build_split64(hfmm_plan_s* P, cudaStream_t st) {
+    if (P->s6_ready || P->ad) return HFMM_OK;
+    const int L = P->L;
+    int* E = nullptr;                                     // [level][3] families, then [kind][level][rhs] expansions
+    const size_t ne = (size_t)3 * (L + 1) + (size_t)2 * (L + 1) * P->max_rhs;
+    HFMM_TRY(plan_alloc(P, (void**)&E, sizeof(int) * ne));
+    P->s6_E = E + 3 * (L + 1);
+    HFMM_CUDA_TRY(cudaMemsetAsync(E, 0x80, sizeof(int) * ne, st));   // far below S6_NONE
+    std::vector<int> sx;
+    std::vector<size_t> off(L + 1, 0);
+    for (int l = 0; l <= L; ++l) {
+        const LevelInfo& lv = P->lev[l];
+        off[l] = sx.size();
+        const double kR = P->k * lv.h / std::sqrt(2.0);
+        for (int n = 0; n <= lv.p; ++n)
+            sx.push_back((int)std::lround(std::min(0.0, n * std::log(0.5 * kR) - std::lgamma(n + 1.0)) / std::log(2.0)));
+    }
+    int* dsx = nullptr;
+    HFMM_TRY(plan_alloc(P, (void**)&dsx, sizeof(int) * sx.size()));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(dsx, sx.data(), sizeof(int) * sx.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // sx is a local
+    auto bytes = [](int nop, int po, int pi) {
+        return 512.0 * ND * nop * ((2 * (2 * po + 1) + 15) / 16) * ((2 * (2 * pi + 1) + 15) / 16);
+    };
+    auto has_free = [&](const LevelInfo& lv) { return !lv.diag_logq && lv.t_free && lv.nv > 0; };
+    auto has_react = [&](const LevelInfo& lv) { return !lv.diag_logq && lv.t_react && lv.nr > 0; };
+    double used = 0.0;
+    for (int l = P->lmin; l <= L; ++l) {
+        const LevelInfo& lv = P->lev[l];
+        used += (has_free(lv) ? bytes(49, lv.p, lv.p) : 0.0) + (has_react(lv) ? bytes(lv.n_react_entries, lv.p, lv.p) : 0.0);
+        if (l > P->lmin) used += bytes(4, lv.p, P->lev[l - 1].p) + bytes(4, P->lev[l - 1].p, lv.p);
+    }
+    if (used > S6_MAX_BYTES) return HFMM_OK;
+    auto make = [&](const cd* T, int kind, int nop, const LevelInfo& o, const LevelInfo& i, int* Ep, uint4** out) -> hfmm_status {
+        S6Op op{T, kind, nop, o.p, i.p, o.s6_sx, i.s6_sx};
+        HFMM_TRY(plan_alloc(P, (void**)out, (size_t)bytes(nop, o.p, i.p)));
+        const int64_t total = (int64_t)(bytes(nop, o.p, i.p) / (16.0 * ND));
+        s6_op_slice_kernel<<<(unsigned)std::min<int64_t>((total + 127) / 128, 64 * 152), 128, 0, st>>>(op, Ep, *out);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        return HFMM_OK;
+    };
+    auto expo = [&](const cd* T, int kind, int nop, const LevelInfo& o, const LevelInfo& i, int* Ep) -> hfmm_status {
+        S6Op op{T, kind, nop, o.p, i.p, o.s6_sx, i.s6_sx};
+        const int64_t total = (int64_t)nop * o.ncoef * i.ncoef;
+        s6_op_exponent_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), 256, 0, st>>>(op, Ep);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        return HFMM_OK;
+    };
+    for (int l = 0; l <= L; ++l) P->lev[l].s6_sx = dsx + off[l];
+    for (int l = P->lmin; l <= L; ++l) {
+        LevelInfo& lv = P->lev[l];
+        lv.s6_Eop = E + 3 * l;
+        const bool fr = has_free(lv), re = has_react(lv);  // diagonal levels translate in diag.cu
+        if (fr) HFMM_TRY(expo(lv.t_free, S6_FREE, 49, lv, lv, lv.s6_Eop));
+        if (re) HFMM_TRY(expo(lv.t_react, S6_REACT, lv.n_react_entries, lv, lv, lv.s6_Eop));
+        if (fr) HFMM_TRY(make(lv.t_free, S6_FREE, 49, lv, lv, lv.s6_Eop, &lv.s6_free));
+        if (re) HFMM_TRY(make(lv.t_react, S6_REACT, lv.n_react_entries, lv, lv, lv.s6_Eop, &lv.s6_react));
+        if (l > P->lmin) {
+            HFMM_TRY(expo(P->lev[l - 1].t_l2l, S6_L2L, 4, lv, P->lev[l - 1], lv.s6_Eop + 1));
+            HFMM_TRY(make(P->lev[l - 1].t_l2l, S6_L2L, 4, lv, P->lev[l - 1], lv.s6_Eop + 1, &lv.s6_l2l));
+        }
+        if (l < L) {
+            HFMM_TRY(expo(lv.t_m2m, S6_M2M, 4, lv, P->lev[l + 1], lv.s6_Eop + 2));
+            HFMM_TRY(make(lv.t_m2m, S6_M2M, 4, lv, P->lev[l + 1], lv.s6_Eop + 2, &lv.s6_m2m));
+        }
+    }
+    P->table_bytes += used;
+    P->s6_ready = true;
+    return HFMM_OK;
+}
+
+// Start of a tree pass: no exponent is known.
+hfmm_status split64_begin(hfmm_plan_s* P, cudaStream_t st) {
+    HFMM_CUDA_TRY(cudaMemsetAsync(P->s6_E, 0x80, sizeof(int) * 2 * (P->L + 1) * P->max_rhs, st));
+    return HFMM_OK;
+}
+
+int* split64_exp(hfmm_plan_s* P, int l, bool loc) { return P->s6_E + ((size_t)(loc ? P->L + 1 : 0) + l) * P->max_rhs; }
+
+// Exponents of a level's expansions that another kernel wrote.
+hfmm_status split64_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[l];
+    const int64_t total = lv.nbox * lv.ncoef;
+    s6_exponent_kernel<<<dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs), 256, 0, st>>>(
+        loc ? lv.loc : lv.mult, lv.nbox, nrhs, lv.p, lv.s6_sx, loc ? 1 : -1, split64_exp(P, l, loc));
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+hfmm_status split64_m2m(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[l];
+    LevelInfo& ch = P->lev[l + 1];
+    S6Args A{};
+    A.l = l; A.L = P->L; A.mode = 0; A.nrhs = nrhs; A.p = lv.p;
+    A.shift = s6_fam(ch.mult, ch, lv.s6_m2m, lv.s6_Eop + 2, split64_exp(P, l + 1, false), -1);
+    A.sxo = lv.s6_sx;
+    A.osign = 1;
+    A.out = lv.mult;
+    A.Eout = split64_exp(P, l, false);
+    ++P->launches;
+    return s6_run(A, st);
+}
+
+// L2L and both M2L lists of level l into loc (diagonal levels: the L2L alone).
+hfmm_status split64_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st) {
+    LevelInfo& lv = P->lev[l];
+    const bool dg = lv.diag_logq > 0;
+    S6Args A{};
+    A.l = l; A.L = P->L; A.mode = 1; A.nrhs = nrhs; A.p = lv.p;
+    A.lb = P->leaf_begin;
+    if (l > P->lmin) {
+        LevelInfo& pa = P->lev[l - 1];
+        A.shift = s6_fam(pa.loc, pa, lv.s6_l2l, lv.s6_Eop + 1, split64_exp(P, l - 1, true), 1);
+    }
+    A.list = s6_fam(lv.mult, lv, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false), -1);
+    A.rops = lv.s6_react;
+    A.vlist = !dg && lv.nv > 0 && (parts & HFMM_PART_FAR_FREE);
+    const bool react = !dg && lv.nr > 0 && (parts & HFMM_PART_FAR_REACT);
+    A.lstar = P->lstar;
+    A.sxo = lv.s6_sx;
+    A.osign = -1;
+    A.out = lv.loc;
+    A.Eout = split64_exp(P, l, true);
+    A.rows = 1 << l;
+    // a bottom-row tile of a fine level has up to 2^(l + 1) reaction steps against
+    // 28 of the others: there they run as a launch of their own over the two rows
+    const bool apart = react && l >= 5;
+    A.rlist = react && !apart;
+    if (!A.vlist && !A.rlist) A.list.src = nullptr;
+    ++P->launches;
+    HFMM_TRY(s6_run(A, st));
+    if (apart) {
+        A.list = s6_fam(lv.mult, lv, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false), -1);
+        A.shift.src = nullptr;
+        A.vlist = 0;
+        A.rlist = 1;
+        A.rows = 2;
+        A.accumulate = 1;
+        ++P->launches;
+        HFMM_TRY(s6_run(A, st));
+    }
+    return HFMM_OK;
+}
