@@ -273,36 +273,12 @@ __global__ void __launch_bounds__(P2P_THREADS) p2p_kernel(const int32_t* lb, int
     }
 }
 
-// Directly summed reaction: one CTA per target leaf with direct pairs.
-__global__ void direct_react_kernel(const int32_t* lb, const int32_t* d_begin, const int32_t* d_src,
-                                    const int64_t* d_blk, const cd* vals, const cd* qs, int64_t n,
-                                    int nrhs, cd* ys) {
-    const int64_t b = blockIdx.x;
-    const int32_t e0 = d_begin[b], e1 = d_begin[b + 1];
-    if (e1 <= e0) return;
-    const int32_t tlo = lb[b], tn = lb[b + 1] - tlo;
-    const int items = nrhs * tn;
-    for (int it = threadIdx.x; it < items; it += blockDim.x) {
-        const int r = it / tn, i = it % tn;
-        cd acc = cmk(0.0, 0.0);
-        for (int32_t e = e0; e < e1; ++e) {
-            const int32_t s = d_src[e];
-            const int32_t slo = lb[s], sn = lb[s + 1] - slo;
-            const cd* G = vals + d_blk[e] + (int64_t)i * sn;
-            const cd* qr = qs + (int64_t)r * n + slo;
-            for (int j = 0; j < sn; ++j) cfma(acc, G[j], qr[j]);
-        }
-        cd* yy = ys + (int64_t)r * n + tlo + i;
-        *yy = cadd(*yy, acc);
-    }
-}
-
 // Near field from per-plan blocks (FP64 plans): for every target leaf T the
 // values (i/4) H0(k |x_t - x_s|) of all its U-list sources s (the 3 x 3
 // neighbourhood in dy, dx order, each leaf's points in order; 0 for s = t),
 // stored source-major, G[off[T] + j * n_T + i], so that the lanes (targets)
-// of a warp read consecutive values.  The plan computes each H0 once; an
-// apply streams the blocks.
+// of a warp read consecutive values.  The plan computes each H0 once and turns the
+// blocks into digit words; an apply streams them (leaf64.cu).
 __global__ void near64_fill_kernel(const int32_t* __restrict__ lb, int L, const double2* __restrict__ xs, double k,
                                    const int64_t* __restrict__ off, cd* __restrict__ G) {
     const int64_t b = blockIdx.x;
@@ -331,44 +307,6 @@ __global__ void near64_fill_kernel(const int32_t* __restrict__ lb, int L, const 
         }
 }
 
-// y[r][t] += sum over the U-list sources s of G[s][t] q[r][s]: a warp per
-// target leaf (four per CTA), lane = target (passes of 32).
-__global__ void __launch_bounds__(128) near64_kernel(const int32_t* __restrict__ lb, int L, int64_t nleaf,
-                                                     const int64_t* __restrict__ off, const cd* __restrict__ G,
-                                                     const cd* __restrict__ qs, int64_t n, int nrhs,
-                                                     cd* __restrict__ ys) {
-    const int64_t b = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (b >= nleaf) return;
-    const int lane = threadIdx.x & 31;
-    const int32_t tlo = lb[b], tn = lb[b + 1] - tlo;
-    if (tn <= 0) return;
-    const int m = 1 << L;
-    const int ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
-    const cd* Gb = G + off[b];
-    for (int r = 0; r < nrhs; ++r)
-        for (int i0 = 0; i0 < tn; i0 += 32) {
-            const int i = i0 + lane;
-            const bool live = i < tn;
-            cd acc = cmk(0.0, 0.0);
-            int64_t j = 0;
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int sx = ix + dx, sy = iy + dy;
-                    if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
-                    const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
-                    const int32_t slo = lb[s], shi = lb[s + 1];
-                    const cd* qr = qs + (int64_t)r * n;
-#pragma unroll 4
-                    for (int32_t js = slo; js < shi; ++js, ++j)
-                        if (live) cfma(acc, Gb[j * tn + i], qr[js]);
-                }
-            if (live) {
-                cd* yy = ys + (int64_t)r * n + tlo + i;
-                *yy = cadd(*yy, acc);
-            }
-        }
-}
-
 int pick_chunk(int p) {
     const int ncoef = 2 * p + 1;
     int c = (int)(40000 / (ncoef * 16 + (p + 1) * 8));
@@ -389,19 +327,36 @@ hfmm_status down64_lists(hfmm_plan_s* P, int l, int nrhs, const cd* mult, cd* lo
     return HFMM_OK;
 }
 
+// P2M of the sorted strengths, from the plan's bases where it holds them.
+static hfmm_status leaves64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[P->L];
+    if (P->s6_ready) HFMM_TRY(split64_begin(P, st));
+    if (P->basis64) HFMM_TRY(launch_p2m64(P, nrhs, st));
+    else {
+        const int chunk = pick_chunk(lv.p);
+        const size_t sm = (size_t)chunk * ((2 * lv.p + 1) * sizeof(cd) + (lv.p + 1) * sizeof(double));
+        p2m_kernel<<<(unsigned)lv.nbox, TB, sm, st>>>(P->leaf_begin, P->xy_sorted, P->q_sorted, P->n, nrhs, P->x0, P->y0,
+                                                     lv.h, P->L, P->k, lv.p, chunk, lv.mult);
+        ++P->launches;
+        HFMM_CUDA_TRY(cudaGetLastError());
+        if (P->s6_ready) HFMM_TRY(split64_exponent(P, P->L, false, nrhs, st));
+    }
+    if (P->s6_ready) HFMM_TRY(split64_slice(P, P->L, false, nrhs, st));
+    if (lv.diag_logq) HFMM_TRY(diag_src(P, P->L, nrhs, st));
+    return HFMM_OK;
+}
+
 // M2M from the leaves up to lmin (leaf multipoles in place), with the spectra
 // of the diagonal levels: on the tensor cores (split64.cu) where the plan holds
 // the operators' slices, else one FP64 thread per output coefficient.
 static hfmm_status upward64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
     const int L = P->L;
-    if (P->s6_ready) {
-        HFMM_TRY(split64_begin(P, st));
-        HFMM_TRY(split64_exponent(P, L, false, nrhs, st));
-    }
     for (int l = L - 1; l >= P->lmin; --l) {
         LevelInfo& lv = P->lev[l];
-        if (P->s6_ready) HFMM_TRY(split64_m2m(P, l, nrhs, st));
-        else {
+        if (P->s6_ready) {
+            HFMM_TRY(split64_m2m(P, l, nrhs, st));
+            if (l > P->lmin || !lv.diag_logq) HFMM_TRY(split64_slice(P, l, false, nrhs, st));
+        } else {
             m2m_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(
                 P->lev[l + 1].mult, lv.t_m2m, P->lev[l + 1].p, lv.p, nrhs, lv.mult);
             ++P->launches;
@@ -433,6 +388,7 @@ static hfmm_status downward64(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t 
             HFMM_TRY(diag_m2l(P, l, nrhs, parts, st));
             if (P->s6_ready && l < L) HFMM_TRY(split64_exponent(P, l, true, nrhs, st));
         }
+        if (P->s6_ready && l < L) HFMM_TRY(split64_slice(P, l, true, nrhs, st));
     }
     return HFMM_OK;
 }
@@ -450,24 +406,21 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
     tm.begin(HFMM_STAGE_GATHER);
     gather_q<<<nb, 256, 0, st>>>(q, P->perm, n, nrhs, adjoint, P->q_sorted);
     ++P->launches;
-    HFMM_CUDA_TRY(cudaMemsetAsync(P->y_sorted, 0, sizeof(cd) * n * nrhs, st));
+    const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0, near = (parts & HFMM_PART_NEAR_FREE) != 0;
+    // sums that leaf64_kernel does not make itself go through y_sorted
+    const bool l2p_here = far && P->basis64, near_here = near && P->near64_vals;
+    const bool extra = P->ad || (far && !l2p_here) || (near && !near_here);
+    if (extra) HFMM_CUDA_TRY(cudaMemsetAsync(P->y_sorted, 0, sizeof(cd) * n * nrhs, st));
     tm.end(HFMM_STAGE_GATHER);
     P->st_bytes[HFMM_STAGE_GATHER] = 2.0 * C * n + 8.0 * n;
     if (P->ad) HFMM_TRY(apply_adaptive(P, nrhs, parts, st));
     else {
-        const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0;
         if (far) {
             // step 2: upward pass
             {
                 LevelInfo& lv = P->lev[L];
-                const int chunk = pick_chunk(lv.p);
-                const size_t sm = (size_t)chunk * ((2 * lv.p + 1) * sizeof(cd) + (lv.p + 1) * sizeof(double));
                 tm.begin(HFMM_STAGE_P2M);
-                p2m_kernel<<<(unsigned)lv.nbox, TB, sm, st>>>(P->leaf_begin, P->xy_sorted, P->q_sorted, n, nrhs,
-                                                             P->x0, P->y0, lv.h, L, P->k, lv.p, chunk, lv.mult);
-                ++P->launches;
-                HFMM_CUDA_TRY(cudaGetLastError());
-                if (lv.diag_logq) HFMM_TRY(diag_src(P, L, nrhs, st));
+                HFMM_TRY(leaves64(P, nrhs, st));
                 tm.end(HFMM_STAGE_P2M);
                 P->st_flops[HFMM_STAGE_P2M] = MAC * n * lv.ncoef;
                 P->st_bytes[HFMM_STAGE_P2M] = C * n + 16.0 * n + C * lv.nbox * lv.ncoef;
@@ -496,48 +449,47 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
                                                 (has_parent ? C * P->lev[l - 1].nbox * P->lev[l - 1].ncoef : 0.0);
             }
             tm.end(HFMM_STAGE_DOWN);
-            // step 4: local expansions at the targets
+            // step 4: local expansions at the targets (with step 5 where the plan holds the bases)
             {
                 LevelInfo& lv = P->lev[L];
-                const int chunk = pick_chunk(lv.p);
-                const size_t sm = (size_t)chunk * ((2 * lv.p + 1) * sizeof(cd) + (lv.p + 1) * sizeof(double));
-                tm.begin(HFMM_STAGE_L2P);
-                l2p_kernel<<<(unsigned)lv.nbox, TB, sm, st>>>(P->leaf_begin, P->xy_sorted, lv.loc, n, nrhs, P->x0,
-                                                             P->y0, lv.h, P->k, lv.p, chunk, P->y_sorted);
-                ++P->launches;
-                HFMM_CUDA_TRY(cudaGetLastError());
-                tm.end(HFMM_STAGE_L2P);
+                if (!l2p_here) {
+                    const int chunk = pick_chunk(lv.p);
+                    const size_t sm = (size_t)chunk * ((2 * lv.p + 1) * sizeof(cd) + (lv.p + 1) * sizeof(double));
+                    tm.begin(HFMM_STAGE_L2P);
+                    l2p_kernel<<<(unsigned)lv.nbox, TB, sm, st>>>(P->leaf_begin, P->xy_sorted, lv.loc, n, nrhs, P->x0,
+                                                                 P->y0, lv.h, P->k, lv.p, chunk, P->y_sorted);
+                    ++P->launches;
+                    HFMM_CUDA_TRY(cudaGetLastError());
+                    tm.end(HFMM_STAGE_L2P);
+                }
                 P->st_flops[HFMM_STAGE_L2P] = MAC * n * lv.ncoef;
                 P->st_bytes[HFMM_STAGE_L2P] = C * lv.nbox * lv.ncoef + 16.0 * n + 2.0 * C * n;
             }
         }
         // step 5: direct interactions
-        if (parts & HFMM_PART_NEAR_FREE) {
-            tm.begin(HFMM_STAGE_P2P);
-            if (P->near64_vals)
-                near64_kernel<<<(unsigned)ceil_div(P->lev[L].nbox, 4), 128, 0, st>>>(
-                    P->leaf_begin, L, P->lev[L].nbox, P->near64_off, P->near64_vals, P->q_sorted, n, nrhs, P->y_sorted);
-            else
-                p2p_kernel<<<(unsigned)P->lev[L].nbox, P2P_THREADS, 0, st>>>(P->leaf_begin, L, P->xy_sorted,
-                                                                             P->q_sorted, n, nrhs, P->k, P->y_sorted);
+        const bool direct = (parts & HFMM_PART_NEAR_REACT) && P->nd > 0;
+        tm.begin(HFMM_STAGE_P2P);
+        if (near && !near_here) {
+            p2p_kernel<<<(unsigned)P->lev[L].nbox, P2P_THREADS, 0, st>>>(P->leaf_begin, L, P->xy_sorted, P->q_sorted, n,
+                                                                         nrhs, P->k, P->y_sorted);
             ++P->launches;
             HFMM_CUDA_TRY(cudaGetLastError());
-            tm.end(HFMM_STAGE_P2P);
+        }
+        HFMM_TRY(launch_leaf64(P, nrhs, near_here, l2p_here, direct, extra ? P->y_sorted : nullptr, adjoint, y, st));
+        tm.end(HFMM_STAGE_P2P);
+        if (near) {
             P->st_flops[HFMM_STAGE_P2P] = MAC * (double)P->p2p_point_pairs;
             P->st_bytes[HFMM_STAGE_P2P] = C * n + 2.0 * C * n + 16.0 * n +
                                           (P->near64_vals ? 16.0 * (double)P->p2p_point_pairs : 0.0);
         }
-        if ((parts & HFMM_PART_NEAR_REACT) && P->nd > 0) {
-            tm.begin(HFMM_STAGE_DIRECT);
-            direct_react_kernel<<<(unsigned)P->lev[L].nbox, TB, 0, st>>>(P->leaf_begin, P->d_begin, P->d_src,
-                                                                         P->d_blk, P->d_vals, P->q_sorted, n,
-                                                                         nrhs, P->y_sorted);
-            ++P->launches;
-            HFMM_CUDA_TRY(cudaGetLastError());
-            tm.end(HFMM_STAGE_DIRECT);
+        if (direct) {
             P->st_flops[HFMM_STAGE_DIRECT] = MAC * (double)P->nd_vals;
             P->st_bytes[HFMM_STAGE_DIRECT] = 16.0 * (double)P->nd_vals;
         }
+    }
+    if (!P->ad) {                          // the leaf kernel wrote the caller's order
+        P->last_stream = st;
+        return HFMM_OK;
     }
     tm.begin(HFMM_STAGE_SCATTER);
     scatter_y<<<nb, 256, 0, st>>>(P->y_sorted, P->perm, n, nrhs, adjoint, y);
@@ -823,15 +775,7 @@ hfmm_status field_grad_fp64(hfmm_plan_s* P, int nrhs, cd* fx, cd* fy, cudaStream
     const int L = P->L;
     HFMM_CUDA_TRY(cudaMemsetAsync(fx, 0, sizeof(cd) * n * nrhs, st));
     HFMM_CUDA_TRY(cudaMemsetAsync(fy, 0, sizeof(cd) * n * nrhs, st));
-    {
-        LevelInfo& lv = P->lev[L];
-        const int chunk = pick_chunk(lv.p);
-        const size_t sm = (size_t)chunk * ((2 * lv.p + 1) * sizeof(cd) + (lv.p + 1) * sizeof(double));
-        p2m_kernel<<<(unsigned)lv.nbox, TB, sm, st>>>(P->leaf_begin, P->xy_sorted, P->q_sorted, n, nrhs, P->x0,
-                                                     P->y0, lv.h, L, P->k, lv.p, chunk, lv.mult);
-        HFMM_CUDA_TRY(cudaGetLastError());
-        if (lv.diag_logq) HFMM_TRY(diag_src(P, L, nrhs, st));
-    }
+    HFMM_TRY(leaves64(P, nrhs, st));
     HFMM_TRY(upward64(P, nrhs, st));
     HFMM_TRY(downward64(P, nrhs, HFMM_PART_ALL, st));
     {
@@ -870,6 +814,7 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
         HFMM_TRY(build_direct_grad(P, st));
         HFMM_TRY(build_near64_grad(P, st));
         HFMM_TRY(build_split64(P, st));
+        HFMM_TRY(build_basis64(P, st));
     }
     cd* ux = P->grad_buf;
     cd* uy = ux + (size_t)n * P->max_rhs;
@@ -963,6 +908,7 @@ hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st) {
                 }
         }
         off[b + 1] = off[b] + tn * ns;
+        P->leaf_max = std::max(P->leaf_max, (int)tn);
     }
     const double bytes = 16.0 * (double)off[nleaf];
     if (bytes > NEAR64_MAX_BYTES) return HFMM_OK;
@@ -973,6 +919,12 @@ hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st) {
                                                         P->near64_vals);
     HFMM_CUDA_TRY(cudaGetLastError());
     P->table_bytes += bytes;
+    // coincident points (infinite entries) have no digit form: the apply then
+    // evaluates H0 per pair
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, sizeof(int)));
+    bool finite = true;
+    HFMM_TRY(near64_to_fixed(P->near64_vals, off[nleaf], P->near64_E, &finite, st));
+    if (!finite) P->near64_vals = nullptr;
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));
     return HFMM_OK;
 }

@@ -1,0 +1,528 @@
+// FP64 leaf passes of the uniform tree: P2M from plan-time bases, and one kernel
+// for everything a target sums at the end (near field, L2P, directly summed
+// reaction, result in the caller's order).
+//
+// Bases.  B_m(x) = J_m(k rho) e^{-i m theta} of every point about its leaf's centre,
+// m = 0 .. p + 1, is computed once per plan: J_{-m} = (-1)^m J_m makes the
+// negative orders conjugates, so one product with B_m serves both m and -m (half
+// the FP64 work and half the bytes of a full basis); order p + 1 serves the
+// position gradient.
+//
+// Near field.  The plan stores (i/4) H0 of every U-list pair (near64_vals, fmm64.cu) as
+// 55-bit fixed-point numbers with one exponent, each as seven base-256 digits: byte
+// pairs (re, re, im, im) of two digits per 32-bit word, so that one AND or byte
+// permute gives a digit of both parts as two f16 (the leading digit is signed; the
+// others are the bytes themselves, read as f16 subnormals u 2^-24).  A leaf's
+// strengths are cut into seven signed digits, which fill seven of the eight
+// columns of an mma.sync m16n8k16: 7 MMAs per real product (2 x 7 for complex)
+// give all 49 digit products of 16 targets x 8 sources, exact in FP32 over 32
+// k-steps (255 x 128 x 512 < 2^24).
+//
+// What bounds it: FP64 instructions (64 clocks each on a sub-partition's pipe) and
+// the latency of the block words.  Measured (one GB300, two layers, 262,144 points,
+// one right-hand side): P2M 745 -> 51 us, near field + L2P + scatter 1370 -> 285 us
+// (the blocks are 0.6 GB, 90 us of HBM; digits cut from 53-bit words with shifts
+// instead of byte permutes took 333 us, FP64 partial sums per lane 453 us, loads
+// without the ring 308 us); 1600 points: P2M 67 -> 11 us, the rest 360 -> 45 us.
+#include <algorithm>
+#include <cmath>
+
+#include "bessel.cuh"
+#include "plan.cuh"
+#include "split64.cuh"
+
+namespace {
+
+constexpr double BASIS64_MAX_BYTES = 8e9;
+
+// B[i][m] = J_m(k rho) e^{-i m theta}, m = 0 .. nb - 1 (one CTA per leaf, a thread per point)
+__global__ void basis64_kernel(const int32_t* __restrict__ lb, const double2* __restrict__ xs, double x0, double y0,
+                               double h, double k, int nb, cd* __restrict__ basis) {
+    extern __shared__ double jt[];
+    const int64_t b = blockIdx.x;
+    const double cx = x0 + (morton_x((uint32_t)b) + 0.5) * h, cy = y0 + (morton_y((uint32_t)b) + 0.5) * h;
+    double* J = jt + (size_t)threadIdx.x * nb;
+    for (int32_t i = lb[b] + threadIdx.x; i < lb[b + 1]; i += blockDim.x) {
+        const double dx = xs[i].x - cx, dy = xs[i].y - cy;
+        bessel_j_seq(k * hypot(dx, dy), nb - 1, J);
+        const cd e1 = cexpi(-atan2(dy, dx));
+        cd e = cmk(1.0, 0.0);
+        cd* B = basis + (int64_t)i * nb;
+        for (int m = 0; m < nb; ++m) {
+            B[m] = cscale(e, J[m]);
+            e = cmul(e, e1);
+        }
+    }
+}
+
+// P2M, a thread per (leaf, right-hand side, m >= 0): with q = (a, b), B = (u, v) the four
+// real sums of a u, b v, a v, b u give alpha_m = sum q B_m and
+// alpha_{-m} = (-1)^m sum q conj(B_m).  Also the level's exponent (split64.cu).
+// PS = 4 lanes split a leaf's points where there are too few items for the GPU.
+template <int PS>
+__global__ void __launch_bounds__(128) p2m64_kernel(const int32_t* __restrict__ lb, const cd* __restrict__ basis,
+                                                    const cd* __restrict__ qs, int64_t n, int64_t nleaf, int nrhs, int p,
+                                                    const int* __restrict__ sx, int* __restrict__ E,
+                                                    cd* __restrict__ mult) {
+    const int np = p + 1, nb = p + 2, nc = 2 * p + 1;
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, it = id / PS;
+    const int r = blockIdx.y, part = (int)(id % PS);
+    const bool live = it < nleaf * np;                     // whole groups of PS lanes
+    const int64_t b = live ? it / np : 0;
+    const int m = live ? (int)(it - b * np) : 0;
+    const int32_t lo = lb[b] + part, hi = live ? lb[b + 1] : 0;
+    const cd* q = qs + (int64_t)r * n;
+    const cd* B = basis + m;
+    double s1 = 0.0, s2 = 0.0, s3 = 0.0, s4 = 0.0;
+#pragma unroll 4
+    for (int32_t j = lo; j < hi; j += PS) {
+        const cd a = __ldg(q + j), u = __ldg(B + (int64_t)j * nb);
+        s1 = fma(a.x, u.x, s1);
+        s2 = fma(a.y, u.y, s2);
+        s3 = fma(a.x, u.y, s3);
+        s4 = fma(a.y, u.x, s4);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 1; o < PS; o <<= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        s3 += __shfl_xor_sync(0xffffffffu, s3, o);
+        s4 += __shfl_xor_sync(0xffffffffu, s4, o);
+    }
+    int e = S6_NONE;
+    if (live) {
+        cd* out = mult + (b * nrhs + r) * nc + p;
+        const cd ap = cmk(s1 - s2, s3 + s4), am = cmk(s1 + s2, s4 - s3);
+        if (part == 0) {
+            out[m] = ap;
+            if (m > 0) out[-m] = (m & 1) ? cneg(am) : am;
+        }
+        if (E) {
+            const int sh = -sx[m];
+            e = max(max(s6_exponent(ap.x, sh), s6_exponent(ap.y, sh)), max(s6_exponent(am.x, sh), s6_exponent(am.y, sh)));
+        }
+    }
+    if (E) {
+        e = __reduce_max_sync(0xffffffffu, e);
+        if ((threadIdx.x & 31) == 0 && e > S6_NONE) atomicMax(E + r, e);
+    }
+}
+
+struct Leaf64Args {
+    const int32_t* lb;
+    int L, nrhs, p;
+    int64_t n;
+    const cd* qs;
+    // near field: digit blocks (null: not here), offsets and their exponent
+    const uint4* G;
+    const int64_t* off;
+    const int* EG;
+    // L2P (loc null: not here)
+    const cd* loc;
+    const cd* basis;
+    // directly summed reaction (d_begin null: none)
+    const int32_t *d_begin, *d_src;
+    const int64_t* d_blk;
+    const cd* dvals;
+    const cd* ys;                    // sums made by other kernels (null: none)
+    const int64_t* perm;
+    bool conj_out;
+    cd* y;
+};
+
+constexpr int LD = 7;                // base-256 digits
+constexpr int LF_RING = 4;            // k-steps of near-field words in flight per warp (2 KB each)
+constexpr int LF_TERMS = 32;         // k-steps per exact FP32 accumulation
+constexpr long long LF_BIAS = 0x808080808080ll;   // 128 sum_{i = 0 .. 5} 256^i
+
+// v 2^(54 - E), the last bit zero, |v| < 2^E (see s6_fixed)
+__device__ __forceinline__ long long lf_fixed(double v, int E) { return (s6_fixed<53>(v, 0, E) - S6_BIAS) * 2; }
+
+// digit i of two numbers (with LF_BIAS) as f16: 1024 + field as bits 0x6400 | field, minus 1152
+__device__ __forceinline__ unsigned lf_digit(long long xb, long long yb, int i) {
+    const unsigned f0 = (unsigned)(int)((xb >> (8 * (LD - 1 - i))) + (i == 0 ? 128 : 0)) & 255u;
+    const unsigned f1 = (unsigned)(int)((yb >> (8 * (LD - 1 - i))) + (i == 0 ? 128 : 0)) & 255u;
+    unsigned h = 0x64006400u | f0 | (f1 << 16), r;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x64806480u));
+    return r;
+}
+
+// values v = 0 .. 3 of the four lanes of a quad -> their sums, value t in lane t
+template <class T>
+__device__ __forceinline__ T quad_scatter(const T (&v)[4], int t) {
+    const bool hi2 = t & 2, hi1 = t & 1;
+    const T k0 = hi2 ? v[2] : v[0], k1 = hi2 ? v[3] : v[1], s0 = hi2 ? v[0] : v[2], s1 = hi2 ? v[1] : v[3];
+    const T a0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 2), a1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 2);
+    return (hi1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, hi1 ? a0 : a1, 1);
+}
+
+// One CTA of W warps per (leaf, right-hand side); a warp per 16 targets, and where a
+// leaf has fewer tiles than warps these split its sources (and orders).  In the
+// MMA layout lane (g, t) = (lane / 4, lane % 4) holds targets g and g + 8 of the
+// tile; its part of the L2P and reaction sums is orders / sources = t mod 4.
+// The digit sums stay integers until lane t converts value t of its quad (real and
+// imaginary part of both targets): FP64 instructions are what this kernel has to
+// save.  W = 1 keeps every warp busy and free of barriers where the launch fills
+// the GPU, W = 4 shortens the chain of a launch with few leaves.
+template <int W>
+__global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Args A) {
+    extern __shared__ __align__(16) double lf_smem[];
+    constexpr int CHUNK = 128 * W, QPT = 4;                             // sources staged at once; per thread
+    const int64_t b = blockIdx.x;
+    const int32_t tlo = A.lb[b], tn = A.lb[b + 1] - tlo;
+    if (tn <= 0) return;
+    const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
+    unsigned* sq = reinterpret_cast<unsigned*>(lf_smem);               // [CHUNK][LD] digit pairs
+    double* red = lf_smem + CHUNK * LD / 2;                             // [W][3][32] (W > 1)
+    uint4* ring = reinterpret_cast<uint4*>(red + (W > 1 ? W * 96 : 0));  // [W][LF_RING][4][32]
+    double* coef = reinterpret_cast<double*>(ring + W * LF_RING * 128);  // [p + 1][4]
+    ring += wid * (LF_RING * 128) + lane;
+    const uint32_t ring_a = (uint32_t)__cvta_generic_to_shared(ring);
+    __shared__ int32_t s_lo[9], s_pre[10];
+    __shared__ int s_e[W];
+    auto sync = [&] { if (W > 1) __syncthreads(); else __syncwarp(); };
+    const cd* q = A.qs + (int64_t)r * A.n;
+    const int p = A.p, nb = p + 2, nc = 2 * p + 1;
+    if (A.G && wid == 0) {                                              // lane u: neighbour u, and the prefix sums
+        const int m = 1 << A.L, sx = (int)morton_x((uint32_t)b) + lane % 3 - 1, sy = (int)morton_y((uint32_t)b) + lane / 3 - 1;
+        int32_t lo = 0, cnt = 0;
+        if (lane < 9 && sx >= 0 && sy >= 0 && sx < m && sy < m) {
+            const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
+            lo = A.lb[s];
+            cnt = A.lb[s + 1] - lo;
+        }
+        int32_t inc = cnt;
+        for (int o = 1; o < 16; o <<= 1) {
+            const int32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += x;
+        }
+        if (lane < 9) { s_lo[lane] = lo; s_pre[lane + 1] = inc; }
+        if (lane == 0) s_pre[0] = 0;
+    }
+    if (A.loc) {
+        // y = (i/4) sum_m beta_m conj-basis: with c = beta_m, d = (-1)^m beta_{-m} and B = (u, v)
+        // re y = sum u w0 + v w1, im y = sum u w2 + v w3
+        const cd* beta = A.loc + (b * A.nrhs + r) * nc + p;
+        for (int m = tid; m <= p; m += W * 32) {
+            const cd c = beta[m];
+            cd d = m > 0 ? beta[-m] : cmk(0.0, 0.0);
+            if (m & 1) d = cneg(d);
+            coef[4 * m] = -0.25 * (c.y + d.y);
+            coef[4 * m + 1] = 0.25 * (c.x - d.x);
+            coef[4 * m + 2] = 0.25 * (c.x + d.x);
+            coef[4 * m + 3] = 0.25 * (c.y - d.y);
+        }
+    }
+    sync();
+    const int ns = A.G ? s_pre[9] : 0;
+    auto strength = [&](int j) {
+        if (j >= ns) return cmk(0.0, 0.0);
+        int u = 0;
+        while (j >= s_pre[u + 1]) ++u;
+        return __ldg(q + s_lo[u] + (j - s_pre[u]));
+    };
+    // the first chunk's strengths stay in registers between their exponent and their digits
+    cd qv[QPT];
+    int Eq = S6_NONE;
+    if (A.G) {
+#pragma unroll
+        for (int u = 0; u < QPT; ++u) qv[u] = strength(tid + u * W * 32);
+#pragma unroll
+        for (int u = 0; u < QPT; ++u) Eq = max(Eq, max(s6_exponent(qv[u].x, 0), s6_exponent(qv[u].y, 0)));
+        for (int j = CHUNK + tid; j < ns; j += W * 32) {
+            const cd v = strength(j);
+            Eq = max(Eq, max(s6_exponent(v.x, 0), s6_exponent(v.y, 0)));
+        }
+        Eq = __reduce_max_sync(0xffffffffu, Eq);
+        if (W > 1) {
+            if (lane == 0) s_e[wid] = Eq;
+            __syncthreads();
+            for (int w = 0; w < W; ++w) Eq = max(Eq, s_e[w]);
+        }
+    }
+    const bool bad = Eq >= S6_NAN / 2;
+    const int EV = max(Eq, S6_NONE) + (A.G ? max(*A.EG, S6_NONE) : 0) - 68;
+    const uint4* Gb = A.G ? A.G + A.off[b] : nullptr;
+
+    const int ntile = (tn + 15) / 16;
+    int staged = -1;                                                     // first source of the staged chunk
+    for (int t0 = 0; t0 < ntile;) {
+        const int tp = min(W, ntile - t0), ks = W / tp;                  // tiles at once, warps per tile
+        const int tile = t0 + wid % tp, part = wid / tp;
+        const bool live = part < ks;
+        const int i0 = 16 * tile + g, i1 = i0 + 8;
+        const bool v0 = live && i0 < tn, v1 = live && i1 < tn;
+        long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};            // (re, im) of target i0, of i1
+        for (int c0 = 0; c0 < ns; c0 += CHUNK) {
+            if (staged != c0) {
+                if (staged >= 0) {
+                    sync();                                              // the old chunk is read
+#pragma unroll
+                    for (int u = 0; u < QPT; ++u) qv[u] = strength(c0 + tid + u * W * 32);
+                }
+#pragma unroll
+                for (int u = 0; u < QPT; ++u) {
+                    const long long xr = lf_fixed(qv[u].x, Eq) + LF_BIAS, xi = lf_fixed(qv[u].y, Eq) + LF_BIAS;
+#pragma unroll
+                    for (int d = 0; d < LD; ++d) sq[(tid + u * W * 32) * LD + d] = lf_digit(xr, xi, d);
+                }
+                staged = c0;
+                sync();
+            }
+            if (!live) continue;
+            const int nk = (min(CHUNK, ns - c0) + 7) / 8;
+            // this lane's words of k-step kk into slot (kk / ks) % LF_RING: (i0, j0), (i1, j0), (i0, j1),
+            // (i1, j1); zeros meet zero strengths or unused rows
+            auto load_G = [&](int kk) {
+                if (kk < nk) {
+                    const int j0 = c0 + 8 * kk + t, j1 = j0 + 4;
+                    const uint4* Gj = Gb + (int64_t)j0 * tn;
+                    const uint32_t dst = ring_a + (kk / ks) % LF_RING * 2048;
+                    const bool a0 = v0 && j0 < ns, a1 = v1 && j0 < ns, b0 = v0 && j1 < ns, b1 = v1 && j1 < ns;
+                    cp_async16(dst, a0 ? Gj + i0 : Gb, a0);
+                    cp_async16(dst + 512, a1 ? Gj + i1 : Gb, a1);
+                    cp_async16(dst + 1024, b0 ? Gj + 4 * (int64_t)tn + i0 : Gb, b0);
+                    cp_async16(dst + 1536, b1 ? Gj + 4 * (int64_t)tn + i1 : Gb, b1);
+                }
+                cp_commit();
+            };
+#pragma unroll
+            for (int u = 0; u < LF_RING - 1; ++u) load_G(part + u * ks);
+            for (int kb = part; kb < nk; kb += LF_TERMS * ks) {
+                float ar[LD][4], ai[LD][4];
+#pragma unroll
+                for (int d = 0; d < LD; ++d)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) ar[d][v] = ai[d][v] = 0.0f;
+                const int ke = min(nk, kb + LF_TERMS * ks);
+                for (int kk = kb; kk < ke; kk += ks) {
+                    cp_wait<LF_RING - 2>();
+                    uint4 w[4];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) w[v] = ring[((kk / ks) % LF_RING * 4 + v) * 32];
+                    load_G(kk + (LF_RING - 1) * ks);
+                    // columns g = strength digits: (qr, -qi) for the real part, (qi, qr) for the imaginary
+                    const unsigned d0 = g < LD ? sq[(8 * kk + t) * LD + g] : 0u;
+                    const unsigned d1 = g < LD ? sq[(8 * kk + t + 4) * LD + g] : 0u;
+                    const uint2 br = make_uint2(d0 ^ 0x80000000u, d1 ^ 0x80000000u);
+                    const uint2 bi = make_uint2(__byte_perm(d0, 0, 0x1032), __byte_perm(d1, 0, 0x1032));
+#pragma unroll
+                    for (int d = 0; d < LD; ++d) {
+                        unsigned a[4];
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            const unsigned x = d < 2 ? w[v].x : d < 4 ? w[v].y : d < 6 ? w[v].z : w[v].w;
+                            if (d == 0) {
+                                const unsigned h = (x & 0x00ff00ffu) | 0x64006400u;
+                                asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(a[v]) : "r"(h), "r"(0x64806480u));
+                            } else a[v] = (d & 1) ? __byte_perm(x, 0, 0x4341) : x & 0x00ff00ffu;
+                        }
+                        const uint4 av = make_uint4(a[0], a[1], a[2], a[3]);
+                        s6_mma(ar[d], av, br);
+                        s6_mma(ai[d], av, bi);
+                    }
+                }
+                // columns 2t, 2t + 1 of the accumulators: order k = digit + column - 2t
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const int row = v >> 1;                              // 0: target i0, 1: i1
+                    float (&acc)[LD][4] = (v & 1) ? ai : ar;
+                    int s[LD + 1];
+#pragma unroll
+                    for (int k = 0; k <= LD; ++k) {
+                        s[k] = 0;
+                        if (k < LD) s[k] = __float2int_rn(acc[k][2 * row] * (k > 0 ? 16777216.0f : 1.0f));
+                        if (k > 0) s[k] += __float2int_rn(acc[k - 1][2 * row + 1] * (k > 1 ? 16777216.0f : 1.0f));
+                    }
+                    hi[v] += ((long long)s[0] << 24) + ((long long)s[1] << 16) + ((long long)s[2] << 8) + s[3];
+                    lo[v] += ((long long)s[4] << 24) + ((long long)s[5] << 16) + ((long long)s[6] << 8) + s[7];
+                }
+            }
+        }
+        double val[4] = {0.0, 0.0, 0.0, 0.0};
+        if (live) {
+            if (A.loc) {
+                const cd* B0 = A.basis + (int64_t)(tlo + (v0 ? i0 : 0)) * nb;
+                const cd* B1 = A.basis + (int64_t)(tlo + (v1 ? i1 : 0)) * nb;
+#pragma unroll 4
+                for (int m = t + 4 * part; m <= p; m += 4 * ks) {
+                    const double w0 = coef[4 * m], w1 = coef[4 * m + 1], w2 = coef[4 * m + 2], w3 = coef[4 * m + 3];
+                    const cd u0 = v0 ? __ldg(B0 + m) : cmk(0.0, 0.0), u1 = v1 ? __ldg(B1 + m) : cmk(0.0, 0.0);
+                    val[0] = fma(u0.x, w0, fma(u0.y, w1, val[0]));
+                    val[1] = fma(u0.x, w2, fma(u0.y, w3, val[1]));
+                    val[2] = fma(u1.x, w0, fma(u1.y, w1, val[2]));
+                    val[3] = fma(u1.x, w2, fma(u1.y, w3, val[3]));
+                }
+            }
+            if (A.d_begin)
+                for (int32_t e = A.d_begin[b]; e < A.d_begin[b + 1]; ++e) {
+                    const int32_t s = A.d_src[e], slo = A.lb[s], sn = A.lb[s + 1] - slo;
+                    const cd* D = A.dvals + A.d_blk[e];
+#pragma unroll 2
+                    for (int j = t + 4 * part; j < sn; j += 4 * ks) {
+                        const cd v = __ldg(q + slo + j);
+                        cd a0 = cmk(val[0], val[1]), a1 = cmk(val[2], val[3]);
+                        if (v0) cfma(a0, __ldg(D + (int64_t)i0 * sn + j), v);
+                        if (v1) cfma(a1, __ldg(D + (int64_t)i1 * sn + j), v);
+                        val[0] = a0.x; val[1] = a0.y; val[2] = a1.x; val[3] = a1.y;
+                    }
+                }
+        }
+        // quad sums: A 2^32 + B, lane t's digits 2^(-16 t) below (what falls under the unit
+        // of B is 2^-70 of the largest product)
+        long long pa[4], pb[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            pa[v] = hi[v] >> (16 * t);
+            pb[v] = t == 0 ? lo[v] : ((hi[v] << (64 - 16 * t)) >> 32 & 0xffffffffll) + (lo[v] >> (16 * t));
+        }
+        long long a = ns > 0 ? quad_scatter(pa, t) : 0, bsum = ns > 0 ? quad_scatter(pb, t) : 0;
+        double x = A.loc || A.d_begin ? quad_scatter(val, t) : 0.0;
+        if (W > 1 && ks > 1) {                                           // parts of a tile, added in order by part 0
+            double* mine = red + (size_t)wid * 96 + lane;
+            __syncthreads();
+            if (live && part > 0) {
+                mine[0] = __longlong_as_double(a);
+                mine[32] = __longlong_as_double(bsum);
+                mine[64] = x;
+            }
+            __syncthreads();
+            if (part == 0)
+                for (int o = 1; o < ks; ++o) {
+                    const double* other = mine + (size_t)o * tp * 96;
+                    a += __double_as_longlong(other[0]);
+                    bsum += __double_as_longlong(other[32]);
+                    x += other[64];
+                }
+        }
+        if (live && part == 0 && (t < 2 ? v0 : v1)) {
+            const int64_t i = tlo + (t < 2 ? i0 : i1);
+            if (ns > 0) x += fma((double)a, 4294967296.0, (double)bsum) * pow2d(EV);
+            if (bad) x = __longlong_as_double(0x7ff8000000000000ll);
+            if (A.ys) x += reinterpret_cast<const double*>(A.ys + (int64_t)r * A.n + i)[t & 1];
+            reinterpret_cast<double*>(A.y + (int64_t)r * A.n + A.perm[i])[t & 1] = (A.conj_out && (t & 1)) ? -x : x;
+        }
+        t0 += tp;
+    }
+}
+
+// (i/4) H0 doubles -> largest exponent; then, in place, digit words.
+__global__ void near64_exponent_kernel(const cd* __restrict__ G, int64_t n, int* __restrict__ E) {
+    int e = S6_NONE;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        e = max(e, max(s6_exponent(G[i].x, 0), s6_exponent(G[i].y, 0)));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0 && e > S6_NONE) atomicMax(E, e);
+}
+
+__global__ void near64_fix_kernel(cd* G, int64_t n, const int* __restrict__ E) {
+    const int e = *E;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const cd v = G[i];
+        const long long x = lf_fixed(v.x, e) + (128ll << 48), y = lf_fixed(v.y, e) + (128ll << 48);
+        unsigned w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {                      // digits 2k, 2k + 1 = bytes 6 - 2k, 5 - 2k
+            const unsigned x0 = (unsigned)(x >> (8 * (6 - 2 * k))) & 255u, y0 = (unsigned)(y >> (8 * (6 - 2 * k))) & 255u;
+            const unsigned x1 = k < 3 ? (unsigned)(x >> (8 * (5 - 2 * k))) & 255u : 0u;
+            const unsigned y1 = k < 3 ? (unsigned)(y >> (8 * (5 - 2 * k))) & 255u : 0u;
+            w[k] = x0 | (x1 << 8) | (y0 << 16) | (y1 << 24);
+        }
+        reinterpret_cast<uint4*>(G)[i] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+}  // namespace
+
+// Plan-time bases of an FP64 plan (a mixed plan's first gradient): skipped above
+// the byte budget (the P2M and L2P then evaluate them in each apply).
+hfmm_status build_basis64(hfmm_plan_s* P, cudaStream_t st) {
+    if (P->basis64 || P->ad) return HFMM_OK;
+    const LevelInfo& lv = P->lev[P->L];
+    const int nb = lv.p + 2;
+    const double bytes = sizeof(cd) * (double)P->n * nb;
+    if (bytes > BASIS64_MAX_BYTES || nb * (int)sizeof(double) > 40000) return HFMM_OK;
+    HFMM_TRY(plan_alloc(P, (void**)&P->basis64, (size_t)bytes));
+    P->buffer_bytes += bytes;
+    const int thr = std::max(1, std::min(64, 5000 / nb));
+    basis64_kernel<<<(unsigned)lv.nbox, thr, (size_t)thr * nb * sizeof(double), st>>>(
+        P->leaf_begin, P->xy_sorted, P->x0, P->y0, lv.h, P->k, nb, P->basis64);
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+// Digit form of `pairs` near-field values in place; *finite = false (and the
+// values unchanged) where an entry is not finite (coincident points).
+hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, bool* finite, cudaStream_t st) {
+    *finite = true;
+    HFMM_CUDA_TRY(cudaMemsetAsync(E, 0x80, sizeof(int), st));
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((pairs + 255) / 256, 16 * 152));
+    near64_exponent_kernel<<<grid, 256, 0, st>>>(vals, pairs, E);
+    HFMM_CUDA_TRY(cudaGetLastError());
+    int e = 0;
+    HFMM_CUDA_TRY(cudaMemcpyAsync(&e, E, sizeof(int), cudaMemcpyDeviceToHost, st));
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+    if (e >= S6_NAN / 2) { *finite = false; return HFMM_OK; }
+    near64_fix_kernel<<<grid, 256, 0, st>>>(vals, pairs, E);
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+// P2M of the sorted strengths into the leaf multipoles (and their exponent).
+hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[P->L];
+    const int64_t items = lv.nbox * (lv.p + 1);
+    const int ps = items < 32 * 1024 ? 4 : 1;        // not by nrhs: it would change the sums' order
+    auto kernel = ps == 4 ? p2m64_kernel<4> : p2m64_kernel<1>;
+    kernel<<<dim3((unsigned)((items * ps + 127) / 128), (unsigned)nrhs), 128, 0, st>>>(
+        P->leaf_begin, P->basis64, P->q_sorted, P->n, lv.nbox, nrhs, lv.p, lv.s6_sx,
+        P->s6_ready ? split64_exp(P, P->L, false) : nullptr, lv.mult);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+// Everything at the targets, into the caller's order: near = the stored blocks,
+// l2p = the leaves' locals, direct = the reaction blocks, ys = other sums.
+hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool direct, const cd* ys, bool conj_out, cd* y,
+                          cudaStream_t st) {
+    const LevelInfo& lv = P->lev[P->L];
+    Leaf64Args A{};
+    A.lb = P->leaf_begin;
+    A.L = P->L;
+    A.nrhs = nrhs;
+    A.p = lv.p;
+    A.n = P->n;
+    A.qs = P->q_sorted;
+    if (near) {
+        A.G = (const uint4*)P->near64_vals;
+        A.off = P->near64_off;
+        A.EG = P->near64_E;
+    }
+    if (l2p) {
+        A.loc = lv.loc;
+        A.basis = P->basis64;
+    }
+    if (direct) {
+        A.d_begin = P->d_begin;
+        A.d_src = P->d_src;
+        A.d_blk = P->d_blk;
+        A.dvals = P->d_vals;
+    }
+    A.ys = ys;
+    A.perm = P->perm;
+    A.conj_out = conj_out;
+    A.y = y;
+    // one warp per leaf from 16 of them per SM on (leaves of at most four tiles), else four
+    const bool one = lv.nbox >= 16 * 152 && P->leaf_max <= 64;
+    const int W = one ? 1 : 4;
+    const size_t sm = sizeof(double) * (128 * W * LD / 2 + (one ? 0 : W * 96) + W * LF_RING * 256 + (l2p ? 4 * (size_t)(lv.p + 1) : 0));
+    auto kernel = one ? leaf64_kernel<1> : leaf64_kernel<4>;
+    if (sm > 47 * 1024)                                    // (static shared memory beside it)
+        HFMM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    kernel<<<dim3((unsigned)lv.nbox, (unsigned)nrhs), W * 32, sm, st>>>(A);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}

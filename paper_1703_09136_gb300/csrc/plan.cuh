@@ -105,6 +105,7 @@ struct LevelInfo {
     const int* s6_sx = nullptr;
     uint4 *s6_free = nullptr, *s6_react = nullptr, *s6_l2l = nullptr, *s6_m2m = nullptr;
     int* s6_Eop = nullptr;
+    unsigned *s6_dmult = nullptr, *s6_dloc = nullptr;   // digits of the level's expansions
 };
 
 // Diagonal form: kept on a level when its weighted difference to the dense
@@ -197,7 +198,10 @@ struct hfmm_plan_s {
     // FP64 near field: (i/4) H0 blocks of every target leaf's U list, built
     // at plan time (fmm64.cu), and their offsets per leaf; null above the budget
     int64_t* near64_off = nullptr;
-    cd* near64_vals = nullptr;
+    cd* near64_vals = nullptr;      // after the fill: base-256 digits (leaf64.cu)
+    int* near64_E = nullptr;        // their exponent
+    int leaf_max = 0;               // largest number of points of a leaf
+    cd* basis64 = nullptr;          // [n][p_L + 2] P2M basis J_m(k rho) e^{-i m theta}, m >= 0
     void* krylov = nullptr;         // hfmm_solve: Krylov vectors (first call; grows with restart)
     size_t krylov_bytes = 0;
     double* krylov_part = nullptr;  // partial sums of its dot products
@@ -321,8 +325,16 @@ double diag_flops(const hfmm_plan_s* P, int l, int nrhs, int parts);
 hfmm_status build_split64(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status split64_begin(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status split64_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st);
+hfmm_status split64_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st);
 hfmm_status split64_m2m(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st);
 hfmm_status split64_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st);
+int* split64_exp(hfmm_plan_s* P, int l, bool loc);
+// leaf64.cu
+hfmm_status build_basis64(hfmm_plan_s* P, cudaStream_t st);
+hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, bool* finite, cudaStream_t st);
+hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st);
+hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool direct, const cd* ys, bool conj_out, cd* y,
+                          cudaStream_t st);
 hfmm_status build_near64_grad(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, bool adjoint,
                        cudaStream_t st);

@@ -26,7 +26,7 @@
 // clocks per SM), mma.sync f16 at 600 TFLOP/s: 21 products leave 28 TFLOP/s.
 // Measured (one GB300, two layers, 262,144 points, one right-hand side): leaf
 // level (order 15, 430k free-space and 49k reaction translations, 3.8 GFLOP)
-// 5.73 -> 0.63 ms, all levels 12.0 -> 1.55 ms, M2M 0.72 -> 0.17 ms; the result
+// 5.73 -> 0.43 ms, all levels 12.0 -> 1.03 ms, M2M 0.72 -> 0.13 ms; the result
 // differs from the FP64 kernels' by 2e-13 (1e-14 at orders where those cancel
 // less), and both are equally far from the direct sum.
 #include <algorithm>
@@ -34,49 +34,12 @@
 #include <vector>
 
 #include "plan.cuh"
+#include "split64.cuh"
 
 namespace {
 
-constexpr int ND = 6;                    // digits
-constexpr int S6_MAXW = 8;               // m-tiles (warps) per CTA
-constexpr int S6_NONE = -(1 << 24);      // exponent of an all-zero level (or below)
-constexpr int S6_NAN = 1 << 20;          // exponent of a level with an infinity or a NaN
-constexpr double S6_MAX_BYTES = 16e9;    // operator slices of one plan
-
-// largest E with |v 2^shift| < 2^E (S6_NONE for zero)
-__device__ __forceinline__ int s6_exponent(double v, int shift) {
-    const long long b = __double_as_longlong(v);
-    const int e = (int)((b >> 52) & 2047);
-    if (e == 2047) return S6_NAN;
-    if (e == 0) return (b & 0xfffffffffffffll) ? -1021 + shift : S6_NONE;
-    return e - 1022 + shift;
-}
-
-// v 2^shift 2^(BITS - E) rounded to an integer plus the digit bias, |v 2^shift| < 2^E
-template <int BITS>
-__device__ __forceinline__ long long s6_fixed(double v, int shift, int E) {
-    const long long b = __double_as_longlong(v);
-    int e = (int)((b >> 52) & 2047);
-    unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
-    if (e) m |= 1ull << 52; else e = 1;
-    const int s = E - shift - e + 1075 - BITS;            // right shift, >= 0 for BITS = 53
-    if (s > 0) m = s > 54 ? 0ull : (m + (1ull << (s - 1))) >> s;
-    const long long x = b < 0 ? -(long long)m : (long long)m;
-    // + 256 sum_{i = 0 .. 4} 512^i: the low five fields then hold digit + 256
-    return x + 0x100804020100ll;
-}
-
-// field of digit i (0 = most significant), digit + 256 in [0, 512]
-__device__ __forceinline__ unsigned s6_field(long long xb, int i) {
-    return i == 0 ? (unsigned)((int)(xb >> 45) + 256) : (unsigned)(xb >> (9 * (ND - 1 - i))) & 511u;
-}
-
-// two digits as f16 (1024 + field as bits 0x6400 | field, minus 1280)
-__device__ __forceinline__ unsigned s6_half2(unsigned f0, unsigned f1) {
-    unsigned h = 0x64006400u + (f0 | (f1 << 16)), r;
-    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x65006500u));
-    return r;
-}
+constexpr int S6_MAXW = 6;               // m-tiles (warps) per CTA
+constexpr double S6_MAX_BYTES = 16e9;    // operator slices of one plan, and its expansions' digits
 
 // ---------------------------------------------------------------------------
 // plan time: operator slices in the A-fragment order of mma.m16n8k16
@@ -137,7 +100,7 @@ __global__ void s6_op_slice_kernel(S6Op o, const int* __restrict__ Ep, uint4* __
         for (int q = 0; q < 4; ++q) {
             const int row = 16 * mt + g + (q & 1) * 8, m = (16 * ks + (q >> 1) * 8) / 2 + t;   // columns 2m, 2m + 1
             const int j = row >> 1;
-            long long x0 = 0x100804020100ll, x1 = 0x100804020100ll;
+            long long x0 = S6_BIAS, x1 = S6_BIAS;
             if (j < no && m < ni) {
                 int sh;
                 const cd v = s6_entry(o, op, j - o.po, m - o.pi, &sh);
@@ -172,17 +135,42 @@ __global__ void s6_exponent_kernel(const cd* __restrict__ a, int64_t nbox, int n
     if ((threadIdx.x & 31) == 0 && e > S6_NONE) atomicMax(E + r, e);
 }
 
+// Digits of a level's expansions in the B-fragment order of mma.m16n8k16:
+// per (box, right-hand side, k-step of eight coefficients, digit) the words
+// [coefficient % 4][coefficient / 4] (32 bytes).  Every source meets up to 27
+// target tiles: cutting it in the product kernel took 60% of that kernel's
+// instructions (leaf level of two layers 0.47 -> 0.34 ms without it).
+__global__ void s6_slice_kernel(const cd* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
+                                int sign, const int* __restrict__ E, unsigned* __restrict__ dig) {
+    const int nc = 2 * p + 1, KS = (2 * nc + 15) / 16, r = blockIdx.y;
+    const int64_t total = nbox * KS * 8;
+    const int e = E[r];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = i / (KS * 8);
+        const int m = (int)(i - b * (KS * 8));
+        long long xr = S6_BIAS, xi = S6_BIAS;
+        if (m < nc) {
+            const cd v = a[(b * nrhs + r) * nc + m];
+            const int sh = sign * sx[abs(m - p)];
+            xr = s6_fixed<53>(v.x, sh, e);
+            xi = s6_fixed<53>(v.y, sh, e);
+        }
+        unsigned* o = dig + ((b * nrhs + r) * KS + (m >> 3)) * (ND * 8) + (m & 3) * 2 + (m >> 2 & 1);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) o[d * 8] = s6_half2(s6_field(xr, d), s6_field(xi, d));
+    }
+}
+
 // ---------------------------------------------------------------------------
 // the product kernel
 // ---------------------------------------------------------------------------
 // One operator family of a launch: sources, their order, scale signs, slices.
 struct S6Fam {
-    const cd* src;
+    const uint4* dig;                // source digits (s6_slice_kernel)
     const uint4* ops;
     const int* Eop;                  // exponent of the family
     const int* Esrc;                 // [nrhs] exponent of the source expansions
-    const int* sx;                   // log2 s of the source level
-    int p, sign;                     // source order; in_shift = sign * sx
+    int p;                           // source order
 };
 
 struct S6Args {
@@ -190,8 +178,8 @@ struct S6Args {
     int nrhs, p;                     // output order
     int tiles;
     const int32_t* lb;               // leaf ranges (downward: empty targets are skipped)
-    S6Fam shift;                     // M2M or L2L (src null: none)
-    S6Fam list;                      // M2L sources (src null: none); ops = free-space operators
+    S6Fam shift;                     // M2M or L2L (dig null: none)
+    S6Fam list;                      // M2L sources (dig null: none); ops = free-space operators
     const uint4* rops;               // reaction operators (null: none)
     int vlist, rlist, lstar;         // lists to run; first level whose bottom-row pair is admissible
     int rows;                        // box rows covered by the launch (downward)
@@ -201,12 +189,6 @@ struct S6Args {
     cd* out;
     int* Eout;                       // [nrhs], or null
 };
-
-__device__ __forceinline__ void s6_mma(float (&c)[4], const uint4& a, const uint2& b) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
-}
 
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
@@ -231,7 +213,7 @@ struct S6Tile {
 };
 
 __device__ __forceinline__ int s6_steps(const S6Args& A, S6Tile& T) {
-    T.nshift = A.shift.src ? (A.mode == 0 ? 4 : 1) : 0;
+    T.nshift = A.shift.dig ? (A.mode == 0 ? 4 : 1) : 0;
     T.nv = T.nr = 0;
     if (A.mode == 1) {
         T.nv = A.vlist ? 36 : 0;      // 6 x 6 offsets of the parents' neighbourhood
@@ -275,15 +257,14 @@ __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s,
 }
 
 // A CTA owns 8 NT target boxes of one row and one column parity (they share every
-// operator) and up to eight m-tiles of 16 output rows, one per warp; it walks the
-// steps, slices the sources' 64-term chunks into shared memory (integer work on
-// the otherwise idle ALUs: slicing on the fly costs a tenth of the products and
-// saves a pass over memory) and multiplies them with the operator fragments, which
-// each warp reads from L2 as it needs them.  Levels with few tiles split a tile's
-// steps over a cluster of up to eight CTAs and add the partial sums in rank order
-// through distributed shared memory, so results do not depend on timing.
+// operator) and up to six m-tiles of 16 output rows, one per warp; it walks the
+// steps, copies the sources' digits of 64 terms into shared memory and multiplies
+// them with the operator fragments, which each warp copies from L2 into a ring of
+// its own.  Levels with few tiles split a tile's steps over a cluster of up to
+// eight CTAs and add the partial sums in rank order through distributed shared
+// memory, so results do not depend on timing.
 template <int NT>
-__global__ void __launch_bounds__(S6_MAXW * 32, 1) s6_kernel(const __grid_constant__ S6Args A) {
+__global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant__ S6Args A) {
     // digits of the sources of one 64-term chunk, in B-fragment order, two buffers
     __shared__ __align__(16) uint2 Bs[2][ND][4][NT][32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
@@ -323,7 +304,7 @@ __global__ void __launch_bounds__(S6_MAXW * 32, 1) s6_kernel(const __grid_consta
         if (!any) return;
     }
     const int nsteps = s6_steps(A, T);
-    const int nis = A.shift.src ? 2 * A.shift.p + 1 : 0, nil = A.list.src ? 2 * A.list.p + 1 : 0;
+    const int nis = A.shift.dig ? 2 * A.shift.p + 1 : 0, nil = A.list.dig ? 2 * A.list.p + 1 : 0;
     const int KSs = (2 * nis + 15) / 16, KSl = (2 * nil + 15) / 16;
 
     float acc[NT][ND][4];
@@ -339,19 +320,20 @@ __global__ void __launch_bounds__(S6_MAXW * 32, 1) s6_kernel(const __grid_consta
 #pragma unroll
             for (int o = 0; o < ND; ++o) acc[t][o][v] = 0.0f;
         }
-    int Es = 0;                       // exponent of the family being staged
     int since = 0;                    // chunks since the integers were last folded
-    // dacc += (digit sums) 2^(Esrc + Eop - 42): order o weighs 2^(9 (10 - o)) of 2^-105
+    // dacc += (digit sums) 2^(Esrc + Eop - 42): order o weighs 2^(9 (10 - o)) of 2^-105.  Four
+    // FP64 instructions a value (the pipe takes 64 clocks for each of a sub-partition's):
+    // orders 0 .. 2 and 3 .. 5 as two integers below 2^51
     auto fold = [&](int E) {
+        const double chi = pow2d(E + 9), clo = pow2d(E - 18);
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                const long long x = ((long long)iacc[t][0][v] << 27) + ((long long)iacc[t][1][v] << 18) +
-                                    ((long long)iacc[t][2][v] << 9) + (long long)iacc[t][3][v];
-                const float lo = acc[t][4][v] + acc[t][5][v] * (1.0f / 512.0f);
-                const double d = (double)x + (double)lo * (1.0 / 512.0);
-                dacc[t][v] += scalbn(d, E);
+                const long long hi = ((long long)iacc[t][0][v] << 18) + ((long long)iacc[t][1][v] << 9) + iacc[t][2][v];
+                const long long lo = ((long long)iacc[t][3][v] << 18) + (__float2ll_rn(acc[t][4][v]) << 9) +
+                                     __float2ll_rn(acc[t][5][v]);
+                dacc[t][v] = fma(int51d(hi), chi, fma(int51d(lo), clo, dacc[t][v]));
                 iacc[t][0][v] = iacc[t][1][v] = iacc[t][2][v] = iacc[t][3][v] = 0;
                 acc[t][4][v] = acc[t][5][v] = 0.0f;
             }
@@ -359,95 +341,136 @@ __global__ void __launch_bounds__(S6_MAXW * 32, 1) s6_kernel(const __grid_consta
     };
     int Ef[2] = {0, 0};               // fold exponents per family
     bool bad = false;
-    if (A.shift.src) {
+    if (A.shift.dig) {
         const int e = A.shift.Esrc[r];
         bad |= e >= S6_NAN / 2;
         Ef[0] = max(e, S6_NONE) + max(*A.shift.Eop, S6_NONE) - 42;
     }
-    if (A.list.src) {
+    if (A.list.dig) {
         const int e = A.list.Esrc[r];
         bad |= e >= S6_NAN / 2;
         Ef[1] = max(e, S6_NONE) + max(*A.list.Eop, S6_NONE) - 42;
     }
 
-    int buf = 0, prev_fam = -1;
-    for (int s = rank; s < nsteps; s += S) {
-        S6Step st;
-        if (!s6_step(A, T, s, MT, KSs, KSl, st)) continue;
-        const S6Fam& F = st.fam ? A.list : A.shift;
-        const int ni = st.fam ? nil : nis, KS = st.fam ? KSl : KSs;
-        if (prev_fam >= 0 && st.fam != prev_fam) fold(Ef[prev_fam]);
-        prev_fam = st.fam;
-        Es = F.Esrc[r];
-        const uint4* op = st.op + (int64_t)mt * KS * (ND * 32) + lane;
-        for (int k0 = 0; k0 < KS; k0 += 4) {
-            const int nk = min(4, KS - k0);
-            // stage: warp w < 4 slices columns w, w + 4, ...; lane = complex coefficient of the chunk
-            const int m = 8 * k0 + lane;
-            if (wid < 4) {
-                cd v[2 * NT];
-                const int sh = m < ni ? F.sign * F.sx[abs(m - F.p)] : 0;
-#pragma unroll
-                for (int u = 0; u < 2 * NT; ++u) {
-                    const int c = 4 * u + wid;
-                    int64_t b = -1;
-                    if (m < ni) {
-                        if (st.fam == 0) {
-                            if (A.mode == 0) b = box0 + c < nbox ? 4 * (box0 + c) + st.child : -1;
-                            else if (c < T.ncol) b = morton((uint32_t)((T.ix0 >> 1) + c), (uint32_t)(T.iy >> 1));
-                        } else if (c < T.ncol) {
-                            const int sx = T.ix0 + 2 * c - st.dx;
-                            if (sx >= 0 && sx < T.n) b = morton((uint32_t)sx, (uint32_t)st.sy);
-                        }
-                    }
-                    v[u] = b >= 0 ? __ldg(F.src + (b * A.nrhs + r) * ni + m) : cmk(0.0, 0.0);
-                }
-                const int kk = lane >> 3, reg = (lane >> 2) & 1;
-#pragma unroll
-                for (int u = 0; u < 2 * NT; ++u) {
-                    const int c = 4 * u + wid, fl = (c & 7) * 4 + (lane & 3);
-                    const long long xr = s6_fixed<53>(v[u].x, sh, Es), xi = s6_fixed<53>(v[u].y, sh, Es);
-#pragma unroll
-                    for (int d = 0; d < ND; ++d)
-                        reinterpret_cast<unsigned*>(&Bs[buf][d][kk][c >> 3][fl])[reg] =
-                            s6_half2(s6_field(xr, d), s6_field(xi, d));
-                }
-            }
-            __syncthreads();
-            if (has_m) {
-#pragma unroll
-                for (int t = 0; t < NT; ++t)
-#pragma unroll
-                    for (int o = 0; o < 4; ++o)
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) acc[t][o][v] = 0.0f;
-                for (int kk = 0; kk < nk; ++kk) {
-                    uint4 a[ND];
-#pragma unroll
-                    for (int d = 0; d < ND; ++d) a[d] = __ldg(op + (int64_t)((k0 + kk) * ND + d) * 32);
-#pragma unroll
-                    for (int t = 0; t < NT; ++t) {
-                        uint2 bb[ND];
-#pragma unroll
-                        for (int d = 0; d < ND; ++d) bb[d] = Bs[buf][d][kk][t][lane];
-#pragma unroll
-                        for (int i = 0; i < ND; ++i)
-#pragma unroll
-                            for (int j = 0; j < ND - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
-                    }
-                }
-#pragma unroll
-                for (int t = 0; t < NT; ++t)
-#pragma unroll
-                    for (int o = 0; o < 4; ++o)
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) iacc[t][o][v] += __float2int_rn(acc[t][o][v]);
-                if (++since == 120) fold(Ef[st.fam]);     // 120 x 2^24 < 2^31
-            }
-            buf ^= 1;
+    // A chunk: up to 64 terms (four k-steps) of one step.  While the tensor cores work on
+    // one chunk the next one's source digits are copied into the other buffer and
+    // the operator fragments into the warp's four-slot ring (two k-steps ahead
+    // across chunks), all asynchronously: a k-step's loads alone take as long as
+    // its 21 NT products.
+    struct Chunk { S6Step st; int s, k0; };
+    auto next = [&](Chunk& c) -> bool {             // the following chunk of this CTA, false at the end
+        if (c.s >= 0) {
+            c.k0 += 4;
+            if (c.k0 < (c.st.fam ? KSl : KSs)) return true;
         }
+        c.k0 = 0;
+        for (c.s = c.s < 0 ? rank : c.s + S; c.s < nsteps; c.s += S)
+            if (s6_step(A, T, c.s, MT, KSs, KSl, c.st)) return true;
+        return false;
+    };
+    // digits of the chunk's columns, 48 pieces of 16 bytes each (k-step, digit, half): a
+    // warp takes columns wid, wid + nw, ..., a lane the pieces lane and lane + 32; one group.
+    // Lane c holds the source box of column c (found once per step).
+    int64_t sbox = -1;
+    auto load_src = [&](const Chunk& c, int buf, bool ok) {
+        if (ok) {
+            if (c.k0 == 0) {
+                sbox = -1;
+                if (c.st.fam == 0) {
+                    if (A.mode == 0) sbox = lane < NC && box0 + lane < nbox ? 4 * (box0 + lane) + c.st.child : -1;
+                    else if (lane < T.ncol) sbox = morton((uint32_t)((T.ix0 >> 1) + lane), (uint32_t)(T.iy >> 1));
+                } else if (lane < T.ncol) {
+                    const int x = T.ix0 + 2 * lane - c.st.dx;
+                    if (x >= 0 && x < T.n) sbox = morton((uint32_t)x, (uint32_t)c.st.sy);
+                }
+            }
+            const int KS = c.st.fam ? KSl : KSs, nk = min(4, KS - c.k0);
+            const uint4* dig = (c.st.fam ? A.list.dig : A.shift.dig) + (int64_t)c.k0 * (2 * ND);
+            const int64_t stride = (int64_t)A.nrhs * KS * (2 * ND), first = (int64_t)r * KS * (2 * ND);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int q = lane + 32 * u, kk = q / 12, d = q % 12 >> 1, h = q & 1;
+                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&Bs[buf][d][kk][0][2 * h]);
+                for (int col = wid; col < NC; col += nw) {
+                    const int64_t b = __shfl_sync(0xffffffffu, sbox, col);
+                    if (kk < nk)
+                        cp_async16(dst + (col >> 3) * 256 + (col & 7) * 32, b >= 0 ? dig + b * stride + first + q : dig, b >= 0);
+                }
+            }
+        }
+        cp_commit();
+    };
+    extern __shared__ __align__(16) uint4 s6_ring[];      // [warps][4][ND][32]
+    const uint4* ring = s6_ring + (size_t)wid * (4 * ND * 32) + lane;
+    const uint32_t ring_a = (uint32_t)__cvta_generic_to_shared(ring);
+    // operator fragments of k-step kk of chunk c into slot kk; one group, empty where there is none
+    auto load_op = [&](const Chunk& c, int kk, bool ok) {
+        const int KS = c.st.fam ? KSl : KSs;
+        if (ok && has_m && c.k0 + kk < KS) {
+            const uint4* op = c.st.op + (((int64_t)mt * KS + c.k0 + kk) * ND) * 32 + lane;
+#pragma unroll
+            for (int d = 0; d < ND; ++d) cp_async16(ring_a + (kk * ND + d) * 512, op + d * 32, true);
+        }
+        cp_commit();
+    };
+    int buf = 0, prev_fam = -1;
+    Chunk cur{{}, -1, 0};
+    bool more = next(cur);
+    load_src(cur, 0, more);
+    load_op(cur, 0, more);
+    load_op(cur, 1, more);
+    while (more) {
+        const int fam = cur.st.fam, nk = min(4, (fam ? KSl : KSs) - cur.k0);
+        load_op(cur, 2, true);
+        load_op(cur, 3, true);
+        cp_wait<4>();                                     // the source digits (four operator groups came after)
+        __syncthreads();
+        more = next(cur);
+        load_src(cur, buf ^ 1, more);
+        if (has_m) {
+            if (prev_fam >= 0 && fam != prev_fam) fold(Ef[prev_fam]);
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+                for (int o = 0; o < 4; ++o)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) acc[t][o][x] = 0.0f;
+        }
+        // groups in flight, in order: this chunk's slots 0 .. 3, the next chunk's digits, its slots 0, 1
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            if (kk < 3) cp_wait<4>(); else cp_wait<3>();
+            if (has_m && kk < nk) {
+                uint4 a[ND];
+#pragma unroll
+                for (int d = 0; d < ND; ++d) a[d] = ring[(kk * ND + d) * 32];
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                    uint2 bb[ND];
+#pragma unroll
+                    for (int d = 0; d < ND; ++d) bb[d] = Bs[buf][d][kk][t][lane];
+#pragma unroll
+                    for (int i = 0; i < ND; ++i)
+#pragma unroll
+                        for (int j = 0; j < ND - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
+                }
+            }
+            if (kk < 2) load_op(cur, kk, more);
+        }
+        if (has_m) {
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+                for (int o = 0; o < 4; ++o)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) iacc[t][o][x] += __float2int_rn(acc[t][o][x]);
+            if (++since == 120) fold(Ef[fam]);            // 120 x 2^24 < 2^31
+        }
+        prev_fam = fam;
+        buf ^= 1;
     }
     if (prev_fam >= 0) fold(Ef[prev_fam]);
+    cp_wait<0>();
 
     // partial sums of the cluster's CTAs, added in rank order by rank 0
     double* part = reinterpret_cast<double*>(&Bs[0][0][0][0][0]);   // [warp][NT][4][32]: 8 NT x 1 KB <= 24 KB NT / 2
@@ -488,7 +511,7 @@ __global__ void __launch_bounds__(S6_MAXW * 32, 1) s6_kernel(const __grid_consta
             if (row >= 2 * no || b < 0) continue;
             const int sh = A.sxo[abs((row >> 1) - A.p)];
             double* o = reinterpret_cast<double*>(A.out + (b * A.nrhs + r) * no) + row;
-            double x = bad ? nan : scalbn(dacc[t][v], A.osign * sh);
+            double x = bad ? nan : dacc[t][v] * pow2d(A.osign * sh);
             if (A.accumulate) x += *o;
             *o = x;
             e = max(e, s6_exponent(x, -A.osign * sh));
@@ -502,13 +525,16 @@ __global__ void __launch_bounds__(S6_MAXW * 32, 1) s6_kernel(const __grid_consta
 template <int NT>
 hfmm_status s6_launch(const S6Args& A, int tiles, int steps, cudaStream_t st) {
     const int MT = (2 * (2 * A.p + 1) + 15) / 16;
-    const int gy = (MT + S6_MAXW - 1) / S6_MAXW, W = std::max(4, (MT + gy - 1) / gy);
-    // CTAs per tile: split the steps over a cluster while the launch leaves SMs idle
+    const int gy = (MT + S6_MAXW - 1) / S6_MAXW, W = (MT + gy - 1) / gy;
+    // CTAs per tile: split the steps over a cluster while one right-hand side leaves SMs
+    // idle (whatever nrhs is, so that a right-hand side's bits do not depend on the others)
     int S = 1;
-    while (S < 8 && (int64_t)tiles * gy * A.nrhs * S * 2 <= 4 * 152 && 2 * S <= steps) S *= 2;
+    while (S < 8 && (int64_t)tiles * gy * S * 2 <= 4 * 152 && 2 * S <= steps) S *= 2;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(tiles * S), (unsigned)gy, (unsigned)A.nrhs);
     cfg.blockDim = dim3(32 * W);
+    cfg.dynamicSmemBytes = (size_t)W * 4 * ND * 512;
+    HFMM_CUDA_TRY(cudaFuncSetAttribute(s6_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, S6_MAXW * 4 * ND * 512));
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -531,28 +557,25 @@ hfmm_status s6_run(S6Args& A, cudaStream_t st) {
         return (int64_t)A.rows * (n > 1 ? 2 : 1) * ((per + nc - 1) / nc);
     };
     const int steps = A.mode == 0 ? 4 : 1 + (A.vlist ? 27 : 0) + (A.rlist ? (int)std::min<int64_t>(n, 1 << 20) : 0);
-    const bool wide = (A.mode == 0 || (n >> 1) > 8) && tiles(16) * gy * A.nrhs >= 2 * 152;
+    const bool wide = (A.mode == 0 || (n >> 1) > 8) && tiles(16) * gy >= 3 * 152;
     A.tiles = (int)tiles(wide ? 16 : 8);
     return wide ? s6_launch<2>(A, A.tiles, steps, st) : s6_launch<1>(A, A.tiles, steps, st);
 }
 
-S6Fam s6_fam(const cd* src, const LevelInfo& sl, const uint4* ops, const int* Eop, const int* Esrc,
-             int sign) {
+S6Fam s6_fam(const unsigned* dig, int p, const uint4* ops, const int* Eop, const int* Esrc) {
     S6Fam f{};
-    f.src = src;
+    f.dig = (const uint4*)dig;
     f.ops = ops;
     f.Eop = Eop;
     f.Esrc = Esrc;
-    f.sx = sl.s6_sx;
-    f.p = sl.p;
-    f.sign = sign;
+    f.p = p;
     return f;
 }
 
 }  // namespace
 
 // Operator slices of every level (plan time, or a mixed plan's first gradient).
-// A plan whose slices would pass the byte budget keeps the FP64 kernels.
+// A plan whose slices or digits would pass the byte budget keeps the FP64 kernels.
 hfmm_status build_split64(hfmm_plan_s* P, cudaStream_t st) {
     if (P->s6_ready || P->ad) return HFMM_OK;
     const int L = P->L;
@@ -585,7 +608,16 @@ hfmm_status build_split64(hfmm_plan_s* P, cudaStream_t st) {
         used += (has_free(lv) ? bytes(49, lv.p, lv.p) : 0.0) + (has_react(lv) ? bytes(lv.n_react_entries, lv.p, lv.p) : 0.0);
         if (l > P->lmin) used += bytes(4, lv.p, P->lev[l - 1].p) + bytes(4, P->lev[l - 1].p, lv.p);
     }
-    if (used > S6_MAX_BYTES) return HFMM_OK;
+    auto digits = [&](const LevelInfo& lv) { return (size_t)lv.nbox * P->max_rhs * ((2 * lv.ncoef + 15) / 16) * (ND * 32); };
+    double dbytes = 0.0;
+    for (int l = P->lmin; l <= L; ++l) dbytes += (l < L ? 2.0 : 1.0) * digits(P->lev[l]);
+    if (used > S6_MAX_BYTES || dbytes > S6_MAX_BYTES) return HFMM_OK;
+    for (int l = P->lmin; l <= L; ++l) {
+        LevelInfo& lv = P->lev[l];
+        HFMM_TRY(plan_alloc(P, (void**)&lv.s6_dmult, digits(lv)));
+        if (l < L) HFMM_TRY(plan_alloc(P, (void**)&lv.s6_dloc, digits(lv)));
+    }
+    P->buffer_bytes += dbytes;
     auto make = [&](const cd* T, int kind, int nop, const LevelInfo& o, const LevelInfo& i, int* Ep, uint4** out) -> hfmm_status {
         S6Op op{T, kind, nop, o.p, i.p, o.s6_sx, i.s6_sx};
         HFMM_TRY(plan_alloc(P, (void**)out, (size_t)bytes(nop, o.p, i.p)));
@@ -643,12 +675,24 @@ hfmm_status split64_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStre
     return HFMM_OK;
 }
 
+// Digits of a level's finished expansions, for the products that read them.
+hfmm_status split64_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[l];
+    const int64_t total = lv.nbox * ((2 * lv.ncoef + 15) / 16 * 8);
+    s6_slice_kernel<<<dim3((unsigned)std::min<int64_t>((total + 127) / 128, 16 * 152), (unsigned)nrhs), 128, 0, st>>>(
+        loc ? lv.loc : lv.mult, lv.nbox, nrhs, lv.p, lv.s6_sx, loc ? 1 : -1, split64_exp(P, l, loc),
+        loc ? lv.s6_dloc : lv.s6_dmult);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
 hfmm_status split64_m2m(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st) {
     LevelInfo& lv = P->lev[l];
     LevelInfo& ch = P->lev[l + 1];
     S6Args A{};
     A.l = l; A.L = P->L; A.mode = 0; A.nrhs = nrhs; A.p = lv.p;
-    A.shift = s6_fam(ch.mult, ch, lv.s6_m2m, lv.s6_Eop + 2, split64_exp(P, l + 1, false), -1);
+    A.shift = s6_fam(ch.s6_dmult, ch.p, lv.s6_m2m, lv.s6_Eop + 2, split64_exp(P, l + 1, false));
     A.sxo = lv.s6_sx;
     A.osign = 1;
     A.out = lv.mult;
@@ -666,9 +710,9 @@ hfmm_status split64_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_
     A.lb = P->leaf_begin;
     if (l > P->lmin) {
         LevelInfo& pa = P->lev[l - 1];
-        A.shift = s6_fam(pa.loc, pa, lv.s6_l2l, lv.s6_Eop + 1, split64_exp(P, l - 1, true), 1);
+        A.shift = s6_fam(pa.s6_dloc, pa.p, lv.s6_l2l, lv.s6_Eop + 1, split64_exp(P, l - 1, true));
     }
-    A.list = s6_fam(lv.mult, lv, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false), -1);
+    A.list = s6_fam(lv.s6_dmult, lv.p, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false));
     A.rops = lv.s6_react;
     A.vlist = !dg && lv.nv > 0 && (parts & HFMM_PART_FAR_FREE);
     const bool react = !dg && lv.nr > 0 && (parts & HFMM_PART_FAR_REACT);
@@ -682,12 +726,12 @@ hfmm_status split64_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_
     // 28 of the others: there they run as a launch of their own over the two rows
     const bool apart = react && l >= 5;
     A.rlist = react && !apart;
-    if (!A.vlist && !A.rlist) A.list.src = nullptr;
+    if (!A.vlist && !A.rlist) A.list.dig = nullptr;
     ++P->launches;
     HFMM_TRY(s6_run(A, st));
     if (apart) {
-        A.list = s6_fam(lv.mult, lv, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false), -1);
-        A.shift.src = nullptr;
+        A.list = s6_fam(lv.s6_dmult, lv.p, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false));
+        A.shift.dig = nullptr;
         A.vlist = 0;
         A.rlist = 1;
         A.rows = 2;

@@ -1,0 +1,72 @@
+// FP64 numbers as six signed base-512 digits in f16 (see split64.cu): exponents,
+// fixed-point words with biased digit fields, digit pairs, and the FP32
+// mma.sync that sums digit products without rounding.
+#pragma once
+
+#include "common.cuh"
+
+constexpr int ND = 6;                    // digits
+constexpr int S6_NONE = -(1 << 24);      // exponent of an all-zero level (or below)
+constexpr long long S6_BIAS = 0x100804020100ll;   // 256 sum_{i = 0 .. 4} 512^i: low five fields = digit + 256
+constexpr int S6_NAN = 1 << 20;          // exponent of a level with an infinity or a NaN
+
+// largest E with |v 2^shift| < 2^E (S6_NONE for zero)
+__device__ __forceinline__ int s6_exponent(double v, int shift) {
+    const long long b = __double_as_longlong(v);
+    const int e = (int)((b >> 52) & 2047);
+    if (e == 2047) return S6_NAN;
+    if (e == 0) return (b & 0xfffffffffffffll) ? -1021 + shift : S6_NONE;
+    return e - 1022 + shift;
+}
+
+// v 2^shift 2^(BITS - E) rounded to an integer plus the digit bias, |v 2^shift| < 2^E
+template <int BITS>
+__device__ __forceinline__ long long s6_fixed(double v, int shift, int E) {
+    const long long b = __double_as_longlong(v);
+    int e = (int)((b >> 52) & 2047);
+    unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
+    if (e) m |= 1ull << 52; else e = 1;
+    const int s = E - shift - e + 1075 - BITS;            // right shift, >= 0 for BITS = 53
+    if (s > 0) m = s > 54 ? 0ull : (m + (1ull << (s - 1))) >> s;
+    const long long x = b < 0 ? -(long long)m : (long long)m;
+    return x + S6_BIAS;
+}
+
+// field of digit i (0 = most significant), digit + 256 in [0, 512]
+__device__ __forceinline__ unsigned s6_field(long long xb, int i) {
+    return i == 0 ? (unsigned)((int)(xb >> 45) + 256) : (unsigned)(xb >> (9 * (ND - 1 - i))) & 511u;
+}
+
+// two digits as f16 (1024 + field as bits 0x6400 | field, minus 1280)
+__device__ __forceinline__ unsigned s6_half2(unsigned f0, unsigned f1) {
+    unsigned h = 0x64006400u + (f0 | (f1 << 16)), r;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x65006500u));
+    return r;
+}
+
+// 2^e as a double (0 below the subnormals, infinite above the range)
+__device__ __forceinline__ double pow2d(int e) {
+    const long long b = e > 1023 ? 0x7ff0000000000000ll : e >= -1022 ? (long long)(e + 1023) << 52
+                        : e >= -1074 ? 1ll << (e + 1074) : 0ll;
+    return __longlong_as_double(b);
+}
+
+// an integer below 2^51 in magnitude as a double: one FP64 addition
+__device__ __forceinline__ double int51d(long long x) {
+    return __longlong_as_double(0x4338000000000000ll + x) - 6755399441055744.0;   // 1.5 2^52
+}
+
+__device__ __forceinline__ void s6_mma(float (&c)[4], const uint4& a, const uint2& b) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
+}
+
+// 16-byte asynchronous copy to shared memory (zeros where !ok), its commit, and
+// the wait until at most N committed groups are in flight
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
