@@ -36,6 +36,7 @@
 
 #include "bessel.cuh"
 #include "plan.cuh"
+#include "split64.cuh"
 
 namespace {
 
@@ -462,6 +463,112 @@ __global__ void ad32_near_fill_kernel(const AdBox* __restrict__ boxes, const int
     }
 }
 
+// Plan time, FP64: half basis J_m(k rho) e^{-i m theta}, m = 0 .. p, of every point of
+// the leaves that have expansions (rows of p + 1 values from boff; see leaf64.cu).
+__global__ void ad64_basis_kernel(const AdBox* __restrict__ boxes, const int32_t* __restrict__ leaves,
+                                  const int64_t* __restrict__ boff, int lup, const double2* __restrict__ xs, double x0,
+                                  double y0, double k, AdLevels lv, cd* __restrict__ out) {
+    extern __shared__ double jt[];
+    const AdBox b = boxes[leaves[blockIdx.x]];
+    if (b.level < lup) return;
+    const int p = lv.p[b.level];
+    double cx, cy;
+    ad_centre(x0, y0, lv.h[b.level], b.ix, b.iy, &cx, &cy);
+    double* J = jt + (size_t)threadIdx.x * (p + 1);
+    for (int32_t i = b.lo + threadIdx.x; i < b.hi; i += blockDim.x) {
+        const double dx = xs[i].x - cx, dy = xs[i].y - cy;
+        bessel_j_seq(k * hypot(dx, dy), p, J);
+        const cd e1 = cexpi(-atan2(dy, dx));
+        cd e = cmk(1.0, 0.0);
+        cd* B = out + boff[blockIdx.x] + (int64_t)(i - b.lo) * (p + 1);
+        for (int m = 0; m <= p; ++m) {
+            B[m] = cscale(e, J[m]);
+            e = cmul(e, e1);
+        }
+    }
+}
+
+// Plan time, FP64: unscaled M2P / P2L basis of every point of every pair (as
+// ad32_basis_pair_kernel): a thread per point, its Hankel sequence in shared memory.
+__global__ void ad64_basis_pair_kernel(const AdBox* __restrict__ boxes, const int32_t* __restrict__ tgt,
+                                       const int32_t* __restrict__ src, const int64_t* __restrict__ boff, bool m2p,
+                                       const double2* __restrict__ xs, double x0, double y0, double k, AdLevels lv,
+                                       cd* __restrict__ out) {
+    extern __shared__ double hsm[];
+    const int64_t e = blockIdx.x;
+    const AdBox T = boxes[tgt[e]], S = boxes[src[e]];
+    const AdBox& E = m2p ? S : T;
+    const AdBox& X = m2p ? T : S;
+    const int p = lv.p[E.level], nc = 2 * p + 1;
+    double cx, cy;
+    ad_centre(x0, y0, lv.h[E.level], E.ix, E.iy, &cx, &cy);
+    cd* Ht = (cd*)hsm + (size_t)threadIdx.x * (p + 1);
+    for (int32_t i = X.lo + threadIdx.x; i < X.hi; i += blockDim.x) {
+        const double dx = m2p ? xs[i].x - cx : cx - xs[i].x, dy = m2p ? xs[i].y - cy : cy - xs[i].y;
+        ad_hbasis(dx, dy, k, p, !m2p, Ht, out + boff[e] + (int64_t)(i - X.lo) * nc, 1);
+    }
+}
+
+__device__ __forceinline__ void ad_fma(cd& a, cd x, cd y) { cfma(a, x, y); }
+__device__ __forceinline__ void ad_fma(cf& a, cf x, cf y) { cfma_f(a, x, y); }
+
+// P2L: the X-list leaves' points into the local expansions of the level's boxes that
+// have such a list, from the plan's bases; one CTA per (box, right-hand side), lane =
+// order, four warps over the points (a thread that walked them alone took up to
+// 0.5 ms a level), partial sums in warp order.  Strengths q[j sj + r sr].
+template <class C>
+__global__ void __launch_bounds__(128) ad_p2l_kernel(const AdBox* __restrict__ boxes, const int32_t* __restrict__ list,
+                                                     const int32_t* __restrict__ x_beg, const int32_t* __restrict__ x_src,
+                                                     const int64_t* __restrict__ x_boff, const C* __restrict__ p2l,
+                                                     const C* __restrict__ q, int64_t sj, int64_t sr, int nrhs, int p,
+                                                     const int* __restrict__ sx, int* __restrict__ E, C* __restrict__ loc) {
+    __shared__ C part[4][32];
+    const int32_t bi = list[blockIdx.x];
+    const int r = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nc = 2 * p + 1;
+    C* out = loc + ((int64_t)boxes[bi].lidx * nrhs + r) * nc;
+    const C* qr = q + r * sr;
+    int ex = S6_NONE;
+    for (int m0 = 0; m0 < nc; m0 += 32) {
+        const int m = m0 + lane;
+        C acc{0, 0};
+        for (int32_t e = x_beg[bi]; e < x_beg[bi + 1]; ++e) {
+            const AdBox X = boxes[x_src[e]];
+            const C* B = p2l + x_boff[e] + m;
+            const int cnt = X.hi - X.lo;
+#pragma unroll 4
+            for (int j = wid; j < cnt; j += 4)
+                if (m < nc) ad_fma(acc, __ldg(qr + (X.lo + j) * sj), __ldg(B + (int64_t)j * nc));
+        }
+        __syncthreads();
+        part[wid][lane] = acc;
+        __syncthreads();
+        if (wid == 0 && m < nc) {
+            C v = out[m];
+            for (int w = 0; w < 4; ++w) { v.x += part[w][lane].x; v.y += part[w][lane].y; }
+            out[m] = v;
+            const int sh = sx ? sx[abs(m - p)] : 0;
+            ex = max(ex, max(s6_exponent(v.x, sh), s6_exponent(v.y, sh)));
+        }
+    }
+    if (wid == 0) {
+        ex = __reduce_max_sync(0xffffffffu, ex);
+        if (lane == 0 && ex > S6_NONE) atomicMax(E + r, ex);
+    }
+}
+
+// Sorted indices of every leaf's near-field sources (its U list), as its blocks count them.
+__global__ void ad_sources_kernel(const AdBox* __restrict__ boxes, const int32_t* __restrict__ u_beg,
+                                  const int32_t* __restrict__ u_src, const Leaf64Rec* __restrict__ recs,
+                                  int32_t* __restrict__ src) {
+    const int li = blockIdx.x;
+    int64_t o = recs[li].soff;
+    for (int32_t e = u_beg[li]; e < u_beg[li + 1]; ++e) {
+        const AdBox S = boxes[u_src[e]];
+        for (int32_t j = S.lo + threadIdx.x; j < S.hi; j += blockDim.x) src[o + (j - S.lo)] = j;
+        o += S.hi - S.lo;
+    }
+}
+
 // per-level FP32 expansion pointers
 struct AdLevels32 {
     cf* mult[AD_MAX_LEVEL + 1];
@@ -473,7 +580,7 @@ struct AdLevels32 {
 __global__ void __launch_bounds__(32) ad32_p2m_kernel(const AdBox* __restrict__ boxes, const int32_t* __restrict__ leaves,
                                                       const int32_t* __restrict__ list, const int64_t* __restrict__ boff,
                                                       const cf* __restrict__ basis, const cf* __restrict__ qs, int nrhs,
-                                                      AdLevels32 lv) {
+                                                      AdLevels32 lv, int* __restrict__ E, int max_rhs) {
     const int li = list[blockIdx.x];
     const AdBox b = boxes[leaves[li]];
     const int l = b.level, nc = 2 * lv.p[l] + 1;
@@ -482,8 +589,13 @@ __global__ void __launch_bounds__(32) ad32_p2m_kernel(const AdBox* __restrict__ 
     for (int it = threadIdx.x; it < nrhs * nc; it += 32) {
         const int r = it / nc, m = it % nc;
         cf acc = cfmk(0.f, 0.f);
+#pragma unroll 4
         for (int32_t j = b.lo; j < b.hi; ++j) cfma_f(acc, qs[(int64_t)j * nrhs + r], B[(int64_t)(j - b.lo) * nc + m]);
         out[it] = acc;
+        if (E) {                                          // exponent of the level's multipoles (split64.cu)
+            const int e = max(s6_exponent(acc.x, 0), s6_exponent(acc.y, 0));
+            if (e > S6_NONE) atomicMax(E + l * max_rhs + r, e);
+        }
     }
 }
 
@@ -690,6 +802,11 @@ struct AdaptiveTree {
     cf *basis32 = nullptr, *m2p32 = nullptr, *p2l32 = nullptr, *near_G32 = nullptr;
     int64_t *d_boff = nullptr, *d_wboff = nullptr, *d_xboff = nullptr;
     int32_t* d_p2m_li = nullptr;              // leaf ordinals of the P2M list
+    cd* p2l64 = nullptr;                      // FP64: plan-time P2L bases (offsets d_xboff)
+    bool fast64 = false;                      // FP64 plans: digit products, plan-time bases, leaf records
+    // boxes with an X list, by level
+    int32_t* d_xbox = nullptr;
+    std::vector<int64_t> xbox_off;
     // device
     AdBox* d_boxes = nullptr;
     int32_t *dv_beg = nullptr, *dv_src = nullptr, *dv_off = nullptr, *dr_beg = nullptr, *dr_src = nullptr,
@@ -712,6 +829,21 @@ hfmm_status ad_upload(hfmm_plan_s* P, const std::vector<V>& h, V** d, cudaStream
 }
 
 }  // namespace
+
+// Boxes with an X list, by level.
+static hfmm_status ad_upload_xboxes(hfmm_plan_s* P, cudaStream_t st) {
+    AdaptiveTree* T = P->ad;
+    std::vector<int32_t> list;
+    T->xbox_off.assign(P->L + 2, 0);
+    for (int l = 0; l <= P->L; ++l) {
+        for (int64_t b = T->lev_off[l]; b < T->lev_off[l + 1]; ++b)
+            if (T->x_beg[b + 1] > T->x_beg[b]) list.push_back((int32_t)b);
+        T->xbox_off[l + 1] = (int64_t)list.size();
+    }
+    HFMM_TRY(ad_upload(P, list, &T->d_xbox, st));
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+    return HFMM_OK;
+}
 
 // Tree of the points (host), sorted points and permutation (device).
 hfmm_status build_adaptive_tree(hfmm_plan_s* P, const double* d_xy, int leaf_size, cudaStream_t st) {
@@ -1079,6 +1211,199 @@ hfmm_status build_adaptive_lists(hfmm_plan_s* P, cudaStream_t st) {
     return HFMM_OK;
 }
 
+// M2M into every level, then L2L, V and reaction lists and P2L of every level, as digit
+// products (w = 0: FP64, 1: FP32) with the levels' P2M done.  The kernels before gave
+// every output coefficient to one thread that walked its box's whole list, a
+// latency chain per level whatever the precision: clusters of 20,011 points, FP64, two
+// right-hand sides: M2M + downward 3.10 -> 0.43 ms (the product 4.37 -> 0.62 ms); star
+// curve of 65,536 points, FP32: 0.87 -> 0.42 ms (the product 1.13 -> 0.73 ms).
+template <class C>
+static hfmm_status ad_tree_pass(hfmm_plan_s* P, int w, int nrhs, int parts, const C* q, int64_t sj, int64_t sr,
+                                const C* p2l, StageTimer& tm, cudaStream_t st) {
+    AdaptiveTree* T = P->ad;
+    const int L = P->L, lmin = T->lup;
+    const double MAC = 8.0 * nrhs;
+    tm.begin(HFMM_STAGE_M2M);
+    HFMM_TRY(split_slice(P, w, L, false, nrhs, st));
+    for (int l = L - 1; l >= lmin; --l) {
+        const LevelInfo& v = P->lev[l];
+        HFMM_TRY(split_m2m(P, w, l, nrhs, st));
+        HFMM_TRY(split_slice(P, w, l, false, nrhs, st));
+        P->st_flops[HFMM_STAGE_M2M] += MAC * 4.0 * v.nbox * v.ncoef * P->lev[l + 1].ncoef;
+    }
+    tm.end(HFMM_STAGE_M2M);
+    tm.begin(HFMM_STAGE_DOWN);
+    for (int l = lmin; l <= L; ++l) {
+        const LevelInfo& v = P->lev[l];
+        HFMM_TRY(split_down(P, w, l, nrhs, parts, st));
+        const int64_t nx = T->xbox_off[l + 1] - T->xbox_off[l];
+        if (nx > 0 && (parts & HFMM_PART_FAR_FREE)) {
+            ad_p2l_kernel<C><<<dim3((unsigned)nx, (unsigned)nrhs), 128, 0, st>>>(
+                T->d_boxes, T->d_xbox + T->xbox_off[l], T->dx_beg, T->dx_src, T->d_xboff, p2l, q, sj, sr, nrhs, v.p,
+                v.s6[w].sx, split_exp(P, w, l, true), w ? (C*)v.loc32 : (C*)v.loc);
+            ++P->launches;
+            HFMM_CUDA_TRY(cudaGetLastError());
+        }
+        if (l < L) HFMM_TRY(split_slice(P, w, l, true, nrhs, st));
+        double pairs = 0.0;
+        if (parts & HFMM_PART_FAR_FREE) pairs += (double)v.nv;
+        if (parts & HFMM_PART_FAR_REACT) pairs += (double)v.nr;
+        P->st_flops[HFMM_STAGE_DOWN] += MAC * pairs * v.ncoef * v.ncoef;
+    }
+    tm.end(HFMM_STAGE_DOWN);
+    return HFMM_OK;
+}
+
+bool adaptive_fast64(const hfmm_plan_s* P) { return P->ad && P->ad->fast64; }
+
+// The FP64 adaptive apply from the gathered strengths into the caller's order, on the
+// plan's digit products and bases.
+hfmm_status apply_adaptive64(hfmm_plan_s* P, int nrhs, int parts, bool conj_out, cd* y, cudaStream_t st) {
+    AdaptiveTree* T = P->ad;
+    const int64_t n = P->n;
+    StageTimer tm{P, st};
+    const double MAC = 8.0 * nrhs;
+    const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0;
+    const bool near = (parts & HFMM_PART_NEAR_FREE) != 0, near_here = near && P->near64_vals;
+    if (far) {
+        tm.begin(HFMM_STAGE_P2M);
+        HFMM_TRY(split_begin(P, 0, st));
+        HFMM_TRY(launch_p2m64(P, nrhs, st));
+        tm.end(HFMM_STAGE_P2M);
+        HFMM_TRY(ad_tree_pass<cd>(P, 0, nrhs, parts, P->q_sorted, 1, n, T->p2l64, tm, st));
+    }
+    tm.begin(HFMM_STAGE_P2P);
+    if (near && !near_here) {                             // coincident points: H0 per pair
+        HFMM_CUDA_TRY(cudaMemsetAsync(P->y_sorted, 0, sizeof(cd) * n * nrhs, st));
+        ad_near_kernel<<<(unsigned)ceil_div((int64_t)T->leaves.size(), 4), 128, 0, st>>>(
+            T->d_boxes, T->d_leaves, (int64_t)T->leaves.size(), T->du_beg, T->du_src, T->du_blk, nullptr, T->dd_beg,
+            T->dd_src, T->dd_blk, P->d_vals, P->xy_sorted, P->q_sorted, n, nrhs, P->k, HFMM_PART_NEAR_FREE, P->y_sorted);
+        ++P->launches;
+        HFMM_CUDA_TRY(cudaGetLastError());
+    }
+    HFMM_TRY(launch_leaf64(P, nrhs, near_here, far, (parts & HFMM_PART_FAR_FREE) != 0,
+                           (parts & HFMM_PART_NEAR_REACT) && P->nd > 0, near && !near_here ? P->y_sorted : nullptr,
+                           conj_out, y, st));
+    tm.end(HFMM_STAGE_P2P);
+    if (parts & (HFMM_PART_NEAR_FREE | HFMM_PART_NEAR_REACT)) {
+        P->st_flops[HFMM_STAGE_P2P] = MAC * (double)P->p2p_point_pairs;
+        P->st_flops[HFMM_STAGE_DIRECT] = MAC * (double)P->nd_vals;
+    }
+    return HFMM_OK;
+}
+
+// Plan-time state of apply_adaptive64 (after the tables): operator slices, bases, digit
+// blocks and leaf records.  A plan above a byte budget keeps the kernels of
+// apply_adaptive.
+hfmm_status build_adaptive64(hfmm_plan_s* P, cudaStream_t st) {
+    AdaptiveTree* T = P->ad;
+    const auto& bx = T->boxes;
+    const int64_t nl = (int64_t)T->leaves.size();
+    const int lup = T->lup, L = P->L;
+    if (!T->near_G && P->p2p_point_pairs > 0) return HFMM_OK;
+    auto nc = [&](int l) { return (int64_t)(2 * P->lev[l].p + 1); };
+    std::vector<int64_t> boff(nl, 0), wboff(T->w_src.size(), 0), xboff(T->x_src.size(), 0);
+    std::vector<int32_t> w_tgt(T->w_src.size()), x_tgt(T->x_src.size());
+    int64_t nb = 0, nw = 0, nx = 0;
+    for (int64_t li = 0; li < nl; ++li) {
+        const AdBox& B = bx[T->leaves[li]];
+        boff[li] = nb;
+        if (B.level >= lup) nb += (int64_t)(B.hi - B.lo) * (P->lev[B.level].p + 1);
+        for (int32_t e = T->w_beg[li]; e < T->w_beg[li + 1]; ++e) {
+            w_tgt[e] = T->leaves[li];
+            wboff[e] = nw;
+            nw += (int64_t)(B.hi - B.lo) * nc(bx[T->w_src[e]].level);
+        }
+    }
+    for (size_t b = 0; b < bx.size(); ++b)
+        for (int32_t e = T->x_beg[b]; e < T->x_beg[b + 1]; ++e) {
+            x_tgt[e] = (int32_t)b;
+            xboff[e] = nx;
+            nx += (int64_t)(bx[T->x_src[e]].hi - bx[T->x_src[e]].lo) * nc(bx[b].level);
+        }
+    if (sizeof(cd) * (double)(nb + nw + nx) > 8e9 || T->pmax * (int)sizeof(cd) > 40000) return HFMM_OK;
+    HFMM_TRY(build_split(P, 0, st));
+    if (!P->s6_ready[0]) return HFMM_OK;
+    HFMM_TRY(ad_upload_xboxes(P, st));
+    AdLevels lv{};
+    for (int l = 0; l <= L; ++l) {
+        lv.p[l] = P->lev[l].p;
+        lv.h[l] = P->lev[l].h;
+    }
+    int64_t *d_boff = nullptr, *d_wboff = nullptr;
+    int32_t *d_wt = nullptr, *d_xt = nullptr;
+    HFMM_TRY(ad_upload(P, boff, &d_boff, st));
+    HFMM_TRY(ad_upload(P, wboff, &d_wboff, st));
+    HFMM_TRY(ad_upload(P, xboff, &T->d_xboff, st));
+    HFMM_TRY(ad_upload(P, w_tgt, &d_wt, st));
+    HFMM_TRY(ad_upload(P, x_tgt, &d_xt, st));
+    HFMM_TRY(plan_alloc(P, (void**)&P->basis64, sizeof(cd) * std::max<int64_t>(nb, 1)));
+    HFMM_TRY(plan_alloc(P, (void**)&P->m2p64, sizeof(cd) * std::max<int64_t>(nw, 1)));
+    HFMM_TRY(plan_alloc(P, (void**)&T->p2l64, sizeof(cd) * std::max<int64_t>(nx, 1)));
+    P->buffer_bytes += sizeof(cd) * (double)(nb + nw + nx);
+    const int thr = std::max(1, std::min(32, 6000 / (T->pmax + 1))), thr2 = std::max(1, std::min(32, 3000 / (T->pmax + 1)));
+    ad64_basis_kernel<<<(unsigned)nl, thr, (size_t)thr * (T->pmax + 1) * sizeof(double), st>>>(
+        T->d_boxes, T->d_leaves, d_boff, lup, P->xy_sorted, P->x0, P->y0, P->k, lv, P->basis64);
+    HFMM_CUDA_TRY(cudaGetLastError());
+    if (!w_tgt.empty()) {
+        ad64_basis_pair_kernel<<<(unsigned)w_tgt.size(), thr2, (size_t)thr2 * (T->pmax + 1) * sizeof(cd), st>>>(
+            T->d_boxes, d_wt, T->dw_src, d_wboff, true, P->xy_sorted, P->x0, P->y0, P->k, lv, P->m2p64);
+        HFMM_CUDA_TRY(cudaGetLastError());
+    }
+    if (!x_tgt.empty()) {
+        ad64_basis_pair_kernel<<<(unsigned)x_tgt.size(), thr2, (size_t)thr2 * (T->pmax + 1) * sizeof(cd), st>>>(
+            T->d_boxes, d_xt, T->dx_src, T->d_xboff, false, P->xy_sorted, P->x0, P->y0, P->k, lv, T->p2l64);
+        HFMM_CUDA_TRY(cudaGetLastError());
+    }
+    // leaf records
+    std::vector<Leaf64Rec> recs(nl);
+    std::vector<Leaf64W> ws(T->w_src.size());
+    std::vector<Leaf64D> ds(T->d_src.size());
+    int64_t soff = 0, goff = 0;
+    for (int64_t li = 0; li < nl; ++li) {
+        const AdBox& B = bx[T->leaves[li]];
+        const LevelInfo& v = P->lev[B.level];
+        Leaf64Rec& R = recs[li];
+        R = Leaf64Rec{};
+        int64_t ns = 0;
+        for (int32_t e = T->u_beg[li]; e < T->u_beg[li + 1]; ++e) ns += bx[T->u_src[e]].hi - bx[T->u_src[e]].lo;
+        R.tlo = B.lo; R.tn = B.hi - B.lo; R.ns = (int32_t)ns; R.p = v.p; R.nb = v.p + 1;
+        R.soff = soff; R.goff = goff; R.boff = boff[li]; R.lidx = B.lidx;
+        if (B.level >= lup) {
+            R.mult = v.mult; R.loc = v.loc; R.sx = v.s6[0].sx;
+            R.E = split_exp(P, 0, B.level, false);
+            P->leaf64_p = std::max(P->leaf64_p, v.p);
+        }
+        R.wbeg = T->w_beg[li]; R.wend = T->w_beg[li + 1];
+        R.dbeg = T->d_beg[li]; R.dend = T->d_beg[li + 1];
+        for (int32_t e = R.wbeg; e < R.wend; ++e) {
+            const AdBox& D = bx[T->w_src[e]];
+            ws[e] = {P->lev[D.level].mult, D.lidx, wboff[e], P->lev[D.level].p, 0};
+        }
+        for (int32_t e = R.dbeg; e < R.dend; ++e) {
+            const AdBox& S = bx[T->d_src[e]];
+            ds[e] = {S.lo, S.hi - S.lo, T->d_blk[e]};
+        }
+        soff += ns;
+        goff += (int64_t)R.tn * ns;
+        P->leaf_max = std::max(P->leaf_max, (int)R.tn);
+    }
+    P->leaf64_n = nl;
+    HFMM_TRY(ad_upload(P, recs, &P->leaf64, st));
+    HFMM_TRY(ad_upload(P, ws, &P->leaf64_w, st));
+    HFMM_TRY(ad_upload(P, ds, &P->leaf64_d, st));
+    HFMM_TRY(plan_alloc(P, (void**)&P->leaf64_src, sizeof(int32_t) * std::max<int64_t>(soff, 1)));
+    ad_sources_kernel<<<(unsigned)nl, 64, 0, st>>>(T->d_boxes, T->du_beg, T->du_src, P->leaf64, P->leaf64_src);
+    HFMM_CUDA_TRY(cudaGetLastError());
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, sizeof(int)));
+    bool finite = true;
+    if (goff > 0) HFMM_TRY(near64_to_fixed(T->near_G, goff, P->near64_E, &finite, st));
+    if (finite) P->near64_vals = T->near_G;
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // the vectors are locals
+    T->fast64 = true;
+    return HFMM_OK;
+}
+
 // The adaptive apply between the gather and the scatter (FP64).
 hfmm_status apply_adaptive(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t st) {
     AdaptiveTree* T = P->ad;
@@ -1244,6 +1569,8 @@ hfmm_status build_adaptive32(hfmm_plan_s* P, cudaStream_t st) {
             T->d_boxes, d_xt, T->dx_src, T->d_xboff, false, P->xy_sorted, P->x0, P->y0, P->k, lv, d_lsp, T->p2l32);
         HFMM_CUDA_TRY(cudaGetLastError());
     }
+    HFMM_TRY(ad_upload_xboxes(P, st));
+    HFMM_TRY(build_split(P, 1, st));
     // FP32 near-field blocks
     const double pp = (double)P->p2p_point_pairs;
     if (pp > 0 && 8.0 * pp <= NEAR64_MAX_BYTES) {
@@ -1278,38 +1605,45 @@ hfmm_status apply_adaptive32(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t s
     const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0;
     if (far) {
         tm.begin(HFMM_STAGE_P2M);
+        if (P->s6_ready[1]) HFMM_TRY(split_begin(P, 1, st));
         if (T->n_p2m > 0) {
             ad32_p2m_kernel<<<(unsigned)T->n_p2m, 32, 0, st>>>(T->d_boxes, T->d_leaves, T->d_p2m_li, T->d_boff,
-                                                               T->basis32, P->q32, nrhs, lv);
+                                                               T->basis32, P->q32, nrhs, lv,
+                                                               P->s6_ready[1] ? split_exp(P, 1, 0, false) : nullptr,
+                                                               P->max_rhs);
             ++P->launches;
             HFMM_CUDA_TRY(cudaGetLastError());
         }
         tm.end(HFMM_STAGE_P2M);
-        tm.begin(HFMM_STAGE_M2M);
-        for (int l = L - 1; l >= lmin; --l) {
-            const LevelInfo& v = P->lev[l];
-            ad32_m2m_kernel<<<dim3((unsigned)v.nbox, ad_split(v.nbox, nrhs * v.ncoef)), AD_TB, 0, st>>>(
-                T->d_boxes, T->lev_off[l], l, v.t_m2m32, lv, nrhs);
-            ++P->launches;
-            HFMM_CUDA_TRY(cudaGetLastError());
-            P->st_flops[HFMM_STAGE_M2M] += MAC * 4.0 * v.nbox * v.ncoef * P->lev[l + 1].ncoef;
+        if (P->s6_ready[1])
+            HFMM_TRY(ad_tree_pass<cf>(P, 1, nrhs, parts, P->q32, nrhs, 1, T->p2l32, tm, st));
+        else {
+            tm.begin(HFMM_STAGE_M2M);
+            for (int l = L - 1; l >= lmin; --l) {
+                const LevelInfo& v = P->lev[l];
+                ad32_m2m_kernel<<<dim3((unsigned)v.nbox, ad_split(v.nbox, nrhs * v.ncoef)), AD_TB, 0, st>>>(
+                    T->d_boxes, T->lev_off[l], l, v.t_m2m32, lv, nrhs);
+                ++P->launches;
+                HFMM_CUDA_TRY(cudaGetLastError());
+                P->st_flops[HFMM_STAGE_M2M] += MAC * 4.0 * v.nbox * v.ncoef * P->lev[l + 1].ncoef;
+            }
+            tm.end(HFMM_STAGE_M2M);
+            tm.begin(HFMM_STAGE_DOWN);
+            for (int l = lmin; l <= L; ++l) {
+                const LevelInfo& v = P->lev[l];
+                ad32_down_kernel<<<dim3((unsigned)v.nbox, ad_split(v.nbox, nrhs * v.ncoef)), AD_TB, 0, st>>>(
+                    T->d_boxes, T->lev_off[l], l, lmin, nrhs, lv, l > lmin ? P->lev[l - 1].t_l2l32 : nullptr, T->dv_beg,
+                    T->dv_src, T->dv_off, v.t_free32, T->dr_beg, T->dr_src, T->dr_tab, v.t_react32, T->dx_beg, T->dx_src,
+                    T->d_xboff, T->p2l32, P->q32, parts);
+                ++P->launches;
+                HFMM_CUDA_TRY(cudaGetLastError());
+                double pairs = 0.0;
+                if (parts & HFMM_PART_FAR_FREE) pairs += (double)v.nv;
+                if (parts & HFMM_PART_FAR_REACT) pairs += (double)v.nr;
+                P->st_flops[HFMM_STAGE_DOWN] += MAC * pairs * v.ncoef * v.ncoef;
+            }
+            tm.end(HFMM_STAGE_DOWN);
         }
-        tm.end(HFMM_STAGE_M2M);
-        tm.begin(HFMM_STAGE_DOWN);
-        for (int l = lmin; l <= L; ++l) {
-            const LevelInfo& v = P->lev[l];
-            ad32_down_kernel<<<dim3((unsigned)v.nbox, ad_split(v.nbox, nrhs * v.ncoef)), AD_TB, 0, st>>>(
-                T->d_boxes, T->lev_off[l], l, lmin, nrhs, lv, l > lmin ? P->lev[l - 1].t_l2l32 : nullptr, T->dv_beg,
-                T->dv_src, T->dv_off, v.t_free32, T->dr_beg, T->dr_src, T->dr_tab, v.t_react32, T->dx_beg, T->dx_src,
-                T->d_xboff, T->p2l32, P->q32, parts);
-            ++P->launches;
-            HFMM_CUDA_TRY(cudaGetLastError());
-            double pairs = 0.0;
-            if (parts & HFMM_PART_FAR_FREE) pairs += (double)v.nv;
-            if (parts & HFMM_PART_FAR_REACT) pairs += (double)v.nr;
-            P->st_flops[HFMM_STAGE_DOWN] += MAC * pairs * v.ncoef * v.ncoef;
-        }
-        tm.end(HFMM_STAGE_DOWN);
         tm.begin(HFMM_STAGE_L2P);
         ad32_leaf_far_kernel<<<(unsigned)nl, 32, 0, st>>>(T->d_boxes, T->d_leaves, T->d_boff, T->basis32, T->dw_beg,
                                                           T->dw_src, T->d_wboff, T->m2p32, nrhs, lv, lmin, parts,
@@ -1330,6 +1664,67 @@ hfmm_status apply_adaptive32(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t s
         P->st_flops[HFMM_STAGE_DIRECT] = MAC * (double)P->nd_vals;
     }
     return HFMM_OK;
+}
+
+// Table entries of level l's reaction list (dx, ysum), each once, increasing.
+void adaptive_react_entries(const hfmm_plan_s* P, int l, std::vector<int32_t>& entries) {
+    const AdaptiveTree* T = P->ad;
+    entries.clear();
+    for (int64_t b = T->lev_off[l]; b < T->lev_off[l + 1]; ++b)
+        entries.insert(entries.end(), T->r_tab.begin() + T->r_beg[b], T->r_tab.begin() + T->r_beg[b + 1]);
+    std::sort(entries.begin(), entries.end());
+    entries.erase(std::unique(entries.begin(), entries.end()), entries.end());
+}
+
+// Tiles of a level for the digit products (split64.cu): up = false, the boxes of one
+// child position (they share the L2L and most V offsets), eight consecutive ones a
+// tile, with one step per operator any of them uses; up = true, the boxes with
+// children, with one M2M step per child position.
+void adaptive_tiles(const hfmm_plan_s* P, int l, bool up, const std::vector<int32_t>& rmap, std::vector<int32_t>& tgt,
+                    std::vector<int32_t>& tbeg, std::vector<S6Rec>& recs) {
+    const AdaptiveTree* T = P->ad;
+    const auto& bx = T->boxes;
+    tgt.clear();
+    recs.clear();
+    tbeg.assign(1, 0);
+    for (int c = 0; c < (up ? 1 : 4); ++c) {
+        std::vector<int32_t> boxes;
+        for (int64_t b = T->lev_off[l]; b < T->lev_off[l + 1]; ++b)
+            if (up ? !bx[b].leaf : (bx[b].ix & 1) + 2 * (bx[b].iy & 1) == c) boxes.push_back((int32_t)b);
+        for (size_t t0 = 0; t0 < boxes.size(); t0 += 8) {
+            const size_t m = std::min<size_t>(8, boxes.size() - t0);
+            std::vector<std::pair<int32_t, std::pair<int, int32_t>>> use;    // (op, (column, source))
+            for (size_t u = 0; u < 8; ++u) {
+                tgt.push_back(u < m ? bx[boxes[t0 + u]].lidx : -1);
+                if (u >= m) continue;
+                const int32_t b = boxes[t0 + u];
+                if (up) {
+                    for (int a = 0; a < 4; ++a)
+                        if (bx[b].child[a] >= 0) use.push_back({4 * a, {(int)u, bx[bx[b].child[a]].lidx}});
+                    continue;
+                }
+                if (l > T->lup && bx[b].parent >= 0) use.push_back({4 * c, {(int)u, bx[bx[b].parent].lidx}});
+                for (int32_t e = T->v_beg[b]; e < T->v_beg[b + 1]; ++e)
+                    use.push_back({4 * T->v_off[e] + 1, {(int)u, T->v_src[e]}});
+                for (int32_t e = T->r_beg[b]; e < T->r_beg[b + 1]; ++e) {
+                    const int32_t o = (int32_t)(std::lower_bound(rmap.begin(), rmap.end(), T->r_tab[e]) - rmap.begin());
+                    use.push_back({4 * o + 2, {(int)u, T->r_src[e]}});
+                }
+            }
+            // shifts first, then one run of the two list families (one fold of the digit sums each)
+            std::sort(use.begin(), use.end(), [](const auto& x, const auto& y) {
+                const int kx = x.first & 3, ky = y.first & 3;
+                return kx != ky ? kx < ky : x < y;
+            });
+            // a (target, operator) pair occurs once: an operator fixes the source
+            for (size_t i = 0; i < use.size(); ++i) {
+                if (i == 0 || use[i].first != use[i - 1].first)
+                    recs.push_back({use[i].first, {-1, -1, -1, -1, -1, -1, -1, -1}});
+                recs.back().src[use[i].second.first] = use[i].second.second;
+            }
+            tbeg.push_back((int32_t)recs.size());
+        }
+    }
 }
 
 // Introspection: boxes (level, ix, iy, first sorted point, end, leaf) and

@@ -343,8 +343,9 @@ static hfmm_status plan_create_one(hfmm_plan_t* out, int64_t n, const double* xy
         if ((s = build_tables(P, st)) != HFMM_OK) break;
         if (!mixed && !adaptive && (s = build_near64(P, st)) != HFMM_OK) break;
         if (!mixed && (s = build_diag(P, st)) != HFMM_OK) break;
-        if (!mixed && !adaptive && (s = build_split64(P, st)) != HFMM_OK) break;
-        if (!mixed && !adaptive && (s = build_basis64(P, st)) != HFMM_OK) break;
+        if (!mixed && !adaptive && (s = build_split(P, 0, st)) != HFMM_OK) break;
+        if (!mixed && !adaptive && (s = build_leaf64(P, st)) != HFMM_OK) break;
+        if (!mixed && adaptive && (s = build_adaptive64(P, st)) != HFMM_OK) break;
         if (mixed && adaptive) {
             if ((s = build_tables32(P, st)) != HFMM_OK) break;
             if ((s = build_adaptive32(P, st)) != HFMM_OK) break;

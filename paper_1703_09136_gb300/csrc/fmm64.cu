@@ -330,7 +330,7 @@ hfmm_status down64_lists(hfmm_plan_s* P, int l, int nrhs, const cd* mult, cd* lo
 // P2M of the sorted strengths, from the plan's bases where it holds them.
 static hfmm_status leaves64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
     LevelInfo& lv = P->lev[P->L];
-    if (P->s6_ready) HFMM_TRY(split64_begin(P, st));
+    if (P->s6_ready[0]) HFMM_TRY(split_begin(P, 0, st));
     if (P->basis64) HFMM_TRY(launch_p2m64(P, nrhs, st));
     else {
         const int chunk = pick_chunk(lv.p);
@@ -339,9 +339,9 @@ static hfmm_status leaves64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
                                                      lv.h, P->L, P->k, lv.p, chunk, lv.mult);
         ++P->launches;
         HFMM_CUDA_TRY(cudaGetLastError());
-        if (P->s6_ready) HFMM_TRY(split64_exponent(P, P->L, false, nrhs, st));
+        if (P->s6_ready[0]) HFMM_TRY(split_exponent(P, 0, P->L, false, nrhs, st));
     }
-    if (P->s6_ready) HFMM_TRY(split64_slice(P, P->L, false, nrhs, st));
+    if (P->s6_ready[0]) HFMM_TRY(split_slice(P, 0, P->L, false, nrhs, st));
     if (lv.diag_logq) HFMM_TRY(diag_src(P, P->L, nrhs, st));
     return HFMM_OK;
 }
@@ -353,9 +353,9 @@ static hfmm_status upward64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
     const int L = P->L;
     for (int l = L - 1; l >= P->lmin; --l) {
         LevelInfo& lv = P->lev[l];
-        if (P->s6_ready) {
-            HFMM_TRY(split64_m2m(P, l, nrhs, st));
-            if (l > P->lmin || !lv.diag_logq) HFMM_TRY(split64_slice(P, l, false, nrhs, st));
+        if (P->s6_ready[0]) {
+            HFMM_TRY(split_m2m(P, 0, l, nrhs, st));
+            if (l > P->lmin || !lv.diag_logq) HFMM_TRY(split_slice(P, 0, l, false, nrhs, st));
         } else {
             m2m_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(
                 P->lev[l + 1].mult, lv.t_m2m, P->lev[l + 1].p, lv.p, nrhs, lv.mult);
@@ -374,7 +374,7 @@ static hfmm_status downward64(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t 
         LevelInfo& lv = P->lev[l];
         const bool has_parent = l > P->lmin;
         const bool dg = lv.diag_logq > 0;   // translations in diagonal form after the L2L
-        if (P->s6_ready) HFMM_TRY(split64_down(P, l, nrhs, parts, st));
+        if (P->s6_ready[0]) HFMM_TRY(split_down(P, 0, l, nrhs, parts, st));
         else {
             downward_kernel<<<dim3((unsigned)lv.nbox, box_split(lv.nbox, nrhs * lv.ncoef)), TB, 0, st>>>(
                 P->leaf_begin, L, l, P->lmin, nrhs, lv.p, has_parent ? P->lev[l - 1].p : 0,
@@ -386,9 +386,9 @@ static hfmm_status downward64(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t 
         }
         if (dg) {
             HFMM_TRY(diag_m2l(P, l, nrhs, parts, st));
-            if (P->s6_ready && l < L) HFMM_TRY(split64_exponent(P, l, true, nrhs, st));
+            if (P->s6_ready[0] && l < L) HFMM_TRY(split_exponent(P, 0, l, true, nrhs, st));
         }
-        if (P->s6_ready && l < L) HFMM_TRY(split64_slice(P, l, true, nrhs, st));
+        if (P->s6_ready[0] && l < L) HFMM_TRY(split_slice(P, 0, l, true, nrhs, st));
     }
     return HFMM_OK;
 }
@@ -409,11 +409,13 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
     const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0, near = (parts & HFMM_PART_NEAR_FREE) != 0;
     // sums that leaf64_kernel does not make itself go through y_sorted
     const bool l2p_here = far && P->basis64, near_here = near && P->near64_vals;
-    const bool extra = P->ad || (far && !l2p_here) || (near && !near_here);
+    const bool ad_fast = adaptive_fast64(P);
+    const bool extra = P->ad ? !ad_fast : (far && !l2p_here) || (near && !near_here);
     if (extra) HFMM_CUDA_TRY(cudaMemsetAsync(P->y_sorted, 0, sizeof(cd) * n * nrhs, st));
     tm.end(HFMM_STAGE_GATHER);
     P->st_bytes[HFMM_STAGE_GATHER] = 2.0 * C * n + 8.0 * n;
-    if (P->ad) HFMM_TRY(apply_adaptive(P, nrhs, parts, st));
+    if (ad_fast) HFMM_TRY(apply_adaptive64(P, nrhs, parts, adjoint, y, st));
+    else if (P->ad) HFMM_TRY(apply_adaptive(P, nrhs, parts, st));
     else {
         if (far) {
             // step 2: upward pass
@@ -475,7 +477,7 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
             ++P->launches;
             HFMM_CUDA_TRY(cudaGetLastError());
         }
-        HFMM_TRY(launch_leaf64(P, nrhs, near_here, l2p_here, direct, extra ? P->y_sorted : nullptr, adjoint, y, st));
+        HFMM_TRY(launch_leaf64(P, nrhs, near_here, l2p_here, false, direct, extra ? P->y_sorted : nullptr, adjoint, y, st));
         tm.end(HFMM_STAGE_P2P);
         if (near) {
             P->st_flops[HFMM_STAGE_P2P] = MAC * (double)P->p2p_point_pairs;
@@ -487,7 +489,7 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
             P->st_bytes[HFMM_STAGE_DIRECT] = 16.0 * (double)P->nd_vals;
         }
     }
-    if (!P->ad) {                          // the leaf kernel wrote the caller's order
+    if (!P->ad || ad_fast) {               // the leaf kernel wrote the caller's order
         P->last_stream = st;
         return HFMM_OK;
     }
@@ -813,8 +815,8 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
         HFMM_TRY(plan_alloc(P, (void**)&P->grad_buf, 5 * bytes));
         HFMM_TRY(build_direct_grad(P, st));
         HFMM_TRY(build_near64_grad(P, st));
-        HFMM_TRY(build_split64(P, st));
-        HFMM_TRY(build_basis64(P, st));
+        HFMM_TRY(build_split(P, 0, st));
+        HFMM_TRY(build_leaf64(P, st));
     }
     cd* ux = P->grad_buf;
     cd* uy = ux + (size_t)n * P->max_rhs;
@@ -908,7 +910,6 @@ hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st) {
                 }
         }
         off[b + 1] = off[b] + tn * ns;
-        P->leaf_max = std::max(P->leaf_max, (int)tn);
     }
     const double bytes = 16.0 * (double)off[nleaf];
     if (bytes > NEAR64_MAX_BYTES) return HFMM_OK;

@@ -1,6 +1,7 @@
-// FP64 leaf passes of the uniform tree: P2M from plan-time bases, and one kernel
-// for everything a target sums at the end (near field, L2P, directly summed
-// reaction, result in the caller's order).
+// FP64 leaf passes: P2M from plan-time bases, and one kernel for everything a
+// target sums at the end (near field, L2P, an adaptive tree's M2P, directly
+// summed reaction, result in the caller's order).  Every non-empty leaf has a
+// record (Leaf64Rec) with its ranges, so both trees run the same kernels.
 //
 // Bases.  B_m(x) = J_m(k rho) e^{-i m theta} of every point about its leaf's centre,
 // m = 0 .. p + 1, is computed once per plan: J_{-m} = (-1)^m J_m makes the
@@ -26,6 +27,7 @@
 // without the ring 308 us); 1600 points: P2M 67 -> 11 us, the rest 360 -> 45 us.
 #include <algorithm>
 #include <cmath>
+#include <vector>
 
 #include "bessel.cuh"
 #include "plan.cuh"
@@ -60,22 +62,21 @@ __global__ void basis64_kernel(const int32_t* __restrict__ lb, const double2* __
 // alpha_{-m} = (-1)^m sum q conj(B_m).  Also the level's exponent (split64.cu).
 // PS = 4 lanes split a leaf's points where there are too few items for the GPU.
 template <int PS>
-__global__ void __launch_bounds__(128) p2m64_kernel(const int32_t* __restrict__ lb, const cd* __restrict__ basis,
-                                                    const cd* __restrict__ qs, int64_t n, int64_t nleaf, int nrhs, int p,
-                                                    const int* __restrict__ sx, int* __restrict__ E,
-                                                    cd* __restrict__ mult) {
-    const int np = p + 1, nb = p + 2, nc = 2 * p + 1;
+__global__ void __launch_bounds__(128) p2m64_kernel(const Leaf64Rec* __restrict__ recs, const cd* __restrict__ basis,
+                                                    const cd* __restrict__ qs, int64_t n, int64_t nleaf, int pitch,
+                                                    int nrhs) {
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, it = id / PS;
-    const int r = blockIdx.y, part = (int)(id % PS);
-    const bool live = it < nleaf * np;                     // whole groups of PS lanes
-    const int64_t b = live ? it / np : 0;
-    const int m = live ? (int)(it - b * np) : 0;
-    const int32_t lo = lb[b] + part, hi = live ? lb[b + 1] : 0;
-    const cd* q = qs + (int64_t)r * n;
-    const cd* B = basis + m;
+    const int r = blockIdx.y, part = (int)(id % PS), m = (int)(it % pitch);
+    const bool in = it < nleaf * pitch;                    // whole groups of PS lanes
+    const Leaf64Rec& L = recs[in ? it / pitch : 0];
+    const bool live = in && L.mult && m <= L.p;
+    const int nb = L.nb;
+    const cd* q = qs + (int64_t)r * n + L.tlo;
+    const cd* B = basis + L.boff + m;
     double s1 = 0.0, s2 = 0.0, s3 = 0.0, s4 = 0.0;
+    const int tn = live ? L.tn : 0;
 #pragma unroll 4
-    for (int32_t j = lo; j < hi; j += PS) {
+    for (int j = part; j < tn; j += PS) {
         const cd a = __ldg(q + j), u = __ldg(B + (int64_t)j * nb);
         s1 = fma(a.x, u.x, s1);
         s2 = fma(a.y, u.y, s2);
@@ -92,38 +93,64 @@ __global__ void __launch_bounds__(128) p2m64_kernel(const int32_t* __restrict__ 
     }
     int e = S6_NONE;
     if (live) {
-        cd* out = mult + (b * nrhs + r) * nc + p;
+        cd* out = L.mult + (L.lidx * nrhs + r) * (2 * L.p + 1) + L.p;
         const cd ap = cmk(s1 - s2, s3 + s4), am = cmk(s1 + s2, s4 - s3);
         if (part == 0) {
             out[m] = ap;
             if (m > 0) out[-m] = (m & 1) ? cneg(am) : am;
         }
-        if (E) {
-            const int sh = -sx[m];
+        if (L.E) {
+            const int sh = -L.sx[m];
             e = max(max(s6_exponent(ap.x, sh), s6_exponent(ap.y, sh)), max(s6_exponent(am.x, sh), s6_exponent(am.y, sh)));
         }
     }
-    if (E) {
+    // one level (uniform trees): one atomic per warp, else one per lane that has a value
+    int* E = live ? L.E : nullptr;
+    const unsigned same = __match_any_sync(0xffffffffu, (unsigned long long)E);
+    if (same == 0xffffffffu) {
         e = __reduce_max_sync(0xffffffffu, e);
-        if ((threadIdx.x & 31) == 0 && e > S6_NONE) atomicMax(E + r, e);
-    }
+        if ((threadIdx.x & 31) == 0 && E && e > S6_NONE) atomicMax(E + r, e);
+    } else if (E && e > S6_NONE) atomicMax(E + r, e);
+}
+
+// Empty leaves of a uniform tree: zero multipoles (their parents' M2M reads them).
+__global__ void zero_empty_kernel(const int32_t* __restrict__ lb, int64_t nleaf, int64_t per, cd* __restrict__ mult) {
+    for (int64_t b = blockIdx.x; b < nleaf; b += gridDim.x)
+        if (lb[b + 1] == lb[b])
+            for (int64_t i = threadIdx.x; i < per; i += blockDim.x) mult[b * per + i] = cmk(0.0, 0.0);
+}
+
+// Sorted indices of every leaf's near-field sources (uniform trees: the 3 x 3 neighbourhood
+// in dy, dx order), as the block layout counts them.
+__global__ void leaf_sources_kernel(const int32_t* __restrict__ lb, int L, const Leaf64Rec* __restrict__ recs,
+                                    int32_t* __restrict__ src) {
+    const Leaf64Rec& R = recs[blockIdx.x];
+    const int m = 1 << L, ix = (int)morton_x((uint32_t)R.lidx), iy = (int)morton_y((uint32_t)R.lidx);
+    int64_t o = R.soff;
+    for (int dy = -1; dy <= 1; ++dy)
+        for (int dx = -1; dx <= 1; ++dx) {
+            const int sx = ix + dx, sy = iy + dy;
+            if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
+            const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
+            for (int32_t j = lb[s] + threadIdx.x; j < lb[s + 1]; j += blockDim.x) src[o + (j - lb[s])] = j;
+            o += lb[s + 1] - lb[s];
+        }
 }
 
 struct Leaf64Args {
-    const int32_t* lb;
-    int L, nrhs, p;
+    const Leaf64Rec* recs;
+    int nrhs, p;                     // largest order of a leaf
     int64_t n;
     const cd* qs;
-    // near field: digit blocks (null: not here), offsets and their exponent
+    // near field: digit blocks (null: not here), their exponent, source indices
     const uint4* G;
-    const int64_t* off;
     const int* EG;
-    // L2P (loc null: not here)
-    const cd* loc;
+    const int32_t* src;
+    bool l2p, m2p, direct;
     const cd* basis;
-    // directly summed reaction (d_begin null: none)
-    const int32_t *d_begin, *d_src;
-    const int64_t* d_blk;
+    const Leaf64W* w;                // M2P
+    const cd* m2pb;
+    const Leaf64D* d;                // directly summed reaction
     const cd* dvals;
     const cd* ys;                    // sums made by other kernels (null: none)
     const int64_t* perm;
@@ -137,7 +164,7 @@ constexpr int LF_TERMS = 32;         // k-steps per exact FP32 accumulation
 constexpr long long LF_BIAS = 0x808080808080ll;   // 128 sum_{i = 0 .. 5} 256^i
 
 // v 2^(54 - E), the last bit zero, |v| < 2^E (see s6_fixed)
-__device__ __forceinline__ long long lf_fixed(double v, int E) { return (s6_fixed<53>(v, 0, E) - S6_BIAS) * 2; }
+__device__ __forceinline__ long long lf_fixed(double v, int E) { return s6_fixed<53>(v, 0, E) * 2; }
 
 // digit i of two numbers (with LF_BIAS) as f16: 1024 + field as bits 0x6400 | field, minus 1152
 __device__ __forceinline__ unsigned lf_digit(long long xb, long long yb, int i) {
@@ -169,9 +196,8 @@ template <int W>
 __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Args A) {
     extern __shared__ __align__(16) double lf_smem[];
     constexpr int CHUNK = 128 * W, QPT = 4;                             // sources staged at once; per thread
-    const int64_t b = blockIdx.x;
-    const int32_t tlo = A.lb[b], tn = A.lb[b + 1] - tlo;
-    if (tn <= 0) return;
+    const Leaf64Rec L = A.recs[blockIdx.x];
+    const int32_t tlo = L.tlo, tn = L.tn;
     const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
     unsigned* sq = reinterpret_cast<unsigned*>(lf_smem);               // [CHUNK][LD] digit pairs
     double* red = lf_smem + CHUNK * LD / 2;                             // [W][3][32] (W > 1)
@@ -179,31 +205,15 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
     double* coef = reinterpret_cast<double*>(ring + W * LF_RING * 128);  // [p + 1][4]
     ring += wid * (LF_RING * 128) + lane;
     const uint32_t ring_a = (uint32_t)__cvta_generic_to_shared(ring);
-    __shared__ int32_t s_lo[9], s_pre[10];
     __shared__ int s_e[W];
     auto sync = [&] { if (W > 1) __syncthreads(); else __syncwarp(); };
     const cd* q = A.qs + (int64_t)r * A.n;
-    const int p = A.p, nb = p + 2, nc = 2 * p + 1;
-    if (A.G && wid == 0) {                                              // lane u: neighbour u, and the prefix sums
-        const int m = 1 << A.L, sx = (int)morton_x((uint32_t)b) + lane % 3 - 1, sy = (int)morton_y((uint32_t)b) + lane / 3 - 1;
-        int32_t lo = 0, cnt = 0;
-        if (lane < 9 && sx >= 0 && sy >= 0 && sx < m && sy < m) {
-            const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
-            lo = A.lb[s];
-            cnt = A.lb[s + 1] - lo;
-        }
-        int32_t inc = cnt;
-        for (int o = 1; o < 16; o <<= 1) {
-            const int32_t x = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += x;
-        }
-        if (lane < 9) { s_lo[lane] = lo; s_pre[lane + 1] = inc; }
-        if (lane == 0) s_pre[0] = 0;
-    }
-    if (A.loc) {
+    const int p = L.p, nb = L.nb, nc = 2 * p + 1;
+    const bool l2p = A.l2p && L.loc;
+    if (l2p) {
         // y = (i/4) sum_m beta_m conj-basis: with c = beta_m, d = (-1)^m beta_{-m} and B = (u, v)
         // re y = sum u w0 + v w1, im y = sum u w2 + v w3
-        const cd* beta = A.loc + (b * A.nrhs + r) * nc + p;
+        const cd* beta = L.loc + (L.lidx * A.nrhs + r) * nc + p;
         for (int m = tid; m <= p; m += W * 32) {
             const cd c = beta[m];
             cd d = m > 0 ? beta[-m] : cmk(0.0, 0.0);
@@ -215,13 +225,9 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
         }
     }
     sync();
-    const int ns = A.G ? s_pre[9] : 0;
-    auto strength = [&](int j) {
-        if (j >= ns) return cmk(0.0, 0.0);
-        int u = 0;
-        while (j >= s_pre[u + 1]) ++u;
-        return __ldg(q + s_lo[u] + (j - s_pre[u]));
-    };
+    const int ns = A.G ? L.ns : 0;
+    const int32_t* src = A.src + L.soff;
+    auto strength = [&](int j) { return j < ns ? __ldg(q + __ldg(src + j)) : cmk(0.0, 0.0); };
     // the first chunk's strengths stay in registers between their exponent and their digits
     cd qv[QPT];
     int Eq = S6_NONE;
@@ -243,7 +249,7 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
     }
     const bool bad = Eq >= S6_NAN / 2;
     const int EV = max(Eq, S6_NONE) + (A.G ? max(*A.EG, S6_NONE) : 0) - 68;
-    const uint4* Gb = A.G ? A.G + A.off[b] : nullptr;
+    const uint4* Gb = A.G ? A.G + L.goff : nullptr;
 
     const int ntile = (tn + 15) / 16;
     int staged = -1;                                                     // first source of the staged chunk
@@ -342,9 +348,9 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
         }
         double val[4] = {0.0, 0.0, 0.0, 0.0};
         if (live) {
-            if (A.loc) {
-                const cd* B0 = A.basis + (int64_t)(tlo + (v0 ? i0 : 0)) * nb;
-                const cd* B1 = A.basis + (int64_t)(tlo + (v1 ? i1 : 0)) * nb;
+            if (l2p) {
+                const cd* B0 = A.basis + L.boff + (int64_t)(v0 ? i0 : 0) * nb;
+                const cd* B1 = A.basis + L.boff + (int64_t)(v1 ? i1 : 0) * nb;
 #pragma unroll 4
                 for (int m = t + 4 * part; m <= p; m += 4 * ks) {
                     const double w0 = coef[4 * m], w1 = coef[4 * m + 1], w2 = coef[4 * m + 2], w3 = coef[4 * m + 3];
@@ -355,16 +361,32 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
                     val[3] = fma(u1.x, w2, fma(u1.y, w3, val[3]));
                 }
             }
-            if (A.d_begin)
-                for (int32_t e = A.d_begin[b]; e < A.d_begin[b + 1]; ++e) {
-                    const int32_t s = A.d_src[e], slo = A.lb[s], sn = A.lb[s + 1] - slo;
-                    const cd* D = A.dvals + A.d_blk[e];
+            if (A.m2p && L.wend > L.wbeg) {                              // (i/4) sum_m a_m H_m e^{i m theta}
+                cd a0 = cmk(0.0, 0.0), a1 = cmk(0.0, 0.0);
+                for (int32_t e = L.wbeg; e < L.wend; ++e) {
+                    const Leaf64W D = A.w[e];
+                    const int nw = 2 * D.p + 1;
+                    const cd* am = D.mult + (D.lidx * A.nrhs + r) * nw;
+                    const cd* M = A.m2pb + D.boff;
 #pragma unroll 2
-                    for (int j = t + 4 * part; j < sn; j += 4 * ks) {
-                        const cd v = __ldg(q + slo + j);
+                    for (int m = t + 4 * part; m < nw; m += 4 * ks) {
+                        const cd a = __ldg(am + m);
+                        if (v0) cfma(a0, a, __ldg(M + (int64_t)i0 * nw + m));
+                        if (v1) cfma(a1, a, __ldg(M + (int64_t)i1 * nw + m));
+                    }
+                }
+                val[0] -= 0.25 * a0.y; val[1] += 0.25 * a0.x; val[2] -= 0.25 * a1.y; val[3] += 0.25 * a1.x;
+            }
+            if (A.direct)
+                for (int32_t e = L.dbeg; e < L.dend; ++e) {
+                    const Leaf64D E = A.d[e];
+                    const cd* D = A.dvals + E.blk;
+#pragma unroll 2
+                    for (int j = t + 4 * part; j < E.sn; j += 4 * ks) {
+                        const cd v = __ldg(q + E.slo + j);
                         cd a0 = cmk(val[0], val[1]), a1 = cmk(val[2], val[3]);
-                        if (v0) cfma(a0, __ldg(D + (int64_t)i0 * sn + j), v);
-                        if (v1) cfma(a1, __ldg(D + (int64_t)i1 * sn + j), v);
+                        if (v0) cfma(a0, __ldg(D + (int64_t)i0 * E.sn + j), v);
+                        if (v1) cfma(a1, __ldg(D + (int64_t)i1 * E.sn + j), v);
                         val[0] = a0.x; val[1] = a0.y; val[2] = a1.x; val[3] = a1.y;
                     }
                 }
@@ -378,7 +400,7 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
             pb[v] = t == 0 ? lo[v] : ((hi[v] << (64 - 16 * t)) >> 32 & 0xffffffffll) + (lo[v] >> (16 * t));
         }
         long long a = ns > 0 ? quad_scatter(pa, t) : 0, bsum = ns > 0 ? quad_scatter(pb, t) : 0;
-        double x = A.loc || A.d_begin ? quad_scatter(val, t) : 0.0;
+        double x = quad_scatter(val, t);
         if (W > 1 && ks > 1) {                                           // parts of a tile, added in order by part 0
             double* mine = red + (size_t)wid * 96 + lane;
             __syncthreads();
@@ -435,23 +457,6 @@ __global__ void near64_fix_kernel(cd* G, int64_t n, const int* __restrict__ E) {
 
 }  // namespace
 
-// Plan-time bases of an FP64 plan (a mixed plan's first gradient): skipped above
-// the byte budget (the P2M and L2P then evaluate them in each apply).
-hfmm_status build_basis64(hfmm_plan_s* P, cudaStream_t st) {
-    if (P->basis64 || P->ad) return HFMM_OK;
-    const LevelInfo& lv = P->lev[P->L];
-    const int nb = lv.p + 2;
-    const double bytes = sizeof(cd) * (double)P->n * nb;
-    if (bytes > BASIS64_MAX_BYTES || nb * (int)sizeof(double) > 40000) return HFMM_OK;
-    HFMM_TRY(plan_alloc(P, (void**)&P->basis64, (size_t)bytes));
-    P->buffer_bytes += bytes;
-    const int thr = std::max(1, std::min(64, 5000 / nb));
-    basis64_kernel<<<(unsigned)lv.nbox, thr, (size_t)thr * nb * sizeof(double), st>>>(
-        P->leaf_begin, P->xy_sorted, P->x0, P->y0, lv.h, P->k, nb, P->basis64);
-    HFMM_CUDA_TRY(cudaGetLastError());
-    return HFMM_OK;
-}
-
 // Digit form of `pairs` near-field values in place; *finite = false (and the
 // values unchanged) where an entry is not finite (coincident points).
 hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, bool* finite, cudaStream_t st) {
@@ -469,59 +474,135 @@ hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, bool* finite, cudaS
     return HFMM_OK;
 }
 
-// P2M of the sorted strengths into the leaf multipoles (and their exponent).
+// Leaf records, near-field source indices and half bases of a uniform FP64 plan
+// (a mixed plan's first gradient).  Without bases (byte budget) the P2M and
+// L2P run on the kernels that evaluate them.
+hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
+    if (P->leaf64 || P->ad) return HFMM_OK;
+    const int L = P->L;
+    const LevelInfo& lv = P->lev[L];
+    const int nb = lv.p + 2, m = 1 << L;
+    const double bytes = sizeof(cd) * (double)P->n * nb;
+    const bool has_basis = bytes <= BASIS64_MAX_BYTES && nb * (int)sizeof(double) <= 40000;
+    const auto& lb = P->h_leaf_begin;
+    std::vector<Leaf64Rec> recs;
+    std::vector<Leaf64D> ds;
+    std::vector<int32_t> dbeg, dsrc;
+    std::vector<int64_t> dblk;
+    if (P->nd > 0) {
+        dbeg.resize((size_t)lv.nbox + 1);
+        dsrc.resize(P->nd);
+        dblk.resize(P->nd);
+        HFMM_CUDA_TRY(cudaMemcpyAsync(dbeg.data(), P->d_begin, sizeof(int32_t) * dbeg.size(), cudaMemcpyDeviceToHost, st));
+        HFMM_CUDA_TRY(cudaMemcpyAsync(dsrc.data(), P->d_src, sizeof(int32_t) * P->nd, cudaMemcpyDeviceToHost, st));
+        HFMM_CUDA_TRY(cudaMemcpyAsync(dblk.data(), P->d_blk, sizeof(int64_t) * P->nd, cudaMemcpyDeviceToHost, st));
+        HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+    }
+    int64_t soff = 0, goff = 0;
+    for (int64_t b = 0; b < lv.nbox; ++b) {
+        const int32_t tn = lb[b + 1] - lb[b];
+        if (tn == 0) continue;
+        const int ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
+        int64_t ns = 0;
+        for (int dy = -1; dy <= 1; ++dy)
+            for (int dx = -1; dx <= 1; ++dx) {
+                const int sx = ix + dx, sy = iy + dy;
+                if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
+                const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
+                ns += lb[s + 1] - lb[s];
+            }
+        Leaf64Rec R{};
+        R.tlo = lb[b]; R.tn = tn; R.ns = (int32_t)ns; R.p = lv.p; R.nb = nb;
+        R.soff = soff; R.goff = goff; R.boff = (int64_t)lb[b] * nb; R.lidx = b;
+        R.mult = lv.mult; R.loc = lv.loc; R.sx = lv.s6[0].sx;
+        R.E = P->s6_ready[0] ? split_exp(P, 0, L, false) : nullptr;
+        R.dbeg = (int32_t)ds.size();
+        if (P->nd > 0)
+            for (int32_t e = dbeg[b]; e < dbeg[b + 1]; ++e)
+                ds.push_back({lb[dsrc[e]], lb[dsrc[e] + 1] - lb[dsrc[e]], dblk[e]});
+        R.dend = (int32_t)ds.size();
+        soff += ns;
+        goff += (int64_t)tn * ns;
+        P->leaf_max = std::max(P->leaf_max, (int)tn);
+        recs.push_back(R);
+    }
+    P->leaf_empty = (int64_t)recs.size() < lv.nbox;
+    P->leaf64_n = (int64_t)recs.size();
+    P->leaf64_p = lv.p;
+    HFMM_TRY(plan_alloc(P, (void**)&P->leaf64, sizeof(Leaf64Rec) * recs.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->leaf64_d, sizeof(Leaf64D) * ds.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->leaf64_src, sizeof(int32_t) * soff));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->leaf64, recs.data(), sizeof(Leaf64Rec) * recs.size(), cudaMemcpyHostToDevice, st));
+    if (!ds.empty())
+        HFMM_CUDA_TRY(cudaMemcpyAsync(P->leaf64_d, ds.data(), sizeof(Leaf64D) * ds.size(), cudaMemcpyHostToDevice, st));
+    leaf_sources_kernel<<<(unsigned)recs.size(), 64, 0, st>>>(P->leaf_begin, L, P->leaf64, P->leaf64_src);
+    HFMM_CUDA_TRY(cudaGetLastError());
+    if (has_basis) {
+        HFMM_TRY(plan_alloc(P, (void**)&P->basis64, (size_t)bytes));
+        P->buffer_bytes += bytes;
+        const int thr = std::max(1, std::min(64, 5000 / nb));
+        basis64_kernel<<<(unsigned)lv.nbox, thr, (size_t)thr * nb * sizeof(double), st>>>(
+            P->leaf_begin, P->xy_sorted, P->x0, P->y0, lv.h, P->k, nb, P->basis64);
+        HFMM_CUDA_TRY(cudaGetLastError());
+    }
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // recs and ds are locals
+    return HFMM_OK;
+}
+
+// P2M of the sorted strengths into the leaf multipoles (and their exponents).
 hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
-    LevelInfo& lv = P->lev[P->L];
-    const int64_t items = lv.nbox * (lv.p + 1);
+    const int pitch = P->leaf64_p + 1;
+    const int64_t items = P->leaf64_n * pitch;
     const int ps = items < 32 * 1024 ? 4 : 1;        // not by nrhs: it would change the sums' order
     auto kernel = ps == 4 ? p2m64_kernel<4> : p2m64_kernel<1>;
+    if (P->leaf_empty) {
+        const LevelInfo& lv = P->lev[P->L];
+        zero_empty_kernel<<<(unsigned)std::min<int64_t>(lv.nbox, 16 * 152), 64, 0, st>>>(
+            P->leaf_begin, lv.nbox, (int64_t)nrhs * lv.ncoef, lv.mult);
+        ++P->launches;
+    }
     kernel<<<dim3((unsigned)((items * ps + 127) / 128), (unsigned)nrhs), 128, 0, st>>>(
-        P->leaf_begin, P->basis64, P->q_sorted, P->n, lv.nbox, nrhs, lv.p, lv.s6_sx,
-        P->s6_ready ? split64_exp(P, P->L, false) : nullptr, lv.mult);
+        P->leaf64, P->basis64, P->q_sorted, P->n, P->leaf64_n, pitch, nrhs);
     ++P->launches;
     HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;
 }
 
 // Everything at the targets, into the caller's order: near = the stored blocks,
-// l2p = the leaves' locals, direct = the reaction blocks, ys = other sums.
-hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool direct, const cd* ys, bool conj_out, cd* y,
-                          cudaStream_t st) {
-    const LevelInfo& lv = P->lev[P->L];
+// l2p = the leaves' locals, m2p = the W lists, direct = the reaction blocks, ys =
+// other sums.
+hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2p, bool direct, const cd* ys,
+                          bool conj_out, cd* y, cudaStream_t st) {
     Leaf64Args A{};
-    A.lb = P->leaf_begin;
-    A.L = P->L;
+    A.recs = P->leaf64;
     A.nrhs = nrhs;
-    A.p = lv.p;
+    A.p = P->leaf64_p;
     A.n = P->n;
     A.qs = P->q_sorted;
-    if (near) {
-        A.G = (const uint4*)P->near64_vals;
-        A.off = P->near64_off;
-        A.EG = P->near64_E;
-    }
-    if (l2p) {
-        A.loc = lv.loc;
-        A.basis = P->basis64;
-    }
-    if (direct) {
-        A.d_begin = P->d_begin;
-        A.d_src = P->d_src;
-        A.d_blk = P->d_blk;
-        A.dvals = P->d_vals;
-    }
+    if (near) A.G = (const uint4*)P->near64_vals;
+    A.EG = P->near64_E;
+    A.src = P->leaf64_src;
+    A.l2p = l2p;
+    A.m2p = m2p;
+    A.direct = direct;
+    A.basis = P->basis64;
+    A.w = P->leaf64_w;
+    A.m2pb = P->m2p64;
+    A.d = P->leaf64_d;
+    A.dvals = P->d_vals;
     A.ys = ys;
     A.perm = P->perm;
     A.conj_out = conj_out;
     A.y = y;
     // one warp per leaf from 16 of them per SM on (leaves of at most four tiles), else four
-    const bool one = lv.nbox >= 16 * 152 && P->leaf_max <= 64;
+    const bool one = P->leaf64_n >= 16 * 152 && P->leaf_max <= 64;
     const int W = one ? 1 : 4;
-    const size_t sm = sizeof(double) * (128 * W * LD / 2 + (one ? 0 : W * 96) + W * LF_RING * 256 + (l2p ? 4 * (size_t)(lv.p + 1) : 0));
+    const size_t sm = sizeof(double) * (128 * W * LD / 2 + (one ? 0 : W * 96) + W * LF_RING * 256 +
+                                        (l2p ? 4 * (size_t)(A.p + 1) : 0));
     auto kernel = one ? leaf64_kernel<1> : leaf64_kernel<4>;
     if (sm > 47 * 1024)                                    // (static shared memory beside it)
         HFMM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    kernel<<<dim3((unsigned)lv.nbox, (unsigned)nrhs), W * 32, sm, st>>>(A);
+    kernel<<<dim3((unsigned)P->leaf64_n, (unsigned)nrhs), W * 32, sm, st>>>(A);
     ++P->launches;
     HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;

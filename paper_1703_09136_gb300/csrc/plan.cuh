@@ -19,6 +19,25 @@
 
 #include "common.cuh"
 
+// Translations as digit products (split64.cu).  Adaptive trees list their tiles:
+// eight targets of a level (-1: none) and their steps, one operator and a source per
+// target each (op = operator * 4 + 0 shift, 1 free-space, 2 reaction; -1: no source).
+struct S6Rec { int32_t op, src[8]; };
+struct S6Tiles {
+    int n = 0;
+    int32_t *tgt = nullptr, *tbeg = nullptr;
+    S6Rec* recs = nullptr;
+};
+// One level: power-of-two scales log2 s(n), operator digit slices, exponents of the
+// operator families (lists, L2L into the level, M2M into it), expansion digits.
+struct S6Lev {
+    const int* sx = nullptr;
+    uint4 *free = nullptr, *react = nullptr, *l2l = nullptr, *m2m = nullptr;
+    int* Eop = nullptr;
+    unsigned *dmult = nullptr, *dloc = nullptr;
+    S6Tiles down, up;
+};
+
 struct LevelInfo {
     int p = 0;
     int ncoef = 1;          // 2p + 1
@@ -99,13 +118,7 @@ struct LevelInfo {
     cd* diag_spec = nullptr;
     double diag_err = -1.0;
     int64_t nonempty = 0;         // non-empty boxes (set by the diagonal-form check)
-    // FP64 translations on the tensor cores (split64.cu): power-of-two scales
-    // log2 s(n), operator digit slices and the exponents of the operator families
-    // (lists, L2L into this level, M2M into this level)
-    const int* s6_sx = nullptr;
-    uint4 *s6_free = nullptr, *s6_react = nullptr, *s6_l2l = nullptr, *s6_m2m = nullptr;
-    int* s6_Eop = nullptr;
-    unsigned *s6_dmult = nullptr, *s6_dloc = nullptr;   // digits of the level's expansions
+    S6Lev s6[2];                  // digit products (split64.cu) of the FP64 and of the FP32 expansions
 };
 
 // Diagonal form: kept on a level when its weighted difference to the dense
@@ -132,6 +145,28 @@ struct NtChunk {
     int32_t nrun;    // runs of consecutive covered leaves (1 or 2)
     int32_t run[2];  // each: width | first column << 8 | first tile row << 16
     int32_t pad;
+};
+
+// FP64 leaf passes (leaf64.cu).  Leaf: targets tlo .. tlo + tn, ns near-field sources
+// (indices from soff, block from goff), order p, basis rows of nb values from boff,
+// expansions of its level (null: none) and index in them, scale and exponent of its
+// multipoles, ranges of its W and directly summed pairs.  W pair: the box's
+// multipoles and the basis of the leaf's points.  Direct pair: sources and block.
+struct Leaf64Rec {
+    int32_t tlo, tn, ns, p, nb, wbeg, wend, dbeg, dend;
+    int64_t soff, goff, boff, lidx;
+    cd *mult, *loc;
+    const int* sx;
+    int* E;
+};
+struct Leaf64W {
+    const cd* mult;
+    int64_t lidx, boff;
+    int32_t p, pad;
+};
+struct Leaf64D {
+    int32_t slo, sn;
+    int64_t blk;
 };
 
 // Adaptive trees (adaptive.cu): deepest level, and the host / device tree.
@@ -201,6 +236,14 @@ struct hfmm_plan_s {
     cd* near64_vals = nullptr;      // after the fill: base-256 digits (leaf64.cu)
     int* near64_E = nullptr;        // their exponent
     int leaf_max = 0;               // largest number of points of a leaf
+    bool leaf_empty = false;        // a uniform tree with empty leaves
+    Leaf64Rec* leaf64 = nullptr;    // non-empty leaves (leaf64.cu), their largest order, near-field source
+    int64_t leaf64_n = 0;           // indices, W and directly summed pairs, M2P bases of the W pairs
+    int leaf64_p = 0;
+    int32_t* leaf64_src = nullptr;
+    Leaf64W* leaf64_w = nullptr;
+    Leaf64D* leaf64_d = nullptr;
+    cd* m2p64 = nullptr;
     cd* basis64 = nullptr;          // [n][p_L + 2] P2M basis J_m(k rho) e^{-i m theta}, m >= 0
     void* krylov = nullptr;         // hfmm_solve: Krylov vectors (first call; grows with restart)
     size_t krylov_bytes = 0;
@@ -233,10 +276,10 @@ struct hfmm_plan_s {
     float* tc_part = nullptr;       // partial sums of split launches (levels with few tiles)
     size_t tc_part_floats = 0;
 
-    // FP64 translations on the tensor cores (split64.cu): slices built, and the
-    // exponents of every level's expansions [multipoles, locals][level][max_rhs]
-    bool s6_ready = false;
-    int* s6_E = nullptr;
+    // digit products (split64.cu): slices built, and the exponents of every level's
+    // expansions [multipoles, locals][level][max_rhs]; 0: FP64, 1: FP32
+    bool s6_ready[2] = {false, false};
+    int* s6_E[2] = {nullptr, nullptr};
 
     // table quadrature: panel-count scale (hfmm_options.quad_scale) and the
     // node-doubling check's largest weighted relative difference and where
@@ -312,6 +355,9 @@ hfmm_status build_diag(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status build_adaptive_tree(hfmm_plan_s* P, const double* d_xy, int leaf_size, cudaStream_t st);
 hfmm_status build_adaptive_lists(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status apply_adaptive(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t st);
+hfmm_status build_adaptive64(hfmm_plan_s* P, cudaStream_t st);
+bool adaptive_fast64(const hfmm_plan_s* P);
+hfmm_status apply_adaptive64(hfmm_plan_s* P, int nrhs, int parts, bool conj_out, cd* y, cudaStream_t st);
 hfmm_status build_adaptive32(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status apply_adaptive32(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t st);
 hfmm_status adaptive_boxes(const hfmm_plan_s* P, int64_t* count, int32_t* out);
@@ -321,20 +367,23 @@ void adaptive_destroy(AdaptiveTree* T);
 hfmm_status diag_src(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st);
 hfmm_status diag_m2l(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st);
 double diag_flops(const hfmm_plan_s* P, int l, int nrhs, int parts);
-// split64.cu
-hfmm_status build_split64(hfmm_plan_s* P, cudaStream_t st);
-hfmm_status split64_begin(hfmm_plan_s* P, cudaStream_t st);
-hfmm_status split64_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st);
-hfmm_status split64_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st);
-hfmm_status split64_m2m(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st);
-hfmm_status split64_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st);
-int* split64_exp(hfmm_plan_s* P, int l, bool loc);
+// split64.cu (w = 0: FP64 expansions, 1: FP32)
+hfmm_status build_split(hfmm_plan_s* P, int w, cudaStream_t st);
+hfmm_status split_begin(hfmm_plan_s* P, int w, cudaStream_t st);
+hfmm_status split_exponent(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st);
+hfmm_status split_slice(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st);
+hfmm_status split_m2m(hfmm_plan_s* P, int w, int l, int nrhs, cudaStream_t st);
+hfmm_status split_down(hfmm_plan_s* P, int w, int l, int nrhs, int parts, cudaStream_t st);
+int* split_exp(hfmm_plan_s* P, int w, int l, bool loc);
+void adaptive_react_entries(const hfmm_plan_s* P, int l, std::vector<int32_t>& entries);
+void adaptive_tiles(const hfmm_plan_s* P, int l, bool up, const std::vector<int32_t>& rmap, std::vector<int32_t>& tgt,
+                    std::vector<int32_t>& tbeg, std::vector<S6Rec>& recs);
 // leaf64.cu
-hfmm_status build_basis64(hfmm_plan_s* P, cudaStream_t st);
+hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, bool* finite, cudaStream_t st);
 hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st);
-hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool direct, const cd* ys, bool conj_out, cd* y,
-                          cudaStream_t st);
+hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2p, bool direct, const cd* ys,
+                          bool conj_out, cd* y, cudaStream_t st);
 hfmm_status build_near64_grad(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, bool adjoint,
                        cudaStream_t st);

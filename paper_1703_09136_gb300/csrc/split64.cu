@@ -1,5 +1,5 @@
-// FP64 translations (M2M, L2L, free-space and reaction M2L) as exact-slice
-// products on the tensor cores.
+// Translations (M2M, L2L, free-space and reaction M2L) as exact-slice products on
+// the tensor cores: FP64 expansions with six digits, FP32 ones with three.
 //
 // Every translation is a real matrix-vector product of length 2 nc (interleaved
 // real and imaginary parts).  The operand and the operator are written as
@@ -22,6 +22,10 @@
 // expansions stay unscaled, so every other kernel reads them as before.  A level
 // that holds an infinity or a NaN makes every output of that right-hand side NaN.
 //
+// FP32 (the mixed path's expansions, already scaled by s): three digits hold 26
+// bits, six products (i + j <= 2) replace the 21, orders 0 and 1 are kept as
+// integers and order 2 in FP32.
+//
 // What bounds it: GB300's FP64 pipe runs at 1.0 TFLOP/s (a warp-wide FMA every 16
 // clocks per SM), mma.sync f16 at 600 TFLOP/s: 21 products leave 28 TFLOP/s.
 // Measured (one GB300, two layers, 262,144 points, one right-hand side): leaf
@@ -41,6 +45,19 @@ namespace {
 constexpr int S6_MAXW = 6;               // m-tiles (warps) per CTA
 constexpr double S6_MAX_BYTES = 16e9;    // operator slices of one plan, and its expansions' digits
 
+// D digits; orders 0 .. NI - 1 are summed as integers, the others in FP32
+template <int D> struct S6Traits;
+template <> struct S6Traits<6> {
+    using C = cd;
+    using R = double;
+    static constexpr int NI = 4;
+};
+template <> struct S6Traits<3> {
+    using C = cf;
+    using R = float;
+    static constexpr int NI = 2;
+};
+
 // ---------------------------------------------------------------------------
 // plan time: operator slices in the A-fragment order of mma.m16n8k16
 // ---------------------------------------------------------------------------
@@ -48,26 +65,33 @@ enum { S6_FREE = 0, S6_REACT = 1, S6_L2L = 2, S6_M2M = 3 };
 
 struct S6Op {
     const cd* T;
+    const int32_t* map;              // table entries of the operators (null: all, in order)
     int kind, nop, po, pi;           // orders of the outputs and the inputs
-    const int* sxo;                  // log2 s of the output level, per |order|
+    const int* sxo;                  // log2 s of the output level, per |order| (null: log s below)
     const int* sxi;
+    const double* lso;               // FP32 expansions: log s, applied to the entries
+    const double* lsi;
 };
 
 __device__ __forceinline__ cd s6_entry(const S6Op& o, int op, int j, int m, int* sh) {
     // output order j, input order m; *sh = -(in_shift + out_shift)
-    const int so = o.sxo[abs(j)], si = o.sxi[abs(m)];
-    if (o.kind == S6_FREE) {
-        *sh = so + si;
-        return o.T[(int64_t)op * (4 * o.po + 1) + (m - j) + 2 * o.po];
+    if (o.map) op = o.map[op];
+    cd v;
+    if (o.kind == S6_FREE) v = o.T[(int64_t)op * (4 * o.po + 1) + (m - j) + 2 * o.po];
+    else if (o.kind == S6_REACT) {
+        v = o.T[(int64_t)op * (4 * o.po + 1) + (-m - j) + 2 * o.po];
+        if (m & 1) v = cneg(v);
+    } else {
+        const int nmax = o.po + o.pi, w = 2 * nmax + 1;   // J_{n-m}(c - P) or J_{m-j}(P - c)
+        v = o.T[(int64_t)op * w + nmax + (m - j)];
     }
-    if (o.kind == S6_REACT) {
-        *sh = so + si;
-        cd v = o.T[(int64_t)op * (4 * o.po + 1) + (-m - j) + 2 * o.po];
-        return (m & 1) ? cneg(v) : v;
+    const int go = o.kind == S6_M2M ? -1 : 1, gi = o.kind == S6_L2L ? -1 : 1;   // s to the power go, gi
+    if (o.sxo) *sh = go * o.sxo[abs(j)] + gi * o.sxi[abs(m)];
+    else {
+        *sh = 0;
+        v = cscale(v, exp(go * o.lso[abs(j)] + gi * o.lsi[abs(m)]));
     }
-    const int nmax = o.po + o.pi, w = 2 * nmax + 1;
-    *sh = o.kind == S6_L2L ? so - si : si - so;
-    return o.T[(int64_t)op * w + nmax + (m - j)];         // J_{n-m}(c - P) or J_{m-j}(P - c)
+    return v;
 }
 
 __global__ void s6_op_exponent_kernel(S6Op o, int* __restrict__ E) {
@@ -85,6 +109,7 @@ __global__ void s6_op_exponent_kernel(S6Op o, int* __restrict__ E) {
 }
 
 // one thread per (op, m-tile, k-step, lane): its eight entries' digits
+template <int D>
 __global__ void s6_op_slice_kernel(S6Op o, const int* __restrict__ Ep, uint4* __restrict__ out) {
     const int no = 2 * o.po + 1, ni = 2 * o.pi + 1;
     const int MT = (2 * no + 15) / 16, KS = (2 * ni + 15) / 16;
@@ -95,31 +120,32 @@ __global__ void s6_op_slice_kernel(S6Op o, const int* __restrict__ Ep, uint4* __
         const int64_t blk = i >> 5;                        // (op, mt, ks)
         const int ks = (int)(blk % KS), mt = (int)((blk / KS) % MT), op = (int)(blk / ((int64_t)KS * MT));
         const int g = lane >> 2, t = lane & 3;
-        unsigned f[ND][4];
+        unsigned f[D][4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int row = 16 * mt + g + (q & 1) * 8, m = (16 * ks + (q >> 1) * 8) / 2 + t;   // columns 2m, 2m + 1
             const int j = row >> 1;
-            long long x0 = S6_BIAS, x1 = S6_BIAS;
+            long long x0 = s6_bias<D>(), x1 = s6_bias<D>();
             if (j < no && m < ni) {
                 int sh;
                 const cd v = s6_entry(o, op, j - o.po, m - o.pi, &sh);
                 // [[Re, -Im], [Im, Re]]
-                x0 = s6_fixed<52>((row & 1) ? v.y : v.x, sh, E);
-                x1 = s6_fixed<52>((row & 1) ? v.x : -v.y, sh, E);
+                x0 += s6_fixed<9 * D - 2>((row & 1) ? v.y : v.x, sh, E);
+                x1 += s6_fixed<9 * D - 2>((row & 1) ? v.x : -v.y, sh, E);
             }
 #pragma unroll
-            for (int d = 0; d < ND; ++d) f[d][q] = s6_half2(s6_field(x0, d), s6_field(x1, d));
+            for (int d = 0; d < D; ++d) f[d][q] = s6_half2(s6_field<D>(x0, d), s6_field<D>(x1, d));
         }
 #pragma unroll
-        for (int d = 0; d < ND; ++d) out[(blk * ND + d) * 32 + lane] = make_uint4(f[d][0], f[d][1], f[d][2], f[d][3]);
+        for (int d = 0; d < D; ++d) out[(blk * D + d) * 32 + lane] = make_uint4(f[d][0], f[d][1], f[d][2], f[d][3]);
     }
 }
 
 // ---------------------------------------------------------------------------
 // level exponents of expansions written by other kernels
 // ---------------------------------------------------------------------------
-__global__ void s6_exponent_kernel(const cd* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
+template <class C>
+__global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
                                    int sign, int* __restrict__ E) {
     const int nc = 2 * p + 1, r = blockIdx.y;
     int e = S6_NONE;
@@ -127,8 +153,8 @@ __global__ void s6_exponent_kernel(const cd* __restrict__ a, int64_t nbox, int n
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / nc;
         const int m = (int)(i % nc) - p;
-        const cd v = a[(b * nrhs + r) * nc + m + p];
-        const int sh = sign * sx[abs(m)];
+        const C v = a[(b * nrhs + r) * nc + m + p];
+        const int sh = sx ? sign * sx[abs(m)] : 0;
         e = max(e, max(s6_exponent(v.x, sh), s6_exponent(v.y, sh)));
     }
     e = __reduce_max_sync(0xffffffffu, e);
@@ -140,7 +166,8 @@ __global__ void s6_exponent_kernel(const cd* __restrict__ a, int64_t nbox, int n
 // [coefficient % 4][coefficient / 4] (32 bytes).  Every source meets up to 27
 // target tiles: cutting it in the product kernel took 60% of that kernel's
 // instructions (leaf level of two layers 0.47 -> 0.34 ms without it).
-__global__ void s6_slice_kernel(const cd* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
+template <int D>
+__global__ void s6_slice_kernel(const typename S6Traits<D>::C* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
                                 int sign, const int* __restrict__ E, unsigned* __restrict__ dig) {
     const int nc = 2 * p + 1, KS = (2 * nc + 15) / 16, r = blockIdx.y;
     const int64_t total = nbox * KS * 8;
@@ -148,16 +175,16 @@ __global__ void s6_slice_kernel(const cd* __restrict__ a, int64_t nbox, int nrhs
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / (KS * 8);
         const int m = (int)(i - b * (KS * 8));
-        long long xr = S6_BIAS, xi = S6_BIAS;
+        long long xr = s6_bias<D>(), xi = s6_bias<D>();
         if (m < nc) {
-            const cd v = a[(b * nrhs + r) * nc + m];
-            const int sh = sign * sx[abs(m - p)];
-            xr = s6_fixed<53>(v.x, sh, e);
-            xi = s6_fixed<53>(v.y, sh, e);
+            const auto v = a[(b * nrhs + r) * nc + m];
+            const int sh = sx ? sign * sx[abs(m - p)] : 0;
+            xr += s6_fixed<9 * D - 1>(v.x, sh, e);
+            xi += s6_fixed<9 * D - 1>(v.y, sh, e);
         }
-        unsigned* o = dig + ((b * nrhs + r) * KS + (m >> 3)) * (ND * 8) + (m & 3) * 2 + (m >> 2 & 1);
+        unsigned* o = dig + ((b * nrhs + r) * KS + (m >> 3)) * (D * 8) + (m & 3) * 2 + (m >> 2 & 1);
 #pragma unroll
-        for (int d = 0; d < ND; ++d) o[d * 8] = s6_half2(s6_field(xr, d), s6_field(xi, d));
+        for (int d = 0; d < D; ++d) o[d * 8] = s6_half2(s6_field<D>(xr, d), s6_field<D>(xi, d));
     }
 }
 
@@ -174,7 +201,8 @@ struct S6Fam {
 };
 
 struct S6Args {
-    int l, L, mode;                  // mode 0: M2M (targets 16 NT consecutive boxes), 1: downward
+    // mode 0: M2M (targets 8 NT consecutive boxes), 1: downward, 2: explicit tiles (adaptive trees)
+    int l, L, mode;
     int nrhs, p;                     // output order
     int tiles;
     const int32_t* lb;               // leaf ranges (downward: empty targets are skipped)
@@ -184,9 +212,12 @@ struct S6Args {
     int vlist, rlist, lstar;         // lists to run; first level whose bottom-row pair is admissible
     int rows;                        // box rows covered by the launch (downward)
     int accumulate;                  // add to the outputs
-    const int* sxo;
+    const int* sxo;                  // (null: no output shift)
     int osign;                       // out_shift = osign * sxo
-    cd* out;
+    const int32_t* tgt;              // mode 2: [tiles][8] targets (-1: none), first step of every tile, steps
+    const int32_t* tbeg;
+    const S6Rec* recs;
+    void* out;
     int* Eout;                       // [nrhs], or null
 };
 
@@ -200,7 +231,7 @@ __device__ __forceinline__ void cluster_sync() {
 struct S6Step {
     int fam;                         // 0 shift, 1 list
     const uint4* op;
-    int dx, sy, child;               // list: source (ix - dx, sy); shift: child position (mode 0)
+    int dx, sy, child;               // list: source (ix - dx, sy); shift: child position (mode 0); mode 2: record
 };
 
 // Steps of a downward tile (row iy, columns ix0, ix0 + 2, ..., ncol of them):
@@ -209,10 +240,14 @@ struct S6Step {
 // dx).  Returns false where a step does not exist for this tile.
 struct S6Tile {
     int iy, ix0, ncol, n;            // n boxes per row
-    int nshift, nv, nr, rspan, ropt0;
+    int nshift, nv, nr, rspan, ropt0, rec0;
 };
 
-__device__ __forceinline__ int s6_steps(const S6Args& A, S6Tile& T) {
+__device__ __forceinline__ int s6_steps(const S6Args& A, S6Tile& T, int tile) {
+    if (A.mode == 2) {
+        T.rec0 = A.tbeg[tile];
+        return A.tbeg[tile + 1] - T.rec0;
+    }
     T.nshift = A.shift.dig ? (A.mode == 0 ? 4 : 1) : 0;
     T.nv = T.nr = 0;
     if (A.mode == 1) {
@@ -227,11 +262,21 @@ __device__ __forceinline__ int s6_steps(const S6Args& A, S6Tile& T) {
     return T.nshift + T.nv + T.nr;
 }
 
+template <int D>
 __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s, int MT, int KSs, int KSl, S6Step& st) {
+    if (A.mode == 2) {               // record: operator * 4 + kind (0 shift, 1 free-space, 2 reaction)
+        st.child = T.rec0 + s;
+        const int op = A.recs[st.child].op, kind = op & 3;
+        st.fam = kind ? 1 : 0;
+        if (kind == 0 ? !A.shift.dig : kind == 1 ? !A.vlist : !A.rlist) return false;
+        st.op = (kind == 0 ? A.shift.ops : kind == 1 ? A.list.ops : A.rops) +
+                (int64_t)(op >> 2) * MT * (kind ? KSl : KSs) * (D * 32);
+        return true;
+    }
     if (s < T.nshift) {
         st.fam = 0;
         st.child = A.mode == 0 ? s : (T.ix0 & 1) + 2 * (T.iy & 1);
-        st.op = A.shift.ops + (int64_t)st.child * MT * KSs * (ND * 32);
+        st.op = A.shift.ops + (int64_t)st.child * MT * KSs * (D * 32);
         return true;
     }
     s -= T.nshift;
@@ -244,7 +289,7 @@ __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s,
         if (st.sy < 0 || st.sy >= T.n) return false;
         st.dx = -ox;
         if (T.ix0 + 2 * (T.ncol - 1) + ox < 0 || T.ix0 + ox >= T.n) return false;
-        st.op = A.list.ops + (int64_t)((st.dx + 3) * 7 + (-oy + 3)) * MT * KSl * (ND * 32);
+        st.op = A.list.ops + (int64_t)((st.dx + 3) * 7 + (-oy + 3)) * MT * KSl * (D * 32);
         return true;
     }
     s -= T.nv;
@@ -252,7 +297,7 @@ __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s,
     st.dx = T.ix0 + 2 * (T.ncol - 1) - s % T.rspan;              // sources from right to left cover [0, n)
     const int dxm = T.n - 1;
     if (abs(st.dx) > dxm) return false;
-    st.op = A.rops + (int64_t)((st.dx + dxm) * 3 + T.iy + st.sy) * MT * KSl * (ND * 32);
+    st.op = A.rops + (int64_t)((st.dx + dxm) * 3 + T.iy + st.sy) * MT * KSl * (D * 32);
     return true;
 }
 
@@ -263,10 +308,12 @@ __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s,
 // its own.  Levels with few tiles split a tile's steps over a cluster of up to
 // eight CTAs and add the partial sums in rank order through distributed shared
 // memory, so results do not depend on timing.
-template <int NT>
+template <int NT, int D>
 __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant__ S6Args A) {
+    using R = typename S6Traits<D>::R;
+    constexpr int NI = S6Traits<D>::NI;
     // digits of the sources of one 64-term chunk, in B-fragment order, two buffers
-    __shared__ __align__(16) uint2 Bs[2][ND][4][NT][32];
+    __shared__ __align__(16) uint2 Bs[2][D][4][NT][32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
     const int S = (int)cluster_size(), rank = (int)cluster_rank();
     const int tile = blockIdx.x / S, r = blockIdx.z;
@@ -278,7 +325,7 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
     S6Tile T;
     int64_t box0 = 0;
     T.n = 1 << A.l;
-    if (A.mode == 0) {
+    if (A.mode != 1) {
         box0 = (int64_t)tile * NC;
         T.iy = T.ix0 = 0;
         T.ncol = NC;
@@ -292,23 +339,24 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
     const int64_t nbox = (int64_t)1 << (2 * A.l);
     auto target = [&](int col) -> int64_t {
         if (A.mode == 0) return box0 + col < nbox ? box0 + col : -1;
+        if (A.mode == 2) return A.tgt[box0 + col];
         if (col >= T.ncol) return -1;
         const int64_t b = morton((uint32_t)(T.ix0 + 2 * col), (uint32_t)T.iy);
         int32_t lo, hi;
         box_range(A.lb, A.L, A.l, b, &lo, &hi);
         return hi > lo ? b : -1;
     };
-    {   // nothing to do where every target is empty (the same for all CTAs of the cluster)
+    if (A.mode == 1) {   // nothing to do where every target is empty (the same for all CTAs of the cluster)
         bool any = false;
         for (int c = 0; c < NC; ++c) any |= target(c) >= 0;
         if (!any) return;
     }
-    const int nsteps = s6_steps(A, T);
+    const int nsteps = s6_steps(A, T, tile);
     const int nis = A.shift.dig ? 2 * A.shift.p + 1 : 0, nil = A.list.dig ? 2 * A.list.p + 1 : 0;
     const int KSs = (2 * nis + 15) / 16, KSl = (2 * nil + 15) / 16;
 
-    float acc[NT][ND][4];
-    int iacc[NT][4][4];
+    float acc[NT][D][4];
+    int iacc[NT][NI][4];
     double dacc[NT][4];
 #pragma unroll
     for (int t = 0; t < NT; ++t)
@@ -316,26 +364,32 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
         for (int v = 0; v < 4; ++v) {
             dacc[t][v] = 0.0;
 #pragma unroll
-            for (int o = 0; o < 4; ++o) iacc[t][o][v] = 0;
+            for (int o = 0; o < NI; ++o) iacc[t][o][v] = 0;
 #pragma unroll
-            for (int o = 0; o < ND; ++o) acc[t][o][v] = 0.0f;
+            for (int o = 0; o < D; ++o) acc[t][o][v] = 0.0f;
         }
     int since = 0;                    // chunks since the integers were last folded
-    // dacc += (digit sums) 2^(Esrc + Eop - 42): order o weighs 2^(9 (10 - o)) of 2^-105.  Four
-    // FP64 instructions a value (the pipe takes 64 clocks for each of a sub-partition's):
-    // orders 0 .. 2 and 3 .. 5 as two integers below 2^51
+    // dacc += (digit sums) 2^E, E = Esrc + Eop - (18 D - 3): order o weighs 512^(2 (D - 1) - o).
+    // Four (two) FP64 instructions a value (the pipe takes 64 clocks for each of a
+    // sub-partition's): orders 0 .. 2 and 3 .. 5 as integers below 2^51
     auto fold = [&](int E) {
-        const double chi = pow2d(E + 9), clo = pow2d(E - 18);
+        const double chi = pow2d(E + 9 * (2 * D - 4)), clo = D == 6 ? pow2d(E + 45) : 0.0;
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                const long long hi = ((long long)iacc[t][0][v] << 18) + ((long long)iacc[t][1][v] << 9) + iacc[t][2][v];
-                const long long lo = ((long long)iacc[t][3][v] << 18) + (__float2ll_rn(acc[t][4][v]) << 9) +
-                                     __float2ll_rn(acc[t][5][v]);
-                dacc[t][v] = fma(int51d(hi), chi, fma(int51d(lo), clo, dacc[t][v]));
-                iacc[t][0][v] = iacc[t][1][v] = iacc[t][2][v] = iacc[t][3][v] = 0;
-                acc[t][4][v] = acc[t][5][v] = 0.0f;
+                long long hi = ((long long)iacc[t][0][v] << 18) + ((long long)iacc[t][1][v] << 9);
+                if (D == 6) {
+                    hi += iacc[t][NI - 2][v];
+                    const long long lo = ((long long)iacc[t][NI - 1][v] << 18) + (__float2ll_rn(acc[t][D - 2][v]) << 9) +
+                                         __float2ll_rn(acc[t][D - 1][v]);
+                    dacc[t][v] = fma(int51d(lo), clo, dacc[t][v]);
+                } else hi += __float2ll_rn(acc[t][D - 1][v]);
+                dacc[t][v] = fma(int51d(hi), chi, dacc[t][v]);
+#pragma unroll
+                for (int o = 0; o < NI; ++o) iacc[t][o][v] = 0;
+#pragma unroll
+                for (int o = NI; o < D; ++o) acc[t][o][v] = 0.0f;
             }
         since = 0;
     };
@@ -344,12 +398,12 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
     if (A.shift.dig) {
         const int e = A.shift.Esrc[r];
         bad |= e >= S6_NAN / 2;
-        Ef[0] = max(e, S6_NONE) + max(*A.shift.Eop, S6_NONE) - 42;
+        Ef[0] = max(e, S6_NONE) + max(*A.shift.Eop, S6_NONE) - (18 * D - 3);
     }
     if (A.list.dig) {
         const int e = A.list.Esrc[r];
         bad |= e >= S6_NAN / 2;
-        Ef[1] = max(e, S6_NONE) + max(*A.list.Eop, S6_NONE) - 42;
+        Ef[1] = max(e, S6_NONE) + max(*A.list.Eop, S6_NONE) - (18 * D - 3);
     }
 
     // A chunk: up to 64 terms (four k-steps) of one step.  While the tensor cores work on
@@ -365,10 +419,10 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
         }
         c.k0 = 0;
         for (c.s = c.s < 0 ? rank : c.s + S; c.s < nsteps; c.s += S)
-            if (s6_step(A, T, c.s, MT, KSs, KSl, c.st)) return true;
+            if (s6_step<D>(A, T, c.s, MT, KSs, KSl, c.st)) return true;
         return false;
     };
-    // digits of the chunk's columns, 48 pieces of 16 bytes each (k-step, digit, half): a
+    // digits of the chunk's columns, 8 D pieces of 16 bytes each (k-step, digit, half): a
     // warp takes columns wid, wid + nw, ..., a lane the pieces lane and lane + 32; one group.
     // Lane c holds the source box of column c (found once per step).
     int64_t sbox = -1;
@@ -376,7 +430,8 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
         if (ok) {
             if (c.k0 == 0) {
                 sbox = -1;
-                if (c.st.fam == 0) {
+                if (A.mode == 2) sbox = lane < NC ? A.recs[c.st.child].src[lane & 7] : -1;
+                else if (c.st.fam == 0) {
                     if (A.mode == 0) sbox = lane < NC && box0 + lane < nbox ? 4 * (box0 + lane) + c.st.child : -1;
                     else if (lane < T.ncol) sbox = morton((uint32_t)((T.ix0 >> 1) + lane), (uint32_t)(T.iy >> 1));
                 } else if (lane < T.ncol) {
@@ -385,31 +440,31 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
                 }
             }
             const int KS = c.st.fam ? KSl : KSs, nk = min(4, KS - c.k0);
-            const uint4* dig = (c.st.fam ? A.list.dig : A.shift.dig) + (int64_t)c.k0 * (2 * ND);
-            const int64_t stride = (int64_t)A.nrhs * KS * (2 * ND), first = (int64_t)r * KS * (2 * ND);
+            const uint4* dig = (c.st.fam ? A.list.dig : A.shift.dig) + (int64_t)c.k0 * (2 * D);
+            const int64_t stride = (int64_t)A.nrhs * KS * (2 * D), first = (int64_t)r * KS * (2 * D);
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int q = lane + 32 * u, kk = q / 12, d = q % 12 >> 1, h = q & 1;
-                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&Bs[buf][d][kk][0][2 * h]);
+            for (int u = 0; u < (8 * D + 31) / 32; ++u) {
+                const int q = lane + 32 * u, kk = q / (2 * D), d = q % (2 * D) >> 1, h = q & 1;
+                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&Bs[buf][d][kk & 3][0][2 * h]);
                 for (int col = wid; col < NC; col += nw) {
                     const int64_t b = __shfl_sync(0xffffffffu, sbox, col);
-                    if (kk < nk)
+                    if (q < 8 * D && kk < nk)
                         cp_async16(dst + (col >> 3) * 256 + (col & 7) * 32, b >= 0 ? dig + b * stride + first + q : dig, b >= 0);
                 }
             }
         }
         cp_commit();
     };
-    extern __shared__ __align__(16) uint4 s6_ring[];      // [warps][4][ND][32]
-    const uint4* ring = s6_ring + (size_t)wid * (4 * ND * 32) + lane;
+    extern __shared__ __align__(16) uint4 s6_ring[];      // [warps][4][D][32]
+    const uint4* ring = s6_ring + (size_t)wid * (4 * D * 32) + lane;
     const uint32_t ring_a = (uint32_t)__cvta_generic_to_shared(ring);
     // operator fragments of k-step kk of chunk c into slot kk; one group, empty where there is none
     auto load_op = [&](const Chunk& c, int kk, bool ok) {
         const int KS = c.st.fam ? KSl : KSs;
         if (ok && has_m && c.k0 + kk < KS) {
-            const uint4* op = c.st.op + (((int64_t)mt * KS + c.k0 + kk) * ND) * 32 + lane;
+            const uint4* op = c.st.op + (((int64_t)mt * KS + c.k0 + kk) * D) * 32 + lane;
 #pragma unroll
-            for (int d = 0; d < ND; ++d) cp_async16(ring_a + (kk * ND + d) * 512, op + d * 32, true);
+            for (int d = 0; d < D; ++d) cp_async16(ring_a + (kk * D + d) * 512, op + d * 32, true);
         }
         cp_commit();
     };
@@ -432,7 +487,7 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
 #pragma unroll
             for (int t = 0; t < NT; ++t)
 #pragma unroll
-                for (int o = 0; o < 4; ++o)
+                for (int o = 0; o < NI; ++o)
 #pragma unroll
                     for (int x = 0; x < 4; ++x) acc[t][o][x] = 0.0f;
         }
@@ -441,18 +496,18 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
         for (int kk = 0; kk < 4; ++kk) {
             if (kk < 3) cp_wait<4>(); else cp_wait<3>();
             if (has_m && kk < nk) {
-                uint4 a[ND];
+                uint4 a[D];
 #pragma unroll
-                for (int d = 0; d < ND; ++d) a[d] = ring[(kk * ND + d) * 32];
+                for (int d = 0; d < D; ++d) a[d] = ring[(kk * D + d) * 32];
 #pragma unroll
                 for (int t = 0; t < NT; ++t) {
-                    uint2 bb[ND];
+                    uint2 bb[D];
 #pragma unroll
-                    for (int d = 0; d < ND; ++d) bb[d] = Bs[buf][d][kk][t][lane];
+                    for (int d = 0; d < D; ++d) bb[d] = Bs[buf][d][kk][t][lane];
 #pragma unroll
-                    for (int i = 0; i < ND; ++i)
+                    for (int i = 0; i < D; ++i)
 #pragma unroll
-                        for (int j = 0; j < ND - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
+                        for (int j = 0; j < D - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
                 }
             }
             if (kk < 2) load_op(cur, kk, more);
@@ -461,7 +516,7 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
 #pragma unroll
             for (int t = 0; t < NT; ++t)
 #pragma unroll
-                for (int o = 0; o < 4; ++o)
+                for (int o = 0; o < NI; ++o)
 #pragma unroll
                     for (int x = 0; x < 4; ++x) iacc[t][o][x] += __float2int_rn(acc[t][o][x]);
             if (++since == 120) fold(Ef[fam]);            // 120 x 2^24 < 2^31
@@ -473,7 +528,7 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
     cp_wait<0>();
 
     // partial sums of the cluster's CTAs, added in rank order by rank 0
-    double* part = reinterpret_cast<double*>(&Bs[0][0][0][0][0]);   // [warp][NT][4][32]: 8 NT x 1 KB <= 24 KB NT / 2
+    double* part = reinterpret_cast<double*>(s6_ring);              // [warp][NT][4][32]: NT KB of a warp's 2 D KB
     if (S > 1) {
         __syncthreads();
         if (rank != 0 && has_m)
@@ -509,12 +564,12 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
             const int row = 16 * mt + (lane >> 2) + (v >> 1) * 8, c = 8 * t + 2 * (lane & 3) + (v & 1);
             const int64_t b = target(c);
             if (row >= 2 * no || b < 0) continue;
-            const int sh = A.sxo[abs((row >> 1) - A.p)];
-            double* o = reinterpret_cast<double*>(A.out + (b * A.nrhs + r) * no) + row;
-            double x = bad ? nan : dacc[t][v] * pow2d(A.osign * sh);
+            const int sh = A.sxo ? A.osign * A.sxo[abs((row >> 1) - A.p)] : 0;
+            R* o = reinterpret_cast<R*>(A.out) + ((b * A.nrhs + r) * no * 2 + row);
+            R x = (R)(bad ? nan : dacc[t][v] * pow2d(sh));
             if (A.accumulate) x += *o;
             *o = x;
-            e = max(e, s6_exponent(x, -A.osign * sh));
+            e = max(e, s6_exponent(x, -sh));
         }
     if (A.Eout) {
         e = __reduce_max_sync(0xffffffffu, e);
@@ -522,7 +577,7 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
     }
 }
 
-template <int NT>
+template <int NT, int D>
 hfmm_status s6_launch(const S6Args& A, int tiles, int steps, cudaStream_t st) {
     const int MT = (2 * (2 * A.p + 1) + 15) / 16;
     const int gy = (MT + S6_MAXW - 1) / S6_MAXW, W = (MT + gy - 1) / gy;
@@ -533,8 +588,9 @@ hfmm_status s6_launch(const S6Args& A, int tiles, int steps, cudaStream_t st) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(tiles * S), (unsigned)gy, (unsigned)A.nrhs);
     cfg.blockDim = dim3(32 * W);
-    cfg.dynamicSmemBytes = (size_t)W * 4 * ND * 512;
-    HFMM_CUDA_TRY(cudaFuncSetAttribute(s6_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, S6_MAXW * 4 * ND * 512));
+    cfg.dynamicSmemBytes = (size_t)W * 4 * D * 512;
+    HFMM_CUDA_TRY(cudaFuncSetAttribute(s6_kernel<NT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       S6_MAXW * 4 * D * 512));
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -542,13 +598,16 @@ hfmm_status s6_launch(const S6Args& A, int tiles, int steps, cudaStream_t st) {
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    HFMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, s6_kernel<NT>, A));
+    HFMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, s6_kernel<NT, D>, A));
     return HFMM_OK;
 }
 
 // Columns per tile: 16 where that still fills the GPU (each operator slice is
 // read once per tile), else 8.
+template <int D>
 hfmm_status s6_run(S6Args& A, cudaStream_t st) {
+    if (A.tiles == 0 && A.mode == 2) return HFMM_OK;
+    if (A.mode == 2) return s6_launch<1, D>(A, A.tiles, 28, st);
     const int64_t n = (int64_t)1 << A.l;
     const int MT = (2 * (2 * A.p + 1) + 15) / 16, gy = (MT + S6_MAXW - 1) / S6_MAXW;
     auto tiles = [&](int nc) -> int64_t {
@@ -559,7 +618,7 @@ hfmm_status s6_run(S6Args& A, cudaStream_t st) {
     const int steps = A.mode == 0 ? 4 : 1 + (A.vlist ? 27 : 0) + (A.rlist ? (int)std::min<int64_t>(n, 1 << 20) : 0);
     const bool wide = (A.mode == 0 || (n >> 1) > 8) && tiles(16) * gy >= 3 * 152;
     A.tiles = (int)tiles(wide ? 16 : 8);
-    return wide ? s6_launch<2>(A, A.tiles, steps, st) : s6_launch<1>(A, A.tiles, steps, st);
+    return wide ? s6_launch<2, D>(A, A.tiles, steps, st) : s6_launch<1, D>(A, A.tiles, steps, st);
 }
 
 S6Fam s6_fam(const unsigned* dig, int p, const uint4* ops, const int* Eop, const int* Esrc) {
@@ -572,172 +631,247 @@ S6Fam s6_fam(const unsigned* dig, int p, const uint4* ops, const int* Eop, const
     return f;
 }
 
-}  // namespace
+template <int D> S6Lev& s6_lev(LevelInfo& lv) { return lv.s6[D == 6 ? 0 : 1]; }
+template <int D> typename S6Traits<D>::C* s6_expansion(const LevelInfo& lv, bool loc);
+template <> cd* s6_expansion<6>(const LevelInfo& lv, bool loc) { return loc ? lv.loc : lv.mult; }
+template <> cf* s6_expansion<3>(const LevelInfo& lv, bool loc) { return loc ? lv.loc32 : lv.mult32; }
 
-// Operator slices of every level (plan time, or a mixed plan's first gradient).
-// A plan whose slices or digits would pass the byte budget keeps the FP64 kernels.
-hfmm_status build_split64(hfmm_plan_s* P, cudaStream_t st) {
-    if (P->s6_ready || P->ad) return HFMM_OK;
+template <int D>
+hfmm_status s6_build(hfmm_plan_s* P, cudaStream_t st) {
+    constexpr int w = D == 6 ? 0 : 1;
+    if (P->s6_ready[w]) return HFMM_OK;
     const int L = P->L;
+    auto bytes = [](int nop, int po, int pi) {
+        return 512.0 * D * nop * ((2 * (2 * po + 1) + 15) / 16) * ((2 * (2 * pi + 1) + 15) / 16);
+    };
+    auto digits = [&](const LevelInfo& lv) { return (size_t)lv.nbox * P->max_rhs * ((2 * lv.ncoef + 15) / 16) * (D * 32); };
+    // reaction entries of an adaptive tree: the ones its lists use
+    std::vector<std::vector<int32_t>> rmap(L + 1);
+    if (P->ad)
+        for (int l = P->lmin; l <= L; ++l) adaptive_react_entries(P, l, rmap[l]);
+    auto has_free = [&](const LevelInfo& lv) { return !lv.diag_logq && lv.t_free && lv.nv > 0; };
+    auto nreact = [&](int l) {
+        const LevelInfo& lv = P->lev[l];
+        if (lv.diag_logq || !lv.t_react || lv.nr == 0) return 0;
+        return P->ad ? (int)rmap[l].size() : lv.n_react_entries;
+    };
+    double used = 0.0, dbytes = 0.0;
+    for (int l = P->lmin; l <= L; ++l) {
+        const LevelInfo& lv = P->lev[l];
+        used += (has_free(lv) ? bytes(49, lv.p, lv.p) : 0.0) + bytes(nreact(l), lv.p, lv.p);
+        if (l > P->lmin) used += bytes(4, lv.p, P->lev[l - 1].p) + bytes(4, P->lev[l - 1].p, lv.p);
+        dbytes += (l < L ? 2.0 : 1.0) * digits(lv);
+    }
+    if (used > S6_MAX_BYTES || dbytes > S6_MAX_BYTES) return HFMM_OK;
     int* E = nullptr;                                     // [level][3] families, then [kind][level][rhs] expansions
     const size_t ne = (size_t)3 * (L + 1) + (size_t)2 * (L + 1) * P->max_rhs;
     HFMM_TRY(plan_alloc(P, (void**)&E, sizeof(int) * ne));
-    P->s6_E = E + 3 * (L + 1);
+    P->s6_E[w] = E + 3 * (L + 1);
     HFMM_CUDA_TRY(cudaMemsetAsync(E, 0x80, sizeof(int) * ne, st));   // far below S6_NONE
     std::vector<int> sx;
     std::vector<size_t> off(L + 1, 0);
+    std::vector<int32_t> maps;
+    std::vector<size_t> moff(L + 1, 0);
     for (int l = 0; l <= L; ++l) {
         const LevelInfo& lv = P->lev[l];
         off[l] = sx.size();
         const double kR = P->k * lv.h / std::sqrt(2.0);
         for (int n = 0; n <= lv.p; ++n)
             sx.push_back((int)std::lround(std::min(0.0, n * std::log(0.5 * kR) - std::lgamma(n + 1.0)) / std::log(2.0)));
+        moff[l] = maps.size();
+        maps.insert(maps.end(), rmap[l].begin(), rmap[l].end());
     }
-    int* dsx = nullptr;
+    int *dsx = nullptr, *dmaps = nullptr;
     HFMM_TRY(plan_alloc(P, (void**)&dsx, sizeof(int) * sx.size()));
     HFMM_CUDA_TRY(cudaMemcpyAsync(dsx, sx.data(), sizeof(int) * sx.size(), cudaMemcpyHostToDevice, st));
-    HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // sx is a local
-    auto bytes = [](int nop, int po, int pi) {
-        return 512.0 * ND * nop * ((2 * (2 * po + 1) + 15) / 16) * ((2 * (2 * pi + 1) + 15) / 16);
+    HFMM_TRY(plan_alloc(P, (void**)&dmaps, sizeof(int) * maps.size()));
+    if (!maps.empty())
+        HFMM_CUDA_TRY(cudaMemcpyAsync(dmaps, maps.data(), sizeof(int) * maps.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // the vectors are locals
+    for (int l = 0; l <= L; ++l) s6_lev<D>(P->lev[l]).sx = D == 6 ? dsx + off[l] : nullptr;
+    auto op_of = [&](const cd* T, int kind, int nop, LevelInfo& o, LevelInfo& i, const int32_t* map) {
+        return S6Op{T, map, kind, nop, o.p, i.p, s6_lev<D>(o).sx, s6_lev<D>(i).sx, o.d_log_s, i.d_log_s};
     };
-    auto has_free = [&](const LevelInfo& lv) { return !lv.diag_logq && lv.t_free && lv.nv > 0; };
-    auto has_react = [&](const LevelInfo& lv) { return !lv.diag_logq && lv.t_react && lv.nr > 0; };
-    double used = 0.0;
-    for (int l = P->lmin; l <= L; ++l) {
-        const LevelInfo& lv = P->lev[l];
-        used += (has_free(lv) ? bytes(49, lv.p, lv.p) : 0.0) + (has_react(lv) ? bytes(lv.n_react_entries, lv.p, lv.p) : 0.0);
-        if (l > P->lmin) used += bytes(4, lv.p, P->lev[l - 1].p) + bytes(4, P->lev[l - 1].p, lv.p);
-    }
-    auto digits = [&](const LevelInfo& lv) { return (size_t)lv.nbox * P->max_rhs * ((2 * lv.ncoef + 15) / 16) * (ND * 32); };
-    double dbytes = 0.0;
-    for (int l = P->lmin; l <= L; ++l) dbytes += (l < L ? 2.0 : 1.0) * digits(P->lev[l]);
-    if (used > S6_MAX_BYTES || dbytes > S6_MAX_BYTES) return HFMM_OK;
-    for (int l = P->lmin; l <= L; ++l) {
-        LevelInfo& lv = P->lev[l];
-        HFMM_TRY(plan_alloc(P, (void**)&lv.s6_dmult, digits(lv)));
-        if (l < L) HFMM_TRY(plan_alloc(P, (void**)&lv.s6_dloc, digits(lv)));
-    }
-    P->buffer_bytes += dbytes;
-    auto make = [&](const cd* T, int kind, int nop, const LevelInfo& o, const LevelInfo& i, int* Ep, uint4** out) -> hfmm_status {
-        S6Op op{T, kind, nop, o.p, i.p, o.s6_sx, i.s6_sx};
-        HFMM_TRY(plan_alloc(P, (void**)out, (size_t)bytes(nop, o.p, i.p)));
-        const int64_t total = (int64_t)(bytes(nop, o.p, i.p) / (16.0 * ND));
-        s6_op_slice_kernel<<<(unsigned)std::min<int64_t>((total + 127) / 128, 64 * 152), 128, 0, st>>>(op, Ep, *out);
-        HFMM_CUDA_TRY(cudaGetLastError());
-        return HFMM_OK;
-    };
-    auto expo = [&](const cd* T, int kind, int nop, const LevelInfo& o, const LevelInfo& i, int* Ep) -> hfmm_status {
-        S6Op op{T, kind, nop, o.p, i.p, o.s6_sx, i.s6_sx};
-        const int64_t total = (int64_t)nop * o.ncoef * i.ncoef;
+    auto expo = [&](const S6Op& op, int* Ep) -> hfmm_status {
+        const int64_t total = (int64_t)op.nop * (2 * op.po + 1) * (2 * op.pi + 1);
         s6_op_exponent_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), 256, 0, st>>>(op, Ep);
         HFMM_CUDA_TRY(cudaGetLastError());
         return HFMM_OK;
     };
-    for (int l = 0; l <= L; ++l) P->lev[l].s6_sx = dsx + off[l];
+    auto make = [&](const S6Op& op, int* Ep, uint4** out) -> hfmm_status {
+        HFMM_TRY(plan_alloc(P, (void**)out, (size_t)bytes(op.nop, op.po, op.pi)));
+        const int64_t total = (int64_t)(bytes(op.nop, op.po, op.pi) / (16.0 * D));
+        s6_op_slice_kernel<D><<<(unsigned)std::min<int64_t>((total + 127) / 128, 64 * 152), 128, 0, st>>>(op, Ep, *out);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        return HFMM_OK;
+    };
     for (int l = P->lmin; l <= L; ++l) {
         LevelInfo& lv = P->lev[l];
-        lv.s6_Eop = E + 3 * l;
-        const bool fr = has_free(lv), re = has_react(lv);  // diagonal levels translate in diag.cu
-        if (fr) HFMM_TRY(expo(lv.t_free, S6_FREE, 49, lv, lv, lv.s6_Eop));
-        if (re) HFMM_TRY(expo(lv.t_react, S6_REACT, lv.n_react_entries, lv, lv, lv.s6_Eop));
-        if (fr) HFMM_TRY(make(lv.t_free, S6_FREE, 49, lv, lv, lv.s6_Eop, &lv.s6_free));
-        if (re) HFMM_TRY(make(lv.t_react, S6_REACT, lv.n_react_entries, lv, lv, lv.s6_Eop, &lv.s6_react));
+        S6Lev& s = s6_lev<D>(lv);
+        HFMM_TRY(plan_alloc(P, (void**)&s.dmult, digits(lv)));
+        if (l < L) HFMM_TRY(plan_alloc(P, (void**)&s.dloc, digits(lv)));
+        s.Eop = E + 3 * l;
+        const int nre = nreact(l);                        // diagonal levels translate in diag.cu
+        const S6Op fr = op_of(lv.t_free, S6_FREE, 49, lv, lv, nullptr);
+        const S6Op re = op_of(lv.t_react, S6_REACT, nre, lv, lv, P->ad ? dmaps + moff[l] : nullptr);
+        if (has_free(lv)) HFMM_TRY(expo(fr, s.Eop));
+        if (nre) HFMM_TRY(expo(re, s.Eop));
+        if (has_free(lv)) HFMM_TRY(make(fr, s.Eop, &s.free));
+        if (nre) HFMM_TRY(make(re, s.Eop, &s.react));
         if (l > P->lmin) {
-            HFMM_TRY(expo(P->lev[l - 1].t_l2l, S6_L2L, 4, lv, P->lev[l - 1], lv.s6_Eop + 1));
-            HFMM_TRY(make(P->lev[l - 1].t_l2l, S6_L2L, 4, lv, P->lev[l - 1], lv.s6_Eop + 1, &lv.s6_l2l));
+            const S6Op op = op_of(P->lev[l - 1].t_l2l, S6_L2L, 4, lv, P->lev[l - 1], nullptr);
+            HFMM_TRY(expo(op, s.Eop + 1));
+            HFMM_TRY(make(op, s.Eop + 1, &s.l2l));
         }
         if (l < L) {
-            HFMM_TRY(expo(lv.t_m2m, S6_M2M, 4, lv, P->lev[l + 1], lv.s6_Eop + 2));
-            HFMM_TRY(make(lv.t_m2m, S6_M2M, 4, lv, P->lev[l + 1], lv.s6_Eop + 2, &lv.s6_m2m));
+            const S6Op op = op_of(lv.t_m2m, S6_M2M, 4, lv, P->lev[l + 1], nullptr);
+            HFMM_TRY(expo(op, s.Eop + 2));
+            HFMM_TRY(make(op, s.Eop + 2, &s.m2m));
+        }
+        if (P->ad) {
+            for (int up = 0; up < 2; ++up) {
+                std::vector<int32_t> tgt, tbeg;
+                std::vector<S6Rec> recs;
+                adaptive_tiles(P, l, up == 1, rmap[l], tgt, tbeg, recs);
+                S6Tiles& t = up ? s.up : s.down;
+                t.n = (int)(tgt.size() / 8);
+                if (t.n == 0) continue;
+                HFMM_TRY(plan_alloc(P, (void**)&t.tgt, sizeof(int32_t) * tgt.size()));
+                HFMM_TRY(plan_alloc(P, (void**)&t.tbeg, sizeof(int32_t) * tbeg.size()));
+                HFMM_TRY(plan_alloc(P, (void**)&t.recs, sizeof(S6Rec) * std::max<size_t>(recs.size(), 1)));
+                HFMM_CUDA_TRY(cudaMemcpyAsync(t.tgt, tgt.data(), sizeof(int32_t) * tgt.size(), cudaMemcpyHostToDevice, st));
+                HFMM_CUDA_TRY(cudaMemcpyAsync(t.tbeg, tbeg.data(), sizeof(int32_t) * tbeg.size(), cudaMemcpyHostToDevice, st));
+                if (!recs.empty())
+                    HFMM_CUDA_TRY(cudaMemcpyAsync(t.recs, recs.data(), sizeof(S6Rec) * recs.size(), cudaMemcpyHostToDevice, st));
+                HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+            }
         }
     }
     P->table_bytes += used;
-    P->s6_ready = true;
+    P->buffer_bytes += dbytes;
+    P->s6_ready[w] = true;
     return HFMM_OK;
 }
 
-// Start of a tree pass: no exponent is known.
-hfmm_status split64_begin(hfmm_plan_s* P, cudaStream_t st) {
-    HFMM_CUDA_TRY(cudaMemsetAsync(P->s6_E, 0x80, sizeof(int) * 2 * (P->L + 1) * P->max_rhs, st));
-    return HFMM_OK;
-}
-
-int* split64_exp(hfmm_plan_s* P, int l, bool loc) { return P->s6_E + ((size_t)(loc ? P->L + 1 : 0) + l) * P->max_rhs; }
-
-// Exponents of a level's expansions that another kernel wrote.
-hfmm_status split64_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
-    LevelInfo& lv = P->lev[l];
-    const int64_t total = lv.nbox * lv.ncoef;
-    s6_exponent_kernel<<<dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs), 256, 0, st>>>(
-        loc ? lv.loc : lv.mult, lv.nbox, nrhs, lv.p, lv.s6_sx, loc ? 1 : -1, split64_exp(P, l, loc));
-    ++P->launches;
-    HFMM_CUDA_TRY(cudaGetLastError());
-    return HFMM_OK;
-}
-
-// Digits of a level's finished expansions, for the products that read them.
-hfmm_status split64_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
-    LevelInfo& lv = P->lev[l];
-    const int64_t total = lv.nbox * ((2 * lv.ncoef + 15) / 16 * 8);
-    s6_slice_kernel<<<dim3((unsigned)std::min<int64_t>((total + 127) / 128, 16 * 152), (unsigned)nrhs), 128, 0, st>>>(
-        loc ? lv.loc : lv.mult, lv.nbox, nrhs, lv.p, lv.s6_sx, loc ? 1 : -1, split64_exp(P, l, loc),
-        loc ? lv.s6_dloc : lv.s6_dmult);
-    ++P->launches;
-    HFMM_CUDA_TRY(cudaGetLastError());
-    return HFMM_OK;
-}
-
-hfmm_status split64_m2m(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st) {
+template <int D>
+hfmm_status s6_m2m(hfmm_plan_s* P, int l, int nrhs, cudaStream_t st) {
+    constexpr int w = D == 6 ? 0 : 1;
     LevelInfo& lv = P->lev[l];
     LevelInfo& ch = P->lev[l + 1];
+    const S6Lev &s = s6_lev<D>(lv), &sc = s6_lev<D>(ch);
     S6Args A{};
-    A.l = l; A.L = P->L; A.mode = 0; A.nrhs = nrhs; A.p = lv.p;
-    A.shift = s6_fam(ch.s6_dmult, ch.p, lv.s6_m2m, lv.s6_Eop + 2, split64_exp(P, l + 1, false));
-    A.sxo = lv.s6_sx;
+    A.l = l; A.L = P->L; A.mode = P->ad ? 2 : 0; A.nrhs = nrhs; A.p = lv.p;
+    A.shift = s6_fam(sc.dmult, ch.p, s.m2m, s.Eop + 2, split_exp(P, w, l + 1, false));
+    A.sxo = s.sx;
     A.osign = 1;
-    A.out = lv.mult;
-    A.Eout = split64_exp(P, l, false);
+    A.out = s6_expansion<D>(lv, false);
+    A.Eout = split_exp(P, w, l, false);
+    A.tiles = s.up.n; A.tgt = s.up.tgt; A.tbeg = s.up.tbeg; A.recs = s.up.recs;
     ++P->launches;
-    return s6_run(A, st);
+    return s6_run<D>(A, st);
 }
 
 // L2L and both M2L lists of level l into loc (diagonal levels: the L2L alone).
-hfmm_status split64_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st) {
+template <int D>
+hfmm_status s6_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st) {
+    constexpr int w = D == 6 ? 0 : 1;
     LevelInfo& lv = P->lev[l];
+    const S6Lev& s = s6_lev<D>(lv);
     const bool dg = lv.diag_logq > 0;
     S6Args A{};
-    A.l = l; A.L = P->L; A.mode = 1; A.nrhs = nrhs; A.p = lv.p;
+    A.l = l; A.L = P->L; A.mode = P->ad ? 2 : 1; A.nrhs = nrhs; A.p = lv.p;
     A.lb = P->leaf_begin;
     if (l > P->lmin) {
         LevelInfo& pa = P->lev[l - 1];
-        A.shift = s6_fam(pa.s6_dloc, pa.p, lv.s6_l2l, lv.s6_Eop + 1, split64_exp(P, l - 1, true));
+        A.shift = s6_fam(s6_lev<D>(pa).dloc, pa.p, s.l2l, s.Eop + 1, split_exp(P, w, l - 1, true));
     }
-    A.list = s6_fam(lv.s6_dmult, lv.p, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false));
-    A.rops = lv.s6_react;
+    const S6Fam list = s6_fam(s.dmult, lv.p, s.free, s.Eop, split_exp(P, w, l, false));
+    A.rops = s.react;
     A.vlist = !dg && lv.nv > 0 && (parts & HFMM_PART_FAR_FREE);
     const bool react = !dg && lv.nr > 0 && (parts & HFMM_PART_FAR_REACT);
     A.lstar = P->lstar;
-    A.sxo = lv.s6_sx;
+    A.sxo = s.sx;
     A.osign = -1;
-    A.out = lv.loc;
-    A.Eout = split64_exp(P, l, true);
+    A.out = s6_expansion<D>(lv, true);
+    A.Eout = split_exp(P, w, l, true);
     A.rows = 1 << l;
+    A.tiles = s.down.n; A.tgt = s.down.tgt; A.tbeg = s.down.tbeg; A.recs = s.down.recs;
     // a bottom-row tile of a fine level has up to 2^(l + 1) reaction steps against
     // 28 of the others: there they run as a launch of their own over the two rows
-    const bool apart = react && l >= 5;
+    const bool apart = react && l >= 5 && !P->ad;
     A.rlist = react && !apart;
-    if (!A.vlist && !A.rlist) A.list.dig = nullptr;
+    if (A.vlist || A.rlist) A.list = list;
     ++P->launches;
-    HFMM_TRY(s6_run(A, st));
+    HFMM_TRY(s6_run<D>(A, st));
     if (apart) {
-        A.list = s6_fam(lv.s6_dmult, lv.p, lv.s6_free, lv.s6_Eop, split64_exp(P, l, false));
+        A.list = list;
         A.shift.dig = nullptr;
         A.vlist = 0;
         A.rlist = 1;
         A.rows = 2;
         A.accumulate = 1;
         ++P->launches;
-        HFMM_TRY(s6_run(A, st));
+        HFMM_TRY(s6_run<D>(A, st));
     }
     return HFMM_OK;
+}
+
+template <int D>
+hfmm_status s6_exponent_of(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[l];
+    const int64_t total = lv.nbox * lv.ncoef;
+    s6_exponent_kernel<<<dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs), 256, 0, st>>>(
+        s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, s6_lev<D>(lv).sx, loc ? 1 : -1,
+        split_exp(P, D == 6 ? 0 : 1, l, loc));
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+template <int D>
+hfmm_status s6_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[l];
+    const S6Lev& s = s6_lev<D>(lv);
+    const int64_t total = lv.nbox * ((2 * lv.ncoef + 15) / 16 * 8);
+    s6_slice_kernel<D><<<dim3((unsigned)std::min<int64_t>((total + 127) / 128, 16 * 152), (unsigned)nrhs), 128, 0, st>>>(
+        s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, s.sx, loc ? 1 : -1, split_exp(P, D == 6 ? 0 : 1, l, loc),
+        loc ? s.dloc : s.dmult);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+}  // namespace
+
+// w = 0: the FP64 expansions, 1: the mixed path's FP32 expansions.
+// Operator slices of every level (plan time, or a mixed plan's first gradient).
+// A plan whose slices or digits would pass the byte budget keeps the SIMT kernels.
+hfmm_status build_split(hfmm_plan_s* P, int w, cudaStream_t st) { return w ? s6_build<3>(P, st) : s6_build<6>(P, st); }
+
+// Start of a tree pass: no exponent is known.
+hfmm_status split_begin(hfmm_plan_s* P, int w, cudaStream_t st) {
+    HFMM_CUDA_TRY(cudaMemsetAsync(P->s6_E[w], 0x80, sizeof(int) * 2 * (P->L + 1) * P->max_rhs, st));
+    return HFMM_OK;
+}
+
+int* split_exp(hfmm_plan_s* P, int w, int l, bool loc) {
+    return P->s6_E[w] + ((size_t)(loc ? P->L + 1 : 0) + l) * P->max_rhs;
+}
+
+// Exponents of a level's expansions that another kernel wrote.
+hfmm_status split_exponent(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st) {
+    return w ? s6_exponent_of<3>(P, l, loc, nrhs, st) : s6_exponent_of<6>(P, l, loc, nrhs, st);
+}
+
+// Digits of a level's finished expansions, for the products that read them.
+hfmm_status split_slice(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st) {
+    return w ? s6_slice<3>(P, l, loc, nrhs, st) : s6_slice<6>(P, l, loc, nrhs, st);
+}
+
+hfmm_status split_m2m(hfmm_plan_s* P, int w, int l, int nrhs, cudaStream_t st) {
+    return w ? s6_m2m<3>(P, l, nrhs, st) : s6_m2m<6>(P, l, nrhs, st);
+}
+
+hfmm_status split_down(hfmm_plan_s* P, int w, int l, int nrhs, int parts, cudaStream_t st) {
+    return w ? s6_down<3>(P, l, nrhs, parts, st) : s6_down<6>(P, l, nrhs, parts, st);
 }

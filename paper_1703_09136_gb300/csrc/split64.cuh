@@ -1,14 +1,21 @@
-// FP64 numbers as six signed base-512 digits in f16 (see split64.cu): exponents,
+// Numbers as signed base-512 digits in f16 (see split64.cu): exponents,
 // fixed-point words with biased digit fields, digit pairs, and the FP32
 // mma.sync that sums digit products without rounding.
 #pragma once
 
 #include "common.cuh"
 
-constexpr int ND = 6;                    // digits
 constexpr int S6_NONE = -(1 << 24);      // exponent of an all-zero level (or below)
-constexpr long long S6_BIAS = 0x100804020100ll;   // 256 sum_{i = 0 .. 4} 512^i: low five fields = digit + 256
 constexpr int S6_NAN = 1 << 20;          // exponent of a level with an infinity or a NaN
+
+// D digits: 9 D - 1 bits; the bias 256 sum_{i = 0 .. D - 2} 512^i makes the low D - 1
+// fields of a word digit + 256
+template <int D>
+__host__ __device__ constexpr long long s6_bias() {
+    long long b = 0;
+    for (int i = 0; i < D - 1; ++i) b = (b << 9) + 256;
+    return b;
+}
 
 // largest E with |v 2^shift| < 2^E (S6_NONE for zero)
 __device__ __forceinline__ int s6_exponent(double v, int shift) {
@@ -18,23 +25,40 @@ __device__ __forceinline__ int s6_exponent(double v, int shift) {
     if (e == 0) return (b & 0xfffffffffffffll) ? -1021 + shift : S6_NONE;
     return e - 1022 + shift;
 }
+__device__ __forceinline__ int s6_exponent(float v, int shift) {
+    const int b = __float_as_int(v), e = (b >> 23) & 255;
+    if (e == 255) return S6_NAN;
+    if (e == 0) return (b & 0x7fffff) ? -125 + shift : S6_NONE;
+    return e - 126 + shift;
+}
 
-// v 2^shift 2^(BITS - E) rounded to an integer plus the digit bias, |v 2^shift| < 2^E
+// v 2^shift 2^(BITS - E) rounded to an integer, |v 2^shift| < 2^E (BITS <= 53; floats: BITS >= 24)
 template <int BITS>
 __device__ __forceinline__ long long s6_fixed(double v, int shift, int E) {
     const long long b = __double_as_longlong(v);
     int e = (int)((b >> 52) & 2047);
     unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
     if (e) m |= 1ull << 52; else e = 1;
-    const int s = E - shift - e + 1075 - BITS;            // right shift, >= 0 for BITS = 53
+    const int s = E - shift - e + 1075 - BITS;            // right shift
     if (s > 0) m = s > 54 ? 0ull : (m + (1ull << (s - 1))) >> s;
-    const long long x = b < 0 ? -(long long)m : (long long)m;
-    return x + S6_BIAS;
+    return b < 0 ? -(long long)m : (long long)m;
+}
+template <int BITS>
+__device__ __forceinline__ long long s6_fixed(float v, int shift, int E) {
+    const int b = __float_as_int(v);
+    int e = (b >> 23) & 255;
+    unsigned m = (unsigned)b & 0x7fffffu;
+    if (e) m |= 1u << 23; else e = 1;
+    const int s = E - shift - e + 150 - BITS;             // right shift, at least 24 - BITS
+    if (s > 0) m = s > 25 ? 0u : (m + (1u << (s - 1))) >> s;
+    else m <<= min(-s, BITS - 24);
+    return b < 0 ? -(long long)m : (long long)m;
 }
 
-// field of digit i (0 = most significant), digit + 256 in [0, 512]
+// field of digit i (0 = most significant) of a biased word, digit + 256 in [0, 512]
+template <int D>
 __device__ __forceinline__ unsigned s6_field(long long xb, int i) {
-    return i == 0 ? (unsigned)((int)(xb >> 45) + 256) : (unsigned)(xb >> (9 * (ND - 1 - i))) & 511u;
+    return i == 0 ? (unsigned)((int)(xb >> (9 * (D - 1))) + 256) : (unsigned)(xb >> (9 * (D - 1 - i))) & 511u;
 }
 
 // two digits as f16 (1024 + field as bits 0x6400 | field, minus 1280)
