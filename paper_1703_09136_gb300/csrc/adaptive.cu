@@ -523,11 +523,13 @@ __global__ void __launch_bounds__(128) ad_p2l_kernel(const AdBox* __restrict__ b
                                                      const C* __restrict__ q, int64_t sj, int64_t sr, int nrhs, int p,
                                                      const int* __restrict__ sx, int* __restrict__ E, C* __restrict__ loc) {
     __shared__ C part[4][32];
+    pdl_start_next();
     const int32_t bi = list[blockIdx.x];
     const int r = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nc = 2 * p + 1;
     C* out = loc + ((int64_t)boxes[bi].lidx * nrhs + r) * nc;
     const C* qr = q + r * sr;
     int ex = S6_NONE;
+    pdl_wait();
     for (int m0 = 0; m0 < nc; m0 += 32) {
         const int m = m0 + lane;
         C acc{0, 0};
@@ -543,7 +545,7 @@ __global__ void __launch_bounds__(128) ad_p2l_kernel(const AdBox* __restrict__ b
         part[wid][lane] = acc;
         __syncthreads();
         if (wid == 0 && m < nc) {
-            C v = out[m];
+            C v = __ldcg(out + m);
             for (int w = 0; w < 4; ++w) { v.x += part[w][lane].x; v.y += part[w][lane].y; }
             out[m] = v;
             const int sh = sx ? sx[abs(m - p)] : 0;
@@ -1238,11 +1240,10 @@ static hfmm_status ad_tree_pass(hfmm_plan_s* P, int w, int nrhs, int parts, cons
         HFMM_TRY(split_down(P, w, l, nrhs, parts, st));
         const int64_t nx = T->xbox_off[l + 1] - T->xbox_off[l];
         if (nx > 0 && (parts & HFMM_PART_FAR_FREE)) {
-            ad_p2l_kernel<C><<<dim3((unsigned)nx, (unsigned)nrhs), 128, 0, st>>>(
-                T->d_boxes, T->d_xbox + T->xbox_off[l], T->dx_beg, T->dx_src, T->d_xboff, p2l, q, sj, sr, nrhs, v.p,
-                v.s6[w].sx, split_exp(P, w, l, true), w ? (C*)v.loc32 : (C*)v.loc);
+            HFMM_CUDA_TRY(pdl_launch(ad_p2l_kernel<C>, dim3((unsigned)nx, (unsigned)nrhs), dim3(128), 0, st, 0, T->d_boxes,
+                                     T->d_xbox + T->xbox_off[l], T->dx_beg, T->dx_src, T->d_xboff, p2l, q, sj, sr, nrhs,
+                                     v.p, v.s6[w].sx, split_exp(P, w, l, true), w ? (C*)v.loc32 : (C*)v.loc));
             ++P->launches;
-            HFMM_CUDA_TRY(cudaGetLastError());
         }
         if (l < L) HFMM_TRY(split_slice(P, w, l, true, nrhs, st));
         double pairs = 0.0;

@@ -65,6 +65,7 @@ template <int PS>
 __global__ void __launch_bounds__(128) p2m64_kernel(const Leaf64Rec* __restrict__ recs, const cd* __restrict__ basis,
                                                     const cd* __restrict__ qs, int64_t n, int64_t nleaf, int pitch,
                                                     int nrhs) {
+    pdl_start_next();
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, it = id / PS;
     const int r = blockIdx.y, part = (int)(id % PS), m = (int)(it % pitch);
     const bool in = it < nleaf * pitch;                    // whole groups of PS lanes
@@ -75,9 +76,10 @@ __global__ void __launch_bounds__(128) p2m64_kernel(const Leaf64Rec* __restrict_
     const cd* B = basis + L.boff + m;
     double s1 = 0.0, s2 = 0.0, s3 = 0.0, s4 = 0.0;
     const int tn = live ? L.tn : 0;
+    pdl_wait();
 #pragma unroll 4
     for (int j = part; j < tn; j += PS) {
-        const cd a = __ldg(q + j), u = __ldg(B + (int64_t)j * nb);
+        const cd a = __ldcg(q + j), u = __ldg(B + (int64_t)j * nb);
         s1 = fma(a.x, u.x, s1);
         s2 = fma(a.y, u.y, s2);
         s3 = fma(a.x, u.y, s3);
@@ -115,6 +117,8 @@ __global__ void __launch_bounds__(128) p2m64_kernel(const Leaf64Rec* __restrict_
 
 // Empty leaves of a uniform tree: zero multipoles (their parents' M2M reads them).
 __global__ void zero_empty_kernel(const int32_t* __restrict__ lb, int64_t nleaf, int64_t per, cd* __restrict__ mult) {
+    pdl_start_next();
+    pdl_wait();
     for (int64_t b = blockIdx.x; b < nleaf; b += gridDim.x)
         if (lb[b + 1] == lb[b])
             for (int64_t i = threadIdx.x; i < per; i += blockDim.x) mult[b * per + i] = cmk(0.0, 0.0);
@@ -195,6 +199,7 @@ __device__ __forceinline__ T quad_scatter(const T (&v)[4], int t) {
 template <int W>
 __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Args A) {
     extern __shared__ __align__(16) double lf_smem[];
+    pdl_start_next();
     constexpr int CHUNK = 128 * W, QPT = 4;                             // sources staged at once; per thread
     const Leaf64Rec L = A.recs[blockIdx.x];
     const int32_t tlo = L.tlo, tn = L.tn;
@@ -210,13 +215,14 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
     const cd* q = A.qs + (int64_t)r * A.n;
     const int p = L.p, nb = L.nb, nc = 2 * p + 1;
     const bool l2p = A.l2p && L.loc;
+    pdl_wait();
     if (l2p) {
         // y = (i/4) sum_m beta_m conj-basis: with c = beta_m, d = (-1)^m beta_{-m} and B = (u, v)
         // re y = sum u w0 + v w1, im y = sum u w2 + v w3
         const cd* beta = L.loc + (L.lidx * A.nrhs + r) * nc + p;
         for (int m = tid; m <= p; m += W * 32) {
-            const cd c = beta[m];
-            cd d = m > 0 ? beta[-m] : cmk(0.0, 0.0);
+            const cd c = __ldcg(beta + m);
+            cd d = m > 0 ? __ldcg(beta - m) : cmk(0.0, 0.0);
             if (m & 1) d = cneg(d);
             coef[4 * m] = -0.25 * (c.y + d.y);
             coef[4 * m + 1] = 0.25 * (c.x - d.x);
@@ -370,7 +376,7 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
                     const cd* M = A.m2pb + D.boff;
 #pragma unroll 2
                     for (int m = t + 4 * part; m < nw; m += 4 * ks) {
-                        const cd a = __ldg(am + m);
+                        const cd a = __ldcg(am + m);
                         if (v0) cfma(a0, a, __ldg(M + (int64_t)i0 * nw + m));
                         if (v1) cfma(a1, a, __ldg(M + (int64_t)i1 * nw + m));
                     }
@@ -557,14 +563,13 @@ hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
     auto kernel = ps == 4 ? p2m64_kernel<4> : p2m64_kernel<1>;
     if (P->leaf_empty) {
         const LevelInfo& lv = P->lev[P->L];
-        zero_empty_kernel<<<(unsigned)std::min<int64_t>(lv.nbox, 16 * 152), 64, 0, st>>>(
-            P->leaf_begin, lv.nbox, (int64_t)nrhs * lv.ncoef, lv.mult);
+        HFMM_CUDA_TRY(pdl_launch(zero_empty_kernel, dim3((unsigned)std::min<int64_t>(lv.nbox, 16 * 152)), dim3(64), 0, st, 0,
+                                 P->leaf_begin, lv.nbox, (int64_t)nrhs * lv.ncoef, lv.mult));
         ++P->launches;
     }
-    kernel<<<dim3((unsigned)((items * ps + 127) / 128), (unsigned)nrhs), 128, 0, st>>>(
-        P->leaf64, P->basis64, P->q_sorted, P->n, P->leaf64_n, pitch, nrhs);
+    HFMM_CUDA_TRY(pdl_launch(kernel, dim3((unsigned)((items * ps + 127) / 128), (unsigned)nrhs), dim3(128), 0, st, 0,
+                             P->leaf64, P->basis64, P->q_sorted, P->n, P->leaf64_n, pitch, nrhs));
     ++P->launches;
-    HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;
 }
 
@@ -602,8 +607,7 @@ hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2
     auto kernel = one ? leaf64_kernel<1> : leaf64_kernel<4>;
     if (sm > 47 * 1024)                                    // (static shared memory beside it)
         HFMM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    kernel<<<dim3((unsigned)P->leaf64_n, (unsigned)nrhs), W * 32, sm, st>>>(A);
+    HFMM_CUDA_TRY(pdl_launch(kernel, dim3((unsigned)P->leaf64_n, (unsigned)nrhs), dim3(W * 32), sm, st, 0, A));
     ++P->launches;
-    HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;
 }

@@ -147,13 +147,15 @@ __global__ void s6_op_slice_kernel(S6Op o, const int* __restrict__ Ep, uint4* __
 template <class C>
 __global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
                                    int sign, int* __restrict__ E) {
+    pdl_start_next();
     const int nc = 2 * p + 1, r = blockIdx.y;
     int e = S6_NONE;
     const int64_t total = nbox * nc;
+    pdl_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / nc;
         const int m = (int)(i % nc) - p;
-        const C v = a[(b * nrhs + r) * nc + m + p];
+        const C v = __ldcg(a + (b * nrhs + r) * nc + m + p);
         const int sh = sx ? sign * sx[abs(m)] : 0;
         e = max(e, max(s6_exponent(v.x, sh), s6_exponent(v.y, sh)));
     }
@@ -169,15 +171,17 @@ __global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nr
 template <int D>
 __global__ void s6_slice_kernel(const typename S6Traits<D>::C* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
                                 int sign, const int* __restrict__ E, unsigned* __restrict__ dig) {
+    pdl_start_next();
     const int nc = 2 * p + 1, KS = (2 * nc + 15) / 16, r = blockIdx.y;
     const int64_t total = nbox * KS * 8;
-    const int e = E[r];
+    pdl_wait();                          // L2 loads: results of kernels that may have run beside this one's start
+    const int e = __ldcg(E + r);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / (KS * 8);
         const int m = (int)(i - b * (KS * 8));
         long long xr = s6_bias<D>(), xi = s6_bias<D>();
         if (m < nc) {
-            const auto v = a[(b * nrhs + r) * nc + m];
+            const auto v = __ldcg(a + (b * nrhs + r) * nc + m);
             const int sh = sx ? sign * sx[abs(m - p)] : 0;
             xr += s6_fixed<9 * D - 1>(v.x, sh, e);
             xi += s6_fixed<9 * D - 1>(v.y, sh, e);
@@ -309,11 +313,12 @@ __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s,
 // eight CTAs and add the partial sums in rank order through distributed shared
 // memory, so results do not depend on timing.
 template <int NT, int D>
-__global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant__ S6Args A) {
+__global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168)) s6_kernel(const __grid_constant__ S6Args A) {
     using R = typename S6Traits<D>::R;
     constexpr int NI = S6Traits<D>::NI;
     // digits of the sources of one 64-term chunk, in B-fragment order, two buffers
     __shared__ __align__(16) uint2 Bs[2][D][4][NT][32];
+    pdl_start_next();
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
     const int S = (int)cluster_size(), rank = (int)cluster_rank();
     const int tile = blockIdx.x / S, r = blockIdx.z;
@@ -337,20 +342,20 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
         T.ncol = min(NC, per - NC * g);
     }
     const int64_t nbox = (int64_t)1 << (2 * A.l);
-    auto target = [&](int col) -> int64_t {
-        if (A.mode == 0) return box0 + col < nbox ? box0 + col : -1;
-        if (A.mode == 2) return A.tgt[box0 + col];
-        if (col >= T.ncol) return -1;
-        const int64_t b = morton((uint32_t)(T.ix0 + 2 * col), (uint32_t)T.iy);
-        int32_t lo, hi;
-        box_range(A.lb, A.L, A.l, b, &lo, &hi);
-        return hi > lo ? b : -1;
-    };
-    if (A.mode == 1) {   // nothing to do where every target is empty (the same for all CTAs of the cluster)
-        bool any = false;
-        for (int c = 0; c < NC; ++c) any |= target(c) >= 0;
-        if (!any) return;
+    // lane c: target of column c (-1: none)
+    int64_t tgt = -1;
+    if (lane < NC) {
+        if (A.mode == 0) tgt = box0 + lane < nbox ? box0 + lane : -1;
+        else if (A.mode == 2) tgt = A.tgt[box0 + lane];
+        else if (lane < T.ncol) {
+            const int64_t b = morton((uint32_t)(T.ix0 + 2 * lane), (uint32_t)T.iy);
+            int32_t lo, hi;
+            box_range(A.lb, A.L, A.l, b, &lo, &hi);
+            if (hi > lo) tgt = b;
+        }
     }
+    // nothing to do where every target is empty (the same for all CTAs of the cluster)
+    if (!__any_sync(0xffffffffu, tgt >= 0)) return;
     const int nsteps = s6_steps(A, T, tile);
     const int nis = A.shift.dig ? 2 * A.shift.p + 1 : 0, nil = A.list.dig ? 2 * A.list.p + 1 : 0;
     const int KSs = (2 * nis + 15) / 16, KSl = (2 * nil + 15) / 16;
@@ -393,24 +398,10 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
             }
         since = 0;
     };
-    int Ef[2] = {0, 0};               // fold exponents per family
-    bool bad = false;
-    if (A.shift.dig) {
-        const int e = A.shift.Esrc[r];
-        bad |= e >= S6_NAN / 2;
-        Ef[0] = max(e, S6_NONE) + max(*A.shift.Eop, S6_NONE) - (18 * D - 3);
-    }
-    if (A.list.dig) {
-        const int e = A.list.Esrc[r];
-        bad |= e >= S6_NAN / 2;
-        Ef[1] = max(e, S6_NONE) + max(*A.list.Eop, S6_NONE) - (18 * D - 3);
-    }
-
     // A chunk: up to 64 terms (four k-steps) of one step.  While the tensor cores work on
     // one chunk the next one's source digits are copied into the other buffer and
-    // the operator fragments into the warp's four-slot ring (two k-steps ahead
-    // across chunks), all asynchronously: a k-step's loads alone take as long as
-    // its 21 NT products.
+    // its operator fragments into the slots of the warp's ring as they fall free,
+    // all asynchronously: a k-step's loads alone take longer than its products.
     struct Chunk { S6Step st; int s, k0; };
     auto next = [&](Chunk& c) -> bool {             // the following chunk of this CTA, false at the end
         if (c.s >= 0) {
@@ -471,14 +462,31 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
     int buf = 0, prev_fam = -1;
     Chunk cur{{}, -1, 0};
     bool more = next(cur);
+    // the operators are the plan's; everything below reads this apply's results.  (The
+    // first digits' group comes after the slots', so the first wait is for all.)
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) load_op(cur, kk, more);
+    pdl_wait();
+    int Ef[2] = {0, 0};               // fold exponents per family
+    bool bad = false;
+    if (A.shift.dig) {
+        const int e = __ldcg(A.shift.Esrc + r);
+        bad |= e >= S6_NAN / 2;
+        Ef[0] = max(e, S6_NONE) + max(*A.shift.Eop, S6_NONE) - (18 * D - 3);
+    }
+    if (A.list.dig) {
+        const int e = __ldcg(A.list.Esrc + r);
+        bad |= e >= S6_NAN / 2;
+        Ef[1] = max(e, S6_NONE) + max(*A.list.Eop, S6_NONE) - (18 * D - 3);
+    }
+
     load_src(cur, 0, more);
-    load_op(cur, 0, more);
-    load_op(cur, 1, more);
+    bool first = true;
     while (more) {
         const int fam = cur.st.fam, nk = min(4, (fam ? KSl : KSs) - cur.k0);
-        load_op(cur, 2, true);
-        load_op(cur, 3, true);
-        cp_wait<4>();                                     // the source digits (four operator groups came after)
+        if (first) cp_wait<0>();                          // the source digits (four operator groups came after)
+        else cp_wait<4>();
+        first = false;
         __syncthreads();
         more = next(cur);
         load_src(cur, buf ^ 1, more);
@@ -491,26 +499,31 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
 #pragma unroll
                     for (int x = 0; x < 4; ++x) acc[t][o][x] = 0.0f;
         }
-        // groups in flight, in order: this chunk's slots 0 .. 3, the next chunk's digits, its slots 0, 1
+        // groups in flight, in order: this chunk's slots, the next chunk's digits, its slots.  Two
+        // k-steps at a time between the waits and copies, which order memory accesses
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            if (kk < 3) cp_wait<4>(); else cp_wait<3>();
-            if (has_m && kk < nk) {
-                uint4 a[D];
+        for (int h = 0; h < 2; ++h) {
+            cp_wait<3>();
+            if (has_m)
 #pragma unroll
-                for (int d = 0; d < D; ++d) a[d] = ring[(kk * D + d) * 32];
+                for (int kk = 2 * h; kk < 2 * h + 2; ++kk)
+                    if (kk < nk) {
+                        uint4 a[D];
 #pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    uint2 bb[D];
+                        for (int d = 0; d < D; ++d) a[d] = ring[(kk * D + d) * 32];
 #pragma unroll
-                    for (int d = 0; d < D; ++d) bb[d] = Bs[buf][d][kk][t][lane];
+                        for (int t = 0; t < NT; ++t) {
+                            uint2 bb[D];
 #pragma unroll
-                    for (int i = 0; i < D; ++i)
+                            for (int d = 0; d < D; ++d) bb[d] = Bs[buf][d][kk][t][lane];
 #pragma unroll
-                        for (int j = 0; j < D - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
-                }
-            }
-            if (kk < 2) load_op(cur, kk, more);
+                            for (int i = 0; i < D; ++i)
+#pragma unroll
+                                for (int j = 0; j < D - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
+                        }
+                    }
+            load_op(cur, 2 * h, more);
+            load_op(cur, 2 * h + 1, more);
         }
         if (has_m) {
 #pragma unroll
@@ -537,20 +550,28 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
 #pragma unroll
                 for (int v = 0; v < 4; ++v) part[((wid * NT + t) * 4 + v) * 32 + lane] = dacc[t][v];
         cluster_sync();
-        if (rank == 0 && has_m)
-            for (int q = 1; q < S; ++q) {
-                uint32_t local = (uint32_t)__cvta_generic_to_shared(part), remote;
-                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(q));
+        if (rank == 0 && has_m) {
+            const uint32_t local = (uint32_t)__cvta_generic_to_shared(part);
 #pragma unroll
-                for (int t = 0; t < NT; ++t)
+            for (int t = 0; t < NT; ++t) {
+                double x[7][4];                                  // all ranks' values in flight at once
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        double x;
-                        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x)
-                                     : "r"(remote + (uint32_t)(((wid * NT + t) * 4 + v) * 32 + lane) * 8u));
-                        dacc[t][v] += x;
+                for (int q = 1; q < 8; ++q)
+                    if (q < S) {
+                        uint32_t remote;
+                        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(q));
+#pragma unroll
+                        for (int v = 0; v < 4; ++v)
+                            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x[q - 1][v])
+                                         : "r"(remote + (uint32_t)(((wid * NT + t) * 4 + v) * 32 + lane) * 8u));
                     }
+#pragma unroll
+                for (int q = 1; q < 8; ++q)
+                    if (q < S)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) dacc[t][v] += x[q - 1][v];
             }
+        }
         cluster_sync();
         if (rank != 0) return;
     }
@@ -562,12 +583,12 @@ __global__ void __maxnreg__(NT == 1 ? 128 : 168) s6_kernel(const __grid_constant
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const int row = 16 * mt + (lane >> 2) + (v >> 1) * 8, c = 8 * t + 2 * (lane & 3) + (v & 1);
-            const int64_t b = target(c);
+            const int64_t b = __shfl_sync(0xffffffffu, tgt, c);
             if (row >= 2 * no || b < 0) continue;
             const int sh = A.sxo ? A.osign * A.sxo[abs((row >> 1) - A.p)] : 0;
             R* o = reinterpret_cast<R*>(A.out) + ((b * A.nrhs + r) * no * 2 + row);
             R x = (R)(bad ? nan : dacc[t][v] * pow2d(sh));
-            if (A.accumulate) x += *o;
+            if (A.accumulate) x += __ldcg(o);
             *o = x;
             e = max(e, s6_exponent(x, -sh));
         }
@@ -585,20 +606,12 @@ hfmm_status s6_launch(const S6Args& A, int tiles, int steps, cudaStream_t st) {
     // idle (whatever nrhs is, so that a right-hand side's bits do not depend on the others)
     int S = 1;
     while (S < 8 && (int64_t)tiles * gy * S * 2 <= 4 * 152 && 2 * S <= steps) S *= 2;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(tiles * S), (unsigned)gy, (unsigned)A.nrhs);
-    cfg.blockDim = dim3(32 * W);
-    cfg.dynamicSmemBytes = (size_t)W * 4 * D * 512;
-    HFMM_CUDA_TRY(cudaFuncSetAttribute(s6_kernel<NT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       S6_MAXW * 4 * D * 512));
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = S;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    HFMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, s6_kernel<NT, D>, A));
+    const size_t sm = (size_t)W * 4 * D * 512;
+    if (sm > 16 * 1024)                                    // beside up to 24 KB of static shared memory
+        HFMM_CUDA_TRY(cudaFuncSetAttribute(s6_kernel<NT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           S6_MAXW * 4 * D * 512));
+    HFMM_CUDA_TRY(pdl_launch(s6_kernel<NT, D>, dim3((unsigned)(tiles * S), (unsigned)gy, (unsigned)A.nrhs), dim3(32 * W),
+                             sm, st, (unsigned)S, A));
     return HFMM_OK;
 }
 
@@ -820,11 +833,11 @@ template <int D>
 hfmm_status s6_exponent_of(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
     LevelInfo& lv = P->lev[l];
     const int64_t total = lv.nbox * lv.ncoef;
-    s6_exponent_kernel<<<dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs), 256, 0, st>>>(
-        s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, s6_lev<D>(lv).sx, loc ? 1 : -1,
-        split_exp(P, D == 6 ? 0 : 1, l, loc));
+    HFMM_CUDA_TRY(pdl_launch(s6_exponent_kernel<typename S6Traits<D>::C>,
+                             dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs), dim3(256), 0, st, 0,
+                             s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, s6_lev<D>(lv).sx, loc ? 1 : -1,
+                             split_exp(P, D == 6 ? 0 : 1, l, loc)));
     ++P->launches;
-    HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;
 }
 
@@ -833,11 +846,11 @@ hfmm_status s6_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st)
     LevelInfo& lv = P->lev[l];
     const S6Lev& s = s6_lev<D>(lv);
     const int64_t total = lv.nbox * ((2 * lv.ncoef + 15) / 16 * 8);
-    s6_slice_kernel<D><<<dim3((unsigned)std::min<int64_t>((total + 127) / 128, 16 * 152), (unsigned)nrhs), 128, 0, st>>>(
-        s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, s.sx, loc ? 1 : -1, split_exp(P, D == 6 ? 0 : 1, l, loc),
-        loc ? s.dloc : s.dmult);
+    HFMM_CUDA_TRY(pdl_launch(s6_slice_kernel<D>,
+                             dim3((unsigned)std::min<int64_t>((total + 127) / 128, 16 * 152), (unsigned)nrhs), dim3(128), 0,
+                             st, 0, s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, s.sx, loc ? 1 : -1,
+                             split_exp(P, D == 6 ? 0 : 1, l, loc), loc ? s.dloc : s.dmult));
     ++P->launches;
-    HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;
 }
 
