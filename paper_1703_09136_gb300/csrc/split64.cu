@@ -215,6 +215,7 @@ struct S6Args {
     const uint4* rops;               // reaction operators (null: none)
     int vlist, rlist, lstar;         // lists to run; first level whose bottom-row pair is admissible
     int rows;                        // box rows covered by the launch (downward)
+    uint8_t voff[4][27];             // V offsets of each child position: (source - target + 3), x + 8 y
     int accumulate;                  // add to the outputs
     const int* sxo;                  // (null: no output shift)
     int osign;                       // out_shift = osign * sxo
@@ -239,9 +240,10 @@ struct S6Step {
 };
 
 // Steps of a downward tile (row iy, columns ix0, ix0 + 2, ..., ncol of them):
-// 0 the L2L, then the offsets (dx, dy), |dx|, |dy| <= 3 outside the 3 x 3
-// neighbourhood whose parents touch, then the reaction pairs (source row,
-// dx).  Returns false where a step does not exist for this tile.
+// 0 the L2L, then the 27 V offsets of the tile's child position, then the reaction
+// pairs (source row, dx).  s6_step returns false where a step does not exist for
+// this tile.  (Walking 36 offsets with divisions and adjacency tests here, or
+// balancing the CTAs by a ballot over such tests, cost microseconds a launch.)
 struct S6Tile {
     int iy, ix0, ncol, n;            // n boxes per row
     int nshift, nv, nr, rspan, ropt0, rec0;
@@ -255,7 +257,7 @@ __device__ __forceinline__ int s6_steps(const S6Args& A, S6Tile& T, int tile) {
     T.nshift = A.shift.dig ? (A.mode == 0 ? 4 : 1) : 0;
     T.nv = T.nr = 0;
     if (A.mode == 1) {
-        T.nv = A.vlist ? 36 : 0;      // 6 x 6 offsets of the parents' neighbourhood
+        T.nv = A.vlist ? 27 : 0;
         if (A.rlist && T.iy < 2) {
             T.ropt0 = (T.iy == 1 || A.l == A.lstar) ? 0 : 1;      // first admissible source row
             const int opts = min(2, T.n) - T.ropt0;
@@ -286,32 +288,23 @@ __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s,
     s -= T.nshift;
     st.fam = 1;
     if (s < T.nv) {
-        // source = parent's neighbourhood: sx = 2 (ixP + a) + u, a = -1 .. 1, u = 0, 1
-        const int ox = s % 6 - 2 - (T.ix0 & 1), oy = s / 6 - 2 - (T.iy & 1);   // source - target
-        if (abs(ox) < 2 && abs(oy) < 2) return false;
+        const int v = A.voff[(T.ix0 & 1) + 2 * (T.iy & 1)][s], ox = (v & 7) - 3, oy = (v >> 3) - 3;
         st.sy = T.iy + oy;
-        if (st.sy < 0 || st.sy >= T.n) return false;
         st.dx = -ox;
-        if (T.ix0 + 2 * (T.ncol - 1) + ox < 0 || T.ix0 + ox >= T.n) return false;
-        st.op = A.list.ops + (int64_t)((st.dx + 3) * 7 + (-oy + 3)) * MT * KSl * (D * 32);
+        if ((unsigned)st.sy >= (unsigned)T.n || T.ix0 + 2 * (T.ncol - 1) + ox < 0 || T.ix0 + ox >= T.n) return false;
+        st.op = A.list.ops + (uint32_t)((st.dx + 3) * 7 + (3 - oy)) * (uint64_t)(MT * KSl * (D * 32));
         return true;
     }
     s -= T.nv;
-    st.sy = T.ropt0 + s / T.rspan;
-    st.dx = T.ix0 + 2 * (T.ncol - 1) - s % T.rspan;              // sources from right to left cover [0, n)
+    st.sy = T.ropt0;
+    if (s >= T.rspan) { s -= T.rspan; ++st.sy; }
+    st.dx = T.ix0 + 2 * (T.ncol - 1) - s;                        // sources from left to right cover [0, n)
     const int dxm = T.n - 1;
     if (abs(st.dx) > dxm) return false;
-    st.op = A.rops + (int64_t)((st.dx + dxm) * 3 + T.iy + st.sy) * MT * KSl * (D * 32);
+    st.op = A.rops + (uint32_t)((st.dx + dxm) * 3 + T.iy + st.sy) * (uint64_t)(MT * KSl * (D * 32));
     return true;
 }
 
-// A CTA owns 8 NT target boxes of one row and one column parity (they share every
-// operator) and up to six m-tiles of 16 output rows, one per warp; it walks the
-// steps, copies the sources' digits of 64 terms into shared memory and multiplies
-// them with the operator fragments, which each warp copies from L2 into a ring of
-// its own.  Levels with few tiles split a tile's steps over a cluster of up to
-// eight CTAs and add the partial sums in rank order through distributed shared
-// memory, so results do not depend on timing.
 template <int NT, int D>
 __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168)) s6_kernel(const __grid_constant__ S6Args A) {
     using R = typename S6Traits<D>::R;
@@ -794,6 +787,13 @@ hfmm_status s6_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st)
     S6Args A{};
     A.l = l; A.L = P->L; A.mode = P->ad ? 2 : 1; A.nrhs = nrhs; A.p = lv.p;
     A.lb = P->leaf_begin;
+    for (int c = 0; c < 4; ++c) {
+        int k = 0;
+        for (int o = 0; o < 36; ++o) {
+            const int ox = o % 6 - 2 - (c & 1), oy = o / 6 - 2 - (c >> 1);
+            if (std::abs(ox) >= 2 || std::abs(oy) >= 2) A.voff[c][k++] = (uint8_t)((ox + 3) + 8 * (oy + 3));
+        }
+    }
     if (l > P->lmin) {
         LevelInfo& pa = P->lev[l - 1];
         A.shift = s6_fam(s6_lev<D>(pa).dloc, pa.p, s.l2l, s.Eop + 1, split_exp(P, w, l - 1, true));
