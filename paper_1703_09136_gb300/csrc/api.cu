@@ -50,6 +50,7 @@ static void plan_free(hfmm_plan_s* P) {
     for (cudaEvent_t e : {P->ev_fork, P->ev_near_done, P->ev_far_done})
         if (e) cudaEventDestroy(e);
     for (void* p : P->allocations) cudaFree(p);
+    if (P->krylov_host) cudaFreeHost(P->krylov_host);
     adaptive_destroy(P->ad);
     delete P;
 }

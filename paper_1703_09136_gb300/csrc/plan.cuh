@@ -247,7 +247,10 @@ struct hfmm_plan_s {
     cd* basis64 = nullptr;          // [n][p_L + 2] P2M basis J_m(k rho) e^{-i m theta}, m >= 0
     void* krylov = nullptr;         // hfmm_solve: Krylov vectors (first call; grows with restart)
     size_t krylov_bytes = 0;
-    double* krylov_part = nullptr;  // partial sums of its dot products
+    double2* krylov_part = nullptr; // its dot products and their partial sums
+    size_t krylov_words = 0;
+    double2* krylov_host = nullptr; // page-locked copy of a Hessenberg column
+    size_t krylov_host_words = 0;
     cd* near64g_x = nullptr;        // d/dx, d/dy of the same blocks (first gradient request)
     cd* near64g_y = nullptr;
     cd* grad_buf = nullptr;         // [5][max_rhs][n]

@@ -2,9 +2,15 @@
 //     (sigma I + A) x = b,   A_ij = u_{x_j}(x_i)  (Sec. 2.4),
 // the dense system of a second-kind integral equation discretised on the
 // plan's points.  Every operator application is one hfmm apply; the Krylov
-// vectors stay on the device (dot products and updates are this file's
-// kernels, accumulated in FP64); the small Hessenberg least-squares problem
-// (Givens rotations) is solved on the host after each Arnoldi step.
+// vectors stay on the device and are orthogonalised there by two passes of
+// classical Gram-Schmidt (as orthogonal as the modified form to rounding; dot
+// products accumulated in FP64): one kernel takes all dot products of a pass, one
+// subtracts all projections.  The host reads one Hessenberg column per Arnoldi
+// step and solves the small least-squares problem (Givens rotations).
+//
+// The modified form took a kernel, a copy and a host round trip per dot product:
+// 1600 points, FP64, 14 steps: 28 ms, of which the applies were 2.3 ms (one GB300).
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -30,29 +36,137 @@ template <> struct Cx<cf> {
     static __device__ __forceinline__ cf mk(double r, double i) { return cfmk((float)r, (float)i); }
 };
 
-// partial sums of sum_i conj(a_i) b_i, one pair of doubles per block
-template <class T>
-__global__ void __launch_bounds__(SV_THREADS) dot_kernel(const T* __restrict__ a, const T* __restrict__ b,
-                                                         int64_t n, double* __restrict__ part) {
-    double sr = 0.0, si = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double ar = Cx<T>::re(a[i]), ai = Cx<T>::im(a[i]), br = Cx<T>::re(b[i]), bi = Cx<T>::im(b[i]);
-        sr += ar * br + ai * bi;
-        si += ar * bi - ai * br;
-    }
-    __shared__ double rr[SV_THREADS / 32], ri[SV_THREADS / 32];
+// sum over the block, in thread 0
+__device__ __forceinline__ double2 sv_block_sum(double sr, double si, double2* red) {
     for (int o = 16; o > 0; o >>= 1) {
         sr += __shfl_down_sync(0xffffffffu, sr, o);
         si += __shfl_down_sync(0xffffffffu, si, o);
     }
-    if ((threadIdx.x & 31) == 0) { rr[threadIdx.x >> 5] = sr; ri[threadIdx.x >> 5] = si; }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_double2(sr, si);
+    __syncthreads();
+    double2 t = make_double2(0.0, 0.0);
+    if (threadIdx.x == 0)
+        for (int w = 0; w < SV_THREADS / 32; ++w) { t.x += red[w].x; t.y += red[w].y; }
+    return t;
+}
+
+// the block that finishes last adds the blocks' partial sums of `cnt` values (part[value][block])
+// in block order into out; *ticket is zero between launches
+__device__ __forceinline__ bool sv_last_block(unsigned* ticket) {
+    __shared__ bool last;
+    __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        double tr = 0.0, ti = 0.0;
-        for (int w = 0; w < SV_THREADS / 32; ++w) { tr += rr[w]; ti += ri[w]; }
-        part[2 * blockIdx.x] = tr;
-        part[2 * blockIdx.x + 1] = ti;
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last) *ticket = 0;
     }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+__device__ __forceinline__ double2 sv_warp_sum(double sr, double si) {
+    for (int o = 16; o > 0; o >>= 1) {
+        sr += __shfl_xor_sync(0xffffffffu, sr, o);
+        si += __shfl_xor_sync(0xffffffffu, si, o);
+    }
+    return make_double2(sr, si);
+}
+
+__device__ __forceinline__ void sv_add_parts(const double2* part, int cnt, double2* out) {
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < cnt; i += SV_THREADS / 32) {
+        double sr = 0.0, si = 0.0;
+        for (unsigned k = lane; k < gridDim.x; k += 32) {
+            const double2 p = __ldcg(part + (size_t)i * gridDim.x + k);
+            sr += p.x;
+            si += p.y;
+        }
+        const double2 s = sv_warp_sum(sr, si);
+        if (lane == 0) out[i] = s;
+    }
+}
+
+// h_i = <v_i, w>, i < cnt (v_i = V + i n); with shift, w += sigma v_{cnt - 1} first (the operator's
+// shift).  A block keeps its part of w in shared memory, a warp takes every eighth vector.
+template <class T>
+__global__ void __launch_bounds__(SV_THREADS) dots_kernel(const T* __restrict__ V, T* __restrict__ w, int64_t n, int chunk,
+                                                          int cnt, int shift, double sr, double si,
+                                                          double2* __restrict__ part, double2* __restrict__ h,
+                                                          unsigned* __restrict__ ticket) {
+    extern __shared__ double2 ws[];
+    const int lane = threadIdx.x & 31;
+    const int64_t lo = (int64_t)blockIdx.x * chunk;
+    const int m = (int)(n - lo < chunk ? n - lo : chunk);
+    for (int i = threadIdx.x; i < m; i += SV_THREADS) {
+        T x = w[lo + i];
+        if (shift) {
+            const T v = V[(int64_t)(cnt - 1) * n + lo + i];
+            const double vr = Cx<T>::re(v), vi = Cx<T>::im(v);
+            x = Cx<T>::mk(Cx<T>::re(x) + sr * vr - si * vi, Cx<T>::im(x) + sr * vi + si * vr);
+            w[lo + i] = x;
+        }
+        ws[i] = make_double2(Cx<T>::re(x), Cx<T>::im(x));
+    }
+    __syncthreads();
+    for (int j = threadIdx.x >> 5; j < cnt; j += SV_THREADS / 32) {
+        const T* v = V + (int64_t)j * n + lo;
+        double tr = 0.0, ti = 0.0;
+#pragma unroll 4
+        for (int i = lane; i < m; i += 32) {
+            const double ar = Cx<T>::re(v[i]), ai = Cx<T>::im(v[i]);
+            const double2 b = ws[i];
+            tr += ar * b.x + ai * b.y;
+            ti += ar * b.y - ai * b.x;
+        }
+        const double2 t = sv_warp_sum(tr, ti);
+        if (lane == 0) part[(size_t)j * gridDim.x + blockIdx.x] = t;
+    }
+    if (sv_last_block(ticket)) sv_add_parts(part, cnt, h);
+}
+
+// w += sgn sum_i c_i v_i, i < cnt; norm: also |w|^2 into *nrm
+template <class T>
+__global__ void __launch_bounds__(SV_THREADS) combine_kernel(const T* V, const double2* __restrict__ c, int cnt,
+                                                             double sgn, T* w, int64_t n, int chunk,
+                                                             double2* __restrict__ part, double2* __restrict__ nrm,
+                                                             unsigned* __restrict__ ticket) {
+    __shared__ double2 red[SV_THREADS / 32];
+    const int64_t lo = (int64_t)blockIdx.x * chunk;
+    double s = 0.0;
+    for (int64_t i = lo + threadIdx.x; i < n && i < lo + chunk; i += SV_THREADS) {
+        double wr = 0.0, wi = 0.0;
+#pragma unroll 4
+        for (int j = 0; j < cnt; ++j) {
+            const double2 a = c[j];
+            const T v = V[(int64_t)j * n + i];
+            const double vr = Cx<T>::re(v), vi = Cx<T>::im(v);
+            wr += a.x * vr - a.y * vi;
+            wi += a.x * vi + a.y * vr;
+        }
+        const T x = Cx<T>::mk(Cx<T>::re(w[i]) + sgn * wr, Cx<T>::im(w[i]) + sgn * wi);
+        w[i] = x;
+        s += Cx<T>::re(x) * Cx<T>::re(x) + Cx<T>::im(x) * Cx<T>::im(x);
+    }
+    if (!nrm) return;
+    const double2 t = sv_block_sum(s, 0.0, red);
+    if (threadIdx.x == 0) part[blockIdx.x] = t;
+    if (sv_last_block(ticket)) sv_add_parts(part, 1, nrm);
+}
+
+// v = w / |w| (v = 0 for |w| = 0); the column h = h1 + h2 and |w|^2 for the host
+template <class T>
+__global__ void __launch_bounds__(SV_THREADS) normalise_kernel(const T* __restrict__ w, const double2* __restrict__ nrm,
+                                                               T* __restrict__ v, int64_t n, int cnt,
+                                                               const double2* __restrict__ h1,
+                                                               const double2* __restrict__ h2, double2* __restrict__ col) {
+    const double d = sqrt(nrm->x), inv = d > 0.0 ? 1.0 / d : 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        v[i] = Cx<T>::mk(inv * Cx<T>::re(w[i]), inv * Cx<T>::im(w[i]));
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i <= cnt; i += SV_THREADS)
+            col[i] = i < cnt ? make_double2(h1[i].x + h2[i].x, h1[i].y + h2[i].y) : *nrm;
 }
 
 // y = alpha x + beta y (alpha, beta complex)
@@ -72,18 +186,39 @@ struct Krylov {
     hfmm_plan_s* P;
     cudaStream_t st;
     int64_t n;
-    double* part;        // device partial sums
-    std::vector<double> hpart;
+    // device: block partial sums, two passes' dot products, a norm, a column; the column's page-locked copy
+    double2 *part, *h1, *h2, *nrm, *col, *host;
+    unsigned* ticket;
+    int chunk;           // vector elements of a block in the Gram-Schmidt kernels
 
-    hfmm_status dot(const T* a, const T* b, zc* out) {
-        dot_kernel<T><<<SV_BLOCKS, SV_THREADS, 0, st>>>(a, b, n, part);
-        HFMM_CUDA_TRY(cudaGetLastError());
-        HFMM_CUDA_TRY(cudaMemcpyAsync(hpart.data(), part, sizeof(double) * 2 * SV_BLOCKS, cudaMemcpyDeviceToHost, st));
+    unsigned blocks() const { return (unsigned)((n + chunk - 1) / chunk); }
+    hfmm_status read(const double2* d, int cnt) {
+        HFMM_CUDA_TRY(cudaMemcpyAsync(host, d, sizeof(double2) * cnt, cudaMemcpyDeviceToHost, st));
         HFMM_CUDA_TRY(cudaStreamSynchronize(st));
-        double r = 0.0, i = 0.0;
-        for (int k = 0; k < SV_BLOCKS; ++k) { r += hpart[2 * k]; i += hpart[2 * k + 1]; }
-        *out = zc(r, i);
         return HFMM_OK;
+    }
+    // |a|^2
+    hfmm_status norm2(T* a, double* out) {
+        combine_kernel<T><<<blocks(), SV_THREADS, 0, st>>>(a, h1, 0, 0.0, a, n, chunk, part, nrm, ticket);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        HFMM_TRY(read(nrm, 1));
+        *out = host[0].x;
+        return HFMM_OK;
+    }
+    // Arnoldi step: w = (sigma + A) v_j minus its projections on v_0 .. v_j, v_{j + 1} = w / |w|;
+    // host[0 .. j] = the Hessenberg column, host[j + 1].x = |w|^2
+    hfmm_status arnoldi(zc sigma, T* V, int j, T* w) {
+        HFMM_TRY(apply(V + (size_t)j * n, w));
+        const unsigned g = blocks();
+        const size_t sm = sizeof(double2) * chunk;
+        dots_kernel<T><<<g, SV_THREADS, sm, st>>>(V, w, n, chunk, j + 1, 1, sigma.real(), sigma.imag(), part, h1, ticket);
+        combine_kernel<T><<<g, SV_THREADS, 0, st>>>(V, h1, j + 1, -1.0, w, n, chunk, part, nullptr, ticket);
+        dots_kernel<T><<<g, SV_THREADS, sm, st>>>(V, w, n, chunk, j + 1, 0, 0.0, 0.0, part, h2, ticket);
+        combine_kernel<T><<<g, SV_THREADS, 0, st>>>(V, h2, j + 1, -1.0, w, n, chunk, part, nrm, ticket);
+        normalise_kernel<T><<<(unsigned)std::min<int64_t>(SV_BLOCKS, (n + SV_THREADS - 1) / SV_THREADS), SV_THREADS, 0, st>>>(
+            w, nrm, V + (size_t)(j + 1) * n, n, j + 1, h1, h2, col);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        return read(col, j + 2);
     }
     // y = a x + b y
     hfmm_status axpby(zc a, const T* x, zc b, T* y) {
@@ -91,12 +226,14 @@ struct Krylov {
         HFMM_CUDA_TRY(cudaGetLastError());
         return HFMM_OK;
     }
+    hfmm_status apply(const T* v, T* y) {
+        if (P->precision == HFMM_MIXED)
+            return apply_mixed(P, 1, (const cf*)v, (cf*)y, HFMM_PART_ALL, false, st);
+        return apply_fp64(P, 1, (const cd*)v, (cd*)y, HFMM_PART_ALL, false, st);
+    }
     // y = sigma v + A v
     hfmm_status op(zc sigma, const T* v, T* y) {
-        if (P->precision == HFMM_MIXED)
-            HFMM_TRY(apply_mixed(P, 1, (const cf*)v, (cf*)y, HFMM_PART_ALL, false, st));
-        else
-            HFMM_TRY(apply_fp64(P, 1, (const cd*)v, (cd*)y, HFMM_PART_ALL, false, st));
+        HFMM_TRY(apply(v, y));
         return axpby(sigma, v, zc(1.0, 0.0), y);
     }
 };
@@ -111,14 +248,32 @@ hfmm_status gmres(hfmm_plan_s* P, zc sigma, const T* b, T* x, double tol, int m,
         HFMM_TRY(plan_alloc(P, (void**)&P->krylov, need));
         P->krylov_bytes = need;
     }
-    if (!P->krylov_part) HFMM_TRY(plan_alloc(P, (void**)&P->krylov_part, sizeof(double) * 2 * SV_BLOCKS));
-    Krylov<T> K{P, st, n, P->krylov_part, std::vector<double>(2 * SV_BLOCKS)};
+    // small arrays: a pass's block sums [m + 1][blocks], its dot products (twice), a norm, a column, the ticket
+    // two blocks per SM where the vectors are long enough, at most 2048 elements a block
+    const int chunk = (int)std::min<int64_t>(2048, std::max<int64_t>(32, (n + 303) / 304));
+    const size_t nblk = (size_t)((n + chunk - 1) / chunk);
+    const size_t words = (size_t)(m + 1) * nblk + 3 * (size_t)(m + 2) + 2;
+    if (!P->krylov_part || P->krylov_words < words) {
+        HFMM_TRY(plan_alloc(P, (void**)&P->krylov_part, sizeof(double2) * words));
+        P->krylov_words = words;
+    }
+    if (!P->krylov_host || P->krylov_host_words < (size_t)m + 2) {
+        if (P->krylov_host) cudaFreeHost(P->krylov_host);
+        P->krylov_host = nullptr;
+        HFMM_CUDA_TRY(cudaMallocHost((void**)&P->krylov_host, sizeof(double2) * ((size_t)m + 2)));
+        P->krylov_host_words = (size_t)m + 2;
+    }
+    double2* small = P->krylov_part;
+    Krylov<T> K{P, st, n, small + 3 * (size_t)(m + 2) + 2, small, small + (m + 2), small + 3 * (size_t)(m + 2),
+                small + 2 * (size_t)(m + 2), P->krylov_host, (unsigned*)(small + 3 * (size_t)(m + 2) + 1), chunk};
+    HFMM_CUDA_TRY(cudaMemsetAsync(K.ticket, 0, sizeof(unsigned), st));
     T* V = (T*)P->krylov;
     T* w = V + (size_t)n * (m + 1);
     auto vec = [&](int j) { return V + (size_t)n * j; };
-    zc bb;
-    HFMM_TRY(K.dot(b, b, &bb));
-    const double bnorm = std::sqrt(bb.real());
+    double bb;
+    HFMM_CUDA_TRY(cudaMemcpyAsync(w, b, sizeof(T) * n, cudaMemcpyDeviceToDevice, st));
+    HFMM_TRY(K.norm2(w, &bb));
+    const double bnorm = std::sqrt(bb);
     *iters = 0;
     *relres = 0.0;
     if (bnorm == 0.0) {
@@ -131,9 +286,9 @@ hfmm_status gmres(hfmm_plan_s* P, zc sigma, const T* b, T* x, double tol, int m,
         // r = b - (sigma x + A x) into V_0
         HFMM_TRY(K.op(sigma, x, vec(0)));
         HFMM_TRY(K.axpby(zc(1.0, 0.0), b, zc(-1.0, 0.0), vec(0)));
-        zc rr;
-        HFMM_TRY(K.dot(vec(0), vec(0), &rr));
-        const double beta = std::sqrt(rr.real());
+        double rr;
+        HFMM_TRY(K.norm2(vec(0), &rr));
+        const double beta = std::sqrt(rr);
         *relres = beta / bnorm;
         if (*relres <= tol) break;
         HFMM_TRY(K.axpby(zc(1.0 / beta, 0.0), vec(0), zc(0.0, 0.0), vec(0)));
@@ -142,18 +297,10 @@ hfmm_status gmres(hfmm_plan_s* P, zc sigma, const T* b, T* x, double tol, int m,
         int j = 0;
         for (; j < m && *iters < maxit; ++j) {
             ++*iters;
-            HFMM_TRY(K.op(sigma, vec(j), w));
-            for (int i = 0; i <= j; ++i) {          // modified Gram-Schmidt
-                zc h;
-                HFMM_TRY(K.dot(vec(i), w, &h));
-                H[(size_t)i * m + j] = h;
-                HFMM_TRY(K.axpby(-h, vec(i), zc(1.0, 0.0), w));
-            }
-            zc ww;
-            HFMM_TRY(K.dot(w, w, &ww));
-            const double hn = std::sqrt(ww.real());
+            HFMM_TRY(K.arnoldi(sigma, V, j, w));
+            for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = zc(K.host[i].x, K.host[i].y);
+            const double hn = std::sqrt(K.host[j + 1].x);
             H[(size_t)(j + 1) * m + j] = hn;
-            if (hn > 0.0) HFMM_TRY(K.axpby(zc(1.0 / hn, 0.0), w, zc(0.0, 0.0), vec(j + 1)));
             // Givens rotations: apply the previous ones to column j, make a new one
             for (int i = 0; i < j; ++i) {
                 const zc a = H[(size_t)i * m + j], c = H[(size_t)(i + 1) * m + j];
@@ -177,15 +324,18 @@ hfmm_status gmres(hfmm_plan_s* P, zc sigma, const T* b, T* x, double tol, int m,
             for (int k = i + 1; k < j; ++k) s -= H[(size_t)i * m + k] * y[k];
             y[i] = s / H[(size_t)i * m + i];
         }
-        for (int i = 0; i < j; ++i) HFMM_TRY(K.axpby(y[i], vec(i), zc(1.0, 0.0), x));
+        for (int i = 0; i < j; ++i) K.host[i] = make_double2(y[i].real(), y[i].imag());
+        HFMM_CUDA_TRY(cudaMemcpyAsync(K.col, K.host, sizeof(double2) * j, cudaMemcpyHostToDevice, st));
+        combine_kernel<T><<<K.blocks(), SV_THREADS, 0, st>>>(V, K.col, j, 1.0, x, n, chunk, K.part, nullptr, K.ticket);
+        HFMM_CUDA_TRY(cudaGetLastError());
         if (*relres <= tol) break;
     }
     // the true residual of the returned x
     HFMM_TRY(K.op(sigma, x, w));
     HFMM_TRY(K.axpby(zc(1.0, 0.0), b, zc(-1.0, 0.0), w));
-    zc rr;
-    HFMM_TRY(K.dot(w, w, &rr));
-    *relres = std::sqrt(rr.real()) / bnorm;
+    double rr;
+    HFMM_TRY(K.norm2(w, &rr));
+    *relres = std::sqrt(rr) / bnorm;
     return HFMM_OK;
 }
 
