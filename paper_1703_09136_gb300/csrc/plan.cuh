@@ -260,6 +260,7 @@ struct hfmm_plan_s {
     void* dj_jobs = nullptr;        // direct-block quadrature jobs and segments (tables.cu)
     void* dj_segs = nullptr;
     int64_t dj_njobs = 0;
+    int dj_tiles = 0;               // tiles of the largest job
     bool tc_on = false;             // every level lmin..L has tensor-core M2M / downward state
     bool tc_l2p = false;            // leaf L2P fused into the tensor-core downward epilogue
     // leaf level with level-wide scales: every leaf multipole row r written with
