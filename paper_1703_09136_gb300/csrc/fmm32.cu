@@ -914,6 +914,15 @@ hfmm_status fork_near_far(hfmm_plan_s* P, cudaStream_t st) {
     return HFMM_OK;
 }
 
+// Directly summed reaction onto y32.
+hfmm_status launch_direct32(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
+    direct32_kernel<<<(unsigned)P->lev[P->L].nbox, 128, 0, st>>>(P->leaf_begin, P->d_begin, P->d_src, P->d_blk,
+                                                                P->d_vals32, P->q32, P->n, nrhs, P->y32);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
 hfmm_status apply_mixed(hfmm_plan_s* P, int nrhs, const cf* q, cf* y, int parts, bool adjoint,
                         cudaStream_t st) {
     const int64_t n = P->n;
@@ -925,17 +934,30 @@ hfmm_status apply_mixed(hfmm_plan_s* P, int nrhs, const cf* q, cf* y, int parts,
     P->leaf_flops = 0.0;
     const double C = 8.0 * nrhs;
     const double MAC = 8.0 * nrhs;
-    tm.begin(HFMM_STAGE_GATHER);
-    const unsigned ntile = (unsigned)ceil_div(n, TP_PTS);
-    if (P->qmax) HFMM_CUDA_TRY(cudaMemsetAsync(P->qmax, 0, sizeof(unsigned) * nrhs, st));
-    gather_q32<<<ntile, TP_THREADS, 0, st>>>(q, P->iperm32, n, nrhs, adjoint, P->q32, P->qmax);
-    ++P->launches;
-    HFMM_CUDA_TRY(cudaMemsetAsync(P->y32, 0, sizeof(cf) * n * nrhs, st));
-    tm.end(HFMM_STAGE_GATHER);
-    P->st_bytes[HFMM_STAGE_GATHER] = 2.0 * C * n + 8.0 * n;
     const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0;
     // few right-hand sides: warp-level kernels (small.cu) instead of the tensor-core tiles
-    const bool small = nrhs <= P->small_rhs && !(P->flags & HFMM_FLAG_SIMT_M2L);
+    const bool small = nrhs <= P->small_rhs && !(P->flags & HFMM_FLAG_SIMT_M2L) && !P->ad;
+    tm.begin(HFMM_STAGE_GATHER);
+    const unsigned ntile = (unsigned)ceil_div(n, TP_PTS);
+    if (small || (P->ad && nrhs <= 4)) {
+        HFMM_TRY(launch_gather_few(P, nrhs, q, adjoint, st));
+    } else {
+        if (P->qmax) HFMM_CUDA_TRY(cudaMemsetAsync(P->qmax, 0, sizeof(unsigned) * nrhs, st));
+        gather_q32<<<ntile, TP_THREADS, 0, st>>>(q, P->iperm32, n, nrhs, adjoint, P->q32, P->qmax);
+        ++P->launches;
+    }
+    if (!small) HFMM_CUDA_TRY(cudaMemsetAsync(P->y32, 0, sizeof(cf) * n * nrhs, st));
+    tm.end(HFMM_STAGE_GATHER);
+    P->st_bytes[HFMM_STAGE_GATHER] = 2.0 * C * n + 8.0 * n;
+    if (small) {
+        HFMM_TRY(apply_small(P, nrhs, parts, adjoint, y, st));
+        if ((parts & HFMM_PART_NEAR_REACT) && P->nd > 0) {
+            P->st_flops[HFMM_STAGE_DIRECT] = MAC * (double)P->nd_vals;
+            P->st_bytes[HFMM_STAGE_DIRECT] = 8.0 * (double)P->nd_vals;
+        }
+        P->last_stream = st;
+        return HFMM_OK;
+    }
     auto large_path = [&]() -> hfmm_status {
         // near free-space field and, unless the downward epilogue does it, the
         // leaves' local expansions (L2P), one fused kernel
@@ -1091,21 +1113,22 @@ hfmm_status apply_mixed(hfmm_plan_s* P, int nrhs, const cf* q, cf* y, int parts,
         return HFMM_OK;
     };
     if (P->ad) HFMM_TRY(apply_adaptive32(P, nrhs, parts, st));   // adaptive tree: its own FP32 passes
-    else HFMM_TRY(small ? apply_small(P, nrhs, parts, st) : large_path());
+    else HFMM_TRY(large_path());
     if ((parts & HFMM_PART_NEAR_REACT) && P->nd > 0 && !P->ad) {
         tm.begin(HFMM_STAGE_DIRECT);
-        direct32_kernel<<<(unsigned)P->lev[L].nbox, 128, 0, st>>>(P->leaf_begin, P->d_begin, P->d_src, P->d_blk,
-                                                                  P->d_vals32, P->q32, n, nrhs, P->y32);
-        ++P->launches;
-        HFMM_CUDA_TRY(cudaGetLastError());
+        HFMM_TRY(launch_direct32(P, nrhs, st));
         tm.end(HFMM_STAGE_DIRECT);
         P->st_flops[HFMM_STAGE_DIRECT] = MAC * (double)P->nd_vals;
         P->st_bytes[HFMM_STAGE_DIRECT] = 8.0 * (double)P->nd_vals;
     }
     tm.begin(HFMM_STAGE_SCATTER);
-    scatter_y32<<<ntile, TP_THREADS, 0, st>>>(P->y32, P->iperm32, n, nrhs, adjoint, y);
-    ++P->launches;
-    HFMM_CUDA_TRY(cudaGetLastError());
+    if (P->ad && nrhs <= 4) {
+        HFMM_TRY(launch_scatter_few(P, nrhs, y, adjoint, st));
+    } else {
+        scatter_y32<<<ntile, TP_THREADS, 0, st>>>(P->y32, P->iperm32, n, nrhs, adjoint, y);
+        ++P->launches;
+        HFMM_CUDA_TRY(cudaGetLastError());
+    }
     tm.end(HFMM_STAGE_SCATTER);
     P->st_bytes[HFMM_STAGE_SCATTER] = 2.0 * C * n + 8.0 * n;
     P->last_stream = st;

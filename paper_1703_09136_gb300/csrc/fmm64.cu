@@ -842,7 +842,7 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
 
 // Offsets of the near-field blocks (every target leaf's U-list pairs) on
 // the device, once per plan; returns the number of pairs in *pairs.
-static hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, bool alloc, cudaStream_t st) {
+hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, bool alloc, cudaStream_t st) {
     const int L = P->L;
     const int64_t nleaf = P->lev[L].nbox;
     const auto& lb = P->h_leaf_begin;

@@ -245,6 +245,7 @@ struct hfmm_plan_s {
     Leaf64D* leaf64_d = nullptr;
     cd* m2p64 = nullptr;
     cd* basis64 = nullptr;          // [n][p_L + 2] P2M basis J_m(k rho) e^{-i m theta}, m >= 0
+    cf* near32_vals = nullptr;      // few-RHS mixed plans: (i/4) H0 blocks in FP32, offsets near64_off
     void* krylov = nullptr;         // hfmm_solve: Krylov vectors (first call; grows with restart)
     size_t krylov_bytes = 0;
     double2* krylov_part = nullptr; // its dot products and their partial sums
@@ -354,6 +355,8 @@ hfmm_status build_direct_grad(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, double* gxy, cudaStream_t st);
 // fmm64.cu
 constexpr double NEAR64_MAX_BYTES = 32e9;   // plan-time FP64 near-field blocks up to this size
+constexpr double NEAR32_MAX_BYTES = 8e9;    // plan-time FP32 blocks of few-RHS mixed plans
+hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, bool alloc, cudaStream_t st);
 hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status build_diag(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status build_adaptive_tree(hfmm_plan_s* P, const double* d_xy, int leaf_size, cudaStream_t st);
@@ -441,8 +444,12 @@ void persist_destroy(PersistBatch* B);
 
 // small.cu: the small-nrhs mixed path (warp-level SIMT kernels, no tensor cores)
 hfmm_status init_small(hfmm_plan_s* P, cudaStream_t st);
-// P2M, M2M, downward pass and near field + L2P of one apply on the sorted q32 / y32
-hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t st);
+hfmm_status build_near_small(hfmm_plan_s* P, cudaStream_t st);
+hfmm_status launch_scatter_few(hfmm_plan_s* P, int nrhs, cf* y, bool conj_out, cudaStream_t st);
+hfmm_status launch_gather_few(hfmm_plan_s* P, int nrhs, const cf* q, bool conj_in, cudaStream_t st);
+// one apply from the sorted q32 into the caller's order
+hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, bool conj_out, cf* y, cudaStream_t st);
+hfmm_status launch_direct32(hfmm_plan_s* P, int nrhs, cudaStream_t st);
 // forks P->near_st (low priority) and P->far_st (high priority) from st
 hfmm_status fork_near_far(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status build_local_coords(hfmm_plan_s* P, cudaStream_t st);

@@ -464,6 +464,225 @@ __global__ void __launch_bounds__(128 * vb_nwc(CPT), CPT == 2 ? 4 : 1)
 }
 
 // ---------------------------------------------------------------------------
+// Caller order -> sorted point-major strengths, a thread per caller point: reads
+// along the points, writes nrhs values (the 64 x 64 tiles of the many-RHS gather
+// take 41 us for 262,144 points and one right-hand side, this 5 us).
+// ---------------------------------------------------------------------------
+__global__ void gather_few_kernel(const cf* __restrict__ q, const int32_t* __restrict__ iperm, int64_t n, int nrhs,
+                                  bool conj_in, cf* __restrict__ qs) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    cf* o = qs + (int64_t)iperm[j] * nrhs;
+    for (int r = 0; r < nrhs; ++r) {
+        const cf v = q[(int64_t)r * n + j];
+        o[r] = conj_in ? cfmk(v.x, -v.y) : v;
+    }
+}
+
+// Sorted fields -> caller order, the same mapping.
+__global__ void scatter_few_kernel(const cf* __restrict__ ys, const int32_t* __restrict__ iperm, int64_t n, int nrhs,
+                                   bool conj_out, cf* __restrict__ y) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const cf* o = ys + (int64_t)iperm[j] * nrhs;
+    for (int r = 0; r < nrhs; ++r) y[(int64_t)r * n + j] = conj_out ? cfmk(o[r].x, -o[r].y) : o[r];
+}
+
+// ---------------------------------------------------------------------------
+// Near field from stored blocks: plans whose applies all come here (max_rhs <=
+// small_rhs) hold (i/4) H0 of every U-list pair in FP32, source-major per target
+// leaf (G[off + j n_T + i], 0 for the target itself), filled once with the table
+// of near_small_kernel.  An apply then streams 8 bytes a pair instead of evaluating
+// the table (25 instructions): two layers, 262,144 points, one right-hand side
+// 255 -> 101 us.  A warp per target leaf; leaves of at most 16 points give each
+// half-warp alternate sources.  Strengths of up to 256 sources wait in shared memory.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int near_sources(const int32_t* lb, int L, int64_t b, int lane, int32_t* lo, int32_t* pre) {
+    const int m = 1 << L, sx = (int)morton_x((uint32_t)b) + lane % 3 - 1, sy = (int)morton_y((uint32_t)b) + lane / 3 - 1;
+    int32_t first = 0, cnt = 0;
+    if (lane < 9 && sx >= 0 && sy >= 0 && sx < m && sy < m) {
+        const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
+        first = lb[s];
+        cnt = lb[s + 1] - first;
+    }
+    int32_t inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const int32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    if (lane < 9) { lo[lane] = first; pre[lane + 1] = inc; }
+    if (lane == 0) pre[0] = 0;
+    __syncwarp();
+    return pre[9];
+}
+
+__global__ void __launch_bounds__(128) near_fill_kernel(const int32_t* __restrict__ lb, int L, int64_t nleaf,
+                                                        const float2* __restrict__ xl, float k, float h,
+                                                        const int64_t* __restrict__ off, cf* __restrict__ G) {
+    __shared__ float tj[H0N][H0D + 1], tr[H0N][H0D + 1];
+    __shared__ int32_t s_lo[4][9], s_pre[4][10];
+    for (int e = threadIdx.x; e < H0N * (H0D + 1); e += blockDim.x) {
+        tj[e / (H0D + 1)][e % (H0D + 1)] = g_h0[0][e / (H0D + 1)][e % (H0D + 1)];
+        tr[e / (H0D + 1)][e % (H0D + 1)] = g_h0[1][e / (H0D + 1)][e % (H0D + 1)];
+    }
+    __syncthreads();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t b = (int64_t)blockIdx.x * 4 + w;
+    if (b >= nleaf) return;
+    const int32_t tlo = lb[b], tn = lb[b + 1] - tlo;
+    if (tn <= 0) return;
+    const int ns = near_sources(lb, L, b, lane, s_lo[w], s_pre[w]);
+    cf* Gb = G + off[b];
+    for (int64_t e = lane; e < (int64_t)ns * tn; e += 32) {
+        const int j = (int)(e / tn), i = (int)(e - (int64_t)j * tn);
+        int u = 0;
+        while (j >= s_pre[w][u + 1]) ++u;
+        const int32_t js = s_lo[w][u] + j - s_pre[w][u], t = tlo + i;
+        cf g = cfmk(0.f, 0.f);
+        if (js != t) {
+            const float2 tp = xl[t], sp = xl[js];
+            const float ddx = (float)(1 - u % 3) * h + (tp.x - sp.x), ddy = (float)(1 - u / 3) * h + (tp.y - sp.y);
+            const float z = k * sqrtf(ddx * ddx + ddy * ddy);
+            if (z < H0_ZMAX) g = green_tab(tj, tr, z);
+            else {
+                const cd h0 = hankel0((double)z);
+                g = cfmk((float)(-0.25 * h0.y), (float)(0.25 * h0.x));
+            }
+        }
+        Gb[e] = g;
+    }
+}
+
+constexpr int NB_SRC = 256;
+
+template <int R>
+__global__ void __launch_bounds__(128) near_blocks_kernel(const int32_t* __restrict__ lb, int L, int64_t nleaf,
+                                                          const int64_t* __restrict__ off, const cf* __restrict__ G,
+                                                          const cf* __restrict__ qs, int nrhs, cf* __restrict__ ys) {
+    __shared__ cf sq[4][NB_SRC][R];
+    __shared__ int32_t s_lo[4][9], s_pre[4][10];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t b = (int64_t)blockIdx.x * 4 + w;
+    if (b >= nleaf) return;
+    const int32_t tlo = lb[b], tn = lb[b + 1] - tlo;
+    if (tn <= 0) return;
+    const int ns = near_sources(lb, L, b, lane, s_lo[w], s_pre[w]);
+    const cf* Gb = G + off[b];
+    const bool split = tn <= 16;
+    const int half = split ? lane >> 4 : 0, step = split ? 2 : 1;
+    for (int r0 = 0; r0 < nrhs; r0 += R) {
+        int staged = -1;
+        for (int i0 = 0; i0 < tn; i0 += 32) {
+            const int i = i0 + (split ? lane & 15 : lane);
+            const bool live = i < tn;
+            cf acc[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = cfmk(0.f, 0.f);
+            for (int c0 = 0; c0 < ns; c0 += NB_SRC) {
+                const int cnt = min(NB_SRC, ns - c0);
+                if (staged != c0) {
+                    __syncwarp();
+                    for (int e = lane; e < cnt; e += 32) {
+                        const int j = c0 + e;
+                        int u = 0;
+                        while (j >= s_pre[w][u + 1]) ++u;
+                        const cf* q = qs + (int64_t)(s_lo[w][u] + j - s_pre[w][u]) * nrhs + r0;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) sq[w][e][r] = r0 + r < nrhs ? q[r] : cfmk(0.f, 0.f);
+                    }
+                    staged = c0;
+                    __syncwarp();
+                }
+                if (!live) continue;
+                const cf* g = Gb + (int64_t)c0 * tn + i;
+#pragma unroll 8
+                for (int j = half; j < cnt; j += step) {
+                    const cf gv = __ldg(g + (int64_t)j * tn);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) cfma(acc[r], gv, sq[w][j][r]);
+                }
+            }
+            __syncwarp();
+            if (split)
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, 16);
+                    acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, 16);
+                }
+            if (live && half == 0)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (r0 + r < nrhs) ys[(int64_t)(tlo + i) * nrhs + r0 + r] = acc[r];
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The leaves' L2P, the other sums (sorted ys, null: none) and the caller's order in one
+// pass: a warp per leaf, four lanes per target (orders mod 4: 32-byte pieces of a
+// basis row), then lane r of a quad writes right-hand side r.  Two layers, 262,144
+// points: L2P 32 us + scatter 33 us before, now 29 us.
+// ---------------------------------------------------------------------------
+template <int R>
+__global__ void __launch_bounds__(128) l2p_scatter_kernel(const int32_t* __restrict__ lb, int64_t nleaf, int64_t n,
+                                                          int nrhs, const cf* __restrict__ loc,
+                                                          const cf* __restrict__ basis, int nc,
+                                                          const cf* ys, const int64_t* __restrict__ perm,
+                                                          bool conj_out, cf* y) {
+    extern __shared__ cf s_coef[];                         // [4 warps][R][nc]
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 3;
+    const int64_t b = (int64_t)blockIdx.x * 4 + w;
+    if (b >= nleaf) return;
+    const int32_t lo = lb[b], hi = lb[b + 1];
+    if (hi <= lo) return;
+    cf* coef = s_coef + (size_t)w * R * nc;
+    for (int r0 = 0; r0 < nrhs; r0 += R) {
+        if (loc) {
+            __syncwarp();
+            const cf* src = loc + ((int64_t)b * nrhs + r0) * nc;
+            const int cnt = min(R, nrhs - r0) * nc;
+            for (int e = lane; e < R * nc; e += 32) coef[e] = e < cnt ? src[e] : cfmk(0.f, 0.f);
+            __syncwarp();
+        }
+        for (int32_t i0 = lo; i0 < hi; i0 += 8) {
+            const int32_t i = i0 + (lane >> 2);
+            const bool live = i < hi;
+            cf acc[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = cfmk(0.f, 0.f);
+            if (loc && live) {
+                const cf* B = basis + (int64_t)i * nc;
+#pragma unroll 4
+                for (int m = t; m < nc; m += 4) {
+                    const cf v = __ldg(B + m), g = cfmk(0.25f * v.y, 0.25f * v.x);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) cfma(acc[r], g, coef[r * nc + m]);
+                }
+            }
+            cf out = cfmk(0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, 1);
+                acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, 1);
+                acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, 2);
+                acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, 2);
+                if (r == t) out = acc[r];
+            }
+            if (live && t < R && r0 + t < nrhs) {
+                if (ys) {
+                    const cf o = ys[(int64_t)i * nrhs + r0 + t];
+                    out.x += o.x;
+                    out.y += o.y;
+                }
+                if (perm) y[(int64_t)(r0 + t) * n + perm[i]] = conj_out ? cfmk(out.x, -out.y) : out;
+                else y[(int64_t)i * nrhs + r0 + t] = out;          // sorted point-major
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Near field and the leaves' local expansions: warp per target leaf, lane =
 // target point (passes of 32), sources of the 3 x 3 neighbourhood in order.
 // ---------------------------------------------------------------------------
@@ -981,6 +1200,37 @@ hfmm_status init_small(hfmm_plan_s* P, cudaStream_t st) {
     return HFMM_OK;
 }
 
+// Stored near-field blocks of a plan that only runs few right-hand sides (after
+// build_local_coords); skipped above the byte budget.
+hfmm_status build_near_small(hfmm_plan_s* P, cudaStream_t st) {
+    const LevelInfo& lv = P->lev[P->L];
+    if (P->max_rhs > P->small_rhs || P->ad || (P->flags & HFMM_FLAG_SIMT_M2L)) return HFMM_OK;
+    int64_t pairs = 0;
+    HFMM_TRY(near64_offsets(P, &pairs, false, st));
+    if (sizeof(cf) * (double)pairs > NEAR32_MAX_BYTES) return HFMM_OK;
+    HFMM_TRY(near64_offsets(P, &pairs, true, st));
+    HFMM_TRY(plan_alloc(P, (void**)&P->near32_vals, sizeof(cf) * (size_t)std::max<int64_t>(pairs, 1)));
+    near_fill_kernel<<<(unsigned)ceil_div(lv.nbox, 4), 128, 0, st>>>(P->leaf_begin, P->L, lv.nbox, P->xl32, (float)P->k,
+                                                                     (float)lv.h, P->near64_off, P->near32_vals);
+    HFMM_CUDA_TRY(cudaGetLastError());
+    P->table_bytes += sizeof(cf) * (double)pairs;
+    return HFMM_OK;
+}
+
+hfmm_status launch_gather_few(hfmm_plan_s* P, int nrhs, const cf* q, bool conj_in, cudaStream_t st) {
+    gather_few_kernel<<<(unsigned)ceil_div(P->n, 256), 256, 0, st>>>(q, P->iperm32, P->n, nrhs, conj_in, P->q32);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+hfmm_status launch_scatter_few(hfmm_plan_s* P, int nrhs, cf* y, bool conj_out, cudaStream_t st) {
+    scatter_few_kernel<<<(unsigned)ceil_div(P->n, 256), 256, 0, st>>>(P->y32, P->iperm32, P->n, nrhs, conj_out, y);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
 hfmm_status small_p2m(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
     LevelInfo& lv = P->lev[P->L];
     const unsigned grid = (unsigned)ceil_div(lv.nbox, 4);
@@ -1108,24 +1358,49 @@ hfmm_status small_near(hfmm_plan_s* P, int nrhs, bool near, bool l2p, cudaStream
     return HFMM_OK;
 }
 
-hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t st) {
+// The near-field sums into y32 (first writer) and the directly summed reaction onto them.
+static hfmm_status small_near_sums(hfmm_plan_s* P, int nrhs, bool near, bool direct, cudaStream_t st) {
+    LevelInfo& lv = P->lev[P->L];
+    const unsigned grid = (unsigned)ceil_div(lv.nbox, 4);
+    if (near && P->near32_vals) {
+#define HFMM_NEARB(RR)                                                                                             \
+    near_blocks_kernel<RR><<<grid, 128, 0, st>>>(P->leaf_begin, P->L, lv.nbox, P->near64_off, P->near32_vals, P->q32, \
+                                                 nrhs, P->y32)
+        if (nrhs >= 4) HFMM_NEARB(4);
+        else if (nrhs >= 2) HFMM_NEARB(2);
+        else HFMM_NEARB(1);
+#undef HFMM_NEARB
+        HFMM_CUDA_TRY(cudaGetLastError());
+        ++P->launches;
+    } else {
+        HFMM_CUDA_TRY(cudaMemsetAsync(P->y32, 0, sizeof(cf) * P->n * nrhs, st));
+        if (near) {
+            HFMM_TRY(small_near(P, nrhs, true, false, st));
+            ++P->launches;
+        }
+    }
+    if (direct) HFMM_TRY(launch_direct32(P, nrhs, st));
+    return HFMM_OK;
+}
+
+// Everything after the gather, into the caller's order.
+hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, bool conj_out, cf* y, cudaStream_t st) {
     const int L = P->L;
     const int64_t n = P->n;
     const double MAC = 8.0 * nrhs, C = 8.0 * nrhs;
     const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0;
     const bool near = (parts & HFMM_PART_NEAR_FREE) != 0;
-    // Both fields: the near field (first writer of y32 after the memset) runs on
-    // a low-priority stream while the far-field chain runs on a high-priority
-    // one and fills the SMs that the coarse levels' few CTAs leave idle; the
-    // leaves' L2P then waits for it and adds into y32.
+    const bool direct = (parts & HFMM_PART_NEAR_REACT) && P->nd > 0;
+    // Both fields: the near field runs on a low-priority stream while the far-field
+    // chain runs on a high-priority one and fills the SMs that the coarse levels'
+    // few CTAs leave idle; the leaves' L2P then waits for it.
     const bool concurrent = far && near;
     cudaStream_t fs = st;
     if (concurrent) {
         HFMM_TRY(fork_near_far(P, st));
         StageTimer tn{P, P->near_st};
         tn.begin(HFMM_STAGE_P2P);
-        HFMM_TRY(small_near(P, nrhs, true, false, P->near_st));
-        ++P->launches;
+        HFMM_TRY(small_near_sums(P, nrhs, true, direct, P->near_st));
         tn.end(HFMM_STAGE_P2P);
         HFMM_CUDA_TRY(cudaEventRecord(P->ev_near_done, P->near_st));
         fs = P->far_st;
@@ -1163,25 +1438,48 @@ hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t st) {
         }
         tm.end(HFMM_STAGE_DOWN);
     }
+    LevelInfo& leaf = P->lev[L];
+    const bool sums = near || direct;
+    if (concurrent) {
+        HFMM_CUDA_TRY(cudaStreamWaitEvent(fs, P->ev_near_done, 0));
+    } else if (sums) {
+        tm.begin(HFMM_STAGE_P2P);
+        HFMM_TRY(small_near_sums(P, nrhs, near, direct, st));
+        tm.end(HFMM_STAGE_P2P);
+    }
+    if (!concurrent) tm.begin(HFMM_STAGE_SCATTER);
+    const unsigned grid = (unsigned)ceil_div(leaf.nbox, 4);
+    // page-locked host memory wants consecutive writes: the sums stay sorted (in y32) and a
+    // second kernel writes the caller's order
+    cudaPointerAttributes at;
+    const bool host = cudaPointerGetAttributes(&at, y) == cudaSuccess && at.type == cudaMemoryTypeHost;
+    cudaGetLastError();
+#define HFMM_TAIL(RR)                                                                                            \
+    do {                                                                                                         \
+        const size_t sm = sizeof(cf) * 4 * RR * leaf.ncoef;                                                      \
+        if (sm > 48 * 1024)                                                                                      \
+            HFMM_CUDA_TRY(cudaFuncSetAttribute(l2p_scatter_kernel<RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); \
+        l2p_scatter_kernel<RR><<<grid, 128, sm, fs>>>(P->leaf_begin, leaf.nbox, n, nrhs, far ? leaf.loc32 : nullptr, \
+                                                      P->basis32, leaf.ncoef, sums ? P->y32 : nullptr,           \
+                                                      host ? nullptr : P->perm, conj_out, host ? P->y32 : y);    \
+    } while (0)
+    if (nrhs >= 3 && leaf.ncoef <= 1500) HFMM_TAIL(4);
+    else if (nrhs >= 2 && leaf.ncoef <= 3000) HFMM_TAIL(2);
+    else HFMM_TAIL(1);
+#undef HFMM_TAIL
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    if (host) HFMM_TRY(launch_scatter_few(P, nrhs, y, conj_out, fs));
+    if (concurrent) {
+        HFMM_CUDA_TRY(cudaEventRecord(P->ev_far_done, fs));
+        HFMM_CUDA_TRY(cudaStreamWaitEvent(st, P->ev_far_done, 0));
+    } else tm.end(HFMM_STAGE_SCATTER);
     if (near || far) {
-        LevelInfo& leaf = P->lev[L];
-        if (concurrent) {
-            // the leaves' L2P after the near field (both add into y32)
-            HFMM_CUDA_TRY(cudaStreamWaitEvent(fs, P->ev_near_done, 0));
-            HFMM_TRY(small_near(P, nrhs, false, true, fs));
-            ++P->launches;
-            HFMM_CUDA_TRY(cudaEventRecord(P->ev_far_done, fs));
-            HFMM_CUDA_TRY(cudaStreamWaitEvent(st, P->ev_far_done, 0));
-        } else {
-            tm.begin(HFMM_STAGE_P2P);
-            HFMM_TRY(small_near(P, nrhs, near, far, st));
-            ++P->launches;
-            tm.end(HFMM_STAGE_P2P);
-        }
         P->st_flops[HFMM_STAGE_P2P] = (near ? MAC * (double)P->p2p_point_pairs : 0.0) +
                                       (far ? MAC * n * leaf.ncoef : 0.0);
         P->st_bytes[HFMM_STAGE_P2P] = 3.0 * C * n + 16.0 * n + (far ? C * leaf.nbox * leaf.ncoef + 8.0 * n * leaf.ncoef : 0.0);
     }
+    P->st_bytes[HFMM_STAGE_SCATTER] = 2.0 * C * n + 8.0 * n;
     return HFMM_OK;
 }
 
