@@ -47,7 +47,9 @@ static void plan_free(hfmm_plan_s* P) {
     }
     if (P->far_st) cudaStreamDestroy(P->far_st);
     if (P->near_st) cudaStreamDestroy(P->near_st);
-    for (cudaEvent_t e : {P->ev_fork, P->ev_near_done, P->ev_far_done})
+    for (cudaEvent_t e : {P->ev_fork, P->ev_near_done, P->ev_far_done, P->ev_up_done})
+        if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : P->ev_react)
         if (e) cudaEventDestroy(e);
     for (void* p : P->allocations) cudaFree(p);
     if (P->krylov_host) cudaFreeHost(P->krylov_host);

@@ -77,7 +77,9 @@ static hfmm_status batch_capture(hfmm_batch_s* B, int nrhs, const void* const* q
     for (int i = 0; !pers && i < B->ninst && e == cudaSuccess && s == HFMM_OK; ++i) {
         e = cudaStreamWaitEvent(B->streams[i], B->fork, 0);
         if (e != cudaSuccess) break;
+        B->plans[i]->in_batch = true;
         s = batch_apply_one(B->plans[i], nrhs, q[i], y[i], adjoint, B->streams[i]);
+        B->plans[i]->in_batch = false;
         if (s != HFMM_OK) break;
         e = cudaEventRecord(B->joins[i], B->streams[i]);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, B->joins[i], 0);

@@ -274,7 +274,12 @@ struct hfmm_plan_s {
     // near field on a low-priority one, both forked from and joined back into the
     // caller's stream (created on first use)
     cudaStream_t far_st = nullptr, near_st = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_near_done = nullptr, ev_far_done = nullptr;
+    // being captured beside other instances: the few-RHS passes then launch without the early start
+    // (split64.cuh), whose waiting CTAs hold places that other instances' kernels could use
+    // (32 x 2048..8192 points, 1 RHS: 2675 us with it, 2598 us without)
+    bool in_batch = false;
+    cudaEvent_t ev_fork = nullptr, ev_near_done = nullptr, ev_far_done = nullptr, ev_up_done = nullptr;
+    std::vector<cudaEvent_t> ev_react;   // per level: its reaction lists' sums (few right-hand sides)
     int* tc_err = nullptr;          // set by the tensor-core pass when a bounded wait gave up
     long tc_spin = 0;               // polls of a bounded device wait (options.spin_limit or the default)
     __half* tc_zero = nullptr;      // 4 KB of zeros: the A half of a missing source box

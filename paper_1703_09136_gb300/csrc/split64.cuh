@@ -2,6 +2,7 @@
 // fixed-point words with biased digit fields, digit pairs, and the FP32
 // mma.sync that sums digit products without rounding.
 #pragma once
+#include <utility>
 
 #include "common.cuh"
 
@@ -100,10 +101,11 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 __device__ __forceinline__ void pdl_start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launch of a kernel that calls pdl_wait() before its first read of earlier results.
+// Launch of a kernel that calls pdl_wait() before its first read of earlier results;
+// pdl = false: an ordinary launch of it.
 template <class... P, class... A>
-inline cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster,
-                              A&&... args) {
+inline cudaError_t pdl_launch_if(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                 unsigned cluster, A&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -111,11 +113,16 @@ inline cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_
     cfg.stream = st;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = cluster;
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = cluster > 0 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster,
+                              A&&... args) {
+    return pdl_launch_if(true, kernel, grid, block, smem, st, cluster, std::forward<A>(args)...);
 }
