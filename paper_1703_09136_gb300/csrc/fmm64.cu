@@ -812,11 +812,39 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
     const int nb = ceil_div(n, 256);
     const size_t bytes = sizeof(cd) * (size_t)n * P->max_rhs;
     if (!P->grad_buf) {
-        HFMM_TRY(plan_alloc(P, (void**)&P->grad_buf, 5 * bytes));
         HFMM_TRY(build_direct_grad(P, st));
         HFMM_TRY(build_near64_grad(P, st));
         HFMM_TRY(build_split(P, 0, st));
         HFMM_TRY(build_leaf64(P, st));
+        P->grad_fused = P->near64g_x && P->basis64;
+        HFMM_TRY(plan_alloc(P, (void**)&P->grad_buf, P->grad_fused ? bytes + 2 * sizeof(double2) * (size_t)n : 5 * bytes));
+    }
+    if (P->grad_fused) {                          // stored blocks and bases (leaf64.cu); else the kernels that evaluate them
+        cd* gc = P->grad_buf;
+        double2* far_sum = (double2*)(gc + (size_t)n * P->max_rhs);
+        double2* near_sum = far_sum + n;
+        gather_q<<<nb, 256, 0, st>>>(q, P->perm, n, nrhs, false, P->q_sorted);
+        gather_q<<<nb, 256, 0, st>>>(g, P->perm, n, nrhs, true, gc);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        HFMM_TRY(fork_near_far(P, st));
+        HFMM_TRY(launch_grad_near(P, nrhs, gc, near_sum, P->near_st));
+        HFMM_CUDA_TRY(cudaEventRecord(P->ev_near_done, P->near_st));
+        HFMM_CUDA_TRY(cudaEventRecord(P->ev_far_done, P->far_st));
+        cd* const qs = P->q_sorted;
+        for (int field = 0; field < 2; ++field) {          // u of q, then w of conj(g)
+            P->q_sorted = field == 0 ? qs : gc;
+            hfmm_status s = leaves64(P, nrhs, st);
+            if (s == HFMM_OK) s = upward64(P, nrhs, st);
+            if (s == HFMM_OK) s = downward64(P, nrhs, HFMM_PART_ALL, st);
+            P->q_sorted = qs;
+            HFMM_TRY(s);
+            if (field == 1) {
+                HFMM_CUDA_TRY(cudaStreamWaitEvent(st, P->ev_near_done, 0));
+                HFMM_CUDA_TRY(cudaStreamWaitEvent(st, P->ev_far_done, 0));
+            }
+            HFMM_TRY(launch_grad_far(P, nrhs, field == 0 ? gc : qs, far_sum, near_sum, field == 0 ? nullptr : gxy, st));
+        }
+        return HFMM_OK;
     }
     cd* ux = P->grad_buf;
     cd* uy = ux + (size_t)n * P->max_rhs;

@@ -461,7 +461,176 @@ __global__ void near64_fix_kernel(cd* G, int64_t n, const int* __restrict__ E) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// Position gradients: out[t] = Re sum_r (conj(g_t) grad u_t + q_t grad w_t), u and w the fields of q
+// and conj(g).  Both fields go through the same blocks, so a pair needs the one complex number
+//   S = sum_r conj(g_t) q_s + q_t conj(g_s)
+// and the real parts of Gx S and Gy S: 8 nrhs + 4 FP64 FMAs instead of 16 nrhs.  The far part is the
+// L2P with the locals of the derivative, from the same bases (order p + 1 included):
+//   d/dx sum_q b_q E_q = (k/2) sum_m (b_{m+1} - b_{m-1}) E_m,   d/dy: (i k/2) sum_m (b_{m+1} + b_{m-1}) E_m.
+// Bound by FP64 FMAs (3.4 M near-field pairs of 40,000 points, one right-hand side: 12 each, 80 us);
+// the pairs run beside both tree passes.  Measured there: near field 2 x 208 us (a lane per target of
+// ten-point leaves) -> 104 us, locals' gradient 2 x 266 us (Bessel sequences evaluated on each
+// call) -> 2 x 27 us; the whole gradient 1578 -> 768 us.
+// ---------------------------------------------------------------------------
+constexpr int GN_TB = 128;
+
+// Near field and direct reaction.  A CTA per leaf: thread (part, i) takes the target i and every
+// parts-th source, so that consecutive lanes read consecutive block entries; parts added in order.
+template <bool ONE>
+__global__ void __launch_bounds__(GN_TB) grad_near_kernel(const Leaf64Rec* __restrict__ recs, const int32_t* __restrict__ src,
+                                                          const cd* __restrict__ Gx, const cd* __restrict__ Gy,
+                                                          const Leaf64D* __restrict__ ds, const cd* __restrict__ Dx,
+                                                          const cd* __restrict__ Dy, const cd* __restrict__ q,
+                                                          const cd* __restrict__ gc, int64_t n, int nrhs,
+                                                          double2* __restrict__ out) {
+    __shared__ double2 near_s[GN_TB], direct_s[GN_TB];
+    const Leaf64Rec& L = recs[blockIdx.x];
+    const int tid = threadIdx.x, ns = L.ns;
+    auto pair_strength = [&](int64_t t, int64_t s, cd qt, cd gt) {
+        cd S = cmk(0.0, 0.0);
+        if (ONE) {
+            cfma(S, gt, __ldg(q + s));
+            cfma(S, qt, __ldg(gc + s));
+        } else
+            for (int r = 0; r < nrhs; ++r) {
+                cfma(S, __ldg(gc + r * n + t), __ldg(q + r * n + s));
+                cfma(S, __ldg(q + r * n + t), __ldg(gc + r * n + s));
+            }
+        return S;
+    };
+    auto add = [](double2& a, cd x, cd y, cd S) {
+        a.x = fma(x.x, S.x, fma(-x.y, S.y, a.x));
+        a.y = fma(y.x, S.x, fma(-y.y, S.y, a.y));
+    };
+    for (int i0 = 0; i0 < L.tn; i0 += GN_TB) {
+        const int tn = min(GN_TB, L.tn - i0), parts = GN_TB / tn;
+        double2 a = make_double2(0.0, 0.0), b = a;
+        if (tid < parts * tn) {
+            {
+                const int i = i0 + tid % tn;
+                const int64_t t = L.tlo + i;
+                const cd qt = __ldg(q + t), gt = __ldg(gc + t);
+                const int32_t* sj = src + L.soff;
+                const int64_t o = L.goff + i;
+#pragma unroll 4
+                for (int j = tid / tn; j < ns; j += parts) {
+                    const int64_t e = o + (int64_t)j * L.tn;
+                    add(a, __ldg(Gx + e), __ldg(Gy + e), pair_strength(t, __ldg(sj + j), qt, gt));
+                }
+            }
+            const int i = i0 + tid / parts;                // entries of a direct block: consecutive sources
+            const int64_t t = L.tlo + i;
+            for (int32_t e = L.dbeg; e < L.dend; ++e) {
+                const Leaf64D E = ds[e];
+                const int64_t o = E.blk + (int64_t)i * E.sn;
+                const cd qt = __ldg(q + t), gt = __ldg(gc + t);
+                for (int j = tid % parts; j < E.sn; j += parts)
+                    add(b, __ldg(Dx + o + j), __ldg(Dy + o + j), pair_strength(t, E.slo + j, qt, gt));
+            }
+        }
+        __syncthreads();                                   // the last chunk's sums are read
+        near_s[tid] = a;
+        direct_s[tid] = b;
+        __syncthreads();
+        if (tid < tn) {
+            double2 v = make_double2(0.0, 0.0);
+            for (int k = 0; k < parts; ++k) {
+                const double2 x = near_s[k * tn + tid], y = direct_s[tid * parts + k];
+                v.x += x.x + y.x;
+                v.y += x.y + y.y;
+            }
+            out[L.tlo + i0 + tid] = v;
+        }
+    }
+}
+
+// Far field of one of the two fields: Re sum_r v_t grad(local field)_t, four lanes a target.
+// Without gxy the sums go to acc; with it, acc, the near field's sums and these go to the caller's order.
+__global__ void __launch_bounds__(64) grad_far_kernel(const Leaf64Rec* __restrict__ recs, const cd* __restrict__ basis,
+                                                      const cd* __restrict__ v, int64_t n, int nrhs, double k,
+                                                      double2* __restrict__ acc, const double2* __restrict__ near_sum,
+                                                      const int64_t* __restrict__ perm, double* __restrict__ gxy) {
+    extern __shared__ __align__(16) double gf_coef[];      // [p + 2][8]
+    const Leaf64Rec& L = recs[blockIdx.x];
+    const int p = L.p, nb = L.nb, nc = 2 * p + 1, t = threadIdx.x & 3;
+    const double f = 0.125 * k;
+    for (int i0 = 0; i0 < L.tn; i0 += 16) {
+        const int i = i0 + (threadIdx.x >> 2);
+        const bool live = i < L.tn;
+        const cd* B = basis + L.boff + (int64_t)(live ? i : 0) * nb;
+        double ax = 0.0, ay = 0.0;
+        for (int r = 0; r < nrhs; ++r) {
+            if (i0 == 0 || nrhs > 1) {
+                const cd* beta = L.loc + (L.lidx * nrhs + r) * nc + p;
+                auto at = [&](int m) { return m >= -p && m <= p ? __ldg(beta + m) : cmk(0.0, 0.0); };
+                __syncthreads();                           // the last coefficients are read
+                for (int m = threadIdx.x; m <= p + 1; m += 64) {
+                    const double sg = m == 0 ? 0.0 : (m & 1) ? -1.0 : 1.0;
+                    const cd up = at(m + 1), lo = at(m - 1), nup = at(1 - m), nlo = at(-1 - m);
+                    const cd cx = csub(up, lo), dx = cscale(csub(nup, nlo), sg);
+                    const cd cy = cmuli(cadd(up, lo)), dy = cscale(cmuli(cadd(nup, nlo)), sg);
+                    double* w = gf_coef + 8 * m;
+                    w[0] = -f * (cx.y + dx.y); w[1] = f * (cx.x - dx.x); w[2] = f * (cx.x + dx.x); w[3] = f * (cx.y - dx.y);
+                    w[4] = -f * (cy.y + dy.y); w[5] = f * (cy.x - dy.x); w[6] = f * (cy.x + dy.x); w[7] = f * (cy.y - dy.y);
+                }
+                __syncthreads();
+            }
+            cd x = cmk(0.0, 0.0), y = x;
+            if (live) {
+#pragma unroll 2
+                for (int m = t; m < nb; m += 4) {
+                    const cd u = __ldg(B + m);
+                    const double* w = gf_coef + 8 * m;
+                    x.x = fma(u.x, w[0], fma(u.y, w[1], x.x));
+                    x.y = fma(u.x, w[2], fma(u.y, w[3], x.y));
+                    y.x = fma(u.x, w[4], fma(u.y, w[5], y.x));
+                    y.y = fma(u.x, w[6], fma(u.y, w[7], y.y));
+                }
+                const cd vt = __ldg(v + (int64_t)r * n + L.tlo + i);
+                ax = fma(vt.x, x.x, fma(-vt.y, x.y, ax));
+                ay = fma(vt.x, y.x, fma(-vt.y, y.y, ay));
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            ax += __shfl_xor_sync(0xffffffffu, ax, o);
+            ay += __shfl_xor_sync(0xffffffffu, ay, o);
+        }
+        if (live && t == 0) {
+            const int64_t j = L.tlo + i;
+            if (gxy) {
+                const double2 a = acc[j], b = near_sum[j];
+                const int64_t c = perm[j];
+                gxy[2 * c] = ax + a.x + b.x;
+                gxy[2 * c + 1] = ay + a.y + b.y;
+            } else acc[j] = make_double2(ax, ay);
+        }
+    }
+}
+
 }  // namespace
+
+// Position gradient: near field and direct reaction of both fields.
+hfmm_status launch_grad_near(hfmm_plan_s* P, int nrhs, const cd* gc, double2* out, cudaStream_t st) {
+    auto kernel = nrhs == 1 ? grad_near_kernel<true> : grad_near_kernel<false>;
+    kernel<<<(unsigned)P->leaf64_n, GN_TB, 0, st>>>(P->leaf64, P->leaf64_src, P->near64g_x, P->near64g_y, P->leaf64_d,
+                                                    P->d_gvals, P->d_gvals ? P->d_gvals + P->nd_vals : nullptr,
+                                                    P->q_sorted, gc, P->n, nrhs, out);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+// Position gradient: the locals' part of one field, v the other field's factor at the targets.
+hfmm_status launch_grad_far(hfmm_plan_s* P, int nrhs, const cd* v, double2* acc, const double2* near_sum, double* gxy,
+                            cudaStream_t st) {
+    grad_far_kernel<<<(unsigned)P->leaf64_n, 64, 8 * sizeof(double) * (P->leaf64_p + 2), st>>>(
+        P->leaf64, P->basis64, v, P->n, nrhs, P->k, acc, near_sum, P->perm, gxy);
+    ++P->launches;
+    HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
 
 // Digit form of `pairs` near-field values in place; *finite = false (and the
 // values unchanged) where an entry is not finite (coincident points).

@@ -254,7 +254,8 @@ struct hfmm_plan_s {
     size_t krylov_host_words = 0;
     cd* near64g_x = nullptr;        // d/dx, d/dy of the same blocks (first gradient request)
     cd* near64g_y = nullptr;
-    cd* grad_buf = nullptr;         // [5][max_rhs][n]
+    cd* grad_buf = nullptr;         // conj(g) and the fields or sums of a gradient
+    bool grad_fused = false;        // gradients from stored blocks and bases (leaf64.cu)
     cd* grad_q = nullptr;           // mixed plans: widened strengths / loss gradient
     cd* grad_g = nullptr;
     cd* d_gvals = nullptr;          // [2][nd_vals]
@@ -393,6 +394,9 @@ void adaptive_tiles(const hfmm_plan_s* P, int l, bool up, const std::vector<int3
 // leaf64.cu
 hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, bool* finite, cudaStream_t st);
+hfmm_status launch_grad_near(hfmm_plan_s* P, int nrhs, const cd* gc, double2* out, cudaStream_t st);
+hfmm_status launch_grad_far(hfmm_plan_s* P, int nrhs, const cd* v, double2* acc, const double2* near_sum, double* gxy,
+                            cudaStream_t st);
 hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st);
 hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2p, bool direct, const cd* ys,
                           bool conj_out, cd* y, cudaStream_t st);
