@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "bessel.cuh"
+#include "hankel.cuh"
 #include "plan.cuh"
 
 namespace {
@@ -686,41 +687,75 @@ __global__ void grad_combine_kernel(const cd* qs, const cd* gs_conj, const cd* u
 // Near-field gradient blocks (built on a plan's first position-gradient
 // request): d/dx and d/dy of (i/4) H0(k |x_t - x_s|) at the target,
 // (i/4)(-k H1(k r)) (x_t - x_s) / r, for the same pairs and layout as the
-// near-field blocks above (0 for s = t).
-__global__ void near64_grad_fill_kernel(const int32_t* __restrict__ lb, int L, const double2* __restrict__ xs,
-                                        double k, const int64_t* __restrict__ off, cd* __restrict__ Gx,
-                                        cd* __restrict__ Gy) {
+// near-field blocks above (0 for s = t).  The entry of (s, t) is minus that of (t, s): a
+// pair is evaluated once, from the leaf that comes first in (y, x), and written to both blocks.
+// Bound by the FP64 work of H1; grid (leaves, parts of a leaf's pairs).  4,099 points (0.5 M
+// entries): 2560 us with every entry's H0 and H1 by the recurrence with divisions -> 451 us.
+constexpr int GFILL_PARTS = 4;
+__global__ void __launch_bounds__(128) near64_grad_fill_kernel(const int32_t* __restrict__ lb, int L,
+                                                               const double2* __restrict__ xs, double k,
+                                                               const int64_t* __restrict__ off, cd* __restrict__ Gx,
+                                                               cd* __restrict__ Gy) {
+    __shared__ int32_t s_lo[5], s_n[5], s_jb[5], s_js[5];  // the leaf itself and the four neighbours after it
+    __shared__ int64_t s_off[5];
     const int64_t b = blockIdx.x;
     const int32_t tlo = lb[b], tn = lb[b + 1] - tlo;
     if (tn <= 0) return;
     const int m = 1 << L;
     const int ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
-    int64_t j0 = 0;
-    for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-            const int sx = ix + dx, sy = iy + dy;
-            if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
-            const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
-            const int32_t slo = lb[s], sn = lb[s + 1] - slo;
-            for (int e = threadIdx.x; e < sn * tn; e += blockDim.x) {
-                const int j = e / tn, i = e % tn;
-                cd gx = cmk(0.0, 0.0), gy = cmk(0.0, 0.0);
-                if (tlo + i != slo + j) {
-                    const double2 a = xs[tlo + i], c = xs[slo + j];
-                    const double ddx = a.x - c.x, ddy = a.y - c.y;
-                    const double r = hypot(ddx, ddy);
-                    cd h0, h1;
-                    hankel01(k * r, &h0, &h1);
-                    const cd cc = cscale(cmuli(h1), -0.25 * k / r);
-                    gx = cscale(cc, ddx);
-                    gy = cscale(cc, ddy);
-                }
-                const int64_t o = off[b] + (j0 + j) * tn + i;
-                Gx[o] = gx;
-                Gy[o] = gy;
+    if (threadIdx.x < 5) {
+        const int u = threadIdx.x, dx = u == 0 ? 0 : u == 1 ? 1 : u - 3, dy = u < 2 ? 0 : 1;
+        const int sx = ix + dx, sy = iy + dy;
+        const bool in = sx >= 0 && sx < m && sy < m;
+        const uint32_t s = in ? morton((uint32_t)sx, (uint32_t)sy) : 0u;
+        // sources of leaf (x, y)'s list before its neighbour at (ex, ey)
+        auto before = [&](int x, int y, int ex, int ey) {
+            int32_t j = 0;
+            for (int v = 0; v < (ey + 1) * 3 + ex + 1; ++v) {
+                const int nx = x + v % 3 - 1, ny = y + v / 3 - 1;
+                if (nx < 0 || ny < 0 || nx >= m || ny >= m) continue;
+                const uint32_t c = morton((uint32_t)nx, (uint32_t)ny);
+                j += lb[c + 1] - lb[c];
             }
-            j0 += sn;
+            return j;
+        };
+        s_lo[u] = in ? lb[s] : 0;
+        s_n[u] = in ? lb[s + 1] - lb[s] : 0;
+        s_off[u] = in ? off[s] : 0;
+        s_jb[u] = in ? before(ix, iy, dx, dy) : 0;
+        s_js[u] = in ? before(sx, sy, -dx, -dy) : 0;
+    }
+    __syncthreads();
+    const int64_t ob = off[b];
+    int64_t base = 0;
+    for (int u = 0; u < 5; ++u) {
+        const int32_t sn = s_n[u], slo = s_lo[u];
+        const int64_t cnt = (int64_t)sn * tn, step = GFILL_PARTS * 128;
+        // the parts' threads go through the leaf's pairs as one sequence
+        int64_t e = ((int64_t)blockIdx.y * 128 + threadIdx.x - base) % step;
+        if (e < 0) e += step;
+        for (; e < cnt; e += step) {
+            const int j = (int)(e / tn), i = (int)(e % tn);
+            if (u == 0 && i > j) continue;
+            cd gx = cmk(0.0, 0.0), gy = gx;
+            if (u != 0 || i != j) {
+                const double2 a = xs[tlo + i], c = xs[slo + j];
+                const double ddx = a.x - c.x, ddy = a.y - c.y;
+                const double r = hypot(ddx, ddy);
+                const cd cc = cscale(cmuli(hankel1(k * r)), -0.25 * k / r);
+                gx = cscale(cc, ddx);
+                gy = cscale(cc, ddy);
+            }
+            const int64_t o = ob + (int64_t)(s_jb[u] + j) * tn + i, o2 = s_off[u] + (int64_t)(s_js[u] + i) * sn + j;
+            Gx[o] = gx;
+            Gy[o] = gy;
+            if (o2 != o) {
+                Gx[o2] = cneg(gx);
+                Gy[o2] = cneg(gy);
+            }
         }
+        base += cnt;
+    }
 }
 
 // fx[r][t] += sum_s Gx[s][t] v[r][s], fy likewise: a warp per target leaf.
@@ -910,7 +945,7 @@ hfmm_status build_near64_grad(hfmm_plan_s* P, cudaStream_t st) {
     HFMM_TRY(near64_offsets(P, &pairs, true, st));
     HFMM_TRY(plan_alloc(P, (void**)&P->near64g_x, sizeof(cd) * std::max<int64_t>(pairs, 1)));
     HFMM_TRY(plan_alloc(P, (void**)&P->near64g_y, sizeof(cd) * std::max<int64_t>(pairs, 1)));
-    near64_grad_fill_kernel<<<(unsigned)P->lev[P->L].nbox, 128, 0, st>>>(P->leaf_begin, P->L, P->xy_sorted, P->k,
+    near64_grad_fill_kernel<<<dim3((unsigned)P->lev[P->L].nbox, GFILL_PARTS), 128, 0, st>>>(P->leaf_begin, P->L, P->xy_sorted, P->k,
                                                                           P->near64_off, P->near64g_x, P->near64g_y);
     HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;
