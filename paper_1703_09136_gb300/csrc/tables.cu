@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "bessel.cuh"
+#include "hankel.cuh"
 #include "plan.cuh"
 
 namespace {
@@ -320,8 +321,9 @@ __device__ Node eval_node(const MedDev& m, const Seg* segs, int s0, int s1, int6
 }
 
 constexpr int CH = 8;                // orders n (and -n) per pass over a tile's nodes
-constexpr int RT_THREADS = 256;
-constexpr int RT_NODES = 1024;       // nodes of a tile (six doubles each in shared memory)
+constexpr int RT_THREADS = 128;
+constexpr int RT_NODES = 512;        // nodes of a tile
+constexpr int RT_NV = 10;            // doubles of a node in shared memory
 
 // sums of v[0 .. 31] over the warp, value l in lane l (31 additions instead of 160)
 __device__ __forceinline__ double warp_scatter32(double (&v)[32]) {
@@ -344,11 +346,14 @@ __device__ __forceinline__ double warp_scatter32(double (&v)[32]) {
 //              lp, lm = log c - t Y +- i xi X, lz = log(k1 / (xi + t)); on the real path lz
 //              and the common real part of lp, lm are real, so P = e^{lr + n lz} and
 //              Q = e^{lr - n lz} are real and multiply two constant phases.
-// A tile's nodes (square roots, sigma, logarithms) are evaluated once into shared
-// memory; each pass of eight orders starts its recurrences from exponentials (as
-// accurate as before) and serves both signs.  FP64 bound (1.0 TFLOP/s): the kernel
-// before evaluated every node once per eight orders and kept complex recurrences for
-// both signs: three layers, 1M points 612 -> 177 ms per rule, impedance, 4099 points 16.2 -> 1.6.
+// A tile's nodes (square roots, sigma, logarithms, the factors and phases that no order changes) are
+// evaluated once into shared memory; each pass of eight orders serves both signs.  The t nodes'
+// recurrences start every pass from exponentials (their range is that of the whole sum, not
+// of one order).  The tau nodes' phases e^{i n tau} go on from pass to pass by e^{8 i tau},
+// which errs less than the cosine of the rounded product n tau.  FP64 bound (1.0 TFLOP/s):
+// nodes once per eight orders and complex recurrences for both signs, three layers, 1M points
+// 612 ms per rule, impedance, 4099 points 16.2 ms; nodes once, 177 and 1.6 ms; factors and
+// phases once too, see the plan times, and 0.86 ms.
 // blockIdx.y splits the tiles; chunks of eight orders c0 .. c0 + nwin; sums[entry][y][2][chunk][32] =
 // (C, S | T_n, T_-n) x re, im.
 __global__ void __launch_bounds__(RT_THREADS) react_sum_kernel(MedDev m, const Entry* __restrict__ ents,
@@ -358,8 +363,8 @@ __global__ void __launch_bounds__(RT_THREADS) react_sum_kernel(MedDev m, const E
     const Entry e = ents[blockIdx.x];
     const int nch = min((e.nmax + CH) / CH - c0, nwin);   // chunks of this launch's window, n = 0 .. nmax
     if (nch <= 0) return;
-    double* nodes = rt_smem;                               // [6][RT_NODES]
-    double* acc = nodes + 6 * RT_NODES;                    // [2][nch][32]
+    double* nodes = rt_smem;                               // [RT_NV][RT_NODES]
+    double* acc = nodes + RT_NV * RT_NODES;                  // [2][nch][32]
     double* red = acc + 2 * nch * 32;                      // [warps][32]
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     for (int i = tid; i < 2 * nch * 32; i += RT_THREADS) acc[i] = 0.0;
@@ -377,14 +382,30 @@ __global__ void __launch_bounds__(RT_THREADS) react_sum_kernel(MedDev m, const E
                 const Node nd = eval_node(m, segs, e.seg0, e.seg1, t0 + i);
                 double* o = nodes + i;
                 if (grp == 0) {
+                    // c e^{i k1 (...)}, e^{i tau}, e^{8 i tau}, e^{i n tau} of the next order
                     const cd b = cmul(nd.c, cexpi(m.k1 * (e.Y * nd.t.x - e.X * nd.t.y)));
-                    o[0] = b.x; o[RT_NODES] = b.y; o[2 * RT_NODES] = nd.u;
+                    const cd first = cexpi((double)(c0 * CH) * nd.u), step = cexpi(CH * nd.u);
+                    o[0] = b.x; o[RT_NODES] = b.y;
+                    o[2 * RT_NODES] = nd.t.y; o[3 * RT_NODES] = nd.t.x;
+                    o[4 * RT_NODES] = step.x; o[5 * RT_NODES] = step.y;
+                    o[6 * RT_NODES] = first.x; o[7 * RT_NODES] = first.y;
                 } else {
                     const cd lc = csub(clogz(nd.c), cscale(nd.t, e.Y)), ix = cmuli(cscale(nd.xi, e.X));
                     const cd lx = clogz(cadd(nd.xi, nd.t));
                     const cd lp = cadd(lc, ix), lm = csub(lc, ix);
-                    o[0] = lp.x; o[RT_NODES] = lp.y; o[2 * RT_NODES] = lm.x; o[3 * RT_NODES] = lm.y;
-                    o[4 * RT_NODES] = lk - lx.x; o[5 * RT_NODES] = -lx.y;      // lz
+                    const cd lz = cmk(lk - lx.x, -lx.y);
+                    cd f, g;
+                    if (lz.y == 0.0 && lp.x == lm.x) {     // real path: z, 1 / z for the imaginary parts' places
+                        o[RT_NODES] = exp(lz.x); o[3 * RT_NODES] = exp(-lz.x);
+                        f = cexpi(lp.y); g = cexpi(lm.y);
+                    } else {
+                        o[RT_NODES] = lp.y; o[3 * RT_NODES] = lm.y;
+                        f = cexpz(lz); g = cexpz(cneg(lz));
+                    }
+                    o[0] = lp.x; o[2 * RT_NODES] = lm.x;
+                    o[4 * RT_NODES] = lz.x; o[5 * RT_NODES] = lz.y;
+                    o[6 * RT_NODES] = f.x; o[7 * RT_NODES] = f.y;
+                    o[8 * RT_NODES] = g.x; o[9 * RT_NODES] = g.y;
                 }
             }
             __syncthreads();
@@ -394,12 +415,12 @@ __global__ void __launch_bounds__(RT_THREADS) react_sum_kernel(MedDev m, const E
                 for (int j = 0; j < 32; ++j) v[j] = 0.0;
                 const double n0 = (c0 + c) * CH;
                 for (int i = tid; i < cnt; i += RT_THREADS) {
-                    const double* o = nodes + i;
+                    double* o = nodes + i;                 // this thread's node in every pass
                     if (grp == 0) {
-                        const double br = o[0], bi = o[RT_NODES], tau = o[2 * RT_NODES];
-                        double s1, c1, sn, cn;
-                        sincos(tau, &s1, &c1);
-                        sincos(n0 * tau, &sn, &cn);
+                        const double br = o[0], bi = o[RT_NODES], c1 = o[2 * RT_NODES], s1 = o[3 * RT_NODES];
+                        double cn = o[6 * RT_NODES], sn = o[7 * RT_NODES];
+                        const cd next = cmul(cmk(cn, sn), cmk(o[4 * RT_NODES], o[5 * RT_NODES]));
+                        o[6 * RT_NODES] = next.x; o[7 * RT_NODES] = next.y;
 #pragma unroll
                         for (int j = 0; j < CH; ++j) {
                             v[4 * j] = fma(br, cn, v[4 * j]);
@@ -411,11 +432,8 @@ __global__ void __launch_bounds__(RT_THREADS) react_sum_kernel(MedDev m, const E
                             cn = x;
                         }
                     } else if (o[5 * RT_NODES] == 0.0 && o[0] == o[2 * RT_NODES]) {   // real path
-                        const double lr = o[0], lz = o[4 * RT_NODES];
-                        double pr, pi, mr, mi;
-                        sincos(o[RT_NODES], &pi, &pr);
-                        sincos(o[3 * RT_NODES], &mi, &mr);
-                        const double z = exp(lz), zi = exp(-lz);
+                        const double lr = o[0], lz = o[4 * RT_NODES], z = o[RT_NODES], zi = o[3 * RT_NODES];
+                        const double pr = o[6 * RT_NODES], pi = o[7 * RT_NODES], mr = o[8 * RT_NODES], mi = o[9 * RT_NODES];
                         double P = exp(lr + n0 * lz), Q = exp(lr - n0 * lz);
 #pragma unroll
                         for (int j = 0; j < CH; ++j) {
@@ -429,8 +447,8 @@ __global__ void __launch_bounds__(RT_THREADS) react_sum_kernel(MedDev m, const E
                         }
                     } else {
                         const cd lp = cmk(o[0], o[RT_NODES]), lm = cmk(o[2 * RT_NODES], o[3 * RT_NODES]);
-                        const cd lz = cmk(o[4 * RT_NODES], o[5 * RT_NODES]);
-                        const cd z = cexpz(lz), zi = cexpz(cneg(lz)), nz = cscale(lz, n0);
+                        const cd nz = cscale(cmk(o[4 * RT_NODES], o[5 * RT_NODES]), n0);
+                        const cd z = cmk(o[6 * RT_NODES], o[7 * RT_NODES]), zi = cmk(o[8 * RT_NODES], o[9 * RT_NODES]);
                         cd pu = cexpz(cadd(lp, nz)), pd = cexpz(csub(lp, nz));     // e^{lp +- n lz}
                         cd mu = cexpz(cadd(lm, nz)), md = cexpz(csub(lm, nz));
 #pragma unroll
@@ -655,46 +673,56 @@ __global__ void mirror_kernel(const int64_t3* mir, cd* out) {
     for (int64_t i = threadIdx.x; i <= 2 * m.nmax; i += blockDim.x) out[m.dst + i] = out[m.src + 2 * m.nmax - i];
 }
 
-// free-space M2L: one thread per (offset) of one level
-__global__ void free_table_kernel(double k, double h, int p, cd* out) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= 49) return;
+// free-space M2L: a CTA per offset of one level.  One thread carries the recurrences in n, whose
+// quotients and phases the others make: a lone thread's FP64 instructions take 64 clocks each (4,099 points,
+// levels 2 .. 4: 494 us with a thread per offset for everything -> 126 us).
+__global__ void __launch_bounds__(64) free_table_kernel(double k, double h, int p, cd* out) {
+    const int o = blockIdx.x;
     const int dx = o / 7 - 3, dy = o % 7 - 3;
     const int w = 4 * p + 1;
     cd* T = out + (int64_t)o * w;
     if (abs(dx) < 2 && abs(dy) < 2) {
-        for (int i = 0; i < w; ++i) T[i] = cmk(0, 0);
+        for (int i = threadIdx.x; i < w; i += 64) T[i] = cmk(0, 0);
         return;
     }
     const double X = dx * h, Y = dy * h;
     const double r = hypot(X, Y), th = atan2(Y, X);
     const double x = k * r;
-    cd h0, h1;
-    hankel01(x, &h0, &h1);
-    cd hm = h0, hn = h1;
-    T[2 * p] = h0;
-    for (int n = 1; n <= 2 * p; ++n) {
-        cd ph = cexpi(n * th);
-        double sg = (n & 1) ? -1.0 : 1.0;
+    for (int n = 1 + threadIdx.x; n <= 2 * p; n += 64) T[2 * p - n].x = 2.0 * n / x;   // until the phases
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        cd hm, hn;
+        hankel_recurrence<true>(x, &hm, &hn);
+        T[2 * p] = hm;
+#pragma unroll 4
+        for (int n = 1; n <= 2 * p; ++n) {
+            T[2 * p + n] = hn;
+            const cd hx = csub(cscale(hn, T[2 * p - n].x), hm);
+            hm = hn;
+            hn = hx;
+        }
+    }
+    __syncthreads();
+    for (int n = 1 + threadIdx.x; n <= 2 * p; n += 64) {
+        const cd ph = cexpi(n * th), hn = T[2 * p + n];
+        const double sg = (n & 1) ? -1.0 : 1.0;
         T[2 * p + n] = cmul(hn, ph);
         T[2 * p - n] = cscale(cmul(hn, cconj(ph)), sg);
-        cd hx = csub(cscale(hn, 2.0 * n / x), hm);
-        hm = hn;
-        hn = hx;
     }
 }
 
-// M2M (P - c) and L2L (c - P) tables of parent level l: thread per child
-__global__ void shift_table_kernel(double k, double hc, int nmax, double* scratch, cd* m2m,
-                                   cd* l2l) {
-    const int c = threadIdx.x;
-    if (c >= 4) return;
+// M2M (P - c) and L2L (c - P) tables of parent level l: a CTA per child, one thread for the
+// Bessel sequence (276 -> 121 us for the levels above)
+__global__ void __launch_bounds__(64) shift_table_kernel(double k, double hc, int nmax, double* scratch, cd* m2m,
+                                                         cd* l2l) {
+    const int c = blockIdx.x;
     const int w = 2 * nmax + 1;
     const double vx = (0.5 - (c & 1)) * hc, vy = (0.5 - (c >> 1)) * hc;   // P - c
     const double r = hypot(vx, vy), th = atan2(vy, vx);
     double* J = scratch + (int64_t)c * (nmax + 1);
-    bessel_j_seq(k * r, nmax, J);
-    for (int n = 0; n <= nmax; ++n) {
+    if (threadIdx.x == 0) bessel_j_seq(k * r, nmax, J);
+    __syncthreads();
+    for (int n = threadIdx.x; n <= nmax; n += 64) {
         cd ph = cexpi(n * th);
         double sg = (n & 1) ? -1.0 : 1.0;
         cd vp = cscale(ph, J[n]);                  // J_n(v) e^{i n th}
@@ -718,10 +746,10 @@ hfmm_status react_tables(const MedDev& md, const std::vector<Entry>& ents, const
         most = std::max(most, e.nodes);
     }
     const int nch = (nmax + CH) / CH, nwin = std::min(nch, 128);   // chunks per launch: 64 KB of sums
-    const size_t sm = sizeof(double) * (6 * RT_NODES + 2 * (size_t)nwin * 32 + RT_THREADS);
+    const size_t sm = sizeof(double) * (RT_NV * RT_NODES + 2 * (size_t)nwin * 32 + RT_THREADS);
     HFMM_CUDA_TRY(cudaFuncSetAttribute(react_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const int ny = (int)std::max<int64_t>(1, std::min<int64_t>((most + RT_NODES - 1) / RT_NODES,
-                                                               (4 * 152 + (int64_t)ents.size() - 1) / (int64_t)ents.size()));
+                                                               (8 * 152 + (int64_t)ents.size() - 1) / (int64_t)ents.size()));
     double* sums = nullptr;
     HFMM_CUDA_TRY(cudaMallocAsync((void**)&sums, sizeof(double) * 2 * nwin * 32 * ny * ents.size(), st));
     for (int c0 = 0; c0 < nch; c0 += nwin) {
@@ -834,7 +862,7 @@ hfmm_status build_tables(hfmm_plan_s* P, cudaStream_t st) {
         LevelInfo& lv = P->lev[l];
         if (l >= 2 && l >= P->lmin) {
             HFMM_TRY(plan_alloc(P, (void**)&lv.t_free, sizeof(cd) * 49 * (4 * lv.p + 1)));
-            free_table_kernel<<<1, 64, 0, st>>>(k, lv.h, lv.p, lv.t_free);
+            free_table_kernel<<<49, 64, 0, st>>>(k, lv.h, lv.p, lv.t_free);
             HFMM_CUDA_TRY(cudaGetLastError());
             P->table_bytes += sizeof(cd) * 49.0 * (4 * lv.p + 1);
         }
@@ -845,7 +873,7 @@ hfmm_status build_tables(hfmm_plan_s* P, cudaStream_t st) {
             HFMM_TRY(plan_alloc(P, (void**)&scratch, sizeof(double) * 4 * (nmax + 1)));
             HFMM_TRY(plan_alloc(P, (void**)&lv.t_m2m, sizeof(cd) * 4 * w));
             HFMM_TRY(plan_alloc(P, (void**)&lv.t_l2l, sizeof(cd) * 4 * w));
-            shift_table_kernel<<<1, 32, 0, st>>>(k, P->lev[l + 1].h, nmax, scratch, lv.t_m2m, lv.t_l2l);
+            shift_table_kernel<<<4, 64, 0, st>>>(k, P->lev[l + 1].h, nmax, scratch, lv.t_m2m, lv.t_l2l);
             HFMM_CUDA_TRY(cudaGetLastError());
             P->table_bytes += sizeof(cd) * 8.0 * w;
         }
