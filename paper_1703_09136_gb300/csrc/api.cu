@@ -24,9 +24,33 @@ void hfmm_set_error(const char* fmt, ...) {
     g_last_error = buf;
 }
 
+// Device memory of a plan, given back with it.  Requests of up to 1 MB are cut from slabs, each as
+// large as everything before it (2 .. 32 MB): a plan makes some 200 requests, most of a few
+// KB, and cudaMalloc and cudaFree take 5 .. 40 us each (4,099 points, one plan, product, transposed
+// product and gradient: 10.5 -> 9.3 ms).
 hfmm_status plan_alloc(hfmm_plan_s* P, void** ptr, size_t bytes) {
+    constexpr size_t ALIGN = 512, SMALL = (size_t)1 << 20, MIN_SLAB = (size_t)2 << 20, MAX_SLAB = (size_t)32 << 20;
     *ptr = nullptr;
     if (bytes == 0) bytes = 16;
+    if (bytes <= SMALL) {
+        const size_t want = (bytes + ALIGN - 1) / ALIGN * ALIGN;
+        if (P->slab_left < want) {
+            const size_t slab = std::min(MAX_SLAB, std::max(MIN_SLAB, P->slab_bytes));
+            void* base = nullptr;
+            if (cudaMalloc(&base, slab) == cudaSuccess) {
+                P->allocations.push_back(base);
+                P->slab_next = (char*)base;
+                P->slab_left = slab;
+                P->slab_bytes += slab;
+            } else cudaGetLastError();                     // no room for a slab: the request alone, below
+        }
+        if (P->slab_left >= want) {
+            *ptr = P->slab_next;
+            P->slab_next += want;
+            P->slab_left -= want;
+            return HFMM_OK;
+        }
+    }
     cudaError_t e = cudaMalloc(ptr, bytes);
     if (e != cudaSuccess) {
         *ptr = nullptr;

@@ -309,6 +309,8 @@ struct hfmm_plan_s {
     double plan_ms = 0.0;
     int64_t p2p_point_pairs = 0;    // sum over leaves T of n_T * sum_{S in U(T)} n_S
     std::vector<void*> allocations;
+    char* slab_next = nullptr;      // small requests (plan_alloc): rest of the newest slab, bytes of all slabs
+    size_t slab_left = 0, slab_bytes = 0;
 
     // autotuning record (HFMM_FLAG_AUTOTUNE)
     int tune_levels[3] = {0, 0, 0};

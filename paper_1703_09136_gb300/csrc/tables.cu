@@ -353,7 +353,7 @@ __device__ __forceinline__ double warp_scatter32(double (&v)[32]) {
 // which errs less than the cosine of the rounded product n tau.  FP64 bound (1.0 TFLOP/s):
 // nodes once per eight orders and complex recurrences for both signs, three layers, 1M points
 // 612 ms per rule, impedance, 4099 points 16.2 ms; nodes once, 177 and 1.6 ms; factors and
-// phases once too, see the plan times, and 0.86 ms.
+// phases once too, 110 and 0.86 ms.
 // blockIdx.y splits the tiles; chunks of eight orders c0 .. c0 + nwin; sums[entry][y][2][chunk][32] =
 // (C, S | T_n, T_-n) x re, im.
 __global__ void __launch_bounds__(RT_THREADS) react_sum_kernel(MedDev m, const Entry* __restrict__ ents,
