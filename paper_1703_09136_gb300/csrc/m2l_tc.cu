@@ -84,7 +84,9 @@ struct TcCfg {
     static constexpr int stages = budget / stage_bytes < 8 ? budget / stage_bytes : 8;
     static_assert(stages >= 2, "ring needs two stages");
     static_assert((2 * stages + 4 + 3) * 8 <= 256, "barrier area fits 256 bytes");
-    static constexpr size_t smem = (size_t)stages * stage_bytes + 256;
+    // the ring, at width 64 rounded up to what the leaf L2P's staging needs (below)
+    static constexpr int area = NB == 64 && stages * stage_bytes < 49664 && 49664 <= budget ? 49664 : stages * stage_bytes;
+    static constexpr size_t smem = (size_t)area + 256;
 };
 constexpr int TC_MAX_NP = 128;         // widest column block (one 128-column TMEM buffer)
 constexpr int TC_RUN_LEVELS = 2;       // finest levels with level-wide scales (the leaves and the level above)
@@ -95,10 +97,14 @@ constexpr int TC_RUN_LEVELS = 2;       // finest levels with level-wide scales (
 // pass computes); used only where the four warps' regions fit the ring.
 template <int NB>
 struct TcL2p {
-    static constexpr int pts = NB == 48 ? 4 : 8;
+    // Four points a pass wherever eight do not fit the ring: else such leaves take a separate L2P
+    // pass that reads the locals back, after a near field that cannot run beside the far field
+    // (three layers, 100,003 points: 33 right-hand sides at nc = 25 1205 -> 983 us; 64 at nc = 31
+    // 1.26 -> 1.01 ms, at nc = 47 1.88 -> 1.74 ms; 20,000 points 0.53 -> 0.37 ms).
+    static constexpr int pts = NB <= 32 || NB == 112 ? 8 : 4;
     static constexpr int buf = pts * (NB / 2) * 8 + pts * 32 * 8;
     static constexpr int warp_bytes = 32 * (NB + 1) * 4 + 2 * buf;
-    static constexpr bool fits = 4 * warp_bytes <= TcCfg<NB>::stages * TcCfg<NB>::stage_bytes;
+    static constexpr bool fits = 4 * warp_bytes <= TcCfg<NB>::area;
 };
 
 bool tc_l2p_fits(int nbw) {
@@ -311,7 +317,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TcCfg<NB>::ctas) m2l_tc_kernel(
     using CFG = TcCfg<NB>;
     constexpr int stage_bytes = CFG::stage_bytes;
     constexpr int TC_STAGES = CFG::stages;
-    uint64_t* full = (uint64_t*)(smem + TC_STAGES * stage_bytes);
+    uint64_t* full = (uint64_t*)(smem + CFG::area);
     uint64_t* empty = full + TC_STAGES;
     uint64_t* dfull = empty + TC_STAGES;
     uint64_t* dfree = dfull + 2;
@@ -420,7 +426,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TcCfg<NB>::ctas) m2l_tc_kernel(
                     // this CTA has completed; one region per warp); the leaf L2P and the
                     // FP32 store read them from there.
                     constexpr int WS = TcL2p<NB>::fits ? TcL2p<NB>::warp_bytes : 32 * (NB + 1) * 4;
-                    static_assert(4 * WS <= TC_STAGES * stage_bytes, "staging fits the ring");
+                    static_assert(4 * WS <= CFG::area, "staging fits the ring");
                     float* bet = (float*)(smem + warp * WS);
 #pragma unroll
                     for (int j = 0; j < NB; ++j) bet[lane * (NB + 1) + j] = acc[j];

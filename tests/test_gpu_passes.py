@@ -1,6 +1,6 @@
 """Fused passes at the sizes where their tiles and splits have edges: position
 gradients and few-right-hand-side mixed applies of leaves with one point, more
-than a warp, more than a CTA and none at all; stored blocks next to coincident
+than a warp, more than a CTA and none at all; the leaves' L2P at every width; stored blocks next to coincident
 points; restarted GMRES at its smallest bases."""
 import numpy as np
 import pytest
@@ -58,6 +58,24 @@ def test_few_rhs_leaf_edges(medium, n, crowd, levels, nrhs):
         assert np.array_equal(np.asarray(host), dev)
         back = plan.adjoint(torch.from_numpy(q).cuda()).cpu().numpy()
         assert direct.rel_l2(back, adj) < MIXED_TOL, direct.rel_l2(back, adj)
+
+
+@pytest.mark.parametrize("p,nrhs", [(7, 5), (13, 33), (15, 64), (17, 65), (23, 33), (25, 5), (31, 64)])
+def test_leaf_l2p_in_the_downward_pass(p, nrhs):
+    """Leaf widths of every staging size (up to 128 columns in the pass, more beside it), ragged right-hand
+    sides, leaves of zero to a dozen points; against the FP64 plan of the same orders."""
+    torch = _torch()
+    from paper_1703_09136_gb300 import MIXED, Plan
+    n, med = 4001, MEDIA["two"]
+    xy = _clustered(n, 0, p)
+    q = W.strengths(1, n, nrhs, salt=p)
+    with Plan(xy, med, tol=1e-6, p=p, levels=5, max_rhs=nrhs) as plan:
+        want = plan.apply(torch.from_numpy(q).cuda()).cpu().numpy()
+    with Plan(xy, med, tol=1e-6, p=p, levels=5, max_rhs=nrhs, precision=MIXED, small_rhs=-1) as plan:
+        columns = 2 * (2 * plan.info["p"][-1] + 1)
+        assert plan.info["leaf_l2p_fused"] == (columns <= 128)      # one column block
+        got = plan.apply(torch.from_numpy(q.astype(np.complex64)).cuda()).cpu().numpy()
+    assert direct.rel_l2(got, want) < MIXED_TOL, direct.rel_l2(got, want)
 
 
 def test_coincident_points_spoil_their_own_targets_only():
