@@ -45,6 +45,7 @@
 #include <vector>
 
 #include "plan.cuh"
+#include "split64.cuh"
 #include "tcgen05.cuh"
 
 namespace {
@@ -269,7 +270,7 @@ __device__ __forceinline__ void tc_store_row(const float (&acc)[NB], int box, in
     if (sdst) {
         // level-wide scale (qmax given): the exponent of the bound 2 max|q_r| qgain
         float m = 0.0f;
-        if (qmax) m = r < nrhs ? 2.0f * __uint_as_float(qmax[r]) * qgain : 0.0f;
+        if (qmax) m = r < nrhs ? 2.0f * __uint_as_float(__ldcg(qmax + r)) * qgain : 0.0f;
         else
 #pragma unroll
             for (int j = 0; j < NB; ++j) m = fmaxf(m, fabsf(acc[j]));
@@ -326,6 +327,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TcCfg<NB>::ctas) m2l_tc_kernel(
     uint32_t* tslot = (uint32_t*)(dfree + 2);
     uint64_t& mdone = *(dfree + 3);
     volatile int& s_abort = *(volatile int*)(dfree + 4);
+    pdl_start_next();
     const TcTile tile = tiles[blockIdx.x];
     const int rc = blockIdx.y;
     const int nbz = Np / NB;
@@ -354,6 +356,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TcCfg<NB>::ctas) m2l_tc_kernel(
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t taddr = *tslot;
+    pdl_wait();                        // everything below reads or writes expansions
     int sbeg = tile.s0, nsteps = tile.s1 - tile.s0;
     if (nseg > 1) {
         const int len = (nsteps + nseg - 1) / nseg;
@@ -377,7 +380,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TcCfg<NB>::ctas) m2l_tc_kernel(
             const float* scs = sec ? psc : asc;
             const int nsb = sec ? nsbp : nsba, sbk = sec ? sbp : sba;
             const float fb = st.kind == 0 ? sfree[st.idx] : st.kind == 1 ? sreact[st.idx] : ssec[st.idx];
-            return scs[(((int64_t)src * nrc + rc) * nsb + st.c0 / sbk) * 64 + rr] * fb;
+            return __ldcg(scs + (((int64_t)src * nrc + rc) * nsb + st.c0 / sbk) * 64 + rr) * fb;
         };
         // one drain per run of steps (a step, or the steps joined by cont); the
         // run's factor is that of any of its steps with a source for this row
@@ -613,6 +616,8 @@ __global__ void tc_reduce_kernel(const TcTile* __restrict__ tiles, int ntiles, i
                                  __half* __restrict__ sdst, float* __restrict__ ssc, int kcd,
                                  const unsigned* __restrict__ qmax, float qgain) {
     constexpr int NQ = NB / 4;
+    pdl_start_next();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nwarp = (int64_t)ntiles * nrcl * nbz * 128;
     const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -630,8 +635,8 @@ __global__ void tc_reduce_kernel(const TcTile* __restrict__ tiles, int ntiles, i
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (jq < NQ)
             for (int sg = 0; sg < nseg; ++sg) {
-                const float4 w = *(const float4*)(part + ((((int64_t)sg * ntiles + t) * nrcl + rc) * nbz + cb) * 128 * NB +
-                                                  (int64_t)row * NB + 4 * jq);
+                const float4 w = __ldcg((const float4*)(part + ((((int64_t)sg * ntiles + t) * nrcl + rc) * nbz + cb) * 128 * NB +
+                                                        (int64_t)row * NB + 4 * jq));
                 v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
             }
         const float a4[4] = {v.x, v.y, v.z, v.w};
@@ -648,7 +653,7 @@ __global__ void tc_reduce_kernel(const TcTile* __restrict__ tiles, int ntiles, i
         if (sdst) {
             float m = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
             for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (qmax) m = r < nrhs ? 2.0f * __uint_as_float(qmax[r]) * qgain : 0.0f;   // level-wide scale
+            if (qmax) m = r < nrhs ? 2.0f * __uint_as_float(__ldcg(qmax + r)) * qgain : 0.0f;   // level-wide scale
             const int e = f16_exp(m);
             if (lane == 0) ssc[(((int64_t)box * nrc + rc) * nbz + cb) * 64 + rr] = pow2f(-e);
             if (jq < NQ && (g0 >> 4) < kcd) {
@@ -786,18 +791,25 @@ hfmm_status launch_nb(hfmm_plan_s* P, const TcLaunch& a, int nrhs, cudaStream_t 
     const int nseg = tc_nseg(a.ntiles, a.nb, nrc, a.maxsteps);
     float* part = nseg > 1 ? P->tc_part : nullptr;
     dim3 grid((unsigned)a.ntiles, (unsigned)nrcl, (unsigned)(a.nb * nseg));
-    m2l_tc_kernel<NB><<<grid, TC2_THREADS, smem, st>>>(
-        (const TcTile*)a.tiles, (const TcStep*)a.steps, a.Bfree, a.Breact, a.Bsec, a.sfree, a.sreact, a.ssec, a.amma,
+    // Early starts (split64.cuh) where the launch is at most about a wave: its prologue (barriers, TMEM) then
+    // hides behind the launch before it.  CTAs of a larger one would wait in places that the near
+    // field can use, and from 2^16 leaves on the near field lasts for the whole far field (three
+    // layers, 64 right-hand sides, 1M points: 6.78 -> 6.97 ms with all launches, 6.80 with the small
+    // ones; 100,003 points, 33: 983 -> 966 us; 20,000 points, 64: 0.37 -> 0.34 ms; 262,144
+    // points, 16: 4.23 -> 4.19 ms).
+    const bool early = !P->in_batch && !a.l2p && P->lev[P->L].nbox < (1 << 16) &&
+                       (int64_t)grid.x * grid.y * grid.z <= 4 * 152;
+    HFMM_CUDA_TRY(pdl_launch_if(
+        early, m2l_tc_kernel<NB>, grid, dim3(TC2_THREADS), smem, st, 0, (const TcTile*)a.tiles, (const TcStep*)a.steps, a.Bfree, a.Breact, a.Bsec, a.sfree, a.sreact, a.ssec, a.amma,
         a.asc, a.nsba, a.sba, a.pmma, a.psc, a.nsbp, a.sbp, P->tc_zero, a.out, nrhs, a.nc, a.kc, a.kc2, nrc, a.np,
         a.sdst, a.ssc, a.kcd, nseg, part, a.l2p ? P->basis32 : nullptr, P->leaf_begin, P->y32, P->tc_spin, P->tc_err,
-        a.qmax, a.qgain);
-    HFMM_CUDA_TRY(cudaGetLastError());
+        a.qmax, a.qgain));
     if (part) {
         const int64_t warps = a.ntiles * nrcl * a.nb * 128;
         const unsigned blocks = (unsigned)std::min<int64_t>((warps + 7) / 8, 8 * 152);
-        tc_reduce_kernel<NB><<<blocks, 256, 0, st>>>((const TcTile*)a.tiles, (int)a.ntiles, nrcl, a.nb, nseg, part,
-                                                      a.out, nrhs, a.nc, nrc, a.sdst, a.ssc, a.kcd, a.qmax, a.qgain);
-        HFMM_CUDA_TRY(cudaGetLastError());
+        HFMM_CUDA_TRY(pdl_launch_if(early, tc_reduce_kernel<NB>, dim3(blocks), dim3(256), 0, st, 0,
+                                    (const TcTile*)a.tiles, (int)a.ntiles, nrcl, a.nb, nseg, part, a.out, nrhs, a.nc, nrc,
+                                    a.sdst, a.ssc, a.kcd, a.qmax, a.qgain));
         ++P->launches;
     }
     return HFMM_OK;
