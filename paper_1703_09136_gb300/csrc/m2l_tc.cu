@@ -270,7 +270,7 @@ __device__ __forceinline__ void tc_store_row(const float (&acc)[NB], int box, in
     if (sdst) {
         // level-wide scale (qmax given): the exponent of the bound 2 max|q_r| qgain
         float m = 0.0f;
-        if (qmax) m = r < nrhs ? 2.0f * __uint_as_float(__ldcg(qmax + r)) * qgain : 0.0f;
+        if (qmax) m = r < nrhs ? 2.0f * __uint_as_float(qmax[r]) * qgain : 0.0f;
         else
 #pragma unroll
             for (int j = 0; j < NB; ++j) m = fmaxf(m, fabsf(acc[j]));
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(TC2_THREADS, TcCfg<NB>::ctas) m2l_tc_kernel(
             const float* scs = sec ? psc : asc;
             const int nsb = sec ? nsbp : nsba, sbk = sec ? sbp : sba;
             const float fb = st.kind == 0 ? sfree[st.idx] : st.kind == 1 ? sreact[st.idx] : ssec[st.idx];
-            return __ldcg(scs + (((int64_t)src * nrc + rc) * nsb + st.c0 / sbk) * 64 + rr) * fb;
+            return scs[(((int64_t)src * nrc + rc) * nsb + st.c0 / sbk) * 64 + rr] * fb;
         };
         // one drain per run of steps (a step, or the steps joined by cont); the
         // run's factor is that of any of its steps with a source for this row
@@ -635,6 +635,7 @@ __global__ void tc_reduce_kernel(const TcTile* __restrict__ tiles, int ntiles, i
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (jq < NQ)
             for (int sg = 0; sg < nseg; ++sg) {
+                // (the level above's sums lay at the same place: not from L1)
                 const float4 w = __ldcg((const float4*)(part + ((((int64_t)sg * ntiles + t) * nrcl + rc) * nbz + cb) * 128 * NB +
                                                         (int64_t)row * NB + 4 * jq));
                 v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
