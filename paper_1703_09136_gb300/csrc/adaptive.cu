@@ -1277,14 +1277,22 @@ hfmm_status apply_adaptive64(hfmm_plan_s* P, int nrhs, int parts, bool conj_out,
     const double MAC = 8.0 * nrhs;
     const bool far = (parts & (HFMM_PART_FAR_FREE | HFMM_PART_FAR_REACT)) != 0;
     const bool near = (parts & HFMM_PART_NEAR_FREE) != 0, near_here = near && P->near64_vals;
+    const bool direct = (parts & HFMM_PART_NEAR_REACT) && P->nd > 0, m2p = (parts & HFMM_PART_FAR_FREE) != 0;
+    const bool aside = far && near_here;
+    cudaStream_t fs = st;
+    if (aside) {
+        HFMM_TRY(fork_near64(P, nrhs, direct, st, &fs));
+        tm.st = fs;
+    }
     if (far) {
         tm.begin(HFMM_STAGE_P2M);
-        HFMM_TRY(split_begin(P, 0, st));
-        HFMM_TRY(launch_p2m64(P, nrhs, st));
+        HFMM_TRY(split_begin(P, 0, fs));
+        HFMM_TRY(launch_p2m64(P, nrhs, fs));
         tm.end(HFMM_STAGE_P2M);
-        HFMM_TRY(ad_tree_pass<cd>(P, 0, nrhs, parts, P->q_sorted, 1, n, T->p2l64, tm, st));
+        HFMM_TRY(ad_tree_pass<cd>(P, 0, nrhs, parts, P->q_sorted, 1, n, T->p2l64, tm, fs));
     }
-    tm.begin(HFMM_STAGE_P2P);
+    if (aside) HFMM_TRY(join_near64(P, nrhs, m2p, conj_out, y, fs, st));
+    else tm.begin(HFMM_STAGE_P2P);
     if (near && !near_here) {                             // coincident points: H0 per pair
         HFMM_CUDA_TRY(cudaMemsetAsync(P->y_sorted, 0, sizeof(cd) * n * nrhs, st));
         ad_near_kernel<<<(unsigned)ceil_div((int64_t)T->leaves.size(), 4), 128, 0, st>>>(
@@ -1293,10 +1301,11 @@ hfmm_status apply_adaptive64(hfmm_plan_s* P, int nrhs, int parts, bool conj_out,
         ++P->launches;
         HFMM_CUDA_TRY(cudaGetLastError());
     }
-    HFMM_TRY(launch_leaf64(P, nrhs, near_here, far, (parts & HFMM_PART_FAR_FREE) != 0,
-                           (parts & HFMM_PART_NEAR_REACT) && P->nd > 0, near && !near_here ? P->y_sorted : nullptr,
-                           conj_out, y, st));
-    tm.end(HFMM_STAGE_P2P);
+    if (!aside) {
+        HFMM_TRY(launch_leaf64(P, nrhs, near_here, far, m2p, direct, near && !near_here ? P->y_sorted : nullptr, conj_out, y,
+                               st));
+        tm.end(HFMM_STAGE_P2P);
+    }
     if (parts & (HFMM_PART_NEAR_FREE | HFMM_PART_NEAR_REACT)) {
         P->st_flops[HFMM_STAGE_P2P] = MAC * (double)P->p2p_point_pairs;
         P->st_flops[HFMM_STAGE_DIRECT] = MAC * (double)P->nd_vals;

@@ -400,6 +400,7 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
     const int L = P->L;
     const int nb = ceil_div(n, 256);
     StageTimer tm{P, st};
+    cudaStream_t fs = st;                 // the far field's stream
     P->launches = 0;
     for (int s = 0; s < HFMM_NUM_STAGES; ++s) { P->st_flops[s] = 0.0; P->st_bytes[s] = 0.0; P->ev_used[s] = false; }
     const double C = 16.0 * nrhs;      // bytes of one complex128 value per right-hand side
@@ -415,6 +416,12 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
     if (extra) HFMM_CUDA_TRY(cudaMemsetAsync(P->y_sorted, 0, sizeof(cd) * n * nrhs, st));
     tm.end(HFMM_STAGE_GATHER);
     P->st_bytes[HFMM_STAGE_GATHER] = 2.0 * C * n + 8.0 * n;
+    const bool direct = (parts & HFMM_PART_NEAR_REACT) && P->nd > 0;
+    const bool aside = !P->ad && l2p_here && near_here;
+    if (aside) {
+        HFMM_TRY(fork_near64(P, nrhs, direct, st, &fs));
+        tm.st = fs;
+    }
     if (ad_fast) HFMM_TRY(apply_adaptive64(P, nrhs, parts, adjoint, y, st));
     else if (P->ad) HFMM_TRY(apply_adaptive(P, nrhs, parts, st));
     else {
@@ -423,13 +430,13 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
             {
                 LevelInfo& lv = P->lev[L];
                 tm.begin(HFMM_STAGE_P2M);
-                HFMM_TRY(leaves64(P, nrhs, st));
+                HFMM_TRY(leaves64(P, nrhs, fs));
                 tm.end(HFMM_STAGE_P2M);
                 P->st_flops[HFMM_STAGE_P2M] = MAC * n * lv.ncoef;
                 P->st_bytes[HFMM_STAGE_P2M] = C * n + 16.0 * n + C * lv.nbox * lv.ncoef;
             }
             tm.begin(HFMM_STAGE_M2M);
-            HFMM_TRY(upward64(P, nrhs, st));
+            HFMM_TRY(upward64(P, nrhs, fs));
             for (int l = L - 1; l >= P->lmin; --l) {
                 const LevelInfo& lv = P->lev[l];
                 P->st_flops[HFMM_STAGE_M2M] += MAC * 4.0 * lv.nbox * lv.ncoef * P->lev[l + 1].ncoef;
@@ -438,7 +445,7 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
             tm.end(HFMM_STAGE_M2M);
             // step 3: downward pass
             tm.begin(HFMM_STAGE_DOWN);
-            HFMM_TRY(downward64(P, nrhs, parts, st));
+            HFMM_TRY(downward64(P, nrhs, parts, fs));
             for (int l = P->lmin; l <= L; ++l) {
                 const LevelInfo& lv = P->lev[l];
                 const bool has_parent = l > P->lmin, dg = lv.diag_logq > 0;
@@ -470,16 +477,19 @@ hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, 
             }
         }
         // step 5: direct interactions
-        const bool direct = (parts & HFMM_PART_NEAR_REACT) && P->nd > 0;
-        tm.begin(HFMM_STAGE_P2P);
-        if (near && !near_here) {
-            p2p_kernel<<<(unsigned)P->lev[L].nbox, P2P_THREADS, 0, st>>>(P->leaf_begin, L, P->xy_sorted, P->q_sorted, n,
-                                                                         nrhs, P->k, P->y_sorted);
-            ++P->launches;
-            HFMM_CUDA_TRY(cudaGetLastError());
+        if (aside) {
+            HFMM_TRY(join_near64(P, nrhs, false, adjoint, y, fs, st));
+        } else {
+            tm.begin(HFMM_STAGE_P2P);
+            if (near && !near_here) {
+                p2p_kernel<<<(unsigned)P->lev[L].nbox, P2P_THREADS, 0, st>>>(P->leaf_begin, L, P->xy_sorted, P->q_sorted, n,
+                                                                             nrhs, P->k, P->y_sorted);
+                ++P->launches;
+                HFMM_CUDA_TRY(cudaGetLastError());
+            }
+            HFMM_TRY(launch_leaf64(P, nrhs, near_here, l2p_here, false, direct, extra ? P->y_sorted : nullptr, adjoint, y, st));
+            tm.end(HFMM_STAGE_P2P);
         }
-        HFMM_TRY(launch_leaf64(P, nrhs, near_here, l2p_here, false, direct, extra ? P->y_sorted : nullptr, adjoint, y, st));
-        tm.end(HFMM_STAGE_P2P);
         if (near) {
             P->st_flops[HFMM_STAGE_P2P] = MAC * (double)P->p2p_point_pairs;
             P->st_bytes[HFMM_STAGE_P2P] = C * n + 2.0 * C * n + 16.0 * n +

@@ -157,7 +157,7 @@ struct Leaf64Args {
     const Leaf64D* d;                // directly summed reaction
     const cd* dvals;
     const cd* ys;                    // sums made by other kernels (null: none)
-    const int64_t* perm;
+    const int64_t* perm;             // null: sorted order
     bool conj_out;
     cd* y;
 };
@@ -428,8 +428,8 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
             const int64_t i = tlo + (t < 2 ? i0 : i1);
             if (ns > 0) x += fma((double)a, 4294967296.0, (double)bsum) * pow2d(EV);
             if (bad) x = __longlong_as_double(0x7ff8000000000000ll);
-            if (A.ys) x += reinterpret_cast<const double*>(A.ys + (int64_t)r * A.n + i)[t & 1];
-            reinterpret_cast<double*>(A.y + (int64_t)r * A.n + A.perm[i])[t & 1] = (A.conj_out && (t & 1)) ? -x : x;
+            if (A.ys) x += __ldcg(reinterpret_cast<const double*>(A.ys + (int64_t)r * A.n + i) + (t & 1));
+            reinterpret_cast<double*>(A.y + (int64_t)r * A.n + (A.perm ? A.perm[i] : i))[t & 1] = (A.conj_out && (t & 1)) ? -x : x;
         }
         t0 += tp;
     }
@@ -742,11 +742,37 @@ hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
     return HFMM_OK;
 }
 
-// Everything at the targets, into the caller's order: near = the stored blocks,
-// l2p = the leaves' locals, m2p = the W lists, direct = the reaction blocks, ys =
-// other sums.
+// Near field and direct reaction into y_sorted on the near stream, beside the far field (whose
+// stream this returns in *fs): they need the strengths alone, and a tree pass leaves SMs idle
+// at its coarse levels (1600 points 138 -> 114 us an apply, two layers, 262,144 points 1528 -> 1461,
+// an adaptive tree of 20,011 points 582 -> 559).
+hfmm_status fork_near64(hfmm_plan_s* P, int nrhs, bool direct, cudaStream_t st, cudaStream_t* fs) {
+    HFMM_TRY(fork_near_far(P, st));
+    StageTimer tn{P, P->near_st};
+    tn.begin(HFMM_STAGE_P2P);
+    HFMM_TRY(launch_leaf64(P, nrhs, true, false, false, direct, nullptr, false, P->y_sorted, P->near_st, true));
+    tn.end(HFMM_STAGE_P2P);
+    HFMM_CUDA_TRY(cudaEventRecord(P->ev_near_done, P->near_st));
+    *fs = P->far_st;
+    return HFMM_OK;
+}
+
+// The last pass: the locals' (and W lists') part on fs plus the near stream's sums; joins back into st.
+hfmm_status join_near64(hfmm_plan_s* P, int nrhs, bool m2p, bool conj_out, cd* y, cudaStream_t fs, cudaStream_t st) {
+    StageTimer tf{P, fs};
+    HFMM_CUDA_TRY(cudaStreamWaitEvent(fs, P->ev_near_done, 0));
+    tf.begin(HFMM_STAGE_L2P);
+    HFMM_TRY(launch_leaf64(P, nrhs, false, true, m2p, false, P->y_sorted, conj_out, y, fs, false));
+    tf.end(HFMM_STAGE_L2P);
+    HFMM_CUDA_TRY(cudaEventRecord(P->ev_far_done, fs));
+    HFMM_CUDA_TRY(cudaStreamWaitEvent(st, P->ev_far_done, 0));
+    return HFMM_OK;
+}
+
+// Everything at the targets, into the caller's order (sorted: the plan's, into y): near = the stored
+// blocks, l2p = the leaves' locals, m2p = the W lists, direct = the reaction blocks, ys = other sums.
 hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2p, bool direct, const cd* ys,
-                          bool conj_out, cd* y, cudaStream_t st) {
+                          bool conj_out, cd* y, cudaStream_t st, bool sorted) {
     Leaf64Args A{};
     A.recs = P->leaf64;
     A.nrhs = nrhs;
@@ -765,7 +791,7 @@ hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2
     A.d = P->leaf64_d;
     A.dvals = P->d_vals;
     A.ys = ys;
-    A.perm = P->perm;
+    A.perm = sorted ? nullptr : P->perm;
     A.conj_out = conj_out;
     A.y = y;
     // one warp per leaf from 16 of them per SM on (leaves of at most four tiles), else four

@@ -401,7 +401,9 @@ hfmm_status launch_grad_far(hfmm_plan_s* P, int nrhs, const cd* v, double2* acc,
                             cudaStream_t st);
 hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st);
 hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2p, bool direct, const cd* ys,
-                          bool conj_out, cd* y, cudaStream_t st);
+                          bool conj_out, cd* y, cudaStream_t st, bool sorted = false);
+hfmm_status fork_near64(hfmm_plan_s* P, int nrhs, bool direct, cudaStream_t st, cudaStream_t* fs);
+hfmm_status join_near64(hfmm_plan_s* P, int nrhs, bool m2p, bool conj_out, cd* y, cudaStream_t fs, cudaStream_t st);
 hfmm_status build_near64_grad(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, bool adjoint,
                        cudaStream_t st);
