@@ -76,7 +76,8 @@ typedef enum {
 } hfmm_medium_kind;
 
 typedef enum {
-    HFMM_FP64 = 0,              /* complex128 in/out, FP64 arithmetic everywhere */
+    HFMM_FP64 = 0,              /* complex128 in/out, FP64 accuracy throughout (translations and
+                                   stored near field as error-free digit products) */
     HFMM_MIXED = 1              /* complex64 in/out, FP32 P2P/P2M/L2P, tensor-core M2L */
 } hfmm_precision;
 
