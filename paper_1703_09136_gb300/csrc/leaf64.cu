@@ -1,7 +1,8 @@
 // FP64 leaf passes: P2M from plan-time bases, and one kernel for everything a
-// target sums at the end (near field, L2P, an adaptive tree's M2P, directly
-// summed reaction, result in the caller's order).  Every non-empty leaf has a
-// record (Leaf64Rec) with its ranges, so both trees run the same kernels.
+// target sums (near field, L2P, an adaptive tree's M2P, directly summed reaction,
+// result in the caller's order), launched twice where both fields are wanted: near
+// field and reaction beside the tree pass, the rest after it.  Every non-empty leaf has
+// a record (Leaf64Rec) with its ranges, so both trees run the same kernels.
 //
 // Bases.  B_m(x) = J_m(k rho) e^{-i m theta} of every point about its leaf's centre,
 // m = 0 .. p + 1, is computed once per plan: J_{-m} = (-1)^m J_m makes the
