@@ -144,9 +144,11 @@ __global__ void s6_op_slice_kernel(S6Op o, const int* __restrict__ Ep, uint4* __
 // ---------------------------------------------------------------------------
 // level exponents of expansions written by other kernels
 // ---------------------------------------------------------------------------
+// Boxes without points (lb: the leaf ranges of a uniform tree, null: every box has some) are left out: nobody
+// writes their locals, so their memory holds what the allocator or a call of another width left there.
 template <class C>
-__global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
-                                   int sign, int* __restrict__ E) {
+__global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nrhs, int p, const int32_t* __restrict__ lb,
+                                   int L, int l, const int* __restrict__ sx, int sign, int* __restrict__ E) {
     pdl_start_next();
     const int nc = 2 * p + 1, r = blockIdx.y;
     int e = S6_NONE;
@@ -155,6 +157,11 @@ __global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nr
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / nc;
         const int m = (int)(i % nc) - p;
+        if (lb) {
+            int32_t lo, hi;
+            box_range(lb, L, l, b, &lo, &hi);
+            if (hi <= lo) continue;
+        }
         const C v = __ldcg(a + (b * nrhs + r) * nc + m + p);
         const int sh = sx ? sign * sx[abs(m)] : 0;
         e = max(e, max(s6_exponent(v.x, sh), s6_exponent(v.y, sh)));
@@ -835,8 +842,8 @@ hfmm_status s6_exponent_of(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream
     const int64_t total = lv.nbox * lv.ncoef;
     HFMM_CUDA_TRY(pdl_launch(s6_exponent_kernel<typename S6Traits<D>::C>,
                              dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs), dim3(256), 0, st, 0,
-                             s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, s6_lev<D>(lv).sx, loc ? 1 : -1,
-                             split_exp(P, D == 6 ? 0 : 1, l, loc)));
+                             s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, P->ad ? nullptr : P->leaf_begin, P->L, l,
+                             s6_lev<D>(lv).sx, loc ? 1 : -1, split_exp(P, D == 6 ? 0 : 1, l, loc)));
     ++P->launches;
     return HFMM_OK;
 }
