@@ -3,16 +3,21 @@
 //
 // Every translation is a real matrix-vector product of length 2 nc (interleaved
 // real and imaginary parts).  The operand and the operator are written as
-// fixed-point numbers of 53 bits and cut into six signed base-512 digits,
-//     x = 2^(E - 53) sum_i d_i 512^(5 - i),  |d_i| <= 256,
-// (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms
-// 59, 2012): a digit is an f16 number, a digit product is below 2^16, and a sum
-// of up to four of them over 64 terms stays within 2^24, so f16 x f16 -> FP32
-// mma.sync accumulates them without rounding.  The 21 digit products
-// with i + j <= 5 are summed per order i + j: orders 0 .. 3 leave the tensor
-// core every 64 terms as integers (int32, over all sources of a target), the two
-// lowest orders stay in FP32 (their rounding is below 2^-60 of the largest
-// term).  What is dropped (orders >= 6) is below the FP64 rounding of the row.
+// fixed-point numbers of 53 and 52 bits and cut into six signed base-512 digits,
+//     x = 2^(E - 53) sum_i d_i 512^(5 - i),  |d_i| <= 256
+// (the splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms
+// 59, 2012): a digit is an f16 number, a digit product is at most 2^16, and sums
+// below 2^24 leave f16 x f16 -> FP32 mma.sync without rounding.  The 26 digit
+// products with i + j <= 6 are summed per order i + j.  Orders 0 .. 4 leave the
+// tensor core every 64 terms as integers (int32, over all sources of a target): orders 0 .. 3
+// stay within 2^24 there; order 4, five products a term, passes it only where the mean product is above
+// 0.8 of the largest possible one.  Orders 5 and 6 stay in FP32: their sums are exact up to 2^24
+// (28 sources at order 45: 2^23.5), and at the worst, all digits of a tile at their limit with one sign, an
+// addition rounds by 2^-53 of the largest term, where an FP64 dot product rounds by 2^-53 of the whole sum so far.
+// Orders >= 7 are dropped.  Error of a target's free-space list against extended precision, of the field at
+// its points, k h = 0.01 .. 25, orders 9 .. 45, sources of one size and of a million sizes:
+// 0.2 .. 1.5e-15, FP64 multiply-adds 0.3 .. 3.6e-15, all 36 products the same as 26 to two
+// digits.  Without order 6 (21 products) it is 1.6e-15 .. 2.7e-14.
 //
 // Scaling: expansions are scaled by powers of two close to
 // s_l(n) = min(1, (k R_l / 2)^n / n!) (a~_n = a_n / s, b~_n = b_n s), which makes
@@ -23,11 +28,11 @@
 // that holds an infinity or a NaN makes every output of that right-hand side NaN.
 //
 // FP32 (the mixed path's expansions, already scaled by s): three digits hold 26
-// bits, six products (i + j <= 2) replace the 21, orders 0 and 1 are kept as
+// bits, six products (i + j <= 2) replace the 26, orders 0 and 1 are kept as
 // integers and order 2 in FP32.
 //
 // What bounds it: GB300's FP64 pipe runs at 1.0 TFLOP/s (a warp-wide FMA every 16
-// clocks per SM), mma.sync f16 at 600 TFLOP/s: 21 products leave 28 TFLOP/s.
+// clocks per SM), mma.sync f16 at 600 TFLOP/s: 26 products leave 23 TFLOP/s.
 // Measured (one GB300, two layers, 262,144 points, one right-hand side): leaf
 // level (order 15, 430k free-space and 49k reaction translations, 3.8 GFLOP)
 // 5.73 -> 0.43 ms, all levels 12.0 -> 1.03 ms, M2M 0.72 -> 0.13 ms; the result
@@ -45,17 +50,17 @@ namespace {
 constexpr int S6_MAXW = 6;               // m-tiles (warps) per CTA
 constexpr double S6_MAX_BYTES = 16e9;    // operator slices of one plan, and its expansions' digits
 
-// D digits; orders 0 .. NI - 1 are summed as integers, the others in FP32
+// D digits; products of orders 0 .. NO - 1 are kept, orders 0 .. NI - 1 summed as integers, the others in FP32
 template <int D> struct S6Traits;
 template <> struct S6Traits<6> {
     using C = cd;
     using R = double;
-    static constexpr int NI = 4;
+    static constexpr int NO = 7, NI = 5;
 };
 template <> struct S6Traits<3> {
     using C = cf;
     using R = float;
-    static constexpr int NI = 2;
+    static constexpr int NO = 3, NI = 2;
 };
 
 // ---------------------------------------------------------------------------
@@ -315,7 +320,7 @@ __device__ __forceinline__ bool s6_step(const S6Args& A, const S6Tile& T, int s,
 template <int NT, int D>
 __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168)) s6_kernel(const __grid_constant__ S6Args A) {
     using R = typename S6Traits<D>::R;
-    constexpr int NI = S6Traits<D>::NI;
+    constexpr int NO = S6Traits<D>::NO, NI = S6Traits<D>::NI;
     // digits of the sources of one 64-term chunk, in B-fragment order, two buffers
     __shared__ __align__(16) uint2 Bs[2][D][4][NT][32];
     pdl_start_next();
@@ -360,7 +365,7 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
     const int nis = A.shift.dig ? 2 * A.shift.p + 1 : 0, nil = A.list.dig ? 2 * A.list.p + 1 : 0;
     const int KSs = (2 * nis + 15) / 16, KSl = (2 * nil + 15) / 16;
 
-    float acc[NT][D][4];
+    float acc[NT][NO][4];
     int iacc[NT][NI][4];
     double dacc[NT][4];
 #pragma unroll
@@ -371,12 +376,13 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
 #pragma unroll
             for (int o = 0; o < NI; ++o) iacc[t][o][v] = 0;
 #pragma unroll
-            for (int o = 0; o < D; ++o) acc[t][o][v] = 0.0f;
+            for (int o = 0; o < NO; ++o) acc[t][o][v] = 0.0f;
         }
     int since = 0;                    // chunks since the integers were last folded
     // dacc += (digit sums) 2^E, E = Esrc + Eop - (18 D - 3): order o weighs 512^(2 (D - 1) - o).
     // Four (two) FP64 instructions a value (the pipe takes 64 clocks for each of a
-    // sub-partition's): orders 0 .. 2 and 3 .. 5 as integers below 2^51
+    // sub-partition's): orders 0 .. 2 and 3 .. 6 as integers below 2^51 (order 6 rounded to order 5's unit, 2^-61
+    // of the largest term)
     auto fold = [&](int E) {
         const double chi = pow2d(E + 9 * (2 * D - 4)), clo = D == 6 ? pow2d(E + 45) : 0.0;
 #pragma unroll
@@ -385,16 +391,16 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
             for (int v = 0; v < 4; ++v) {
                 long long hi = ((long long)iacc[t][0][v] << 18) + ((long long)iacc[t][1][v] << 9);
                 if (D == 6) {
-                    hi += iacc[t][NI - 2][v];
-                    const long long lo = ((long long)iacc[t][NI - 1][v] << 18) + (__float2ll_rn(acc[t][D - 2][v]) << 9) +
-                                         __float2ll_rn(acc[t][D - 1][v]);
+                    hi += iacc[t][2][v];
+                    const long long lo = ((long long)iacc[t][NI - 2][v] << 18) + ((long long)iacc[t][NI - 1][v] << 9) +
+                                         __float2ll_rn(fmaf(acc[t][NO - 1][v], 0x1p-9f, acc[t][NO - 2][v]));
                     dacc[t][v] = fma(int51d(lo), clo, dacc[t][v]);
                 } else hi += __float2ll_rn(acc[t][D - 1][v]);
                 dacc[t][v] = fma(int51d(hi), chi, dacc[t][v]);
 #pragma unroll
                 for (int o = 0; o < NI; ++o) iacc[t][o][v] = 0;
 #pragma unroll
-                for (int o = NI; o < D; ++o) acc[t][o][v] = 0.0f;
+                for (int o = NI; o < NO; ++o) acc[t][o][v] = 0.0f;
             }
         since = 0;
     };
@@ -519,7 +525,7 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
 #pragma unroll
                             for (int i = 0; i < D; ++i)
 #pragma unroll
-                                for (int j = 0; j < D - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
+                                for (int j = 0; j < D && j < NO - i; ++j) s6_mma(acc[t][i + j], a[i], bb[j]);
                         }
                     }
             load_op(cur, 2 * h, more);
@@ -532,7 +538,7 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
                 for (int o = 0; o < NI; ++o)
 #pragma unroll
                     for (int x = 0; x < 4; ++x) iacc[t][o][x] += __float2int_rn(acc[t][o][x]);
-            if (++since == 120) fold(Ef[fam]);            // 120 x 2^24 < 2^31
+            if (++since == 96) fold(Ef[fam]);             // 96 x 5 x 2^22 < 2^31
         }
         prev_fam = fam;
         buf ^= 1;
