@@ -92,4 +92,13 @@ void hfmm_set_error(const char* fmt, ...);
         if (_s != HFMM_OK) return _s;          \
     } while (0)
 
+// Dynamic shared memory above the default 48 KB for a launch of sm bytes beside at most static_bytes of static
+// ones.  The limit belongs to the kernel, not to the launch: every launch sets the same one (all that a CTA can have),
+// since another host thread may launch the kernel for another plan between this call and the launch.
+template <class K>
+inline cudaError_t smem_limit(K* kernel, size_t sm, int static_bytes = 1024) {
+    if (sm + static_bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - static_bytes);
+}
+
 static inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }

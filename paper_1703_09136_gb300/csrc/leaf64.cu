@@ -801,8 +801,7 @@ hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2
     const size_t sm = sizeof(double) * (128 * W * LD / 2 + (one ? 0 : W * 96) + W * LF_RING * 256 +
                                         (l2p ? 4 * (size_t)(A.p + 1) : 0));
     auto kernel = one ? leaf64_kernel<1> : leaf64_kernel<4>;
-    if (sm > 47 * 1024)                                    // (static shared memory beside it)
-        HFMM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HFMM_CUDA_TRY(smem_limit(kernel, sm));
     HFMM_CUDA_TRY(pdl_launch(kernel, dim3((unsigned)P->leaf64_n, (unsigned)nrhs), dim3(W * 32), sm, st, 0, A));
     ++P->launches;
     return HFMM_OK;

@@ -1160,7 +1160,7 @@ hfmm_status launch_down_ru(hfmm_plan_s* P, int l, int nrhs, int parts, int nchun
     const bool has_parent = l > P->lmin;
     const size_t sm = smem_bytes(R, U, ncs_max);
     auto kern = down_small_kernel<R, U>;
-    HFMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HFMM_CUDA_TRY(smem_limit(kern, sm));
     HFMM_CUDA_TRY(pdl_launch_if(
         !P->in_batch, kern, dim3((unsigned)(lv.nbox * nchunk)), dim3(SM_W * 32), sm, st, 0, P->leaf_begin, P->L, l, P->lmin, nrhs, lv.p,
         has_parent ? P->lev[l - 1].p : 0, has_parent ? P->lev[l - 1].loc32 : nullptr,
@@ -1175,7 +1175,7 @@ hfmm_status launch_m2m_ru(hfmm_plan_s* P, int l, int nrhs, int nchunk, int ncs_m
     LevelInfo& lv = P->lev[l];
     const size_t sm = smem_bytes(R, U, ncs_max);
     auto kern = m2m_small_kernel<R, U>;
-    HFMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HFMM_CUDA_TRY(smem_limit(kern, sm));
     HFMM_CUDA_TRY(pdl_launch_if(!P->in_batch, kern, dim3((unsigned)(lv.nbox * nchunk)), dim3(SM_W * 32), sm, st, 0, P->leaf_begin, P->L, l,
                              P->lev[l + 1].mult32, lv.t_m2m32, P->lev[l + 1].p, lv.p, nrhs, nchunk, ncs_max, lv.mult32));
     return HFMM_OK;
@@ -1277,7 +1277,7 @@ hfmm_status launch_react_u(hfmm_plan_s* P, int l, int nrhs, int parts, int nchun
     LevelInfo& lv = P->lev[l];
     const size_t sm = sizeof(cf) * ((size_t)NW * ncs_max + (size_t)NW * U * 32);
     auto kern = down_small_kernel<1, U, NW>;
-    HFMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HFMM_CUDA_TRY(smem_limit(kern, sm));
     if (lv.n_rtgt == 0) return HFMM_OK;
     kern<<<(unsigned)(lv.n_rtgt * nchunk), NW * 32, sm, st>>>(
         P->leaf_begin, P->L, l, P->lmin, nrhs, lv.p, 0, nullptr, nullptr, lv.mult32, nullptr, lv.v_src, lv.v_off,
@@ -1325,7 +1325,7 @@ hfmm_status small_down(hfmm_plan_s* P, int l, int nrhs, int parts, bool react_do
         const int32_t* vb = ((parts & HFMM_PART_FAR_FREE) && lv.nv) ? lv.v_begin : nullptr;
 #define HFMM_VBLOCK(C)                                                                                              \
     do {                                                                                                            \
-        HFMM_CUDA_TRY(cudaFuncSetAttribute(vblock_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); \
+        HFMM_CUDA_TRY(smem_limit(vblock_kernel<C>, sm));                                                             \
         HFMM_CUDA_TRY(pdl_launch_if(!P->in_batch, vblock_kernel<C>, grid, dim3(128 * vb_nwc(C)), sm, st, 0, P->leaf_begin, P->L, l, nrhs, nc, \
                                  npp, ploc, tl2l, lv.mult32, vb, lv.v_off, lv.t_free32, react_done ? lv.r_begin : nullptr,   \
                                  lv.loc32));                                                                        \
@@ -1352,7 +1352,7 @@ hfmm_status small_down(hfmm_plan_s* P, int l, int nrhs, int parts, bool react_do
         const size_t sm = sizeof(cf) * ((size_t)nw * ncs_max + (size_t)nw * 32);
         if (sm <= 200 * 1024) {
             auto kern = nw == 32 ? down_small_kernel<1, 1, 32> : down_small_kernel<1, 1, 16>;
-            HFMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            HFMM_CUDA_TRY(smem_limit(kern, sm));
             HFMM_CUDA_TRY(pdl_launch_if(
                 !P->in_batch, kern, dim3((unsigned)ncta), dim3(nw * 32), sm, st, 0, P->leaf_begin, P->L, l, P->lmin, nrhs, lv.p,
                 has_parent ? P->lev[l - 1].p : 0, has_parent ? P->lev[l - 1].loc32 : nullptr,
@@ -1505,8 +1505,7 @@ hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, bool conj_out, cf* 
 #define HFMM_TAIL(RR)                                                                                            \
     do {                                                                                                         \
         const size_t sm = sizeof(cf) * 4 * RR * leaf.ncoef;                                                      \
-        if (sm > 48 * 1024)                                                                                      \
-            HFMM_CUDA_TRY(cudaFuncSetAttribute(l2p_scatter_kernel<RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)); \
+        HFMM_CUDA_TRY(smem_limit(l2p_scatter_kernel<RR>, sm));                                                   \
         HFMM_CUDA_TRY(pdl_launch_if(!P->in_batch, l2p_scatter_kernel<RR>, dim3(grid), dim3(128), sm, fs, 0, P->leaf_begin, leaf.nbox, n, nrhs, \
                                  far ? leaf.loc32 : nullptr, P->basis32, leaf.ncoef, sums ? P->y32 : nullptr,    \
                                  host ? nullptr : P->perm, conj_out, host ? P->y32 : y));                        \
@@ -1558,7 +1557,7 @@ template <int R>
 hfmm_status persist_grid(PersistBatch* B, int* grid) {
     const size_t sm = persist_smem(B, R);
     auto kern = persist_kernel<R>;
-    HFMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HFMM_CUDA_TRY(smem_limit(kern, sm, 4096));
     int per_sm = 0, dev = 0, nsm = 0;
     HFMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SM_W * 32, sm));
     HFMM_CUDA_TRY(cudaGetDevice(&dev));

@@ -747,7 +747,7 @@ hfmm_status react_tables(const MedDev& md, const std::vector<Entry>& ents, const
     }
     const int nch = (nmax + CH) / CH, nwin = std::min(nch, 128);   // chunks per launch: 64 KB of sums
     const size_t sm = sizeof(double) * (RT_NV * RT_NODES + 2 * (size_t)nwin * 32 + RT_THREADS);
-    HFMM_CUDA_TRY(cudaFuncSetAttribute(react_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HFMM_CUDA_TRY(smem_limit(react_sum_kernel, sm));
     const int ny = (int)std::max<int64_t>(1, std::min<int64_t>((most + RT_NODES - 1) / RT_NODES,
                                                                (8 * 152 + (int64_t)ents.size() - 1) / (int64_t)ents.size()));
     double* sums = nullptr;
