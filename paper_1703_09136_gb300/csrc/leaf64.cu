@@ -427,7 +427,7 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
         }
         if (live && part == 0 && (t < 2 ? v0 : v1)) {
             const int64_t i = tlo + (t < 2 ? i0 : i1);
-            if (ns > 0) x += fma((double)a, 4294967296.0, (double)bsum) * pow2d(EV);
+            if (ns > 0) x += scale2d(fma((double)a, 4294967296.0, (double)bsum), EV);
             if (bad) x = __longlong_as_double(0x7ff8000000000000ll);
             if (A.ys) x += __ldcg(reinterpret_cast<const double*>(A.ys + (int64_t)r * A.n + i) + (t & 1));
             reinterpret_cast<double*>(A.y + (int64_t)r * A.n + (A.perm ? A.perm[i] : i))[t & 1] = (A.conj_out && (t & 1)) ? -x : x;

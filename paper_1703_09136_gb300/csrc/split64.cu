@@ -379,7 +379,8 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
             for (int o = 0; o < NO; ++o) acc[t][o][v] = 0.0f;
         }
     int since = 0;                    // chunks since the integers were last folded
-    // dacc += (digit sums) 2^E, E = Esrc + Eop - (18 D - 3): order o weighs 512^(2 (D - 1) - o).
+    // dacc += (digit sums) 2^E, E = Esrc + Eop - (18 D - 3) less the larger of the families' E, which the
+    // epilogue puts back (so that no intermediate power of two leaves the range): order o weighs 512^(2 (D - 1) - o).
     // Four (two) FP64 instructions a value (the pipe takes 64 clocks for each of a
     // sub-partition's): orders 0 .. 2 and 3 .. 6 as integers below 2^51 (order 6 rounded to order 5's unit, 2^-61
     // of the largest term)
@@ -473,7 +474,7 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) load_op(cur, kk, more);
     pdl_wait();
-    int Ef[2] = {0, 0};               // fold exponents per family
+    int Ef[2] = {4 * S6_NONE, 4 * S6_NONE};   // fold exponents per family
     bool bad = false;
     if (A.shift.dig) {
         const int e = __ldcg(A.shift.Esrc + r);
@@ -485,6 +486,9 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
         bad |= e >= S6_NAN / 2;
         Ef[1] = max(e, S6_NONE) + max(*A.list.Eop, S6_NONE) - (18 * D - 3);
     }
+    const int Emax = D == 6 ? max(Ef[0], Ef[1]) : 0;       // (FP32's exponents cannot leave the range)
+    Ef[0] -= Emax;
+    Ef[1] -= Emax;
 
     load_src(cur, 0, more);
     bool first = true;
@@ -593,7 +597,7 @@ __global__ void __maxnreg__(D == 3 ? (NT == 1 ? 96 : 128) : (NT == 1 ? 128 : 168
             if (row >= 2 * no || b < 0) continue;
             const int sh = A.sxo ? A.osign * A.sxo[abs((row >> 1) - A.p)] : 0;
             R* o = reinterpret_cast<R*>(A.out) + ((b * A.nrhs + r) * no * 2 + row);
-            R x = (R)(bad ? nan : dacc[t][v] * pow2d(sh));
+            R x = (R)(bad ? nan : D == 6 ? scale2d(dacc[t][v], Emax + sh) : dacc[t][v] * pow2d(Emax + sh));
             if (A.accumulate) x += __ldcg(o);
             *o = x;
             e = max(e, s6_exponent(x, -sh));

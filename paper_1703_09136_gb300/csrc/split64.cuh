@@ -23,7 +23,10 @@ __device__ __forceinline__ int s6_exponent(double v, int shift) {
     const long long b = __double_as_longlong(v);
     const int e = (int)((b >> 52) & 2047);
     if (e == 2047) return S6_NAN;
-    if (e == 0) return (b & 0xfffffffffffffll) ? -1021 + shift : S6_NONE;
+    if (e == 0) {                                         // m 2^-1074
+        const long long m = b & 0xfffffffffffffll;
+        return m ? -1010 - __clzll(m) + shift : S6_NONE;
+    }
     return e - 1022 + shift;
 }
 __device__ __forceinline__ int s6_exponent(float v, int shift) {
@@ -42,6 +45,7 @@ __device__ __forceinline__ long long s6_fixed(double v, int shift, int E) {
     if (e) m |= 1ull << 52; else e = 1;
     const int s = E - shift - e + 1075 - BITS;            // right shift
     if (s > 0) m = s > 54 ? 0ull : (m + (1ull << (s - 1))) >> s;
+    else m <<= min(-s, 51);                               // subnormals alone
     return b < 0 ? -(long long)m : (long long)m;
 }
 template <int BITS>
@@ -74,6 +78,13 @@ __device__ __forceinline__ double pow2d(int e) {
     const long long b = e > 1023 ? 0x7ff0000000000000ll : e >= -1022 ? (long long)(e + 1023) << 52
                         : e >= -1074 ? 1ll << (e + 1074) : 0ll;
     return __longlong_as_double(b);
+}
+
+// x 2^e for any e (a product with one power of two loses digits where that power alone is subnormal or infinite)
+__device__ __forceinline__ double scale2d(double x, int e) {
+    const int f = max(-1000, min(1000, e));
+    x *= pow2d(f);
+    return e == f ? x : x * pow2d(e - f);
 }
 
 // an integer below 2^51 in magnitude as a double: one FP64 addition
