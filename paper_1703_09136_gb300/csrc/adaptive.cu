@@ -1293,7 +1293,7 @@ hfmm_status apply_adaptive64(hfmm_plan_s* P, int nrhs, int parts, bool conj_out,
     }
     if (aside) HFMM_TRY(join_near64(P, nrhs, m2p, conj_out, y, fs, st));
     else tm.begin(HFMM_STAGE_P2P);
-    if (near && !near_here) {                             // coincident points: H0 per pair
+    if (near && !near_here) {                             // too many coincident points: H0 per pair
         HFMM_CUDA_TRY(cudaMemsetAsync(P->y_sorted, 0, sizeof(cd) * n * nrhs, st));
         ad_near_kernel<<<(unsigned)ceil_div((int64_t)T->leaves.size(), 4), 128, 0, st>>>(
             T->d_boxes, T->d_leaves, (int64_t)T->leaves.size(), T->du_beg, T->du_src, T->du_blk, nullptr, T->dd_beg,
@@ -1416,11 +1416,12 @@ hfmm_status build_adaptive64(hfmm_plan_s* P, cudaStream_t st) {
     HFMM_TRY(plan_alloc(P, (void**)&P->leaf64_src, sizeof(int32_t) * std::max<int64_t>(soff, 1)));
     ad_sources_kernel<<<(unsigned)nl, 64, 0, st>>>(T->d_boxes, T->du_beg, T->du_src, P->leaf64, P->leaf64_src);
     HFMM_CUDA_TRY(cudaGetLastError());
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, sizeof(int)));
-    bool finite = true;
-    if (goff > 0) HFMM_TRY(near64_to_fixed(T->near_G, goff, P->near64_E, &finite, st));
-    if (finite) P->near64_vals = T->near_G;
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, 4 * sizeof(int)));
+    bool fixed = true;
+    if (goff > 0) HFMM_TRY(near64_to_fixed(T->near_G, goff, P->near64_E, &P->near64_infinite, &fixed, st));
+    if (fixed) P->near64_vals = T->near_G;
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // the vectors are locals
+    HFMM_TRY(near64_upload_infinite(P, recs, st));
     T->fast64 = true;
     return HFMM_OK;
 }

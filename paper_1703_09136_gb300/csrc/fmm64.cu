@@ -993,12 +993,10 @@ hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st) {
                                                         P->near64_vals);
     HFMM_CUDA_TRY(cudaGetLastError());
     P->table_bytes += bytes;
-    // coincident points (infinite entries) have no digit form: the apply then
-    // evaluates H0 per pair
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, sizeof(int)));
-    bool finite = true;
-    HFMM_TRY(near64_to_fixed(P->near64_vals, off[nleaf], P->near64_E, &finite, st));
-    if (!finite) P->near64_vals = nullptr;
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, 4 * sizeof(int)));
+    bool fixed = true;
+    HFMM_TRY(near64_to_fixed(P->near64_vals, off[nleaf], P->near64_E, &P->near64_infinite, &fixed, st));
+    if (!fixed) P->near64_vals = nullptr;
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));
     return HFMM_OK;
 }

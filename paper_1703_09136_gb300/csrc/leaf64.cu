@@ -436,19 +436,38 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
     }
 }
 
-// (i/4) H0 doubles -> largest exponent; then, in place, digit words.
-__global__ void near64_exponent_kernel(const cd* __restrict__ G, int64_t n, int* __restrict__ E) {
+// (i/4) H0 doubles -> largest exponent; then, in place, digit words.  Entries that are not finite (coincident points)
+// have no digits: they are counted, listed (near64_list_kernel) and leave zeros.
+__device__ __forceinline__ int near64_exponent(cd v) { return max(s6_exponent(v.x, 0), s6_exponent(v.y, 0)); }
+
+__global__ void near64_exponent_kernel(const cd* __restrict__ G, int64_t n, int* __restrict__ E,
+                                       unsigned long long* __restrict__ infinite) {
     int e = S6_NONE;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        e = max(e, max(s6_exponent(G[i].x, 0), s6_exponent(G[i].y, 0)));
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int x = near64_exponent(G[i]);
+        if (x < S6_NAN) e = max(e, x);
+        else atomicAdd(infinite, 1ull);
+    }
     e = __reduce_max_sync(0xffffffffu, e);
     if ((threadIdx.x & 31) == 0 && e > S6_NONE) atomicMax(E, e);
+}
+
+__global__ void near64_list_kernel(const cd* __restrict__ G, int64_t n, unsigned long long* __restrict__ next,
+                                   NearInfinite* __restrict__ out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const cd v = G[i];
+        if (near64_exponent(v) < S6_NAN) continue;
+        NearInfinite& o = out[atomicAdd(next, 1ull)];
+        o.pair = i;
+        o.val = v;
+    }
 }
 
 __global__ void near64_fix_kernel(cd* G, int64_t n, const int* __restrict__ E) {
     const int e = *E;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const cd v = G[i];
+        cd v = G[i];
+        if (near64_exponent(v) >= S6_NAN) v = cmk(0.0, 0.0);
         const long long x = lf_fixed(v.x, e) + (128ll << 48), y = lf_fixed(v.y, e) + (128ll << 48);
         unsigned w[4];
 #pragma unroll
@@ -459,6 +478,30 @@ __global__ void near64_fix_kernel(cd* G, int64_t n, const int* __restrict__ E) {
             w[k] = x0 | (x1 << 8) | (y0 << 16) | (y1 << 24);
         }
         reinterpret_cast<uint4*>(G)[i] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// The listed entries onto the sums that leaf64_kernel wrote: a warp per (target that has some, right-hand side).
+__global__ void __launch_bounds__(128) near64_infinite_kernel(const int32_t* __restrict__ tgt, const int64_t* __restrict__ beg,
+                                                              const int32_t* __restrict__ src, const cd* __restrict__ val,
+                                                              int64_t ntgt, const cd* __restrict__ qs, int64_t n, int nrhs,
+                                                              const int64_t* __restrict__ perm, bool conj_out,
+                                                              cd* __restrict__ y) {
+    const int lane = threadIdx.x & 31;
+    const int64_t total = ntgt * nrhs;
+    for (int64_t id = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5); id < total; id += (int64_t)gridDim.x * 4) {
+        const int64_t t = id % ntgt, r = id / ntgt;
+        cd a = cmk(0.0, 0.0);
+        for (int64_t e = beg[t] + lane; e < beg[t + 1]; e += 32) cfma(a, val[e], qs[r * n + src[e]]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+            a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+        }
+        if (lane == 0) {
+            cd* o = y + r * n + (perm ? perm[tgt[t]] : tgt[t]);
+            *o = cadd(*o, conj_out ? cconj(a) : a);
+        }
     }
 }
 
@@ -633,20 +676,82 @@ hfmm_status launch_grad_far(hfmm_plan_s* P, int nrhs, const cd* v, double2* acc,
     return HFMM_OK;
 }
 
-// Digit form of `pairs` near-field values in place; *finite = false (and the
-// values unchanged) where an entry is not finite (coincident points).
-hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, bool* finite, cudaStream_t st) {
-    *finite = true;
+// Digit form of `pairs` near-field values in place (E: their exponent, and two words behind it a counter), the entries that are not finite (coincident
+// points) in *infinite; *fixed = false (and the values unchanged) where those are more than NEAR64_INFINITE_MAX.
+hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, std::vector<NearInfinite>* infinite, bool* fixed,
+                            cudaStream_t st) {
+    *fixed = true;
+    infinite->clear();
+    unsigned long long* count = (unsigned long long*)(E + 2);
+    HFMM_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(*count), st));
     HFMM_CUDA_TRY(cudaMemsetAsync(E, 0x80, sizeof(int), st));
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((pairs + 255) / 256, 16 * 152));
-    near64_exponent_kernel<<<grid, 256, 0, st>>>(vals, pairs, E);
+    near64_exponent_kernel<<<grid, 256, 0, st>>>(vals, pairs, E, count);
     HFMM_CUDA_TRY(cudaGetLastError());
-    int e = 0;
-    HFMM_CUDA_TRY(cudaMemcpyAsync(&e, E, sizeof(int), cudaMemcpyDeviceToHost, st));
+    unsigned long long ninf = 0;
+    HFMM_CUDA_TRY(cudaMemcpyAsync(&ninf, count, sizeof(ninf), cudaMemcpyDeviceToHost, st));
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));
-    if (e >= S6_NAN / 2) { *finite = false; return HFMM_OK; }
+    if (ninf > NEAR64_INFINITE_MAX) *fixed = false;
+    else if (ninf > 0) {
+        NearInfinite* list = nullptr;
+        HFMM_CUDA_TRY(cudaMallocAsync((void**)&list, sizeof(NearInfinite) * ninf, st));
+        HFMM_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(*count), st));
+        near64_list_kernel<<<grid, 256, 0, st>>>(vals, pairs, count, list);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        infinite->resize(ninf);
+        HFMM_CUDA_TRY(cudaMemcpyAsync(infinite->data(), list, sizeof(NearInfinite) * ninf, cudaMemcpyDeviceToHost, st));
+        HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+        HFMM_CUDA_TRY(cudaFreeAsync(list, st));
+        std::sort(infinite->begin(), infinite->end(), [](const NearInfinite& a, const NearInfinite& b) { return a.pair < b.pair; });
+    }
+    if (!*fixed) return HFMM_OK;
     near64_fix_kernel<<<grid, 256, 0, st>>>(vals, pairs, E);
     HFMM_CUDA_TRY(cudaGetLastError());
+    return HFMM_OK;
+}
+
+// The listed entries by target, from the leaf records (in the order of their blocks) and near-field source indices.
+hfmm_status near64_upload_infinite(hfmm_plan_s* P, const std::vector<Leaf64Rec>& recs, cudaStream_t st) {
+    const auto& list = P->near64_infinite;
+    if (list.empty()) return HFMM_OK;
+    int64_t nsrc = 0;
+    for (const Leaf64Rec& R : recs) nsrc = std::max(nsrc, R.soff + R.ns);
+    std::vector<int32_t> src(nsrc);
+    HFMM_CUDA_TRY(cudaMemcpyAsync(src.data(), P->leaf64_src, sizeof(int32_t) * nsrc, cudaMemcpyDeviceToHost, st));
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+    struct Item { int32_t t, s; cd v; };
+    std::vector<Item> items;
+    size_t r = 0;
+    for (const NearInfinite& e : list) {
+        while (e.pair >= recs[r].goff + (int64_t)recs[r].tn * recs[r].ns) ++r;
+        const int64_t o = e.pair - recs[r].goff;           // source-major within the block
+        items.push_back({recs[r].tlo + (int32_t)(o % recs[r].tn), src[recs[r].soff + o / recs[r].tn], e.val});
+    }
+    std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.t < b.t; });
+    std::vector<int32_t> tgt, isrc;
+    std::vector<int64_t> beg;
+    std::vector<cd> val;
+    for (const Item& it : items) {
+        if (tgt.empty() || tgt.back() != it.t) {
+            tgt.push_back(it.t);
+            beg.push_back((int64_t)val.size());
+        }
+        isrc.push_back(it.s);
+        val.push_back(it.v);
+    }
+    beg.push_back((int64_t)val.size());
+    P->near64_inf_n = (int64_t)tgt.size();
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_tgt, sizeof(int32_t) * tgt.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_beg, sizeof(int64_t) * beg.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_src, sizeof(int32_t) * isrc.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_val, sizeof(cd) * val.size()));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_tgt, tgt.data(), sizeof(int32_t) * tgt.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_beg, beg.data(), sizeof(int64_t) * beg.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_src, isrc.data(), sizeof(int32_t) * isrc.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_val, val.data(), sizeof(cd) * val.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+    P->near64_infinite.clear();
+    P->near64_infinite.shrink_to_fit();
     return HFMM_OK;
 }
 
@@ -722,7 +827,7 @@ hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
         HFMM_CUDA_TRY(cudaGetLastError());
     }
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // recs and ds are locals
-    return HFMM_OK;
+    return near64_upload_infinite(P, recs, st);
 }
 
 // P2M of the sorted strengths into the leaf multipoles (and their exponents).
@@ -804,5 +909,12 @@ hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2
     HFMM_CUDA_TRY(smem_limit(kernel, sm));
     HFMM_CUDA_TRY(pdl_launch(kernel, dim3((unsigned)P->leaf64_n, (unsigned)nrhs), dim3(W * 32), sm, st, 0, A));
     ++P->launches;
+    if (near && P->near64_inf_n > 0) {
+        const unsigned grid = (unsigned)std::min<int64_t>((P->near64_inf_n * nrhs + 3) / 4, 16 * 152);
+        near64_infinite_kernel<<<grid, 128, 0, st>>>(P->near64_inf_tgt, P->near64_inf_beg, P->near64_inf_src, P->near64_inf_val,
+                                                     P->near64_inf_n, P->q_sorted, P->n, nrhs, A.perm, conj_out, y);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        ++P->launches;
+    }
     return HFMM_OK;
 }
