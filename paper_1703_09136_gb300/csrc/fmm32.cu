@@ -925,6 +925,10 @@ hfmm_status launch_direct32(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
 
 hfmm_status apply_mixed(hfmm_plan_s* P, int nrhs, const cf* q, cf* y, int parts, bool adjoint,
                         cudaStream_t st) {
+    if (P->ad && nrhs > RHS_SLICE)
+        return rhs_slices(P, nrhs, [&](int r0, int nr) {
+            return apply_mixed(P, nr, q + (int64_t)r0 * P->n, y + (int64_t)r0 * P->n, parts, adjoint, st);
+        });
     const int64_t n = P->n;
     const int L = P->L;
     StageTimer tm{P, st};

@@ -396,6 +396,10 @@ static hfmm_status downward64(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t 
 
 hfmm_status apply_fp64(hfmm_plan_s* P, int nrhs, const cd* q, cd* y, int parts, bool adjoint,
                        cudaStream_t st) {
+    if (nrhs > RHS_SLICE)
+        return rhs_slices(P, nrhs, [&](int r0, int nr) {
+            return apply_fp64(P, nr, q + (int64_t)r0 * P->n, y + (int64_t)r0 * P->n, parts, adjoint, st);
+        });
     const int64_t n = P->n;
     const int L = P->L;
     const int nb = ceil_div(n, 256);
@@ -850,9 +854,23 @@ hfmm_status field_grad_fp64(hfmm_plan_s* P, int nrhs, cd* fx, cd* fy, cudaStream
     return HFMM_OK;
 }
 
+__global__ void grad_add_kernel(const double* __restrict__ part, int64_t count, double* __restrict__ gxy) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < count) gxy[i] += part[i];
+}
+
 }  // namespace
 
 hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, double* gxy, cudaStream_t st) {
+    if (nrhs > RHS_SLICE) {
+        if (!P->grad_part) HFMM_TRY(plan_alloc(P, (void**)&P->grad_part, sizeof(double) * 2 * P->n));
+        return rhs_slices(P, nrhs, [&](int r0, int nr) -> hfmm_status {
+            HFMM_TRY(apply_grad_fp64(P, nr, q + (int64_t)r0 * P->n, g + (int64_t)r0 * P->n, r0 ? P->grad_part : gxy, st));
+            if (r0) grad_add_kernel<<<ceil_div(2 * P->n, 256), 256, 0, st>>>(P->grad_part, 2 * P->n, gxy);
+            HFMM_CUDA_TRY(cudaGetLastError());
+            return HFMM_OK;
+        });
+    }
     const int64_t n = P->n;
     const int nb = ceil_div(n, 256);
     const size_t bytes = sizeof(cd) * (size_t)n * P->max_rhs;

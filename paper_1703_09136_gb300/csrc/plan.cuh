@@ -268,6 +268,7 @@ struct hfmm_plan_s {
     size_t krylov_host_words = 0;
     cd* near64g_x = nullptr;        // d/dx, d/dy of the same blocks (first gradient request)
     cd* near64g_y = nullptr;
+    double* grad_part = nullptr;    // one slice's part of a gradient of more than RHS_SLICE right-hand sides
     cd* grad_buf = nullptr;         // conj(g) and the fields or sums of a gradient
     bool grad_fused = false;        // gradients from stored blocks and bases (leaf64.cu)
     cd* grad_q = nullptr;           // mixed plans: widened strengths / loss gradient
@@ -355,6 +356,24 @@ struct StageTimer {
         if (P->events_ready) cudaEventRecord(P->ev[s][1], st);
     }
 };
+
+// Passes with the right-hand sides in a grid dimension take at most 65,535 of them: a wider apply is made of
+// several, f(r0, nr) of the right-hand sides r0 .. r0 + nr - 1, and counts their work together.
+constexpr int RHS_SLICE = 65535;
+template <class F>
+hfmm_status rhs_slices(hfmm_plan_s* P, int nrhs, F&& f) {
+    int64_t launches = 0;
+    double flops[HFMM_NUM_STAGES] = {}, bytes[HFMM_NUM_STAGES] = {};
+    for (int r0 = 0; r0 < nrhs; r0 += RHS_SLICE) {
+        const hfmm_status s = f(r0, nrhs - r0 < RHS_SLICE ? nrhs - r0 : RHS_SLICE);
+        if (s != HFMM_OK) return s;
+        launches += P->launches;
+        for (int i = 0; i < HFMM_NUM_STAGES; ++i) { flops[i] += P->st_flops[i]; bytes[i] += P->st_bytes[i]; }
+    }
+    P->launches = launches;
+    for (int i = 0; i < HFMM_NUM_STAGES; ++i) { P->st_flops[i] = flops[i]; P->st_bytes[i] = bytes[i]; }
+    return HFMM_OK;
+}
 
 // allocation helper that records the pointer in the plan
 hfmm_status plan_alloc(hfmm_plan_s* P, void** ptr, size_t bytes);
