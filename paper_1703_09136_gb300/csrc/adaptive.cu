@@ -1314,9 +1314,8 @@ hfmm_status apply_adaptive64(hfmm_plan_s* P, int nrhs, int parts, bool conj_out,
 }
 
 // Plan-time state of apply_adaptive64 (after the tables): operator slices, bases, digit
-// blocks and leaf records.  A plan above a byte budget keeps the kernels of
-// apply_adaptive.
-hfmm_status build_adaptive64(hfmm_plan_s* P, cudaStream_t st) {
+// blocks and leaf records.
+static hfmm_status ad64_build(hfmm_plan_s* P, cudaStream_t st) {
     AdaptiveTree* T = P->ad;
     const auto& bx = T->boxes;
     const int64_t nl = (int64_t)T->leaves.size();
@@ -1342,7 +1341,8 @@ hfmm_status build_adaptive64(hfmm_plan_s* P, cudaStream_t st) {
             xboff[e] = nx;
             nx += (int64_t)(bx[T->x_src[e]].hi - bx[T->x_src[e]].lo) * nc(bx[b].level);
         }
-    if (sizeof(cd) * (double)(nb + nw + nx) > 8e9 || T->pmax * (int)sizeof(cd) > 40000) return HFMM_OK;
+    const double basis_bytes = sizeof(cd) * (double)(nb + nw + nx);
+    if (basis_bytes > 8e9 || T->pmax * (int)sizeof(cd) > 40000 || !optional_fits(basis_bytes)) return HFMM_OK;
     HFMM_TRY(build_split(P, 0, st));
     if (!P->s6_ready[0]) return HFMM_OK;
     HFMM_TRY(ad_upload_xboxes(P, st));
@@ -1420,10 +1420,32 @@ hfmm_status build_adaptive64(hfmm_plan_s* P, cudaStream_t st) {
     bool fixed = true;
     if (goff > 0) HFMM_TRY(near64_to_fixed(T->near_G, goff, P->near64_E, &P->near64_infinite, &fixed, st));
     if (fixed) P->near64_vals = T->near_G;
+    T->fast64 = true;                                     // from here on near_G holds digits
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // the vectors are locals
-    HFMM_TRY(near64_upload_infinite(P, recs, st));
-    T->fast64 = true;
-    return HFMM_OK;
+    return near64_upload_infinite(P, recs, st);
+}
+
+// A plan above a byte budget or the device's memory keeps the kernels of apply_adaptive.
+hfmm_status build_adaptive64(hfmm_plan_s* P, cudaStream_t st) {
+    AdaptiveTree* T = P->ad;
+    return plan_optional(P,
+                         [&] {
+                             const hfmm_status s = ad64_build(P, st);
+                             if (s == HFMM_ERR_OOM && T->fast64) {
+                                 hfmm_set_error("out of memory for the list of coincident points");
+                                 return HFMM_ERR_CUDA;
+                             }
+                             return s;
+                         },
+                         [&] {
+                             split_forget(P, 0);
+                             leaf64_forget(P);
+                             T->d_xbox = nullptr;
+                             T->xbox_off.clear();
+                             T->d_xboff = nullptr;
+                             T->p2l64 = nullptr;
+                             P->near64_E = nullptr;
+                         });
 }
 
 // The adaptive apply between the gather and the scatter (FP64).

@@ -54,6 +54,7 @@ hfmm_status plan_alloc(hfmm_plan_s* P, void** ptr, size_t bytes) {
     cudaError_t e = cudaMalloc(ptr, bytes);
     if (e != cudaSuccess) {
         *ptr = nullptr;
+        cudaGetLastError();                                // (the callers that go on without must not find it)
         hfmm_set_error("cudaMalloc(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? HFMM_ERR_OOM : HFMM_ERR_CUDA;
     }

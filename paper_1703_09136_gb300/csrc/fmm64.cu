@@ -875,12 +875,30 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
     const int nb = ceil_div(n, 256);
     const size_t bytes = sizeof(cd) * (size_t)n * P->max_rhs;
     if (!P->grad_buf) {
-        HFMM_TRY(build_direct_grad(P, st));
-        HFMM_TRY(build_near64_grad(P, st));
-        HFMM_TRY(build_split(P, 0, st));
-        HFMM_TRY(build_leaf64(P, st));
-        P->grad_fused = P->near64g_x && P->basis64;
-        HFMM_TRY(plan_alloc(P, (void**)&P->grad_buf, P->grad_fused ? bytes + 2 * sizeof(double2) * (size_t)n : 5 * bytes));
+        // all of it or none: a call that ran out of memory leaves the plan as it was, for another try
+        const PlanMark mark(P);
+        const bool had_off = P->near64_off, had_leaves = P->leaf64;
+        auto build = [&]() -> hfmm_status {
+            HFMM_TRY(build_direct_grad(P, st));
+            HFMM_TRY(build_near64_grad(P, st));
+            if (!had_leaves) {                            // a mixed plan (an FP64 plan's records know whether it has digits)
+                HFMM_TRY(build_split(P, 0, st));
+                HFMM_TRY(build_leaf64(P, st));
+            }
+            P->grad_fused = P->near64g_x && P->basis64;
+            return plan_alloc(P, (void**)&P->grad_buf, P->grad_fused ? bytes + 2 * sizeof(double2) * (size_t)n : 5 * bytes);
+        };
+        const hfmm_status s = build();
+        if (s != HFMM_OK) {
+            mark.back(P);
+            P->d_gvals = P->near64g_x = P->near64g_y = nullptr;
+            if (!had_off) P->near64_off = nullptr;
+            if (!had_leaves) {
+                split_forget(P, 0);
+                leaf64_forget(P);
+            }
+            return s;
+        }
     }
     if (P->grad_fused) {                          // stored blocks and bases (leaf64.cu); else the kernels that evaluate them
         cd* gc = P->grad_buf;

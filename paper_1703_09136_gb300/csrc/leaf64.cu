@@ -764,7 +764,7 @@ hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
     const LevelInfo& lv = P->lev[L];
     const int nb = lv.p + 2, m = 1 << L;
     const double bytes = sizeof(cd) * (double)P->n * nb;
-    const bool has_basis = bytes <= BASIS64_MAX_BYTES && nb * (int)sizeof(double) <= 40000;
+    const bool has_basis = bytes <= BASIS64_MAX_BYTES && nb * (int)sizeof(double) <= 40000 && optional_fits(bytes);
     const auto& lb = P->h_leaf_begin;
     std::vector<Leaf64Rec> recs;
     std::vector<Leaf64D> ds;
@@ -818,8 +818,10 @@ hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
         HFMM_CUDA_TRY(cudaMemcpyAsync(P->leaf64_d, ds.data(), sizeof(Leaf64D) * ds.size(), cudaMemcpyHostToDevice, st));
     leaf_sources_kernel<<<(unsigned)recs.size(), 64, 0, st>>>(P->leaf_begin, L, P->leaf64, P->leaf64_src);
     HFMM_CUDA_TRY(cudaGetLastError());
-    if (has_basis) {
-        HFMM_TRY(plan_alloc(P, (void**)&P->basis64, (size_t)bytes));
+    if (has_basis)
+        HFMM_TRY(plan_optional(P, [&] { return plan_alloc(P, (void**)&P->basis64, (size_t)bytes); },
+                               [&] { P->basis64 = nullptr; }));
+    if (P->basis64) {
         P->buffer_bytes += bytes;
         const int thr = std::max(1, std::min(64, 5000 / nb));
         basis64_kernel<<<(unsigned)lv.nbox, thr, (size_t)thr * nb * sizeof(double), st>>>(
@@ -828,6 +830,17 @@ hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
     }
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // recs and ds are locals
     return near64_upload_infinite(P, recs, st);
+}
+
+// The plan's memory of its leaf records and bases is gone.
+void leaf64_forget(hfmm_plan_s* P) {
+    P->leaf64 = nullptr;
+    P->leaf64_w = nullptr;
+    P->leaf64_d = nullptr;
+    P->leaf64_src = nullptr;
+    P->basis64 = P->m2p64 = nullptr;
+    P->leaf64_n = 0;
+    P->leaf64_p = P->leaf_max = 0;
 }
 
 // P2M of the sorted strengths into the leaf multipoles (and their exponents).

@@ -378,6 +378,43 @@ hfmm_status rhs_slices(hfmm_plan_s* P, int nrhs, F&& f) {
 // allocation helper that records the pointer in the plan
 hfmm_status plan_alloc(hfmm_plan_s* P, void** ptr, size_t bytes);
 
+// What a plan held at a point of its building, and the way back there: the allocations since then are given
+// back (cudaFree waits for the kernels that use the memory).
+struct PlanMark {
+    size_t kept, slab_left, slab_bytes;
+    char* slab_next;
+    double table_bytes, buffer_bytes;
+    explicit PlanMark(const hfmm_plan_s* P)
+        : kept(P->allocations.size()), slab_left(P->slab_left), slab_bytes(P->slab_bytes), slab_next(P->slab_next),
+          table_bytes(P->table_bytes), buffer_bytes(P->buffer_bytes) {}
+    void back(hfmm_plan_s* P) const {
+        for (; P->allocations.size() > kept; P->allocations.pop_back()) cudaFree(P->allocations.back());
+        P->slab_left = slab_left; P->slab_bytes = slab_bytes; P->slab_next = slab_next;
+        P->table_bytes = table_bytes; P->buffer_bytes = buffer_bytes;
+    }
+};
+
+// Stores that only make a plan faster (digits and operator slices, bases, FP32 blocks) are not worth a plan that does
+// not fit: one of 16 MB or more is made only where as much again stays free for the plan's later
+// buffers and the caller (asking takes 7 us), and where an allocation fails all the same, what the store had taken is
+// given back and the kernels that do without it run.
+inline bool optional_fits(double bytes) {
+    if (bytes < 16e6) return true;
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) { cudaGetLastError(); return true; }
+    return bytes <= 0.5 * (double)free_bytes;
+}
+// build(), and where the device memory runs out in it the way back, with undo() for the pointers
+template <class B, class U>
+hfmm_status plan_optional(hfmm_plan_s* P, B&& build, U&& undo) {
+    const PlanMark mark(P);
+    const hfmm_status s = build();
+    if (s != HFMM_ERR_OOM) return s;
+    mark.back(P);
+    undo();
+    return HFMM_OK;
+}
+
 // tree.cu
 hfmm_status build_tree(hfmm_plan_s* P, const double* d_xy, cudaStream_t st);
 hfmm_status build_lists(hfmm_plan_s* P, cudaStream_t st);
@@ -417,6 +454,7 @@ hfmm_status diag_m2l(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st
 double diag_flops(const hfmm_plan_s* P, int l, int nrhs, int parts);
 // split64.cu (w = 0: FP64 expansions, 1: FP32)
 hfmm_status build_split(hfmm_plan_s* P, int w, cudaStream_t st);
+void split_forget(hfmm_plan_s* P, int w);
 hfmm_status split_begin(hfmm_plan_s* P, int w, cudaStream_t st);
 hfmm_status split_exponent(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st);
 hfmm_status split_slice(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st);
@@ -428,6 +466,7 @@ void adaptive_tiles(const hfmm_plan_s* P, int l, bool up, const std::vector<int3
                     std::vector<int32_t>& tbeg, std::vector<S6Rec>& recs);
 // leaf64.cu
 hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st);
+void leaf64_forget(hfmm_plan_s* P);
 hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, std::vector<NearInfinite>* infinite, bool* fixed,
                             cudaStream_t st);
 hfmm_status near64_upload_infinite(hfmm_plan_s* P, const std::vector<Leaf64Rec>& recs, cudaStream_t st);

@@ -1221,9 +1221,12 @@ hfmm_status build_near_small(hfmm_plan_s* P, cudaStream_t st) {
     if (P->max_rhs > P->small_rhs || P->ad || (P->flags & HFMM_FLAG_SIMT_M2L)) return HFMM_OK;
     int64_t pairs = 0;
     HFMM_TRY(near64_offsets(P, &pairs, false, st));
-    if (sizeof(cf) * (double)pairs > NEAR32_MAX_BYTES) return HFMM_OK;
+    if (sizeof(cf) * (double)pairs > NEAR32_MAX_BYTES || !optional_fits(sizeof(cf) * (double)pairs)) return HFMM_OK;
     HFMM_TRY(near64_offsets(P, &pairs, true, st));
-    HFMM_TRY(plan_alloc(P, (void**)&P->near32_vals, sizeof(cf) * (size_t)std::max<int64_t>(pairs, 1)));
+    HFMM_TRY(plan_optional(P, [&] { return plan_alloc(P, (void**)&P->near32_vals,
+                                                      sizeof(cf) * (size_t)std::max<int64_t>(pairs, 1)); },
+                           [&] { P->near32_vals = nullptr; }));
+    if (!P->near32_vals) return HFMM_OK;
     near_fill_kernel<<<(unsigned)ceil_div(lv.nbox, 4), 128, 0, st>>>(P->leaf_begin, P->L, lv.nbox, P->xl32, (float)P->k,
                                                                      (float)lv.h, P->near64_off, P->near32_vals);
     HFMM_CUDA_TRY(cudaGetLastError());

@@ -685,7 +685,7 @@ hfmm_status s6_build(hfmm_plan_s* P, cudaStream_t st) {
         if (l > P->lmin) used += bytes(4, lv.p, P->lev[l - 1].p) + bytes(4, P->lev[l - 1].p, lv.p);
         dbytes += (l < L ? 2.0 : 1.0) * digits(lv);
     }
-    if (used > S6_MAX_BYTES || dbytes > S6_MAX_BYTES) return HFMM_OK;
+    if (used > S6_MAX_BYTES || dbytes > S6_MAX_BYTES || !optional_fits(used + dbytes)) return HFMM_OK;
     int* E = nullptr;                                     // [level][3] families, then [kind][level][rhs] expansions
     const size_t ne = (size_t)3 * (L + 1) + (size_t)2 * (L + 1) * P->max_rhs;
     HFMM_TRY(plan_alloc(P, (void**)&E, sizeof(int) * ne));
@@ -875,8 +875,17 @@ hfmm_status s6_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st)
 
 // w = 0: the FP64 expansions, 1: the mixed path's FP32 expansions.
 // Operator slices of every level (plan time, or a mixed plan's first gradient).
-// A plan whose slices or digits would pass the byte budget keeps the SIMT kernels.
-hfmm_status build_split(hfmm_plan_s* P, int w, cudaStream_t st) { return w ? s6_build<3>(P, st) : s6_build<6>(P, st); }
+// A plan whose slices or digits would pass the byte budget or the device's memory keeps the SIMT kernels.
+hfmm_status build_split(hfmm_plan_s* P, int w, cudaStream_t st) {
+    return plan_optional(P, [&] { return w ? s6_build<3>(P, st) : s6_build<6>(P, st); }, [&] { split_forget(P, w); });
+}
+
+// The plan's memory of its slices is gone.
+void split_forget(hfmm_plan_s* P, int w) {
+    P->s6_ready[w] = false;
+    P->s6_E[w] = nullptr;
+    for (LevelInfo& lv : P->lev) lv.s6[w] = S6Lev{};
+}
 
 // Start of a tree pass: no exponent is known.
 hfmm_status split_begin(hfmm_plan_s* P, int w, cudaStream_t st) {

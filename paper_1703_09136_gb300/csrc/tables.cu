@@ -748,16 +748,24 @@ hfmm_status react_tables(const MedDev& md, const std::vector<Entry>& ents, const
     const int nch = (nmax + CH) / CH, nwin = std::min(nch, 128);   // chunks per launch: 64 KB of sums
     const size_t sm = sizeof(double) * (RT_NV * RT_NODES + 2 * (size_t)nwin * 32 + RT_THREADS);
     HFMM_CUDA_TRY(smem_limit(react_sum_kernel, sm));
-    const int ny = (int)std::max<int64_t>(1, std::min<int64_t>((most + RT_NODES - 1) / RT_NODES,
-                                                               (8 * 152 + (int64_t)ents.size() - 1) / (int64_t)ents.size()));
+    int ny = (int)std::max<int64_t>(1, std::min<int64_t>((most + RT_NODES - 1) / RT_NODES,
+                                                         (8 * 152 + (int64_t)ents.size() - 1) / (int64_t)ents.size()));
+    // the splits' sums, from the pool; where its granularity (32 MB) does not fit, one split's alone
     double* sums = nullptr;
-    HFMM_CUDA_TRY(cudaMallocAsync((void**)&sums, sizeof(double) * 2 * nwin * 32 * ny * ents.size(), st));
+    const size_t one = sizeof(double) * 2 * nwin * 32 * ents.size();
+    const bool pooled = cudaMallocAsync((void**)&sums, one * ny, st) == cudaSuccess;
+    if (!pooled) {
+        cudaGetLastError();
+        ny = 1;
+        HFMM_CUDA_TRY(cudaMalloc((void**)&sums, one));
+    }
     for (int c0 = 0; c0 < nch; c0 += nwin) {
         react_sum_kernel<<<dim3((unsigned)ents.size(), (unsigned)ny), RT_THREADS, sm, st>>>(md, dents, dsegs, c0, nwin, sums);
         react_finish_kernel<<<(unsigned)ents.size(), 128, 0, st>>>(dents, sums, ny, c0, nwin, out);
     }
     const cudaError_t err = cudaGetLastError();
-    cudaFreeAsync(sums, st);
+    if (pooled) cudaFreeAsync(sums, st);
+    else cudaFree(sums);
     HFMM_CUDA_TRY(err);
     return HFMM_OK;
 }
