@@ -303,6 +303,7 @@ struct Krylov {
     double2 *part, *h1, *h2, *nrm, *col, *host;
     unsigned* ticket;
     int chunk;           // vector elements of a block in the Gram-Schmidt kernels
+    bool one_cluster;    // cgs_kernel takes a whole step
 
     unsigned blocks() const { return (unsigned)((n + chunk - 1) / chunk); }
     hfmm_status read(const double2* d, int cnt) {
@@ -318,17 +319,38 @@ struct Krylov {
         *out = host[0].x;
         return HFMM_OK;
     }
+    size_t cgs_smem(int cnt) const {
+        return sizeof(double2) * ((size_t)((n + CGS_CTAS - 1) / CGS_CTAS) + 4 * (size_t)cnt + CGS_THREADS + 1);
+    }
+    // Whether a basis of m vectors is orthogonalised by cgs_kernel: short vectors, and a device (or the part of
+    // one that this process has) that can place a cluster of 16 CTAs with their shared memory.
+    hfmm_status choose_cgs(int m) {
+        one_cluster = false;
+        if (n > CGS_MAX || m > CGS_MAX_RESTART) return HFMM_OK;
+        HFMM_CUDA_TRY(cudaFuncSetAttribute(cgs_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        HFMM_CUDA_TRY(cudaFuncSetAttribute(cgs_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(CGS_CTAS);
+        cfg.blockDim = dim3(CGS_THREADS);
+        cfg.dynamicSmemBytes = cgs_smem(m);
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = CGS_CTAS;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        one_cluster = cudaOccupancyMaxActiveClusters(&clusters, cgs_kernel<T>, &cfg) == cudaSuccess && clusters > 0;
+        cudaGetLastError();
+        return HFMM_OK;
+    }
     // Arnoldi step: w = (sigma + A) v_j minus its projections on v_0 .. v_j, v_{j + 1} = w / |w|;
     // host[0 .. j] = the Hessenberg column, host[j + 1].x = |w|^2
     hfmm_status arnoldi(zc sigma, T* V, int j, T* w) {
         HFMM_TRY(apply(V + (size_t)j * n, w));
-        if (n <= CGS_MAX && j < CGS_MAX_RESTART) {         // the column goes straight to the host's pages
+        if (one_cluster) {                                 // the column goes straight to the host's pages
             const int part_n = (int)((n + CGS_CTAS - 1) / CGS_CTAS), cnt = j + 1;
-            const size_t bytes = sizeof(double2) * ((size_t)part_n + 4 * (size_t)cnt + CGS_THREADS + 1);
-            auto kernel = cgs_kernel<T>;
-            HFMM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            HFMM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-            HFMM_CUDA_TRY(pdl_launch_if(false, kernel, dim3(CGS_CTAS), dim3(CGS_THREADS), bytes, st, CGS_CTAS, V,
+            HFMM_CUDA_TRY(pdl_launch_if(false, cgs_kernel<T>, dim3(CGS_CTAS), dim3(CGS_THREADS), cgs_smem(cnt), st, CGS_CTAS, V,
                                         V + (size_t)(j + 1) * n, w, n, part_n, cnt, sigma.real(), sigma.imag(), host));
             HFMM_CUDA_TRY(cudaStreamSynchronize(st));
             return HFMM_OK;
@@ -389,7 +411,8 @@ hfmm_status gmres(hfmm_plan_s* P, zc sigma, const T* b, T* x, double tol, int m,
     }
     double2* small = P->krylov_part;
     Krylov<T> K{P, st, n, small + 3 * (size_t)(m + 2) + 2, small, small + (m + 2), small + 3 * (size_t)(m + 2),
-                small + 2 * (size_t)(m + 2), P->krylov_host, (unsigned*)(small + 3 * (size_t)(m + 2) + 1), chunk};
+                small + 2 * (size_t)(m + 2), P->krylov_host, (unsigned*)(small + 3 * (size_t)(m + 2) + 1), chunk, false};
+    HFMM_TRY(K.choose_cgs(m));
     HFMM_CUDA_TRY(cudaMemsetAsync(K.ticket, 0, sizeof(unsigned), st));
     T* V = (T*)P->krylov;
     T* w = V + (size_t)n * (m + 1);
