@@ -896,17 +896,31 @@ extern "C" hfmm_status hfmm_debug_green_f32(int32_t n, const double* z, float* g
     return HFMM_OK;
 }
 
+// A stream or an event of a plan, made once.  A call that could not make one leaves it null (not with what the
+// runtime wrote there before it failed), so that a later call tries again and plan_free destroys what was made.
+hfmm_status ensure_stream(cudaStream_t* s, int priority) {
+    cudaStream_t made = nullptr;
+    if (!*s) HFMM_CUDA_TRY(cudaStreamCreateWithPriority(&made, cudaStreamNonBlocking, priority));
+    if (made) *s = made;
+    return HFMM_OK;
+}
+hfmm_status ensure_event(cudaEvent_t* e) {
+    cudaEvent_t made = nullptr;
+    if (!*e) HFMM_CUDA_TRY(cudaEventCreateWithFlags(&made, cudaEventDisableTiming));
+    if (made) *e = made;
+    return HFMM_OK;
+}
+
 // The near field on a low-priority stream concurrently with the far-field
 // chain on a high-priority one (both created on first use), forked from st
 // after everything already queued there.
 hfmm_status fork_near_far(hfmm_plan_s* P, cudaStream_t st) {
-    if (!P->far_st) {
+    if (!P->ev_far_done) {                                // the last of them
         int least = 0, greatest = 0;
         HFMM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-        HFMM_CUDA_TRY(cudaStreamCreateWithPriority(&P->far_st, cudaStreamNonBlocking, greatest));
-        HFMM_CUDA_TRY(cudaStreamCreateWithPriority(&P->near_st, cudaStreamNonBlocking, least));
-        for (cudaEvent_t* e : {&P->ev_fork, &P->ev_near_done, &P->ev_far_done})
-            HFMM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+        HFMM_TRY(ensure_stream(&P->far_st, greatest));
+        HFMM_TRY(ensure_stream(&P->near_st, least));
+        for (cudaEvent_t* e : {&P->ev_fork, &P->ev_near_done, &P->ev_far_done}) HFMM_TRY(ensure_event(e));
     }
     HFMM_CUDA_TRY(cudaEventRecord(P->ev_fork, st));
     HFMM_CUDA_TRY(cudaStreamWaitEvent(P->far_st, P->ev_fork, 0));

@@ -539,6 +539,8 @@ hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, bool conj_out, cf* 
 hfmm_status launch_direct32(hfmm_plan_s* P, int nrhs, cudaStream_t st);
 // forks P->near_st (low priority) and P->far_st (high priority) from st
 hfmm_status fork_near_far(hfmm_plan_s* P, cudaStream_t st);
+hfmm_status ensure_stream(cudaStream_t* s, int priority);
+hfmm_status ensure_event(cudaEvent_t* e);
 hfmm_status build_local_coords(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status fill_near_tiles(hfmm_plan_s* P, int64_t nchunks, int64_t total_rows, cudaStream_t st);
 // p2p_tc.cu

@@ -1431,10 +1431,10 @@ hfmm_status apply_small(hfmm_plan_s* P, int nrhs, int parts, bool conj_out, cf* 
         HFMM_TRY(small_near_sums(P, nrhs, true, direct, P->near_st));
         tn.end(HFMM_STAGE_P2P);
         HFMM_CUDA_TRY(cudaEventRecord(P->ev_near_done, P->near_st));
-        if (P->ev_react.empty()) {
-            P->ev_react.assign(L + 1, nullptr);
-            for (cudaEvent_t& e : P->ev_react) HFMM_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-            HFMM_CUDA_TRY(cudaEventCreateWithFlags(&P->ev_up_done, cudaEventDisableTiming));
+        if (!P->ev_up_done) {                              // the last of them, as in fork_near_far
+            P->ev_react.resize(L + 1, nullptr);
+            for (cudaEvent_t& e : P->ev_react) HFMM_TRY(ensure_event(&e));
+            HFMM_TRY(ensure_event(&P->ev_up_done));
         }
         fs = P->far_st;
     }

@@ -406,7 +406,9 @@ hfmm_status gmres(hfmm_plan_s* P, zc sigma, const T* b, T* x, double tol, int m,
     if (!P->krylov_host || P->krylov_host_words < (size_t)m + 2) {
         if (P->krylov_host) cudaFreeHost(P->krylov_host);
         P->krylov_host = nullptr;
-        HFMM_CUDA_TRY(cudaMallocHost((void**)&P->krylov_host, sizeof(double2) * ((size_t)m + 2)));
+        double2* made = nullptr;
+        HFMM_CUDA_TRY(cudaMallocHost((void**)&made, sizeof(double2) * ((size_t)m + 2)));
+        P->krylov_host = made;
         P->krylov_host_words = (size_t)m + 2;
     }
     double2* small = P->krylov_part;
