@@ -340,7 +340,7 @@ static hfmm_status leaves64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
                                                      lv.h, P->L, P->k, lv.p, chunk, lv.mult);
         ++P->launches;
         HFMM_CUDA_TRY(cudaGetLastError());
-        if (P->s6_ready[0]) HFMM_TRY(split_exponent(P, 0, P->L, false, nrhs, st));
+        if (P->s6_ready[0]) HFMM_TRY(split_exponent(P, P->L, false, nrhs, st));
     }
     if (P->s6_ready[0]) HFMM_TRY(split_slice(P, 0, P->L, false, nrhs, st));
     if (lv.diag_logq) HFMM_TRY(diag_src(P, P->L, nrhs, st));
@@ -387,7 +387,7 @@ static hfmm_status downward64(hfmm_plan_s* P, int nrhs, int parts, cudaStream_t 
         }
         if (dg) {
             HFMM_TRY(diag_m2l(P, l, nrhs, parts, st));
-            if (P->s6_ready[0] && l < L) HFMM_TRY(split_exponent(P, 0, l, true, nrhs, st));
+            if (P->s6_ready[0] && l < L) HFMM_TRY(split_exponent(P, l, true, nrhs, st));
         }
         if (P->s6_ready[0] && l < L) HFMM_TRY(split_slice(P, 0, l, true, nrhs, st));
     }
@@ -949,31 +949,33 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
     return HFMM_OK;
 }
 
-// Offsets of the near-field blocks (every target leaf's U-list pairs) on
-// the device, once per plan; returns the number of pairs in *pairs.
-hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, bool alloc, cudaStream_t st) {
-    const int L = P->L;
-    const int64_t nleaf = P->lev[L].nbox;
+// Points of leaf b's U list (the 3 x 3 neighbourhood of a uniform tree).
+int64_t u_list_points(const hfmm_plan_s* P, int64_t b) {
     const auto& lb = P->h_leaf_begin;
-    const int m = 1 << L;
+    const int m = 1 << P->L, ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
+    int64_t ns = 0;
+    for (int dy = -1; dy <= 1; ++dy)
+        for (int dx = -1; dx <= 1; ++dx) {
+            const int sx = ix + dx, sy = iy + dy;
+            if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
+            const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
+            ns += lb[s + 1] - lb[s];
+        }
+    return ns;
+}
+
+// Number of the near-field blocks' pairs (every target leaf's U list), and where that is at most max_pairs the
+// blocks' offsets on the device, once per plan.
+hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, double max_pairs, cudaStream_t st) {
+    const int64_t nleaf = P->lev[P->L].nbox;
+    const auto& lb = P->h_leaf_begin;
     std::vector<int64_t> off(nleaf + 1, 0);
     for (int64_t b = 0; b < nleaf; ++b) {
         const int64_t tn = lb[b + 1] - lb[b];
-        int64_t ns = 0;
-        if (tn > 0) {
-            const int ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int sx = ix + dx, sy = iy + dy;
-                    if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
-                    const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
-                    ns += lb[s + 1] - lb[s];
-                }
-        }
-        off[b + 1] = off[b] + tn * ns;
+        off[b + 1] = off[b] + (tn > 0 ? tn * u_list_points(P, b) : 0);
     }
     *pairs = off[nleaf];
-    if (alloc && !P->near64_off) {
+    if ((double)*pairs <= max_pairs && !P->near64_off) {
         HFMM_TRY(plan_alloc(P, (void**)&P->near64_off, sizeof(int64_t) * (nleaf + 1)));
         HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_off, off.data(), sizeof(int64_t) * (nleaf + 1),
                                       cudaMemcpyHostToDevice, st));
@@ -986,9 +988,8 @@ hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, bool alloc, cudaStrea
 // (skipped above the byte budget: the gradient then evaluates H1 per pair).
 hfmm_status build_near64_grad(hfmm_plan_s* P, cudaStream_t st) {
     int64_t pairs = 0;
-    HFMM_TRY(near64_offsets(P, &pairs, false, st));
+    HFMM_TRY(near64_offsets(P, &pairs, NEAR64_MAX_BYTES / 32.0, st));
     if (32.0 * (double)pairs > NEAR64_MAX_BYTES) return HFMM_OK;
-    HFMM_TRY(near64_offsets(P, &pairs, true, st));
     HFMM_TRY(plan_alloc(P, (void**)&P->near64g_x, sizeof(cd) * std::max<int64_t>(pairs, 1)));
     HFMM_TRY(plan_alloc(P, (void**)&P->near64g_y, sizeof(cd) * std::max<int64_t>(pairs, 1)));
     near64_grad_fill_kernel<<<dim3((unsigned)P->lev[P->L].nbox, GFILL_PARTS), 128, 0, st>>>(P->leaf_begin, P->L, P->xy_sorted, P->k,
@@ -1000,38 +1001,18 @@ hfmm_status build_near64_grad(hfmm_plan_s* P, cudaStream_t st) {
 // Plan-time near-field blocks of an FP64 plan (skipped above the byte budget:
 // the apply then evaluates H0 per pair).
 hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st) {
-    const int L = P->L;
-    const int64_t nleaf = P->lev[L].nbox;
-    const auto& lb = P->h_leaf_begin;
-    const int m = 1 << L;
-    std::vector<int64_t> off(nleaf + 1, 0);
-    for (int64_t b = 0; b < nleaf; ++b) {
-        const int64_t tn = lb[b + 1] - lb[b];
-        int64_t ns = 0;
-        if (tn > 0) {
-            const int ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int sx = ix + dx, sy = iy + dy;
-                    if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
-                    const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
-                    ns += lb[s + 1] - lb[s];
-                }
-        }
-        off[b + 1] = off[b] + tn * ns;
-    }
-    const double bytes = 16.0 * (double)off[nleaf];
+    int64_t pairs = 0;
+    HFMM_TRY(near64_offsets(P, &pairs, NEAR64_MAX_BYTES / 16.0, st));
+    const double bytes = 16.0 * (double)pairs;
     if (bytes > NEAR64_MAX_BYTES) return HFMM_OK;
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_off, sizeof(int64_t) * (nleaf + 1)));
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_vals, sizeof(cd) * std::max<int64_t>(off[nleaf], 1)));
-    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_off, off.data(), sizeof(int64_t) * (nleaf + 1), cudaMemcpyHostToDevice, st));
-    near64_fill_kernel<<<(unsigned)nleaf, 128, 0, st>>>(P->leaf_begin, L, P->xy_sorted, P->k, P->near64_off,
-                                                        P->near64_vals);
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_vals, sizeof(cd) * std::max<int64_t>(pairs, 1)));
+    near64_fill_kernel<<<(unsigned)P->lev[P->L].nbox, 128, 0, st>>>(P->leaf_begin, P->L, P->xy_sorted, P->k, P->near64_off,
+                                                                    P->near64_vals);
     HFMM_CUDA_TRY(cudaGetLastError());
     P->table_bytes += bytes;
     HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, 4 * sizeof(int)));
     bool fixed = true;
-    HFMM_TRY(near64_to_fixed(P->near64_vals, off[nleaf], P->near64_E, &P->near64_infinite, &fixed, st));
+    HFMM_TRY(near64_to_fixed(P->near64_vals, pairs, P->near64_E, &P->near64_infinite, &fixed, st));
     if (!fixed) P->near64_vals = nullptr;
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));
     return HFMM_OK;

@@ -762,7 +762,7 @@ hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
     if (P->leaf64 || P->ad) return HFMM_OK;
     const int L = P->L;
     const LevelInfo& lv = P->lev[L];
-    const int nb = lv.p + 2, m = 1 << L;
+    const int nb = lv.p + 2;
     const double bytes = sizeof(cd) * (double)P->n * nb;
     const bool has_basis = bytes <= BASIS64_MAX_BYTES && nb * (int)sizeof(double) <= 40000 && optional_fits(bytes);
     const auto& lb = P->h_leaf_begin;
@@ -783,15 +783,7 @@ hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
     for (int64_t b = 0; b < lv.nbox; ++b) {
         const int32_t tn = lb[b + 1] - lb[b];
         if (tn == 0) continue;
-        const int ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
-        int64_t ns = 0;
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int sx = ix + dx, sy = iy + dy;
-                if (sx < 0 || sy < 0 || sx >= m || sy >= m) continue;
-                const uint32_t s = morton((uint32_t)sx, (uint32_t)sy);
-                ns += lb[s + 1] - lb[s];
-            }
+        const int64_t ns = u_list_points(P, b);
         Leaf64Rec R{};
         R.tlo = lb[b]; R.tn = tn; R.ns = (int32_t)ns; R.p = lv.p; R.nb = nb;
         R.soff = soff; R.goff = goff; R.boff = (int64_t)lb[b] * nb; R.lidx = b;

@@ -93,9 +93,9 @@ constexpr int TC_MAX_NP = 128;         // widest column block (one 128-column TM
 constexpr int TC_RUN_LEVELS = 2;       // finest levels with level-wide scales (the leaves and the level above)
 
 // Shared memory of the leaf L2P in the downward epilogue, per drain warp: its
-// 32 rows of beta~ (stride NB + 1) and two buffers of the basis rows of 8
-// points and its rows of y for them (the next pass's data arrive while this
-// pass computes); used only where the four warps' regions fit the ring.
+// 32 rows of beta~ (stride NB + 1) and two buffers of the basis rows of four or
+// eight points and its rows of y for them (the next pass's data arrive while this
+// pass computes); the four warps' regions lie in the ring.
 template <int NB>
 struct TcL2p {
     // Four points a pass wherever eight do not fit the ring: else such leaves take a separate L2P
@@ -105,22 +105,8 @@ struct TcL2p {
     static constexpr int pts = NB <= 32 || NB == 112 ? 8 : 4;
     static constexpr int buf = pts * (NB / 2) * 8 + pts * 32 * 8;
     static constexpr int warp_bytes = 32 * (NB + 1) * 4 + 2 * buf;
-    static constexpr bool fits = 4 * warp_bytes <= TcCfg<NB>::area;
+    static_assert(4 * warp_bytes <= TcCfg<NB>::area, "the four warps' regions fit the ring");
 };
-
-bool tc_l2p_fits(int nbw) {
-    switch (nbw) {
-        case 16: return TcL2p<16>::fits;
-        case 32: return TcL2p<32>::fits;
-        case 48: return TcL2p<48>::fits;
-        case 64: return TcL2p<64>::fits;
-        case 80: return TcL2p<80>::fits;
-        case 96: return TcL2p<96>::fits;
-        case 112: return TcL2p<112>::fits;
-        case 128: return TcL2p<128>::fits;
-    }
-    return false;
-}
 
 struct TcTile { int32_t b0, b1, s0, s1; };          // boxes (-1: empty), step range
 // kind 0 free M2L, 1 reaction M2L, 2 secondary source (L2L parent or M2M child);
@@ -424,20 +410,20 @@ __global__ void __launch_bounds__(TC2_THREADS, TcCfg<NB>::ctas) m2l_tc_kernel(
             const int box = tgt ? tile.b1 : tile.b0;   // uniform over the warp
             if (box >= 0) {
                 tc_store_row<NB>(acc, box, row, rc, cb, nbz, n0, nrhs, nc, nrc, nullptr, sdst, ssc, kcd, qmax, qgain);
-                if ((TcL2p<NB>::fits && l2p_basis) || out) {
+                if (l2p_basis || out) {
                     // The warp's 32 rows of the result go to the ring once (every MMA of
                     // this CTA has completed; one region per warp); the leaf L2P and the
                     // FP32 store read them from there.
-                    constexpr int WS = TcL2p<NB>::fits ? TcL2p<NB>::warp_bytes : 32 * (NB + 1) * 4;
+                    constexpr int WS = TcL2p<NB>::warp_bytes;
                     static_assert(4 * WS <= CFG::area, "staging fits the ring");
                     float* bet = (float*)(smem + warp * WS);
 #pragma unroll
                     for (int j = 0; j < NB; ++j) bet[lane * (NB + 1) + j] = acc[j];
                     __syncwarp();
-                    if (TcL2p<NB>::fits && l2p_basis) {
+                    if (l2p_basis) {
                         // L2P of the leaf (Algorithm 1, step 4), one column block:
                         // y[t][r] += sum_m beta~[r][m] (i/4) conj(B[t][m]) over the leaf's
-                        // points t, eight points per pass.  The basis rows and this
+                        // points t, four or eight points per pass.  The basis rows and this
                         // warp's rows of y of the next pass are copied (cp.async, second
                         // buffer) while this pass computes; the sum reads beta~ by row and
                         // the basis as broadcasts (each beta~ load feeds 32 FMAs).
@@ -1066,7 +1052,7 @@ hfmm_status build_tc(hfmm_plan_s* P, cudaStream_t st) {
     // leaf row (one column block, no step split) and its staging fits the ring
     {
         const LevelInfo& lf = P->lev[L];
-        P->tc_l2p = lf.tc_nb == 1 && tc_nseg(lf.tc_ntiles, 1, nrc, lf.tc_maxsteps) == 1 && tc_l2p_fits(lf.tc_nbw);
+        P->tc_l2p = lf.tc_nb == 1 && tc_nseg(lf.tc_ntiles, 1, nrc, lf.tc_maxsteps) == 1;
     }
     HFMM_TRY(plan_alloc(P, (void**)&P->tc_err, sizeof(int)));
     HFMM_CUDA_TRY(cudaMemsetAsync(P->tc_err, 0, sizeof(int), st));

@@ -434,7 +434,8 @@ hfmm_status apply_grad_fp64(hfmm_plan_s* P, int nrhs, const cd* q, const cd* g, 
 // fmm64.cu
 constexpr double NEAR64_MAX_BYTES = 32e9;   // plan-time FP64 near-field blocks up to this size
 constexpr double NEAR32_MAX_BYTES = 8e9;    // plan-time FP32 blocks of few-RHS mixed plans
-hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, bool alloc, cudaStream_t st);
+hfmm_status near64_offsets(hfmm_plan_s* P, int64_t* pairs, double max_pairs, cudaStream_t st);
+int64_t u_list_points(const hfmm_plan_s* P, int64_t b);
 hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status build_diag(hfmm_plan_s* P, cudaStream_t st);
 hfmm_status build_adaptive_tree(hfmm_plan_s* P, const double* d_xy, int leaf_size, cudaStream_t st);
@@ -456,7 +457,7 @@ double diag_flops(const hfmm_plan_s* P, int l, int nrhs, int parts);
 hfmm_status build_split(hfmm_plan_s* P, int w, cudaStream_t st);
 void split_forget(hfmm_plan_s* P, int w);
 hfmm_status split_begin(hfmm_plan_s* P, int w, cudaStream_t st);
-hfmm_status split_exponent(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st);
+hfmm_status split_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st);
 hfmm_status split_slice(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st);
 hfmm_status split_m2m(hfmm_plan_s* P, int w, int l, int nrhs, cudaStream_t st);
 hfmm_status split_down(hfmm_plan_s* P, int w, int l, int nrhs, int parts, cudaStream_t st);

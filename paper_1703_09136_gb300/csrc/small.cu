@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(NW * 32) down_small_kernel(
     const int nr0 = ((parts & HFMM_PART_FAR_REACT) && r_begin) ? r_begin[b] : 0;
     const int nr1 = ((parts & HFMM_PART_FAR_REACT) && r_begin) ? r_begin[b + 1] : 0;
     const int nsrc = (has_parent ? 1 : 0) + (nv1 - nv0) + (nr1 - nr0);
-    if (react_add && nsrc == 0) return;        // uniform over the CTA
+    if (react_add && nsrc == 0) return;        // uniform over the CTA (launched without an early start)
     pdl_wait();
     for (int r0 = 0; r0 < nrhs; r0 += R) {
         const int rows = min(R, nrhs - r0);
@@ -699,21 +699,18 @@ __global__ void __launch_bounds__(128) l2p_scatter_kernel(const int32_t* __restr
 }
 
 // ---------------------------------------------------------------------------
-// Near field and the leaves' local expansions: warp per target leaf, lane =
-// target point (passes of 32), sources of the 3 x 3 neighbourhood in order.
+// Near field without stored blocks: warp per target leaf, lane = target point
+// (passes of 32), sources of the 3 x 3 neighbourhood in order.
 // ---------------------------------------------------------------------------
 template <int R>
 __global__ void __launch_bounds__(128) near_small_kernel(const int32_t* __restrict__ lb, int L, int64_t nleaf,
                                                          const float2* __restrict__ xl, const cf* __restrict__ qs,
-                                                         int nrhs, float k, float h, int near,
-                                                         const cf* __restrict__ loc, const cf* __restrict__ basis,
-                                                         int nc, cf* __restrict__ ys) {
+                                                         int nrhs, float k, float h, cf* __restrict__ ys) {
     __shared__ float tj[H0N][H0D + 1], tr[H0N][H0D + 1];
-    if (near)   // an L2P-only pass needs no table
-        for (int e = threadIdx.x; e < H0N * (H0D + 1); e += blockDim.x) {
-            tj[e / (H0D + 1)][e % (H0D + 1)] = g_h0[0][e / (H0D + 1)][e % (H0D + 1)];
-            tr[e / (H0D + 1)][e % (H0D + 1)] = g_h0[1][e / (H0D + 1)][e % (H0D + 1)];
-        }
+    for (int e = threadIdx.x; e < H0N * (H0D + 1); e += blockDim.x) {
+        tj[e / (H0D + 1)][e % (H0D + 1)] = g_h0[0][e / (H0D + 1)][e % (H0D + 1)];
+        tr[e / (H0D + 1)][e % (H0D + 1)] = g_h0[1][e / (H0D + 1)][e % (H0D + 1)];
+    }
     __syncthreads();
     const int64_t b = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     if (b >= nleaf) return;
@@ -722,10 +719,10 @@ __global__ void __launch_bounds__(128) near_small_kernel(const int32_t* __restri
     if (thi <= tlo) return;
     const int ix = (int)morton_x((uint32_t)b), iy = (int)morton_y((uint32_t)b);
     const int mside = 1 << L;
-    // leaves of at most 16 points: the two half-warps take alternate sources
-    // (and alternate L2P coefficients) of the same 16 targets, then add
+    // leaves of at most 16 points: the two half-warps take alternate sources of
+    // the same 16 targets, then add
     const bool split = thi - tlo <= 16;
-    const int half = split ? lane >> 4 : 0, nper = split ? 2 : 4, mstep = split ? 2 : 1;
+    const int half = split ? lane >> 4 : 0, nper = split ? 2 : 4;
     for (int r0 = 0; r0 < nrhs; r0 += R) {
         for (int32_t t0 = tlo; t0 < thi; t0 += 32) {
             const int32_t t = t0 + (split ? lane & 15 : lane);
@@ -734,7 +731,7 @@ __global__ void __launch_bounds__(128) near_small_kernel(const int32_t* __restri
             cf acc[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = cfmk(0.f, 0.f);
-            for (int dy = -1; dy <= 1 && near; ++dy)
+            for (int dy = -1; dy <= 1; ++dy)
                 for (int dx = -1; dx <= 1; ++dx) {
                     const int sx = ix + dx, sy = iy + dy;
                     if (sx < 0 || sy < 0 || sx >= mside || sy >= mside) continue;
@@ -775,19 +772,6 @@ __global__ void __launch_bounds__(128) near_small_kernel(const int32_t* __restri
                         }
                     }
                 }
-            if (loc) {
-                // L2P: (i/4) sum_m b~[r][m] conj(B[t][m])
-#pragma unroll 4
-                for (int m = half; m < nc; m += mstep) {
-                    const cf B = live ? basis[(int64_t)t * nc + m] : cfmk(0.f, 0.f);
-                    const cf g = cfmk(0.25f * B.y, 0.25f * B.x);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const cf bt = r0 + r < nrhs ? loc[((int64_t)b * nrhs + r0 + r) * nc + m] : cfmk(0.f, 0.f);
-                        cfma(acc[r], g, bt);
-                    }
-                }
-            }
             if (split) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
@@ -1154,8 +1138,7 @@ size_t smem_bytes(int R, int U, int ncs_max) {
 }
 
 template <int R, int U>
-hfmm_status launch_down_ru(hfmm_plan_s* P, int l, int nrhs, int parts, int nchunk, int ncs_max, bool react_add,
-                           cudaStream_t st) {
+hfmm_status launch_down_ru(hfmm_plan_s* P, int l, int nrhs, int parts, int nchunk, int ncs_max, cudaStream_t st) {
     LevelInfo& lv = P->lev[l];
     const bool has_parent = l > P->lmin;
     const size_t sm = smem_bytes(R, U, ncs_max);
@@ -1166,7 +1149,7 @@ hfmm_status launch_down_ru(hfmm_plan_s* P, int l, int nrhs, int parts, int nchun
         has_parent ? P->lev[l - 1].p : 0, has_parent ? P->lev[l - 1].loc32 : nullptr,
         has_parent ? P->lev[l - 1].t_l2l32 : nullptr, lv.mult32, lv.nv ? lv.v_begin : nullptr, lv.v_src, lv.v_off,
         lv.t_free32, lv.nr ? lv.r_begin : nullptr, lv.r_src, lv.r_tab, lv.t_react32, parts, nchunk, ncs_max, lv.loc32,
-        react_add, nullptr));
+        false, nullptr));
     return HFMM_OK;
 }
 
@@ -1220,9 +1203,8 @@ hfmm_status build_near_small(hfmm_plan_s* P, cudaStream_t st) {
     const LevelInfo& lv = P->lev[P->L];
     if (P->max_rhs > P->small_rhs || P->ad || (P->flags & HFMM_FLAG_SIMT_M2L)) return HFMM_OK;
     int64_t pairs = 0;
-    HFMM_TRY(near64_offsets(P, &pairs, false, st));
+    HFMM_TRY(near64_offsets(P, &pairs, NEAR32_MAX_BYTES / sizeof(cf), st));
     if (sizeof(cf) * (double)pairs > NEAR32_MAX_BYTES || !optional_fits(sizeof(cf) * (double)pairs)) return HFMM_OK;
-    HFMM_TRY(near64_offsets(P, &pairs, true, st));
     HFMM_TRY(plan_optional(P, [&] { return plan_alloc(P, (void**)&P->near32_vals,
                                                       sizeof(cf) * (size_t)std::max<int64_t>(pairs, 1)); },
                            [&] { P->near32_vals = nullptr; }));
@@ -1365,18 +1347,17 @@ hfmm_status small_down(hfmm_plan_s* P, int l, int nrhs, int parts, bool react_do
             return HFMM_OK;
         }
     }
-    HFMM_SMALL_DISPATCH(launch_down_ru, P, l, nrhs, parts, nchunk, ncs_max, false, st)
+    HFMM_SMALL_DISPATCH(launch_down_ru, P, l, nrhs, parts, nchunk, ncs_max, st)
     hfmm_set_error("small downward pass: no kernel for R=%d U=%d", R, U);
     return HFMM_ERR_UNSUPPORTED;
 }
 
-hfmm_status small_near(hfmm_plan_s* P, int nrhs, bool near, bool l2p, cudaStream_t st) {
+hfmm_status small_near(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
     LevelInfo& lv = P->lev[P->L];
     const unsigned grid = (unsigned)ceil_div(lv.nbox, 4);
-    const cf* loc = l2p ? lv.loc32 : nullptr;
 #define HFMM_NEAR(RR)                                                                                            \
     near_small_kernel<RR><<<grid, 128, 0, st>>>(P->leaf_begin, P->L, lv.nbox, P->xl32, P->q32, nrhs, (float)P->k, \
-                                                (float)lv.h, near ? 1 : 0, loc, P->basis32, lv.ncoef, P->y32)
+                                                (float)lv.h, P->y32)
     if (nrhs >= 8) HFMM_NEAR(8);
     else if (nrhs >= 4) HFMM_NEAR(4);
     else if (nrhs >= 2) HFMM_NEAR(2);
@@ -1403,7 +1384,7 @@ static hfmm_status small_near_sums(hfmm_plan_s* P, int nrhs, bool near, bool dir
     } else {
         HFMM_CUDA_TRY(cudaMemsetAsync(P->y32, 0, sizeof(cf) * P->n * nrhs, st));
         if (near) {
-            HFMM_TRY(small_near(P, nrhs, true, false, st));
+            HFMM_TRY(small_near(P, nrhs, st));
             ++P->launches;
         }
     }

@@ -149,10 +149,9 @@ __global__ void s6_op_slice_kernel(S6Op o, const int* __restrict__ Ep, uint4* __
 // ---------------------------------------------------------------------------
 // level exponents of expansions written by other kernels
 // ---------------------------------------------------------------------------
-// Boxes without points (lb: the leaf ranges of a uniform tree, null: every box has some) are left out: nobody
+// Boxes without points (lb: the leaf ranges) are left out: nobody
 // writes their locals, so their memory holds what the allocator or a call of another width left there.
-template <class C>
-__global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nrhs, int p, const int32_t* __restrict__ lb,
+__global__ void s6_exponent_kernel(const cd* __restrict__ a, int64_t nbox, int nrhs, int p, const int32_t* __restrict__ lb,
                                    int L, int l, const int* __restrict__ sx, int sign, int* __restrict__ E) {
     pdl_start_next();
     const int nc = 2 * p + 1, r = blockIdx.y;
@@ -162,13 +161,11 @@ __global__ void s6_exponent_kernel(const C* __restrict__ a, int64_t nbox, int nr
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / nc;
         const int m = (int)(i % nc) - p;
-        if (lb) {
-            int32_t lo, hi;
-            box_range(lb, L, l, b, &lo, &hi);
-            if (hi <= lo) continue;
-        }
-        const C v = __ldcg(a + (b * nrhs + r) * nc + m + p);
-        const int sh = sx ? sign * sx[abs(m)] : 0;
+        int32_t lo, hi;
+        box_range(lb, L, l, b, &lo, &hi);
+        if (hi <= lo) continue;
+        const cd v = __ldcg(a + (b * nrhs + r) * nc + m + p);
+        const int sh = sign * sx[abs(m)];
         e = max(e, max(s6_exponent(v.x, sh), s6_exponent(v.y, sh)));
     }
     e = __reduce_max_sync(0xffffffffu, e);
@@ -630,7 +627,7 @@ hfmm_status s6_launch(const S6Args& A, int tiles, int steps, cudaStream_t st) {
 template <int D>
 hfmm_status s6_run(S6Args& A, cudaStream_t st) {
     if (A.tiles == 0 && A.mode == 2) return HFMM_OK;
-    if (A.mode == 2) return s6_launch<1, D>(A, A.tiles, 28, st);
+    if (D == 3 || A.mode == 2) return s6_launch<1, D>(A, A.tiles, 28, st);     // FP32 digits: adaptive trees alone
     const int64_t n = (int64_t)1 << A.l;
     const int MT = (2 * (2 * A.p + 1) + 15) / 16, gy = (MT + S6_MAXW - 1) / S6_MAXW;
     auto tiles = [&](int nc) -> int64_t {
@@ -641,7 +638,7 @@ hfmm_status s6_run(S6Args& A, cudaStream_t st) {
     const int steps = A.mode == 0 ? 4 : 1 + (A.vlist ? 27 : 0) + (A.rlist ? (int)std::min<int64_t>(n, 1 << 20) : 0);
     const bool wide = (A.mode == 0 || (n >> 1) > 8) && tiles(16) * gy >= 3 * 152;
     A.tiles = (int)tiles(wide ? 16 : 8);
-    return wide ? s6_launch<2, D>(A, A.tiles, steps, st) : s6_launch<1, D>(A, A.tiles, steps, st);
+    return wide ? s6_launch<2, 6>(A, A.tiles, steps, st) : s6_launch<1, D>(A, A.tiles, steps, st);
 }
 
 S6Fam s6_fam(const unsigned* dig, int p, const uint4* ops, const int* Eop, const int* Esrc) {
@@ -847,18 +844,6 @@ hfmm_status s6_down(hfmm_plan_s* P, int l, int nrhs, int parts, cudaStream_t st)
 }
 
 template <int D>
-hfmm_status s6_exponent_of(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
-    LevelInfo& lv = P->lev[l];
-    const int64_t total = lv.nbox * lv.ncoef;
-    HFMM_CUDA_TRY(pdl_launch(s6_exponent_kernel<typename S6Traits<D>::C>,
-                             dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs), dim3(256), 0, st, 0,
-                             s6_expansion<D>(lv, loc), lv.nbox, nrhs, lv.p, P->ad ? nullptr : P->leaf_begin, P->L, l,
-                             s6_lev<D>(lv).sx, loc ? 1 : -1, split_exp(P, D == 6 ? 0 : 1, l, loc)));
-    ++P->launches;
-    return HFMM_OK;
-}
-
-template <int D>
 hfmm_status s6_slice(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
     LevelInfo& lv = P->lev[l];
     const S6Lev& s = s6_lev<D>(lv);
@@ -897,9 +882,15 @@ int* split_exp(hfmm_plan_s* P, int w, int l, bool loc) {
     return P->s6_E[w] + ((size_t)(loc ? P->L + 1 : 0) + l) * P->max_rhs;
 }
 
-// Exponents of a level's expansions that another kernel wrote.
-hfmm_status split_exponent(hfmm_plan_s* P, int w, int l, bool loc, int nrhs, cudaStream_t st) {
-    return w ? s6_exponent_of<3>(P, l, loc, nrhs, st) : s6_exponent_of<6>(P, l, loc, nrhs, st);
+// Exponents of a level's FP64 expansions that another kernel wrote (uniform trees).
+hfmm_status split_exponent(hfmm_plan_s* P, int l, bool loc, int nrhs, cudaStream_t st) {
+    LevelInfo& lv = P->lev[l];
+    const int64_t total = lv.nbox * lv.ncoef;
+    HFMM_CUDA_TRY(pdl_launch(s6_exponent_kernel, dim3((unsigned)std::min<int64_t>((total + 255) / 256, 8 * 152), nrhs),
+                             dim3(256), 0, st, 0, s6_expansion<6>(lv, loc), lv.nbox, nrhs, lv.p, P->leaf_begin, P->L, l,
+                             lv.s6[0].sx, loc ? 1 : -1, split_exp(P, 0, l, loc)));
+    ++P->launches;
+    return HFMM_OK;
 }
 
 // Digits of a level's finished expansions, for the products that read them.
