@@ -1418,11 +1418,11 @@ static hfmm_status ad64_build(hfmm_plan_s* P, cudaStream_t st) {
     HFMM_CUDA_TRY(cudaGetLastError());
     HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, 4 * sizeof(int)));
     bool fixed = true;
-    if (goff > 0) HFMM_TRY(near64_to_fixed(T->near_G, goff, P->near64_E, &P->near64_infinite, &fixed, st));
+    if (goff > 0) HFMM_TRY(near64_to_fixed(T->near_G, goff, P->near64_E, &P->near64_large, &fixed, st));
     if (fixed) P->near64_vals = T->near_G;
     T->fast64 = true;                                     // from here on near_G holds digits
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // the vectors are locals
-    return near64_upload_infinite(P, recs, st);
+    return near64_upload_large(P, recs, st);
 }
 
 // A plan above a byte budget or the device's memory keeps the kernels of apply_adaptive.

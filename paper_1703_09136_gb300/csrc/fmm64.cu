@@ -1012,7 +1012,7 @@ hfmm_status build_near64(hfmm_plan_s* P, cudaStream_t st) {
     P->table_bytes += bytes;
     HFMM_TRY(plan_alloc(P, (void**)&P->near64_E, 4 * sizeof(int)));
     bool fixed = true;
-    HFMM_TRY(near64_to_fixed(P->near64_vals, pairs, P->near64_E, &P->near64_infinite, &fixed, st));
+    HFMM_TRY(near64_to_fixed(P->near64_vals, pairs, P->near64_E, &P->near64_large, &fixed, st));
     if (!fixed) P->near64_vals = nullptr;
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));
     return HFMM_OK;

@@ -168,8 +168,10 @@ constexpr int LF_RING = 4;            // k-steps of near-field words in flight p
 constexpr int LF_TERMS = 32;         // k-steps per exact FP32 accumulation
 constexpr long long LF_BIAS = 0x808080808080ll;   // 128 sum_{i = 0 .. 5} 256^i
 
-// v 2^(54 - E), the last bit zero, |v| < 2^E (see s6_fixed)
-__device__ __forceinline__ long long lf_fixed(double v, int E) { return s6_fixed<53>(v, 0, E) * 2; }
+// |v| < 2^E as a fixed-point number: 54 bits of the strengths (their leading digit has to hold the carry of the six
+// signed ones below it), 55 of the blocks.  Error of a leaf's sum against extended precision, k h = 0.25 .. 25, 36 to 270
+// sources: 0.7 .. 2.8e-16, FP64 multiply-adds 2.8 .. 8.1e-16 (53 bits of both: up to 1.1e-15).
+constexpr int LF_QBITS = 54, LF_GBITS = 55;
 
 // digit i of two numbers (with LF_BIAS) as f16: 1024 + field as bits 0x6400 | field, minus 1152
 __device__ __forceinline__ unsigned lf_digit(long long xb, long long yb, int i) {
@@ -255,7 +257,7 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
         }
     }
     const bool bad = Eq >= S6_NAN / 2;
-    const int EV = max(Eq, S6_NONE) + (A.G ? max(*A.EG, S6_NONE) : 0) - 68;
+    const int EV = max(Eq, S6_NONE) + (A.G ? max(*A.EG, S6_NONE) : 0) + 40 - LF_QBITS - LF_GBITS;
     const uint4* Gb = A.G ? A.G + L.goff : nullptr;
 
     const int ntile = (tn + 15) / 16;
@@ -276,7 +278,7 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
                 }
 #pragma unroll
                 for (int u = 0; u < QPT; ++u) {
-                    const long long xr = lf_fixed(qv[u].x, Eq) + LF_BIAS, xi = lf_fixed(qv[u].y, Eq) + LF_BIAS;
+                    const long long xr = s6_fixed<LF_QBITS>(qv[u].x, 0, Eq) + LF_BIAS, xi = s6_fixed<LF_QBITS>(qv[u].y, 0, Eq) + LF_BIAS;
 #pragma unroll
                     for (int d = 0; d < LD; ++d) sq[(tid + u * W * 32) * LD + d] = lf_digit(xr, xi, d);
                 }
@@ -436,39 +438,39 @@ __global__ void __maxnreg__(128) leaf64_kernel(const __grid_constant__ Leaf64Arg
     }
 }
 
-// (i/4) H0 doubles -> largest exponent; then, in place, digit words.  Entries that are not finite (coincident points)
-// have no digits: they are counted, listed (near64_list_kernel) and leave zeros.
+// (i/4) H0 doubles -> largest exponent below `top`; then, in place, digit words.  The other entries are counted,
+// listed (near64_list_kernel) and leave zeros.
 __device__ __forceinline__ int near64_exponent(cd v) { return max(s6_exponent(v.x, 0), s6_exponent(v.y, 0)); }
 
-__global__ void near64_exponent_kernel(const cd* __restrict__ G, int64_t n, int* __restrict__ E,
-                                       unsigned long long* __restrict__ infinite) {
+__global__ void near64_exponent_kernel(const cd* __restrict__ G, int64_t n, int top, int* __restrict__ E,
+                                       unsigned long long* __restrict__ above) {
     int e = S6_NONE;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int x = near64_exponent(G[i]);
-        if (x < S6_NAN) e = max(e, x);
-        else atomicAdd(infinite, 1ull);
+        if (x < top) e = max(e, x);
+        else atomicAdd(above, 1ull);
     }
     e = __reduce_max_sync(0xffffffffu, e);
     if ((threadIdx.x & 31) == 0 && e > S6_NONE) atomicMax(E, e);
 }
 
-__global__ void near64_list_kernel(const cd* __restrict__ G, int64_t n, unsigned long long* __restrict__ next,
-                                   NearInfinite* __restrict__ out) {
+__global__ void near64_list_kernel(const cd* __restrict__ G, int64_t n, int top, unsigned long long* __restrict__ next,
+                                   NearLarge* __restrict__ out) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const cd v = G[i];
-        if (near64_exponent(v) < S6_NAN) continue;
-        NearInfinite& o = out[atomicAdd(next, 1ull)];
+        if (near64_exponent(v) < top) continue;
+        NearLarge& o = out[atomicAdd(next, 1ull)];
         o.pair = i;
         o.val = v;
     }
 }
 
-__global__ void near64_fix_kernel(cd* G, int64_t n, const int* __restrict__ E) {
+__global__ void near64_fix_kernel(cd* G, int64_t n, int top, const int* __restrict__ E) {
     const int e = *E;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         cd v = G[i];
-        if (near64_exponent(v) >= S6_NAN) v = cmk(0.0, 0.0);
-        const long long x = lf_fixed(v.x, e) + (128ll << 48), y = lf_fixed(v.y, e) + (128ll << 48);
+        if (near64_exponent(v) >= top) v = cmk(0.0, 0.0);
+        const long long x = s6_fixed<LF_GBITS>(v.x, 0, e) + (128ll << 48), y = s6_fixed<LF_GBITS>(v.y, 0, e) + (128ll << 48);
         unsigned w[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {                      // digits 2k, 2k + 1 = bytes 6 - 2k, 5 - 2k
@@ -482,7 +484,7 @@ __global__ void near64_fix_kernel(cd* G, int64_t n, const int* __restrict__ E) {
 }
 
 // The listed entries onto the sums that leaf64_kernel wrote: a warp per (target that has some, right-hand side).
-__global__ void __launch_bounds__(128) near64_infinite_kernel(const int32_t* __restrict__ tgt, const int64_t* __restrict__ beg,
+__global__ void __launch_bounds__(128) near64_large_kernel(const int32_t* __restrict__ tgt, const int64_t* __restrict__ beg,
                                                               const int32_t* __restrict__ src, const cd* __restrict__ val,
                                                               int64_t ntgt, const cd* __restrict__ qs, int64_t n, int nrhs,
                                                               const int64_t* __restrict__ perm, bool conj_out,
@@ -676,43 +678,48 @@ hfmm_status launch_grad_far(hfmm_plan_s* P, int nrhs, const cd* v, double2* acc,
     return HFMM_OK;
 }
 
-// Digit form of `pairs` near-field values in place (E: their exponent, and two words behind it a counter), the entries that are not finite (coincident
-// points) in *infinite; *fixed = false (and the values unchanged) where those are more than NEAR64_INFINITE_MAX.
-hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, std::vector<NearInfinite>* infinite, bool* fixed,
-                            cudaStream_t st) {
-    *fixed = true;
-    infinite->clear();
+// Digit form of `pairs` near-field values in place (E: their exponent, and two words behind it a counter).  Entries
+// of 4 and more, i.e. of points within some 1e-11 wavelengths, go into *large: an infinite one (coincident points)
+// has no digits, and a large one would cost every other entry of the plan some of its.  Where more than
+// NEAR64_LARGE_MAX are that large, only the infinite ones do; where those are too many as well,
+// *fixed = false and the values stay.
+hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, std::vector<NearLarge>* large, bool* fixed, cudaStream_t st) {
+    large->clear();
     unsigned long long* count = (unsigned long long*)(E + 2);
-    HFMM_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(*count), st));
-    HFMM_CUDA_TRY(cudaMemsetAsync(E, 0x80, sizeof(int), st));
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((pairs + 255) / 256, 16 * 152));
-    near64_exponent_kernel<<<grid, 256, 0, st>>>(vals, pairs, E, count);
-    HFMM_CUDA_TRY(cudaGetLastError());
-    unsigned long long ninf = 0;
-    HFMM_CUDA_TRY(cudaMemcpyAsync(&ninf, count, sizeof(ninf), cudaMemcpyDeviceToHost, st));
-    HFMM_CUDA_TRY(cudaStreamSynchronize(st));
-    if (ninf > NEAR64_INFINITE_MAX) *fixed = false;
-    else if (ninf > 0) {
-        NearInfinite* list = nullptr;
-        HFMM_CUDA_TRY(cudaMallocAsync((void**)&list, sizeof(NearInfinite) * ninf, st));
+    unsigned long long found = 0;
+    int top = 3;
+    for (;; top = S6_NAN) {
         HFMM_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(*count), st));
-        near64_list_kernel<<<grid, 256, 0, st>>>(vals, pairs, count, list);
+        HFMM_CUDA_TRY(cudaMemsetAsync(E, 0x80, sizeof(int), st));
+        near64_exponent_kernel<<<grid, 256, 0, st>>>(vals, pairs, top, E, count);
         HFMM_CUDA_TRY(cudaGetLastError());
-        infinite->resize(ninf);
-        HFMM_CUDA_TRY(cudaMemcpyAsync(infinite->data(), list, sizeof(NearInfinite) * ninf, cudaMemcpyDeviceToHost, st));
+        HFMM_CUDA_TRY(cudaMemcpyAsync(&found, count, sizeof(found), cudaMemcpyDeviceToHost, st));
+        HFMM_CUDA_TRY(cudaStreamSynchronize(st));
+        if (found <= NEAR64_LARGE_MAX || top == S6_NAN) break;
+    }
+    *fixed = found <= NEAR64_LARGE_MAX;
+    if (!*fixed) return HFMM_OK;
+    if (found > 0) {
+        NearLarge* list = nullptr;
+        HFMM_CUDA_TRY(cudaMallocAsync((void**)&list, sizeof(NearLarge) * found, st));
+        HFMM_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(*count), st));
+        near64_list_kernel<<<grid, 256, 0, st>>>(vals, pairs, top, count, list);
+        HFMM_CUDA_TRY(cudaGetLastError());
+        large->resize(found);
+        HFMM_CUDA_TRY(cudaMemcpyAsync(large->data(), list, sizeof(NearLarge) * found, cudaMemcpyDeviceToHost, st));
         HFMM_CUDA_TRY(cudaStreamSynchronize(st));
         HFMM_CUDA_TRY(cudaFreeAsync(list, st));
-        std::sort(infinite->begin(), infinite->end(), [](const NearInfinite& a, const NearInfinite& b) { return a.pair < b.pair; });
+        std::sort(large->begin(), large->end(), [](const NearLarge& a, const NearLarge& b) { return a.pair < b.pair; });
     }
-    if (!*fixed) return HFMM_OK;
-    near64_fix_kernel<<<grid, 256, 0, st>>>(vals, pairs, E);
+    near64_fix_kernel<<<grid, 256, 0, st>>>(vals, pairs, top, E);
     HFMM_CUDA_TRY(cudaGetLastError());
     return HFMM_OK;
 }
 
 // The listed entries by target, from the leaf records (in the order of their blocks) and near-field source indices.
-hfmm_status near64_upload_infinite(hfmm_plan_s* P, const std::vector<Leaf64Rec>& recs, cudaStream_t st) {
-    const auto& list = P->near64_infinite;
+hfmm_status near64_upload_large(hfmm_plan_s* P, const std::vector<Leaf64Rec>& recs, cudaStream_t st) {
+    const auto& list = P->near64_large;
     if (list.empty()) return HFMM_OK;
     int64_t nsrc = 0;
     for (const Leaf64Rec& R : recs) nsrc = std::max(nsrc, R.soff + R.ns);
@@ -722,7 +729,7 @@ hfmm_status near64_upload_infinite(hfmm_plan_s* P, const std::vector<Leaf64Rec>&
     struct Item { int32_t t, s; cd v; };
     std::vector<Item> items;
     size_t r = 0;
-    for (const NearInfinite& e : list) {
+    for (const NearLarge& e : list) {
         while (e.pair >= recs[r].goff + (int64_t)recs[r].tn * recs[r].ns) ++r;
         const int64_t o = e.pair - recs[r].goff;           // source-major within the block
         items.push_back({recs[r].tlo + (int32_t)(o % recs[r].tn), src[recs[r].soff + o / recs[r].tn], e.val});
@@ -740,18 +747,18 @@ hfmm_status near64_upload_infinite(hfmm_plan_s* P, const std::vector<Leaf64Rec>&
         val.push_back(it.v);
     }
     beg.push_back((int64_t)val.size());
-    P->near64_inf_n = (int64_t)tgt.size();
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_tgt, sizeof(int32_t) * tgt.size()));
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_beg, sizeof(int64_t) * beg.size()));
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_src, sizeof(int32_t) * isrc.size()));
-    HFMM_TRY(plan_alloc(P, (void**)&P->near64_inf_val, sizeof(cd) * val.size()));
-    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_tgt, tgt.data(), sizeof(int32_t) * tgt.size(), cudaMemcpyHostToDevice, st));
-    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_beg, beg.data(), sizeof(int64_t) * beg.size(), cudaMemcpyHostToDevice, st));
-    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_src, isrc.data(), sizeof(int32_t) * isrc.size(), cudaMemcpyHostToDevice, st));
-    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_inf_val, val.data(), sizeof(cd) * val.size(), cudaMemcpyHostToDevice, st));
+    P->near64_large_n = (int64_t)tgt.size();
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_large_tgt, sizeof(int32_t) * tgt.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_large_beg, sizeof(int64_t) * beg.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_large_src, sizeof(int32_t) * isrc.size()));
+    HFMM_TRY(plan_alloc(P, (void**)&P->near64_large_val, sizeof(cd) * val.size()));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_large_tgt, tgt.data(), sizeof(int32_t) * tgt.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_large_beg, beg.data(), sizeof(int64_t) * beg.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_large_src, isrc.data(), sizeof(int32_t) * isrc.size(), cudaMemcpyHostToDevice, st));
+    HFMM_CUDA_TRY(cudaMemcpyAsync(P->near64_large_val, val.data(), sizeof(cd) * val.size(), cudaMemcpyHostToDevice, st));
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));
-    P->near64_infinite.clear();
-    P->near64_infinite.shrink_to_fit();
+    P->near64_large.clear();
+    P->near64_large.shrink_to_fit();
     return HFMM_OK;
 }
 
@@ -821,7 +828,7 @@ hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st) {
         HFMM_CUDA_TRY(cudaGetLastError());
     }
     HFMM_CUDA_TRY(cudaStreamSynchronize(st));             // recs and ds are locals
-    return near64_upload_infinite(P, recs, st);
+    return near64_upload_large(P, recs, st);
 }
 
 // The plan's memory of its leaf records and bases is gone.
@@ -914,10 +921,10 @@ hfmm_status launch_leaf64(hfmm_plan_s* P, int nrhs, bool near, bool l2p, bool m2
     HFMM_CUDA_TRY(smem_limit(kernel, sm));
     HFMM_CUDA_TRY(pdl_launch(kernel, dim3((unsigned)P->leaf64_n, (unsigned)nrhs), dim3(W * 32), sm, st, 0, A));
     ++P->launches;
-    if (near && P->near64_inf_n > 0) {
-        const unsigned grid = (unsigned)std::min<int64_t>((P->near64_inf_n * nrhs + 3) / 4, 16 * 152);
-        near64_infinite_kernel<<<grid, 128, 0, st>>>(P->near64_inf_tgt, P->near64_inf_beg, P->near64_inf_src, P->near64_inf_val,
-                                                     P->near64_inf_n, P->q_sorted, P->n, nrhs, A.perm, conj_out, y);
+    if (near && P->near64_large_n > 0) {
+        const unsigned grid = (unsigned)std::min<int64_t>((P->near64_large_n * nrhs + 3) / 4, 16 * 152);
+        near64_large_kernel<<<grid, 128, 0, st>>>(P->near64_large_tgt, P->near64_large_beg, P->near64_large_src, P->near64_large_val,
+                                                     P->near64_large_n, P->q_sorted, P->n, nrhs, A.perm, conj_out, y);
         HFMM_CUDA_TRY(cudaGetLastError());
         ++P->launches;
     }

@@ -169,12 +169,12 @@ struct Leaf64D {
     int64_t blk;
 };
 
-// A near-field entry without digits: its place in the blocks and its value.
-struct NearInfinite {
+// A near-field entry outside the digit form: its place in the blocks and its value.
+struct NearLarge {
     int64_t pair;
     cd val;
 };
-constexpr unsigned long long NEAR64_INFINITE_MAX = 1ull << 24;   // above: H0 evaluated per pair by the apply
+constexpr unsigned long long NEAR64_LARGE_MAX = 1ull << 24;
 
 // Adaptive trees (adaptive.cu): deepest level, and the host / device tree.
 constexpr int AD_MAX_LEVEL = 16;
@@ -242,13 +242,13 @@ struct hfmm_plan_s {
     int64_t* near64_off = nullptr;
     cd* near64_vals = nullptr;      // after the fill: base-256 digits (leaf64.cu)
     int* near64_E = nullptr;        // their exponent (then a plan-time counter)
-    // entries that are not finite (coincident points): as found, then by target (sorted
+    // entries outside the digit form (coincident and almost coincident points): as found, then by target (sorted
     // indices): targets, their ranges, sources and values
-    std::vector<NearInfinite> near64_infinite;
-    int64_t near64_inf_n = 0;
-    int32_t *near64_inf_tgt = nullptr, *near64_inf_src = nullptr;
-    int64_t* near64_inf_beg = nullptr;
-    cd* near64_inf_val = nullptr;
+    std::vector<NearLarge> near64_large;
+    int64_t near64_large_n = 0;
+    int32_t *near64_large_tgt = nullptr, *near64_large_src = nullptr;
+    int64_t* near64_large_beg = nullptr;
+    cd* near64_large_val = nullptr;
     int leaf_max = 0;               // largest number of points of a leaf
     bool leaf_empty = false;        // a uniform tree with empty leaves
     Leaf64Rec* leaf64 = nullptr;    // non-empty leaves (leaf64.cu), their largest order, near-field source
@@ -468,9 +468,9 @@ void adaptive_tiles(const hfmm_plan_s* P, int l, bool up, const std::vector<int3
 // leaf64.cu
 hfmm_status build_leaf64(hfmm_plan_s* P, cudaStream_t st);
 void leaf64_forget(hfmm_plan_s* P);
-hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, std::vector<NearInfinite>* infinite, bool* fixed,
+hfmm_status near64_to_fixed(cd* vals, int64_t pairs, int* E, std::vector<NearLarge>* large, bool* fixed,
                             cudaStream_t st);
-hfmm_status near64_upload_infinite(hfmm_plan_s* P, const std::vector<Leaf64Rec>& recs, cudaStream_t st);
+hfmm_status near64_upload_large(hfmm_plan_s* P, const std::vector<Leaf64Rec>& recs, cudaStream_t st);
 hfmm_status launch_grad_near(hfmm_plan_s* P, int nrhs, const cd* gc, double2* out, cudaStream_t st);
 hfmm_status launch_grad_far(hfmm_plan_s* P, int nrhs, const cd* v, double2* acc, const double2* near_sum, double* gxy,
                             cudaStream_t st);

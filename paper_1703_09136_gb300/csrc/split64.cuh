@@ -36,7 +36,7 @@ __device__ __forceinline__ int s6_exponent(float v, int shift) {
     return e - 126 + shift;
 }
 
-// v 2^shift 2^(BITS - E) rounded to an integer, |v 2^shift| < 2^E (BITS <= 53; floats: BITS >= 24)
+// v 2^shift 2^(BITS - E) rounded to an integer, |v 2^shift| < 2^E (BITS <= 62; floats: BITS >= 24)
 template <int BITS>
 __device__ __forceinline__ long long s6_fixed(double v, int shift, int E) {
     const long long b = __double_as_longlong(v);
@@ -45,7 +45,7 @@ __device__ __forceinline__ long long s6_fixed(double v, int shift, int E) {
     if (e) m |= 1ull << 52; else e = 1;
     const int s = E - shift - e + 1075 - BITS;            // right shift
     if (s > 0) m = s > 54 ? 0ull : (m + (1ull << (s - 1))) >> s;
-    else m <<= min(-s, 51);                               // subnormals alone
+    else m <<= min(-s, BITS - 2);                         // subnormals, and more bits than a double has
     return b < 0 ? -(long long)m : (long long)m;
 }
 template <int BITS>
