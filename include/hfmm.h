@@ -76,8 +76,12 @@ typedef enum {
 } hfmm_medium_kind;
 
 typedef enum {
-    HFMM_FP64 = 0,              /* complex128 in/out, FP64 accuracy throughout (translations and
-                                   stored near field as error-free digit products) */
+    HFMM_FP64 = 0,              /* complex128 in/out, FP64 accuracy throughout.  Translations and stored
+                                   near field run as products of base-512 and base-256 digits on
+                                   the tensor cores: fixed-point numbers of 52 to 55 bits with one
+                                   exponent per level (near field: per plan and per leaf's
+                                   sources) and right-hand side, whose rounding measures no
+                                   larger than that of FP64 multiply-adds */
     HFMM_MIXED = 1              /* complex64 in/out, FP32 P2P/P2M/L2P, tensor-core M2L */
 } hfmm_precision;
 

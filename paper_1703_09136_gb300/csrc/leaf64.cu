@@ -517,7 +517,8 @@ __global__ void __launch_bounds__(128) near64_large_kernel(const int32_t* __rest
 // Bound by FP64 FMAs (3.4 M near-field pairs of 40,000 points, one right-hand side: 12 each, 80 us);
 // the pairs run beside both tree passes.  Measured there: near field 2 x 208 us (a lane per target of
 // ten-point leaves) -> 104 us, locals' gradient 2 x 266 us (Bessel sequences evaluated on each
-// call) -> 2 x 27 us; the whole gradient 1578 -> 768 us.
+// call) -> 2 x 27 us; the whole gradient 1578 -> 768 us (804 with order 6
+// of the digit products).
 // ---------------------------------------------------------------------------
 constexpr int GN_TB = 128;
 
@@ -862,8 +863,8 @@ hfmm_status launch_p2m64(hfmm_plan_s* P, int nrhs, cudaStream_t st) {
 
 // Near field and direct reaction into y_sorted on the near stream, beside the far field (whose
 // stream this returns in *fs): they need the strengths alone, and a tree pass leaves SMs idle
-// at its coarse levels (1600 points 138 -> 114 us an apply, two layers, 262,144 points 1528 -> 1461,
-// an adaptive tree of 20,011 points 582 -> 559).
+// at its coarse levels (before order 6 joined the digit products: 1600 points 138 -> 114 us an apply, two
+// layers, 262,144 points 1528 -> 1461, an adaptive tree of 20,011 points 582 -> 559; with it 116, 1578 and 570).
 hfmm_status fork_near64(hfmm_plan_s* P, int nrhs, bool direct, cudaStream_t st, cudaStream_t* fs) {
     HFMM_TRY(fork_near_far(P, st));
     StageTimer tn{P, P->near_st};

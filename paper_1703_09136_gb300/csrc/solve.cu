@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(SV_THREADS) normalise_kernel(const T* __restri
 // the CTAs' sums added in rank order.  For vectors of up to CGS_MAX elements: five kernels took 60 us there
 // (1600 points), each mostly its start and the two latencies of its reduction; sixteen SMs have
 // the FP64 rate for the 16 n (j + 1) FMAs up to a few thousand points.  1600 points, 38 steps a
-// solve: 8.95 -> 8.61 ms.
+// solve: 8.95 -> 8.61 ms (7.8 with the applies of today).
 constexpr int CGS_CTAS = 16, CGS_THREADS = 512, CGS_WARPS = CGS_THREADS / 32;
 constexpr int64_t CGS_MAX = 4096;
 constexpr int CGS_MAX_RESTART = 1024;

@@ -24,7 +24,9 @@
 // every operator entry O(1); the exponent E is one number per level, kind
 // of expansion and right-hand side (largest scaled coefficient, found by the
 // kernel that writes the expansions) and one per operator family.  The stored
-// expansions stay unscaled, so every other kernel reads them as before.  A level
+// expansions stay unscaled, so every other kernel reads them as before.  A coefficient
+// 2^-b of its level's largest keeps 53 - b bits (an operator's entry 52 - b): one strength 1e12
+// times the others leaves every target as near the FP64 kernels' as their own rounding.  A level
 // that holds an infinity or a NaN makes every output of that right-hand side NaN.
 //
 // FP32 (the mixed path's expansions, already scaled by s): three digits hold 26
@@ -35,9 +37,10 @@
 // clocks per SM), mma.sync f16 at 600 TFLOP/s: 26 products leave 23 TFLOP/s.
 // Measured (one GB300, two layers, 262,144 points, one right-hand side): leaf
 // level (order 15, 430k free-space and 49k reaction translations, 3.8 GFLOP)
-// 5.73 -> 0.43 ms, all levels 12.0 -> 1.03 ms, M2M 0.72 -> 0.13 ms; the result
-// differs from the FP64 kernels' by 2e-13 (1e-14 at orders where those cancel
-// less), and both are equally far from the direct sum.
+// 5.73 -> 0.46 ms, all levels 12.0 -> 1.10 ms, M2M 0.72 -> 0.13 ms (launch lists; 0.42,
+// 0.99 and 0.12 ms with the orders 0 .. 5 alone).  The result of
+// dense translations differs from the FP64 kernels' by 5.3e-15, and theirs by 3 to 6e-15 from
+// their own with the strengths times three.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -176,7 +179,7 @@ __global__ void s6_exponent_kernel(const cd* __restrict__ a, int64_t nbox, int n
 // per (box, right-hand side, k-step of eight coefficients, digit) the words
 // [coefficient % 4][coefficient / 4] (32 bytes).  Every source meets up to 27
 // target tiles: cutting it in the product kernel took 60% of that kernel's
-// instructions (leaf level of two layers 0.47 -> 0.34 ms without it).
+// instructions (leaf level of two layers, orders 0 .. 5: 0.47 -> 0.34 ms without it).
 template <int D>
 __global__ void s6_slice_kernel(const typename S6Traits<D>::C* __restrict__ a, int64_t nbox, int nrhs, int p, const int* __restrict__ sx,
                                 int sign, const int* __restrict__ E, unsigned* __restrict__ dig) {
